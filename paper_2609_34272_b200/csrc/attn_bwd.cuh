@@ -37,7 +37,8 @@
 // staying deterministic and needing no counter.  Barrier set-up, the TMEM allocation and the launch latency
 // are paid once; the step pipeline (stage ring, score buffers) runs on across tile boundaries, the stationary
 // tile of the next work item is fetched by its own warp as soon as the last score product of the current one
-// has been issued and completed, and the epilogue of one tile overlaps the first steps of the next.
+// has been issued and completed, and a warpgroup of its own runs the epilogue of one tile during the first steps of the
+// next.
 #pragma once
 #include "sm100_primitives.cuh"
 
@@ -67,6 +68,18 @@ struct BwdCfg {
   static constexpr int kSliceCols = kStepRows / kSlices;
   static constexpr int kCompute = 128 * kWG;                      // compute threads
   static constexpr int kThreads = 128 + kCompute;                 // stage producer, 2 MMA warps, tile loader; compute warpgroups
+  // dQ-side kernel: one more warpgroup, which prepares the next tile's row constants and writes a finished tile out while
+  // the compute warpgroups are already in the next one (before, 512 threads went through three barriers and the epilogue
+  // together at each tile: 1.2-1.8 us at d = 64, 3.4 us at d = 128, with the tensor core idle but for the next tile's first
+  // scores).  Measured, dQ side alone, before -> after: 16 packed documents of 16384 rows, 16 heads, d = 64: 169 -> 152 us;
+  // 96 heads x 1000 x 128, causal: 88 -> 81 us; 16 heads x 4096 x 64, causal (3.5 tiles per CTA): 80.7 -> 79.0 us.
+  // Registers: 768 x 80 at launch.  At d = 128 they are re-dealt 4 x 88 + 48 + 80 (80 for the compute warps spills there:
+  // 4 heads x 16384: 519 us, with 88: 498 us); at d = 64 they stay as they are (re-dealt: 83 instead of 79 us, the step
+  // loop is scheduled differently).
+  static constexpr int kDqEpiWarp = 4 + 4 * kWG, kDqThreads = kThreads + 128;
+  static constexpr bool kDqMoveRegs = (D == 128);
+  static constexpr int kDqRegsCompute = 88, kDqRegsAux = 48, kDqRegsEpi = 80;
+  static_assert(kWG * kDqRegsCompute + kDqRegsAux + kDqRegsEpi <= 6 * 80, "register shares");
   // Output staging for the TMA stores: its own buffer where shared memory allows (d = 64), else over the stationary tile.
   static constexpr bool kSepStaging = (D == 64);
   // TMEM columns: buffer b holds S at 128 b and dP at 128 b + 64; accumulators follow
@@ -77,13 +90,8 @@ struct BwdCfg {
   static constexpr int kDqStages = (D == 64) ? 6 : 4;
   static constexpr int kDqStageBytes = 2 * kStepTileBytes;
   static constexpr int kDqResBufs = (D == 64) ? 2 : 1;             // stationary (Q, dO) buffers
-  // d = 64 (two stationary buffers): D = rowsum(dO o O), LSE and the row-constant tile of a tile are prepared by the
-  // stationary-tile loader's warp as soon as the tile's dO has landed, i.e. while the tile before it still runs; the
-  // compute warps only pick the two values up.  At d = 128 there is one stationary buffer and the compute warps do it at
-  // the tile's start.
-  static constexpr bool kLoaderStats = (D == 64);
-  static constexpr int kDqSmemBytes = kDqResBufs * 2 * kBigTileBytes + kDqStages * kDqStageBytes + (kSepStaging ? 2 * kBigTileBytes : 0) +
-                                      1024;
+  static constexpr int kDqStagingBytes = 4 * 32 * 128;             // each epilogue warp: 32 rows x 64 columns of dQ
+  static constexpr int kDqSmemBytes = kDqResBufs * 2 * kBigTileBytes + kDqStages * kDqStageBytes + kDqStagingBytes + 1024;
   // dK/dV-side kernel: K, V resident; ring of (Q, dO, Z, stats) step tiles
   static constexpr int kDkvStages = (D == 64) ? 5 : 3;
   static constexpr int kDkvStageBytes = 3 * kStepTileBytes + kExtBlockBytes;   // + the step's 64-row block of the row-constant tile
@@ -170,7 +178,7 @@ __device__ __forceinline__ void store_rows_clipped(const uint8_t *stage, int sla
 }
 
 enum BwdWaitCode {
-  kDqWaitQ = 0x21, kDqWaitKV = 0x22, kDqWaitKVEmpty = 0x23, kDqWaitSdP = 0x24, kDqWaitTR = 0x25, kDqWaitAcc = 0x26, kDqWaitBuf = 0x27, kDqWaitResFree = 0x28, kDqWaitAccFree = 0x29,
+  kDqWaitQ = 0x21, kDqWaitKV = 0x22, kDqWaitKVEmpty = 0x23, kDqWaitSdP = 0x24, kDqWaitTR = 0x25, kDqWaitAcc = 0x26, kDqWaitBuf = 0x27, kDqWaitResFree = 0x28, kDqWaitAccFree = 0x29, kDqWaitStats = 0x2a, kDqWaitMass = 0x2b,
   kDkvWaitKV = 0x31, kDkvWaitQ = 0x32, kDkvWaitQEmpty = 0x33, kDkvWaitSdP = 0x34, kDkvWaitTR = 0x35, kDkvWaitAcc = 0x36, kDkvWaitBuf = 0x37, kDkvWaitResFree = 0x38, kDkvWaitAccFree = 0x39
 };
 
@@ -310,20 +318,53 @@ __device__ __forceinline__ void write_row_constants(float *stats, size_t block, 
   *reinterpret_cast<uint4 *>(blk + 128) = make_uint4(n0 | (n1 << 16), n2, 0u, 0u);
 }
 
+// D_i = sum_c dO_ic O_ic from the saved BF16 output, FP32 (Algorithm 1 line 1), of the ROWS tile rows from `r0` on, by one
+// warp: 16-byte loads (D / 8 lanes share a row), eight elements by sequential FMAs, the partial sums by a butterfly.  Rows
+// from `rows_valid` on get zero.
+template <int D, int ROWS>
+__device__ __forceinline__ void saved_output_dots(const __nv_bfloat16 *O, const __nv_bfloat16 *dO, int r0, int rows_valid, float *sD) {
+  constexpr int L = D / 8, RPI = 32 / L, kIters = ROWS / RPI, kBatch = kIters < 4 ? kIters : 4;   // loads in flight per tensor
+  const int lane = threadIdx.x & 31, sub = lane / L, part = lane % L;
+#pragma unroll 1
+  for (int it0 = 0; it0 < kIters; it0 += kBatch) {
+    uint4 a[kBatch], b[kBatch];
+#pragma unroll
+    for (int it = 0; it < kBatch; ++it) {
+      const int r = r0 + (it0 + it) * RPI + sub;
+      a[it] = b[it] = make_uint4(0u, 0u, 0u, 0u);
+      if (r < rows_valid) {
+        a[it] = __ldg(reinterpret_cast<const uint4 *>(O + static_cast<size_t>(r) * D) + part);
+        b[it] = __ldg(reinterpret_cast<const uint4 *>(dO + static_cast<size_t>(r) * D) + part);
+      }
+    }
+#pragma unroll
+    for (int it = 0; it < kBatch; ++it) {
+      const uint32_t aw[4] = {a[it].x, a[it].y, a[it].z, a[it].w}, bw[4] = {b[it].x, b[it].y, b[it].z, b[it].w};
+      float acc = 0.f;
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        acc = fmaf(bf16_lo_to_f32(aw[w]), bf16_lo_to_f32(bw[w]), acc);
+        acc = fmaf(bf16_hi_to_f32(aw[w]), bf16_hi_to_f32(bw[w]), acc);
+      }
+#pragma unroll
+      for (int off = L / 2; off >= 1; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+      if (part == 0) sD[r0 + (it0 + it) * RPI + sub] = acc;
+    }
+  }
+}
+
 // ============================================================================================
 // dQ side
 // ============================================================================================
 template <int D, bool CAUSAL>
-__global__ void __launch_bounds__(BwdCfg<D>::kThreads, 1)
+__global__ void __launch_bounds__(BwdCfg<D>::kDqThreads, 1)
 bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
               const __grid_constant__ CUtensorMap tmdO,   // box 64 x 128 rows
               const __grid_constant__ CUtensorMap tmK,    // box 64 x 64 rows
               const __grid_constant__ CUtensorMap tmV,    // box 64 x 64 rows
-              const __grid_constant__ CUtensorMap tmdQ,   // store, box 64 x 128 rows
-              const __grid_constant__ CUtensorMap tmZ,    // store, box 64 x 128 rows
-              const __nv_bfloat16 *__restrict__ Og, const __nv_bfloat16 *__restrict__ dOg,
+              const __nv_bfloat16 *__restrict__ Qg, const __nv_bfloat16 *__restrict__ Og, const __nv_bfloat16 *__restrict__ dOg,
               const float *__restrict__ LSE, float *__restrict__ stats,
-              __nv_bfloat16 *__restrict__ dQg, __nv_bfloat16 *__restrict__ Zg,   // plain-store targets of clipped tiles
+              __nv_bfloat16 *__restrict__ dQg, __nv_bfloat16 *__restrict__ Zg,
               const int4 *__restrict__ plan, int nblk,                          // packed sequences: tile list; 64-row statistic blocks per head
               int N, int Nk, int BH, int Hq, int G, int total_tiles, const ItemOrder order, float scale_log2, float alpha, unsigned flags, int *status) {
   // N: query rows per head (own operand), Nk: key rows per head.  Causal support of query i: keys j <= i + (L_k - L_q).
@@ -333,13 +374,15 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t *sRes = smem;                                        // buffer rb: Q tile, then dO tile
   uint8_t *sKV = sRes + R * 2 * C::kBigTileBytes;              // stage s: K step tile, then V step tile
-  uint8_t *sOut = sKV + S * C::kDqStageBytes;                  // staging (dQ tile, then Z tile) when separate
+  uint8_t *sStaging = sKV + S * C::kDqStageBytes;              // epilogue warp w: 4096 w
 
   __shared__ uint64_t bar_res_full[R], bar_res_free[R], bar_kv_full[S], bar_kv_empty[S];
-  __shared__ uint64_t bar_sdp_full[NB], bar_tr_ready[NB], bar_acc_done, bar_acc_free, bar_drain[2], bar_stats_ready[R];
+  __shared__ uint64_t bar_sdp_full[NB], bar_tr_ready[NB], bar_acc_done, bar_acc_free, bar_drain[2];
+  __shared__ uint64_t bar_stats_ready[2], bar_mass_ready[2], bar_mass_free[2];
   __shared__ uint32_t tmem_base_smem;
   __shared__ int cta_abort, cta_skip;
-  __shared__ float s_rho[C::kWG - 1][128], s_m[C::kWG - 1][128], s_lam[128], s_D[R][128], s_lse[R][128];
+  // per tile parity: row constants for the compute warpgroups, their row masses for the epilogue
+  __shared__ float s_D[2][128], s_lse[2][128], s_rho[2][C::kWG][128], s_m[2][C::kWG][128];
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) cta_skip = *reinterpret_cast<volatile int *>(status);
@@ -351,11 +394,12 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
   AbortState ab{status, &cta_abort};
   if (threadIdx.x == 0) {
     cta_abort = 0;
-    for (int r = 0; r < R; ++r) { mbar_init(&bar_res_full[r], 1); mbar_init(&bar_res_free[r], 2); mbar_init(&bar_stats_ready[r], 32); }
+    for (int r = 0; r < R; ++r) { mbar_init(&bar_res_full[r], 1); mbar_init(&bar_res_free[r], 1); }
+    for (int p = 0; p < 2; ++p) { mbar_init(&bar_stats_ready[p], 128); mbar_init(&bar_mass_ready[p], C::kCompute); mbar_init(&bar_mass_free[p], 128); }
     for (int s = 0; s < S; ++s) { mbar_init(&bar_kv_full[s], 1); mbar_init(&bar_kv_empty[s], 1); }
     for (int b = 0; b < NB; ++b) { mbar_init(&bar_sdp_full[b], 1); mbar_init(&bar_tr_ready[b], 128 * C::kSlices); }
     mbar_init(&bar_acc_done, 1);
-    mbar_init(&bar_acc_free, C::kCompute);
+    mbar_init(&bar_acc_free, 128);
     mbar_init(&bar_drain[0], 1);
     mbar_init(&bar_drain[1], 1);
     fence_mbar_init();
@@ -363,7 +407,6 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
   if (warp == 1) { tmem_alloc(&tmem_base_smem, C::kTmemCols); tmem_relinquish(); }
   if (warp == 0 && lane == 0) {
     tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmdO); tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV);
-    tma_prefetch_desc(&tmdQ); tma_prefetch_desc(&tmZ);
   }
   tc_fence_before();
   __syncthreads();
@@ -387,6 +430,8 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
     return max(1, (max(kend, 0) + C::kStepRows - 1) / C::kStepRows);
   };
 
+  if (warp < 4) {
+  if constexpr (C::kDqMoveRegs) setmaxnreg_dec<C::kDqRegsAux>();
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer of the streamed (K, V) step tiles
     if (lane == 0) {
@@ -414,13 +459,12 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
       }
     }
   } else if (warp == 3) {
-    // ---------------------------------------------------------------- TMA loader of the stationary (Q, dO) tiles; with
-    // kLoaderStats the whole warp then prepares the tile's row constants (see below)
-    int ti = 0;
-    for (int lin = sched.next(); lin >= 0; lin = sched.next(), ++ti) {
-      const int rb = ti % R, bh = hix(lin);
-      const TileInfo tl = tile_of(lin);
-      if (lane == 0) {
+    // ---------------------------------------------------------------- TMA loader of the stationary (Q, dO) tiles
+    if (lane == 0) {
+      int ti = 0;
+      for (int lin = sched.next(); lin >= 0; lin = sched.next(), ++ti) {
+        const int rb = ti % R, bh = hix(lin);
+        const TileInfo tl = tile_of(lin);
         if (ti >= R) mbar_wait(&bar_res_free[rb], ((ti / R) - 1) & 1, ab, kDqWaitResFree);
         mbar_expect_tx(&bar_res_full[rb], 2 * C::kBigTileBytes);
         uint8_t *dst = sRes + rb * 2 * C::kBigTileBytes;
@@ -429,53 +473,9 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
           tma_load_3d(dst + C::kBigTileBytes + s * C::kBigSlabBytes, &tmdO, &bar_res_full[rb], s * 64, tl.row0, bh);
         }
       }
-      __syncwarp();
-      if (C::kLoaderStats && ti > 0) {       // the first tile's are computed by the (then idle) compute warps: sixteen warps are faster
-        // D_i = sum_c dO_ic O_ic from the saved BF16 output, FP32 (Algorithm 1 line 1), LSE, and the row-constant tile
-        // for the dK/dV side, for the four rows lane, lane + 32, ... of the tile: dO from the stationary tile in shared
-        // memory, O from global memory.  The sum keeps the order of the d = 128 path (eight elements by sequential FMAs,
-        // the eight partial sums by a butterfly).  The buffer pair rb is free: lane 0 has seen its release above.
-        mbar_wait(&bar_res_full[rb], (ti / R) & 1, ab, kDqWaitQ);
-        const size_t head_row0 = static_cast<size_t>(bh) * N;
-        const uint8_t *sdO = sRes + rb * 2 * C::kBigTileBytes + C::kBigTileBytes;
-#pragma unroll
-        for (int it = 0; it < 4; ++it) {
-          const int r = lane + 32 * it, qrow = tl.row0 + r;
-          float part[D / 8];
-#pragma unroll
-          for (int c = 0; c < D / 8; ++c) {
-            uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
-            if (qrow < tl.seq_end) {
-              a = __ldg(reinterpret_cast<const uint4 *>(Og + (head_row0 + qrow) * D) + c);
-              b = *reinterpret_cast<const uint4 *>(sdO + (c >> 3) * C::kBigSlabBytes + swz128_offset(r, c & 7));
-            }
-            const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b.x, b.y, b.z, b.w};
-            float acc = 0.f;
-#pragma unroll
-            for (int w = 0; w < 4; ++w) {
-              acc = fmaf(bf16_lo_to_f32(aw[w]), bf16_lo_to_f32(bw[w]), acc);
-              acc = fmaf(bf16_hi_to_f32(aw[w]), bf16_hi_to_f32(bw[w]), acc);
-            }
-            part[c] = acc;
-          }
-#pragma unroll
-          for (int off = D / 16; off >= 1; off >>= 1)
-#pragma unroll
-            for (int c = 0; c < off; ++c) part[c] += part[c + off];
-          const float Dv = part[0];
-          const float lse_row = (qrow < tl.seq_end) ? LSE[head_row0 + qrow] : 0.f;
-          s_D[rb][r] = Dv;
-          s_lse[rb][r] = lse_row;
-          const int rel = qrow - tl.seq0;                  // row inside the sequence
-          if (rel < ((tl.seq_end - tl.seq0 + 63) / 64) * 64)
-            write_row_constants(stats, (static_cast<size_t>(bh) * nblk + tl.blk0 + (rel >> 6)), rel & 63, -lse_row * 1.4426950408889634f, Dv, scale_log2);
-        }
-        mbar_arrive(&bar_stats_ready[rb]);
-      }
-    }
-    if (lane == 0 && cta_abort) {
-      for (int q = (ti > R ? ti - R : 0); q < ti; ++q)
-        for (int spin = 0; spin < 100000 && !mbar_try_wait(&bar_res_full[q % R], (q / R) & 1); ++spin) {}
+      if (cta_abort)
+        for (int q = (ti > R ? ti - R : 0); q < ti; ++q)
+          for (int spin = 0; spin < 100000 && !mbar_try_wait(&bar_res_full[q % R], (q / R) & 1); ++spin) {}
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- tensor-core issuer 1: scores
@@ -546,63 +546,39 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
       }
     }
     drain_mmas_if_aborted(&bar_drain[1], ab);
-  } else {
+  }
+  } else if (warp < C::kDqEpiWarp) {
     // ---------------------------------------------------------------- compute: thread <-> (query row, key slice of every kGroups-th step)
+    if constexpr (C::kDqMoveRegs) setmaxnreg_inc<C::kDqRegsCompute>();
     const int wg = (warp - 4) >> 2, grp = wg / C::kSlices, slice = wg % C::kSlices;
     const int row = 32 * (warp & 3) + lane;
     const uint32_t lane_addr = static_cast<uint32_t>(32 * (warp & 3)) << 16;
     const uint32_t slice_addr = tmem_base + lane_addr + C::kSliceCols * slice;
     int g0 = 0, ti = 0;
-    constexpr int L = D / 8, RPI = 32 / L;               // D computation: lanes per row, rows per warp-wide load
-    const int sub = lane / L, part = lane % L;
     for (int lin = sched.next(); lin >= 0; lin = sched.next(), ++ti) {
       const TileInfo tl = tile_of(lin);
-      const int bh = hix(lin), T = steps_of(tl), rb = ti % R;
-      const size_t head_row0 = static_cast<size_t>(bh) * N;
+      const int T = steps_of(tl), par = ti & 1;
       const int qrow = tl.row0 + row;                  // this thread's query row within the head (past seq_end in a ragged tile)
 #ifdef GPROJ_TRACE
       const unsigned long long ev_n0 = global_ns(); const long long ev_c0 = clock64(); unsigned long long ev_n1 = 0, ev_n2 = 0;
 #endif
-
-      float Dv, lse_row;
-      if (C::kLoaderStats && ti > 0) {
-        // prepared by the loader's warp while the previous tile ran
-        mbar_wait(&bar_res_full[rb], (ti / R) & 1, ab, kDqWaitQ);       // the tile's Q is read in the epilogue
-        mbar_wait(&bar_stats_ready[rb], ((ti - 1) / R) & 1, ab, kDqWaitQ);
-        Dv = s_D[rb][row];
-        lse_row = s_lse[rb][row];
-      } else {
-        if (C::kLoaderStats) mbar_wait(&bar_res_full[rb], (ti / R) & 1, ab, kDqWaitQ);
-        // D_i = sum_c dO_ic O_ic from the saved BF16 output, FP32 (Algorithm 1 line 1): each of the 16 compute warps
-        // takes eight rows, 16-byte loads (D/8 lanes share a row) and a shuffle reduction.
-#pragma unroll
-        for (int it = 0; it < 8 / RPI; ++it) {
-          const int r = 8 * (warp - 4) + it * RPI + sub;
-          uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
-          if (tl.row0 + r < tl.seq_end) {
-            a = __ldg(reinterpret_cast<const uint4 *>(Og + (head_row0 + tl.row0 + r) * D) + part);
-            b = __ldg(reinterpret_cast<const uint4 *>(dOg + (head_row0 + tl.row0 + r) * D) + part);
-          }
-          const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b.x, b.y, b.z, b.w};
-          float acc = 0.f;
-#pragma unroll
-          for (int w = 0; w < 4; ++w) {
-            acc = fmaf(bf16_lo_to_f32(aw[w]), bf16_lo_to_f32(bw[w]), acc);
-            acc = fmaf(bf16_hi_to_f32(aw[w]), bf16_hi_to_f32(bw[w]), acc);
-          }
-#pragma unroll
-          for (int off = L / 2; off >= 1; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-          if (part == 0) s_D[rb][r] = acc;
+      if (ti == 0) {
+        // The first tile's constants come from these warps, which have nothing else to do yet.
+        constexpr int kRows = 128 / (4 * C::kWG);
+        const size_t row0 = static_cast<size_t>(hix(lin)) * N + tl.row0;
+        const float lse_row = (qrow < tl.seq_end) ? LSE[row0 + row] : 0.f;
+        saved_output_dots<D, kRows>(Og + row0 * D, dOg + row0 * D, kRows * (warp - 4), tl.seq_end - tl.row0, s_D[0]);
+        named_bar_sync(1, C::kCompute);
+        if (wg == 0) {
+          s_lse[0][row] = lse_row;
+          const int rel = qrow - tl.seq0;
+          if (rel < ((tl.seq_end - tl.seq0 + 63) / 64) * 64)
+            write_row_constants(stats, static_cast<size_t>(hix(lin)) * nblk + tl.blk0 + (rel >> 6), rel & 63, -lse_row * 1.4426950408889634f, s_D[0][row], scale_log2);
+          mbar_arrive(&bar_stats_ready[0]);
         }
-        named_bar_sync(2, C::kCompute);
-        Dv = s_D[rb][row];
-        lse_row = (qrow < tl.seq_end) ? LSE[head_row0 + qrow] : 0.f;
-        // Row constants for the dK/dV side, per 64-row block of a sequence (the last one padded with zeros).
-        const int rel = qrow - tl.seq0;                  // row inside the sequence
-        if (wg == 0 && rel < ((tl.seq_end - tl.seq0 + 63) / 64) * 64)
-          write_row_constants(stats, static_cast<size_t>(bh) * nblk + tl.blk0 + (rel >> 6), rel & 63, -lse_row * 1.4426950408889634f, Dv, scale_log2);
       }
-      const float neg_lse2 = -lse_row * 1.4426950408889634f;
+      mbar_wait(&bar_stats_ready[par], (ti >> 1) & 1, ab, kDqWaitStats);
+      const float Dv = s_D[par][row], neg_lse2 = -s_lse[par][row] * 1.4426950408889634f;
 
       uint64_t rho2 = f32x2(0.f, 0.f), msum2 = f32x2(0.f, 0.f);
 #ifdef GPROJ_TRACE
@@ -628,93 +604,124 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
         tc_fence_before();
         mbar_arrive(&bar_tr_ready[b]);
       }
-
 #ifdef GPROJ_TRACE
       ev_n2 = global_ns();
 #endif
-      // ---- row statistics of all warpgroups (fixed order), lambda = rho / m with the zero-mass rule (Algorithm 1 line 14)
+      // hand this warpgroup's share of the row masses to the epilogue and go on with the next tile
       float rho_lo, rho_hi, m_lo, m_hi;
       f32x2_split(rho2, rho_lo, rho_hi);
       f32x2_split(msum2, m_lo, m_hi);
-      float rho_t = rho_lo + rho_hi, m_t = m_lo + m_hi;
-      if (wg > 0) { s_rho[wg - 1][row] = rho_t; s_m[wg - 1][row] = m_t; }
-      if (C::kSepStaging && threadIdx.x == 128) bulk_wait_group_read0();   // the previous tile's stores have left the staging buffer
-      named_bar_sync(1, C::kCompute);
-      if (wg == 0) {
-#pragma unroll
-        for (int w = 0; w < C::kWG - 1; ++w) { rho_t += s_rho[w][row]; m_t += s_m[w][row]; }
-        s_lam[row] = (m_t != 0.f) ? __fdiv_rn(rho_t, m_t) : 0.f;
-      }
-      named_bar_sync(1, C::kCompute);
-      const float lam = s_lam[row];
-      const float lam_q = (flags & kFlagNoQCorrection) ? 0.f : lam;
-      const float lam_k = (flags & kFlagNoKCorrection) ? 0.f : lam;
-
-      mbar_wait(&bar_acc_done, ti & 1, ab, kDqWaitAcc);
-      tc_fence_after();
-      // The 16-column chunks of the epilogue are dealt round-robin to the warpgroups.  Results are staged in the
-      // TMA (128-byte swizzled) layout and written out by TMA stores: Z = -BF16(lambda q), dQ.
-      uint8_t *sQt = sRes + rb * 2 * C::kBigTileBytes, *sdOt = sQt + C::kBigTileBytes;
-      uint8_t *stage_dq = C::kSepStaging ? sOut : sdOt, *stage_z = C::kSepStaging ? sOut + C::kBigTileBytes : sQt;
-      constexpr int kCh = D / (16 * C::kWG);               // 16-column epilogue chunks per warpgroup
-      uint32_t a[kCh][16], b[kCh][16];
-#pragma unroll
-      for (int nch = 0; nch < kCh; ++nch) {
-        const int cc = wg + nch * C::kWG;
-        tmem_ld16(tmem_base + C::kColAcc0 + lane_addr + 16 * cc, a[nch]);
-        tmem_ld16(tmem_base + C::kColAcc1 + lane_addr + 16 * cc, b[nch]);
-      }
-      tmem_wait_ld();
-      tc_fence_before();
-      mbar_arrive(&bar_acc_free);          // the accumulators may be overwritten by the next tile
-#pragma unroll
-      for (int nch = 0; nch < kCh; ++nch) {
-        const int cc = wg + nch * C::kWG;
-        const uint32_t slab = (cc >> 2) * C::kBigSlabBytes;
-#pragma unroll
-        for (int v = 0; v < 2; ++v) {
-          const uint32_t off = slab + swz128_offset(row, 2 * (cc & 3) + v);
-          const uint4 qv = *reinterpret_cast<const uint4 *>(sQt + off);
-          const uint32_t qw[4] = {qv.x, qv.y, qv.z, qv.w};
-          uint32_t dqw[4], zw[4];
-#pragma unroll
-          for (int w = 0; w < 4; ++w) {
-            const int i = 8 * v + 2 * w;
-            const float g0v = __fmul_rn(alpha, __fsub_rn(__uint_as_float(a[nch][i]), __fmul_rn(lam_q, __uint_as_float(b[nch][i]))));
-            const float g1v = __fmul_rn(alpha, __fsub_rn(__uint_as_float(a[nch][i + 1]), __fmul_rn(lam_q, __uint_as_float(b[nch][i + 1]))));
-            dqw[w] = pack_bf16x2(g0v, g1v);
-            // z = BF16(fl32[lambda q]); the sign flip is exact
-            zw[w] = pack_bf16x2(__fmul_rn(lam_k, bf16_lo_to_f32(qw[w])), __fmul_rn(lam_k, bf16_hi_to_f32(qw[w]))) ^ 0x80008000u;
-          }
-          *reinterpret_cast<uint4 *>(stage_dq + off) = make_uint4(dqw[0], dqw[1], dqw[2], dqw[3]);
-          *reinterpret_cast<uint4 *>(stage_z + off) = make_uint4(zw[0], zw[1], zw[2], zw[3]);
-        }
-      }
-      fence_proxy_async_smem();
-      named_bar_sync(1, C::kCompute);
-      if (tile_store_by_tma(tl, N)) {
-        if (threadIdx.x == 128) {
-          for (int sl = 0; sl < C::kSlabs; ++sl) {
-            tma_store_3d(&tmdQ, stage_dq + sl * C::kBigSlabBytes, sl * 64, tl.row0, bh);
-            tma_store_3d(&tmZ, stage_z + sl * C::kBigSlabBytes, sl * 64, tl.row0, bh);
-          }
-          bulk_commit_group();
-          if (!C::kSepStaging) bulk_wait_group_read0();   // staging shares the Q / dO buffer: reads must finish first
-          mbar_arrive(&bar_res_free[rb]);                 // second arrival: the epilogue no longer needs this buffer
-        }
-      } else {
-        // ragged last tile of a packed sequence that another sequence follows: rows past its end are not ours to write
-        if (wg < 2) store_rows_clipped<D>(wg == 0 ? stage_dq : stage_z, C::kBigSlabBytes,
-                                         (wg == 0 ? dQg : Zg) + (head_row0 + tl.row0) * D, row, tl.seq_end - tl.row0);
-        named_bar_sync(1, C::kCompute);
-        if (threadIdx.x == 128) mbar_arrive(&bar_res_free[rb]);
-      }
+      if (ti >= 2) mbar_wait(&bar_mass_free[par], ((ti >> 1) - 1) & 1, ab, kDqWaitMass);
+      s_rho[par][wg][row] = rho_lo + rho_hi;
+      s_m[par][wg][row] = m_lo + m_hi;
+      mbar_arrive(&bar_mass_ready[par]);
 #ifdef GPROJ_TRACE
       if ((threadIdx.x & 127) == 0) tile_event(1 + wg, lin, T, ev_n0, ev_n1, ev_n2, global_ns(), ev_c0, clock64());
 #endif
       g0 += T;
     }
-    if (threadIdx.x == 128) bulk_wait_group_read0();
+  } else {
+    // ---------------------------------------------------------------- row constants one tile ahead, and the epilogue: thread <-> query row
+    // (keeps the 80 registers of the launch)
+    const int ew = warp - C::kDqEpiWarp, row = 32 * ew + lane;
+    const uint32_t lane_addr = static_cast<uint32_t>(32 * ew) << 16;
+    auto row_constants = [&](int lin, int par) {
+      const TileInfo tl = tile_of(lin);
+      const int bh = hix(lin);
+      const size_t row0 = static_cast<size_t>(bh) * N + tl.row0;
+      const float lse_row = (tl.row0 + row < tl.seq_end) ? LSE[row0 + row] : 0.f;
+      saved_output_dots<D, 32>(Og + row0 * D, dOg + row0 * D, 32 * ew, tl.seq_end - tl.row0, s_D[par]);
+      __syncwarp();
+      s_lse[par][row] = lse_row;
+      const int rel = tl.row0 + row - tl.seq0;             // row inside the sequence; its last 64-row block is padded with zeros
+      if (rel < ((tl.seq_end - tl.seq0 + 63) / 64) * 64)
+        write_row_constants(stats, static_cast<size_t>(bh) * nblk + tl.blk0 + (rel >> 6), rel & 63, -lse_row * 1.4426950408889634f, s_D[par][row], scale_log2);
+      mbar_arrive(&bar_stats_ready[par]);
+    };
+    int ti = 0, lin = sched.next();
+    while (lin >= 0) {
+      const int next = sched.next(), par = ti & 1;
+      // The constants of tile ti + 1 overwrite those of tile ti - 1, whose readers have all handed in their row masses.
+      if (next >= 0) row_constants(next, par ^ 1);
+      const TileInfo tl = tile_of(lin);
+      // q of this warp's 32 rows, D / 8 lanes to a row (whole lines per load and store; one row per thread touches 32
+      // lines with every instruction and took 2.2 us instead of 1 us of the tail at d = 128), the first kQ loads ahead of
+      // the wait
+      constexpr int L = D / 8, RPI = 32 / L, kIters = 32 / RPI;
+      const int sub = lane / L, part = lane % L;
+      const size_t wrow0 = (static_cast<size_t>(hix(lin)) * N + tl.row0 + 32 * ew) * D;
+      const int wrows = tl.seq_end - tl.row0 - 32 * ew;    // rows of this warp that exist
+      constexpr int kQ = D == 128 ? 8 : 4;                 // loads in flight (80 registers at d = 64)
+      uint4 qv[kQ];
+      auto fetch_q = [&](int h) {
+#pragma unroll
+        for (int k = 0; k < kQ; ++k) {
+          const int r = (kQ * h + k) * RPI + sub;
+          qv[k] = r < wrows ? __ldg(reinterpret_cast<const uint4 *>(Qg + wrow0 + static_cast<size_t>(r) * D) + part) : make_uint4(0u, 0u, 0u, 0u);
+        }
+      };
+      fetch_q(0);
+      // row masses of all warpgroups (fixed order), lambda = rho / m with the zero-mass rule (Algorithm 1 line 14)
+      mbar_wait(&bar_mass_ready[par], (ti >> 1) & 1, ab, kDqWaitMass);
+      float rho_t = s_rho[par][0][row], m_t = s_m[par][0][row];
+#pragma unroll
+      for (int w = 1; w < C::kWG; ++w) { rho_t += s_rho[par][w][row]; m_t += s_m[par][w][row]; }
+      mbar_arrive(&bar_mass_free[par]);
+      const float lam = (m_t != 0.f) ? __fdiv_rn(rho_t, m_t) : 0.f;
+      const float lam_q = (flags & kFlagNoQCorrection) ? 0.f : lam, lam_k = (flags & kFlagNoKCorrection) ? 0.f : lam;
+      // z = BF16(fl32[lambda q]), stored negated (the sign flip is exact), while the last products still run
+#pragma unroll
+      for (int h = 0; h < kIters / kQ; ++h) {
+#pragma unroll
+        for (int k = 0; k < kQ; ++k) {
+          const int r = (kQ * h + k) * RPI + sub;
+          const float lr = __shfl_sync(0xffffffffu, lam_k, r);
+          const uint32_t qw[4] = {qv[k].x, qv[k].y, qv[k].z, qv[k].w};
+          uint32_t zw[4];
+#pragma unroll
+          for (int w = 0; w < 4; ++w)
+            zw[w] = pack_bf16x2(__fmul_rn(lr, bf16_lo_to_f32(qw[w])), __fmul_rn(lr, bf16_hi_to_f32(qw[w]))) ^ 0x80008000u;
+          if (r < wrows) reinterpret_cast<uint4 *>(Zg + wrow0 + static_cast<size_t>(r) * D)[part] = make_uint4(zw[0], zw[1], zw[2], zw[3]);
+        }
+        if (h + 1 < kIters / kQ) fetch_q(h + 1);
+      }
+      mbar_wait(&bar_acc_done, ti & 1, ab, kDqWaitAcc);
+      tc_fence_after();
+      uint8_t *stg = sStaging + 4096 * ew;
+#pragma unroll
+      for (int hd = 0; hd < D / 64; ++hd) {
+#pragma unroll
+        for (int cc = 0; cc < 4; ++cc) {
+          uint32_t a[16], b[16];
+          tmem_ld16(tmem_base + C::kColAcc0 + lane_addr + 64 * hd + 16 * cc, a);
+          tmem_ld16(tmem_base + C::kColAcc1 + lane_addr + 64 * hd + 16 * cc, b);
+          tmem_wait_ld();
+          if (hd == D / 64 - 1 && cc == 3) { tc_fence_before(); mbar_arrive(&bar_acc_free); }   // the accumulators may be overwritten by the next tile
+#pragma unroll
+          for (int v = 0; v < 2; ++v) {
+            uint32_t dqw[4];
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+              const int i = 8 * v + 2 * w;
+              const float g0v = __fmul_rn(alpha, __fsub_rn(__uint_as_float(a[i]), __fmul_rn(lam_q, __uint_as_float(b[i]))));
+              const float g1v = __fmul_rn(alpha, __fsub_rn(__uint_as_float(a[i + 1]), __fmul_rn(lam_q, __uint_as_float(b[i + 1]))));
+              dqw[w] = pack_bf16x2(g0v, g1v);
+            }
+            *reinterpret_cast<uint4 *>(stg + swz128_offset(lane, 2 * cc + v)) = make_uint4(dqw[0], dqw[1], dqw[2], dqw[3]);
+          }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const int r = 4 * k + (lane >> 3);
+          const uint4 v = *reinterpret_cast<const uint4 *>(stg + swz128_offset(r, lane & 7));
+          if (r < wrows) reinterpret_cast<uint4 *>(dQg + wrow0 + static_cast<size_t>(r) * D + 64 * hd)[lane & 7] = v;
+        }
+        __syncwarp();
+      }
+      lin = next;
+      ++ti;
+    }
   }
 
   tc_fence_before();

@@ -436,11 +436,11 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
   float *stats = static_cast<float *>(workspace);   // per 64-row block: the row-constant tile (see stats_blocks_bytes)
   __nv_bfloat16 *Zneg = reinterpret_cast<__nv_bfloat16 *>(static_cast<uint8_t *>(workspace) + stats_sz);
 
-  CUtensorMap mQ128, mdO128, mK64, mV64, mK128, mV128, mQ64, mdO64, mZ64, mdQst, mZst, mdKst, mdVst;
+  CUtensorMap mQ128, mdO128, mK64, mV64, mK128, mV128, mQ64, mdO64, mZ64, mZst, mdKst, mdVst;
   bool ok = make_map(&mQ128, Q, BH, N, d, 128) && make_map(&mdO128, dO, BH, N, d, 128) && make_map(&mK64, K, BHkv, Nk, d, 64) &&
             make_map(&mV64, V, BHkv, Nk, d, 64) && make_map(&mK128, K, BHkv, Nk, d, 128) && make_map(&mV128, V, BHkv, Nk, d, 128) &&
             make_map(&mQ64, Q, BH, N, d, 64) && make_map(&mdO64, dO, BH, N, d, 64) && make_map(&mZ64, Zneg, BH, N, d, 64) &&
-            make_map(&mdQst, dQ, BH, N, d, 128) && make_map(&mZst, Zneg, BH, N, d, 128) && make_map(&mdKst, dK, BHkv, Nk, d, 128) &&
+            make_map(&mZst, Zneg, BH, N, d, 128) && make_map(&mdKst, dK, BHkv, Nk, d, 128) &&
             make_map(&mdVst, dV, BHkv, Nk, d, 128);
   if (!ok) return GPROJ_ERR_CUDA;
 
@@ -458,8 +458,8 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
 #define GPROJ_LAUNCH_BWD(DD, CC)                                                                                        \
   do {                                                                                                                  \
     if (run_dq)                                                                                                         \
-      bwd_dq_kernel<DD, CC><<<grid, BwdCfg<DD>::kThreads, BwdCfg<DD>::kDqSmemBytes, s>>>(                               \
-          mQ128, mdO128, mK64, mV64, mdQst, mZst, Ob, dOb, LSE, stats, static_cast<__nv_bfloat16 *>(dQ), Zneg, plan_q, nblk,   \
+      bwd_dq_kernel<DD, CC><<<grid, BwdCfg<DD>::kDqThreads, BwdCfg<DD>::kDqSmemBytes, s>>>(                               \
+          mQ128, mdO128, mK64, mV64, static_cast<const __nv_bfloat16 *>(Q), Ob, dOb, LSE, stats, static_cast<__nv_bfloat16 *>(dQ), Zneg, plan_q, nblk,   \
           N, Nk, BH, H, G, total_tiles, group_q, scale_log2, softmax_scale,                                           \
           flags,                                                                                                        \
           st->status_ptr);                                                                                              \
@@ -475,8 +475,8 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
 #define GPROJ_LAUNCH_BWD_W128(CC)                                                                                       \
   do {                                                                                                                  \
     if (run_dq)                                                                                                         \
-      bwd_dq_kernel<64, CC><<<grid, BwdCfg<64>::kThreads, BwdCfg<64>::kDqSmemBytes, s>>>(                                \
-          mQ128, mdO128, mK64, mV64, mdQst, mZst, Ob, dOb, LSE, stats, static_cast<__nv_bfloat16 *>(dQ), Zneg, plan_q,    \
+      bwd_dq_kernel<64, CC><<<grid, BwdCfg<64>::kDqThreads, BwdCfg<64>::kDqSmemBytes, s>>>(                                \
+          mQ128, mdO128, mK64, mV64, static_cast<const __nv_bfloat16 *>(Q), Ob, dOb, LSE, stats, static_cast<__nv_bfloat16 *>(dQ), Zneg, plan_q,    \
           nblk, N, Nk, BH, H, G, total_tiles, group_q, scale_log2, softmax_scale, flags, st->status_ptr);                 \
     if (run_dkv)                                                                                                        \
       launch_after(bwd_dkv_w128_kernel<CC>, grid_kv, BwdW128::kThreads, BwdW128::kDkvSmemBytes, s, run_dq,               \
