@@ -464,8 +464,8 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
           flags,                                                                                                        \
           st->status_ptr);                                                                                              \
     if (run_dkv)                                                                                                        \
-      launch_after(bwd_dkv_kernel<DD, CC>, grid_kv, BwdCfg<DD>::kThreads, BwdCfg<DD>::kDkvSmemBytes, s, run_dq,            \
-          mK128, mV128, mQ64, mdO64, mZ64, mdKst, mdVst, stats, static_cast<__nv_bfloat16 *>(dK),                        \
+      launch_after(bwd_dkv_kernel<DD, CC>, grid_kv, BwdCfg<DD>::kDkvThreads, BwdCfg<DD>::kDkvSmemBytes, s, run_dq,            \
+          mK128, mV128, mQ64, mdO64, mZ64, stats, static_cast<__nv_bfloat16 *>(dK),                        \
           static_cast<__nv_bfloat16 *>(dV), plan_kv, nblk, Nk, N, BHkv, Hkv, G, total_kv_tiles, group_kv, scale_log2, softmax_scale, \
           flags,                                                                                                        \
           st->status_ptr);                                                                                              \
