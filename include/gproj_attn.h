@@ -275,7 +275,7 @@ int gproj_fp32_attn_bwd(const void *Q, const void *K, const void *V, const void 
  * arithmetic; what the shift removes is the common component of the keys that the leaked row mass multiplies, not
  * the leak itself (Section 2).  The paper's experiments use it only as a baseline; so does this library.
  *   X, Y: DEVICE BF16, [B][Hkv][N][d] (dense) or [Hkv][T][d] with HOST offsets cu_seqlens (packed; the mean is taken
- *   inside each sequence; empty sequences are skipped); Y may be X.  One launch per sequence, on `stream`.
+ *   inside each sequence; empty sequences are skipped); Y may be X.  One launch per 512 non-empty sequences, on `stream`.
  *   Errors: GPROJ_ERR_NULL, GPROJ_ERR_SHAPE (d not 64 / 128, non-positive sizes, malformed offsets), GPROJ_ERR_ALIGN,
  *   GPROJ_ERR_ARCH, GPROJ_ERR_CUDA.
  */

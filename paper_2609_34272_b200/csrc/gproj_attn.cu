@@ -949,13 +949,24 @@ static int smooth_rows(const void *X, void *Y, int heads, long long rows_total, 
   const __nv_bfloat16 *x = static_cast<const __nv_bfloat16 *>(X);
   __nv_bfloat16 *y = static_cast<__nv_bfloat16 *>(Y);
   int launches = 0;
-  const int n = cu_seqlens ? num_seqs : 1;
-  for (int q = 0; q < n; ++q) {
-    const int r0 = cu_seqlens ? cu_seqlens[q] : 0, rows = cu_seqlens ? cu_seqlens[q + 1] - r0 : static_cast<int>(rows_total);
-    if (rows == 0) continue;
-    if (d == 64) smooth_rows_kernel<64><<<heads, kSmoothThreads, 0, s>>>(x, y, rows_total * d, r0, rows);
-    else         smooth_rows_kernel<128><<<heads, kSmoothThreads, 0, s>>>(x, y, rows_total * d, r0, rows);
-    ++launches;
+  const int n = cu_seqlens ? num_seqs : 1, whole[2] = {0, static_cast<int>(rows_total)};
+  const int *cu = cu_seqlens ? cu_seqlens : whole;
+  SmoothOffsets off;
+  for (int q = 0; q < n;) {
+    int m = 0;                                        // non-empty sequences of this launch; empty ones drop out of the offsets
+    off.cu[0] = cu[q];
+    while (q < n && m < kSmoothMaxSeqs) {
+      if (cu[q + 1] > cu[q]) off.cu[++m] = cu[q + 1];
+      ++q;
+    }
+    if (m == 0) continue;
+    for (int h0 = 0; h0 < heads; h0 += 65535) {       // heads along y, whose limit is 65535
+      const dim3 grid(static_cast<unsigned>(m * kSmoothCluster), static_cast<unsigned>(std::min(heads - h0, 65535)));
+      const long long at = static_cast<long long>(h0) * rows_total * d;
+      if (d == 64) smooth_rows_kernel<64><<<grid, kSmoothThreads, 0, s>>>(x + at, y + at, rows_total * d, off);
+      else         smooth_rows_kernel<128><<<grid, kSmoothThreads, 0, s>>>(x + at, y + at, rows_total * d, off);
+      ++launches;
+    }
   }
   if (cudaGetLastError() != cudaSuccess) return GPROJ_ERR_CUDA;
   tl_launch_count = launches;
