@@ -15,6 +15,9 @@
 //   split (2)     one item = one query tile; warpgroup t takes the key tiles j = t (mod 2) with its own running
 //                 maximum, normaliser and accumulator, and warpgroup 0 merges the two halves at the end.  Used when
 //                 pairs would leave SMs idle and for packed sequences.
+//   cluster (3)   one item = one query tile on a cluster of 2, 4 or 8 CTAs that share its key tiles in the same way and
+//                 merge 4, 8 or 16 parts through distributed shared memory.  Used when even single tiles leave SMs
+//                 idle: a block of new queries behind a key history, a short batch.
 // Softmax arithmetic (FMA_SOFTMAX = false, the default): online softmax on the UNSCALED logits with the
 // subtract-before-scale rounding of
 // Eq. "gproj-forward": z = exp2(fl32[ fl32(x - x_max) * (alpha log2 e) ]); l accumulates the FP32 z, the value
@@ -46,6 +49,8 @@ struct FwdCfg {
   static constexpr bool kSepP = (D == 64);             // P~ in its own TMEM columns
   static constexpr uint32_t kColS = 0, kColO = 256, kColP = 256 + 2 * D;   // S_t at 128 t, O_t at 256 + D t, P_t at kColP + 64 t
   static constexpr int kThreads = 384;
+  static constexpr int kMaxCluster = 8;
+  static_assert(256 * (4 * D + 16) <= 2 * kTileBytes + kStages * 2 * kTileBytes, "the cluster merge goes over the Q and K / V tiles");
 };
 
 enum FwdWaitCode {
@@ -84,15 +89,20 @@ __device__ __forceinline__ float softmax_exp_store(const uint32_t (&xr)[4][32], 
 }
 
 // MODE: 0 = pairs of query tiles, 1 = pairs whose warpgroups take turns in the exponential phase, 2 = single tiles with
-// the key range split between the warpgroups.
+// the key range split between the warpgroups, 3 = single tiles with the key range split over the warpgroups of a cluster of
+// CTAs (one tile per cluster; the parts of all CTAs are merged through distributed shared memory).
 template <int D, bool CAUSAL, bool FMA_SOFTMAX, int MODE>
 __global__ void __launch_bounds__(384, 1)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                 const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
-                __nv_bfloat16 *__restrict__ Og, const int4 *__restrict__ plan, float *__restrict__ LSE, int N, int Nk, int BH, int Hq, int G, int tiles_per_item, int total_items, const ItemOrder order, float scale_log2, float alpha,
+                __nv_bfloat16 *__restrict__ Og, const int4 *__restrict__ plan, float *__restrict__ LSE, int N, int Nk, int BH, int Hq, int G, int fold_rows, int tiles_per_item, int total_items, const ItemOrder order, float scale_log2, float alpha,
                 int *status) {
+  // fold > 0 (cluster mode only): the query axis of a KV head is its G query heads' rows laid end to end, `fold` rows each
+  // (grouped queries with few rows); row r then sees the keys of query r mod fold.
   using C = FwdCfg<D>;
   constexpr int S = C::kStages;
+  constexpr bool kCluster = (MODE == 3);
+  const int fold = kCluster ? fold_rows : 0;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t *sQ = smem;                              // tile 0, then tile 1 (each later reused to stage O_t)
@@ -101,23 +111,28 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   __shared__ int s_item[4][2];
   __shared__ uint64_t bar_q_full[2], bar_q_free[2], bar_k_full[S], bar_v_full[S], bar_kv_empty[S];
   __shared__ uint64_t bar_s_full[2], bar_s_free[2], bar_p_ready[2], bar_pv_done[2], bar_o_free[2], bar_turn[2], bar_merge, bar_drain[2];
-  __shared__ float s_m1[2][128], s_l1[2][128];   // split mode: running maximum and normaliser of the second warpgroup
+  __shared__ float s_m1[2][128], s_l1[2][128];   // split mode: running maximum and normaliser of the second warpgroup, by item parity (with a cluster: of both)
   __shared__ uint32_t tmem_base_smem;
   __shared__ int cta_abort, cta_skip;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) cta_skip = *reinterpret_cast<volatile int *>(status);
   __syncthreads();
-  if (cta_skip != 0) return;   // an earlier wait gave up: drain the rest of the grid quickly
+  // An earlier wait gave up: drain the rest of the grid quickly.  The CTAs of a cluster wait for one another at the end, so
+  // they run on with every wait falling through instead.
+  if (!kCluster && cta_skip != 0) return;
 
   const int n_qt = (N + C::kBlockM - 1) / C::kBlockM;   // the last tile may be ragged: rows past N load as zero, stores clip
   const int TPI = tiles_per_item;                  // 2: a pair of query tiles per work item; 1: single tiles, key range split
-  constexpr bool split = (MODE == 2);              // one query tile; warpgroup t takes the key tiles j = t (mod 2), merged at the end
+  constexpr bool split = (MODE >= 2);              // one query tile; warpgroup t takes the key tiles j = t (mod 2), merged at the end
+  // Key tile j of the item belongs to CTA (j / 2) mod ncta of the cluster (ncta = 1 without a cluster), warpgroup j mod 2.
+  const int ncta = kCluster ? cluster_size() : 1, crank = kCluster ? cluster_rank() : 0;
+  auto mine = [&](int j) { return !kCluster || ((j >> 1) % ncta) == crank; };
   constexpr bool TURNS = (MODE == 1);
   const int n_pairs = (n_qt + TPI - 1) / TPI;
   AbortState ab{status, &cta_abort};
   if (threadIdx.x == 0) {
-    cta_abort = 0;
+    cta_abort = kCluster ? cta_skip : 0;
     mbar_init(&bar_merge, 128);
     for (int b = 0; b < 2; ++b) {
       mbar_init(&bar_q_full[b], 1);
@@ -145,6 +160,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   auto tix = [&](int lin) { return order.rank(lin); };
   auto hix = [&](int lin) { return order.head(lin); };
   TileSched sched(total_items);
+  if (kCluster) { sched.G /= ncta; sched.c /= ncta; }
   auto decode_rank = [&](int rank) {       // rank: position of the item's tile (pair) in its head's list, longest first
     Item it;
     if (plan != nullptr) {
@@ -156,16 +172,16 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       it.seq0 = 0; it.len = N; it.qt0 = TPI * pair; it.nq = min(TPI, n_qt - it.qt0);
       it.kseq0 = 0; it.klen = Nk;
     }
-    it.off = it.klen - it.len;
+    it.off = it.klen - (fold > 0 ? fold : it.len);
     // key tiles up to the last key the item's last row sees; at least one (fully masked if the item sees no key at all)
-    const int kend = CAUSAL ? min(it.klen, (it.qt0 + it.nq) * C::kBlockM + it.off) : it.klen;
+    const int kend = (CAUSAL && fold == 0) ? min(it.klen, (it.qt0 + it.nq) * C::kBlockM + it.off) : it.klen;
     it.n_kt = max(1, (max(kend, 0) + C::kBlockN - 1) / C::kBlockN);
     return it;
   };
   auto decode = [&](int lin) { return decode_rank(tix(lin)); };
   // query tile t of the item takes part in key step j?  (key tile 0 always, so that every tile has a first step)
   auto active = [&](const Item &it, int t, int j) {
-    return t < it.nq && (!CAUSAL || j <= max(0, ((it.qt0 + t) * C::kBlockM + C::kBlockM - 1 + it.off) >> 7));
+    return t < it.nq && (!CAUSAL || fold > 0 || j <= max(0, ((it.qt0 + t) * C::kBlockM + C::kBlockM - 1 + it.off) >> 7));
   };
 
   // Q buffers: a pair item fills both tile slots of the one buffer; single-tile items (split mode) alternate between the
@@ -180,7 +196,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       for (int lin = sched.next(); lin >= 0; lin = sched.next()) {
         const Item it = decode(lin);
         const int bh = hix(lin), T = it.n_kt;
-        for (int j = 0; j < T; ++j, ++g) {
+        for (int j = 0; j < T; ++j) {
+          if (!mine(j)) continue;
           const int st = g % S;
           if (g >= S) mbar_wait(&bar_kv_empty[st], ((g / S) - 1) & 1, ab, kFwdWaitKVEmpty);
           uint8_t *dK = sKV + st * 2 * C::kTileBytes, *dV = dK + C::kTileBytes;
@@ -189,6 +206,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           for (int s = 0; s < C::kSlabs; ++s) tma_load_3d(dK + s * C::kSlabBytes, &tmK, &bar_k_full[st], s * 64, krow, kvh);
           mbar_expect_tx(&bar_v_full[st], C::kTileBytes);
           for (int s = 0; s < C::kSlabs; ++s) tma_load_3d(dV + s * C::kSlabBytes, &tmV, &bar_v_full[st], s * 64, krow, kvh);
+          ++g;
         }
       }
       // Every load is consumed by an MMA the epilogue waits for, so nothing is in flight at exit unless the
@@ -236,7 +254,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       const int T = it.n_kt;
       const int qb = q_buf(ti);
       mbar_wait(&bar_q_full[qb], q_use(ti) & 1, ab, kFwdWaitQ);
-      for (int j = 0; j < T; ++j, ++g) {
+      for (int j = 0; j < T; ++j) {
+        if (!mine(j)) continue;
         const int st = g % S;
         mbar_wait(&bar_k_full[st], (g / S) & 1, ab, kFwdWaitK);
         const SmemDesc dscK = dscK0.advanced(st * 2 * C::kTileBytes);
@@ -262,6 +281,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           __syncwarp();
           ++cnt[t];
         }
+        ++g;
       }
     }
     drain_mmas_if_aborted(&bar_drain[0], ab);
@@ -273,14 +293,15 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     for (int lin = sched.next(); lin >= 0; lin = sched.next(), ++ti) {
       const Item it = decode(lin);
       const int T = it.n_kt;
-      for (int j = 0; j < T; ++j, ++g) {
+      for (int j = 0; j < T; ++j) {
+        if (!mine(j)) continue;
         const int st = g % S;
         mbar_wait(&bar_v_full[st], (g / S) & 1, ab, kFwdWaitV);
         const SmemDesc dscV = dscV0.advanced(st * 2 * C::kTileBytes);
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
           if (split ? ((j & 1) != t) : !active(it, t, j)) continue;
-          const bool first = split ? (j < 2) : (j == 0);     // first product into O_t in this work item
+          const bool first = split ? (j < 2 * crank + 2) : (j == 0);     // first product into O_t in this work item
           if (first && ti > 0) mbar_wait(&bar_o_free[t], (ti - 1) & 1, ab, kFwdWaitOFree);   // previous epilogue has read O_t
           mbar_wait(&bar_p_ready[t], cnt[t] & 1, ab, kFwdWaitP);
           tc_fence_after();
@@ -297,6 +318,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         }
         if (elect_one_sync()) umma_commit(&bar_kv_empty[st]);    // every MMA that reads this K / V stage has been issued
         __syncwarp();
+        ++g;
       }
     }
     drain_mmas_if_aborted(&bar_drain[1], ab);
@@ -318,9 +340,12 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       // Masking, reduced to two numbers per tile: column c of key tile j is outside the row's support when
       // 128 j + c > rk, with rk the last key the row sees (causal diagonal and end of the keys, whichever comes first);
       // no key tile before jm needs the test for any row of the tile.
-      const int rk = CAUSAL ? min(row + qt * C::kBlockM + it.off, it.klen - 1) : it.klen - 1;
-      const int jl = CAUSAL ? max(0, (qt * C::kBlockM + C::kBlockM - 1 + it.off) >> 7) : T;   // last key tile of this query tile
-      const int jm = CAUSAL ? min((qt * C::kBlockM + it.off + 1) >> 7, it.klen >> 7) : (it.klen >> 7);
+      const int q_lo = fold > 0 ? 0 : qt * C::kBlockM, q_row = fold > 0 ? (qt * C::kBlockM + row) % fold : qt * C::kBlockM + row;   // first query of the tile, this row's query
+      const int rk = CAUSAL ? min(q_row + it.off, it.klen - 1) : it.klen - 1;
+      const int jl = (CAUSAL && fold == 0) ? max(0, (qt * C::kBlockM + C::kBlockM - 1 + it.off) >> 7) : T;   // last key tile of this query tile
+      const int jm = CAUSAL ? min((q_lo + it.off + 1) >> 7, it.klen >> 7) : (it.klen >> 7);
+      // A warp none of whose rows exist (a short block of queries) only keeps the barriers going.
+      const bool live = qt * C::kBlockM + 32 * (warp & 3) < it.len;
       if (!split && t >= it.nq) {
         // Odd number of query tiles: the last pair has no second tile.  This warpgroup is in step with the item (it has
         // waited for its Q above), so it may hand back the slot without any barrier running ahead of its waiters.
@@ -335,8 +360,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       // Both tiles of the pair exist: the warpgroups alternate in the exponential phase, step by step, tile 0 first.
       const bool take_turns = TURNS && it.nq == 2;
       const int cnt_item0 = cnt;
-      for (int j = split ? t : 0; j < T; j += split ? 2 : 1) {
-        const bool first = split ? (j < 2) : (j == 0);     // this warpgroup's first key tile of the item
+      for (int j = split ? 2 * crank + t : 0; j < T; j += split ? 2 * ncta : 1) {
+        const bool first = split ? (j < 2 * crank + 2) : (j == 0);     // this warpgroup's first key tile of the item
         if (!split && j > jl) {
           // no work in this step (causal: the first tile of the pair ends one key tile earlier): pass the turn on
           if (take_turns) {
@@ -348,6 +373,13 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         }
         mbar_wait(&bar_s_full[t], cnt & 1, ab, kFwdWaitS);
         tc_fence_after();
+        if (kCluster && !live) {
+          if (C::kSepP) mbar_arrive(&bar_s_free[t]);
+          if (!first) mbar_wait(&bar_pv_done[t], (cnt - 1) & 1, ab, kFwdWaitPV);
+          mbar_arrive(&bar_p_ready[t]);
+          ++cnt;
+          continue;
+        }
         uint32_t xr[4][32];
 #pragma unroll
         for (int c = 0; c < 4; ++c) tmem_ld32(tS + 32 * c, xr[c]);
@@ -420,6 +452,13 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 #endif
       // ---- epilogue: O = BF16(acc / l) staged in the TMA layout over this tile's Q, LSE = alpha x_max + ln l
       if (cnt > cnt_item0) { mbar_wait(&bar_pv_done[t], (cnt - 1) & 1, ab, kFwdWaitPV); tc_fence_after(); }
+      if (kCluster) {
+        // the merge is below, by all threads of the cluster
+        s_m1[t][row] = m_run;
+        s_l1[t][row] = l_run;
+        tc_fence_before();
+        break;
+      }
       if (split && t == 1) {
         // hand this half's statistics to warpgroup 0, which merges the two accumulators (l = 0: no key tiles here).
         // With two Q slots this warpgroup could finish a second item before warpgroup 0 has looked at the first one's
@@ -500,6 +539,68 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 #ifdef GPROJ_TRACE
       if (row == 0) tile_event(20 + t, lin, T, ev_n0, ev_n0, ev_n2, global_ns(), ev_c0, clock64());
 #endif
+    }
+  }
+
+  if (kCluster) {
+    // Merge of the 2 ncta partial results of the cluster's tile: O = sum_w O_w s_w / L with s_w = exp2((m_w - M) alpha log2 e),
+    // M = max m_w, L = sum l_w s_w.  Every softmax thread scales its own accumulator row and sends it to the CTA that
+    // finishes the row (128 / ncta rows each), over that CTA's consumed Q and K / V tiles; the sums are taken in a fixed
+    // order.
+    constexpr int kRowBytes = D * 4 + 16;                    // padded: rows of consecutive threads start in different banks
+    const int own = 128 / ncta, nsrc = 2 * ncta;
+    cluster_sync();                                          // statistics written; every product of every CTA is complete
+    const Item it = decode(sched.c);
+    const int bh = hix(sched.c), tile_row0 = it.qt0 * C::kBlockM;
+    const int t = (warp - 4) >> 2, row = 32 * (warp & 3) + lane;
+    float M = -INFINITY, L = 0.f;
+    if (warp >= 4) {
+      tc_fence_after();
+      const uint32_t am = smem_u32(&s_m1[0][row]), al = smem_u32(&s_l1[0][row]);
+      float mw[2 * C::kMaxCluster], lw[2 * C::kMaxCluster];  // every load issued before the first use: a remote load takes some 200 clk
+#pragma unroll
+      for (int w = 0; w < 2 * C::kMaxCluster; ++w) {
+        const bool in = w < nsrc;
+        mw[w] = in ? cluster_load_f32(cluster_map_shared(am, w >> 1) + 512 * (w & 1)) : -INFINITY;
+        lw[w] = in ? cluster_load_f32(cluster_map_shared(al, w >> 1) + 512 * (w & 1)) : 0.f;
+      }
+#pragma unroll
+      for (int w = 0; w < 2 * C::kMaxCluster; ++w) M = fmaxf(M, mw[w]);
+      M = fmaxf(M, kFwdMaxFloor);                            // a part without key tiles has m = -inf, l = 0
+#pragma unroll
+      for (int w = 0; w < 2 * C::kMaxCluster; ++w) L += lw[w] * fast_exp2(__fmul_rn(__fsub_rn(mw[w], M), scale_log2));
+      const bool has = s_l1[t][row] > 0.f;                   // otherwise the accumulator may never have been written
+      const float a = has && L > 0.f ? fast_exp2(__fmul_rn(__fsub_rn(s_m1[t][row], M), scale_log2)) / L : 0.f;
+      const uint32_t dst = cluster_map_shared(smem_u32(smem) + static_cast<uint32_t>(((2 * crank + t) * own + row % own) * kRowBytes), row / own);
+      const uint32_t tO = tmem_base + C::kColO + D * t + (static_cast<uint32_t>(32 * (warp & 3)) << 16);
+#pragma unroll
+      for (int c = 0; c < D / 16; ++c) {
+        uint32_t o[16];
+        tmem_ld16(tO + 16 * c, o);
+        tmem_wait_ld();
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          float f[4];
+#pragma unroll
+          for (int w = 0; w < 4; ++w) f[w] = has ? __uint_as_float(o[4 * v + w]) * a : 0.f;
+          cluster_store_f4(dst + 64 * c + 16 * v, f[0], f[1], f[2], f[3]);
+        }
+      }
+      tc_fence_before();
+      const int qrel = tile_row0 + row;
+      if (t == 0 && row / own == crank && qrel < it.len)
+        LSE[static_cast<size_t>(bh) * N + it.seq0 + qrel] = (L > 0.f) ? fmaf(M, alpha, logf(L)) : INFINITY;
+    }
+    cluster_sync();
+    for (int i = threadIdx.x; i < own * (D / 4); i += C::kThreads) {
+      const int r = i / (D / 4), c4 = i % (D / 4), qrel = tile_row0 + crank * own + r;
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int w = 0; w < nsrc; ++w) {
+        const float4 v = *reinterpret_cast<const float4 *>(smem + (w * own + r) * kRowBytes + 16 * c4);
+        acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+      }
+      if (qrel < it.len)
+        *reinterpret_cast<uint2 *>(Og + (static_cast<size_t>(bh) * N + it.seq0 + qrel) * D + 4 * c4) = make_uint2(pack_bf16x2(acc.x, acc.y), pack_bf16x2(acc.z, acc.w));
     }
   }
 

@@ -52,6 +52,7 @@ struct DeviceState {
   bool arch_ok = false;
   int *status_ptr = nullptr;
   int sm_count = 0;
+  int fwd_clusters[2][4] = {};   // forward with clusters of 2, 4, 8 CTAs (entries 1, 2, 3) at d = 64 and d = 128: how many run at once
   // host-buffer entry point only: copy-in and copy-out streams and the events that order them against the caller's stream
   bool pipe_ready = false;
   cudaStream_t in_stream = nullptr, out_stream = nullptr;
@@ -67,6 +68,27 @@ thread_local int tl_launch_count = 0;
 template <typename Kernel>
 cudaError_t allow_smem(Kernel kernel, int bytes) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+
+cudaLaunchAttribute cluster_attr(int size) {
+  cudaLaunchAttribute a = {};
+  a.id = cudaLaunchAttributeClusterDimension;
+  a.val.clusterDim.x = static_cast<unsigned>(size);
+  a.val.clusterDim.y = a.val.clusterDim.z = 1;
+  return a;
+}
+
+// How many clusters of `size` CTAs of `kernel` the device runs at once.
+template <typename... Params>
+cudaError_t max_clusters(void (*kernel)(Params...), int size, int threads, int smem, int *out) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(size));
+  cfg.blockDim = dim3(static_cast<unsigned>(threads));
+  cfg.dynamicSmemBytes = static_cast<size_t>(smem);
+  cudaLaunchAttribute attr = cluster_attr(size);
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaOccupancyMaxActiveClusters(out, kernel, &cfg);
 }
 
 // One-time, per-device set-up: capability check, status word address, shared-memory opt-in.
@@ -118,6 +140,14 @@ int device_state(DeviceState **out) {
       ok &= allow_smem(bwd_dq_kernel<128, false>, BwdCfg<128>::kDqSmemBytes) == cudaSuccess;
       ok &= allow_smem(bwd_dkv_kernel<128, true>, BwdCfg<128>::kDkvSmemBytes) == cudaSuccess;
       ok &= allow_smem(bwd_dkv_kernel<128, false>, BwdCfg<128>::kDkvSmemBytes) == cudaSuccess;
+      ok &= allow_smem(attn_fwd_kernel<64, true, false, 3>, FwdCfg<64>::kSmemBytes) == cudaSuccess;
+      ok &= allow_smem(attn_fwd_kernel<64, false, false, 3>, FwdCfg<64>::kSmemBytes) == cudaSuccess;
+      ok &= allow_smem(attn_fwd_kernel<128, true, false, 3>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
+      ok &= allow_smem(attn_fwd_kernel<128, false, false, 3>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
+      for (int lg = 1; ok && lg < 4; ++lg) {
+        ok &= max_clusters(attn_fwd_kernel<64, true, false, 3>, 1 << lg, FwdCfg<64>::kThreads, FwdCfg<64>::kSmemBytes, &st.fwd_clusters[0][lg]) == cudaSuccess;
+        ok &= max_clusters(attn_fwd_kernel<128, true, false, 3>, 1 << lg, FwdCfg<128>::kThreads, FwdCfg<128>::kSmemBytes, &st.fwd_clusters[1][lg]) == cudaSuccess;
+      }
       if (!ok) { (void)cudaGetLastError(); return GPROJ_ERR_CUDA; }
     }
     st.ready = true;
@@ -168,8 +198,22 @@ void launch_after(void (*kernel)(Params...), dim3 grid, int threads, size_t smem
   (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);   // the caller reads cudaGetLastError()
 }
 
+// Launch `ctas` CTAs in clusters of `size`.
+template <typename... Params, typename... Args>
+void launch_cluster(void (*kernel)(Params...), int ctas, int size, int threads, size_t smem, cudaStream_t s, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(ctas));
+  cfg.blockDim = dim3(static_cast<unsigned>(threads));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr = cluster_attr(size);
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);   // the caller reads cudaGetLastError()
+}
+
 int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE, int B, int H, int Hkv, int N, int Nk, int d,
-               float softmax_scale, int causal, unsigned fwd_flags, const int4 *plan, int n_plan_tiles, void *stream);
+               float softmax_scale, int causal, unsigned fwd_flags, const int4 *plan, int n_plan_tiles, int longest_keys, void *stream);
 int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const float *LSE, const void *dO,
                void *dQ, void *dK, void *dV, int B, int H, int Hkv, int N, int Nk, int d, float softmax_scale, int causal,
                void *workspace, size_t workspace_bytes, unsigned flags, const int4 *plan_q, const int4 *plan_kv,
@@ -197,7 +241,7 @@ int gproj_attn_fwd_gqa(const void *Q, const void *K, const void *V, void *O, flo
 
 int gproj_attn_fwd_ex(const void *Q, const void *K, const void *V, void *O, float *LSE, int B, int H, int Hkv, int N,
                       int d, float softmax_scale, int causal, unsigned fwd_flags, void *stream) {
-  return launch_fwd(Q, K, V, O, LSE, B, H, Hkv, N, N, d, softmax_scale, causal, fwd_flags, nullptr, 0, stream);
+  return launch_fwd(Q, K, V, O, LSE, B, H, Hkv, N, N, d, softmax_scale, causal, fwd_flags, nullptr, 0, 0, stream);
 }
 
 }  // extern "C"
@@ -322,22 +366,45 @@ bool fwd_prefers_single_tiles(int BH, int n_qt, int sms) {
   return t_single < t_pairs;
 }
 
+// CTAs per query tile of the forward (its base-two logarithm): with few tiles and long key ranges a tile's key range is
+// split over a cluster of 2, 4 or 8 CTAs, as many as leave each of their two warpgroups at least two 128-key tiles and let
+// all clusters run at once (`fit`: how many clusters of 2^lg CTAs do).  Beyond one wave the split only adds its merge, and
+// below 16 key tiles the launch and the merge of a cluster (about 6 us) cost what they save.  Measured, one CTA per tile ->
+// cluster: 8 x (16 query, 4 KV heads) x 16 queries behind 16384 keys, d = 64: 109.7 -> 51.8 us (with the query heads
+// folded, see launch_fwd), behind 8192: 58.5 -> 33.0, behind 4096: 33.2 -> 22.9, behind 2048: 20.6 -> 18.6; 4 x 8 heads x 1
+// query behind 16384 keys, d = 128: 201 -> 72 us; 4 heads x 1000 x 128 (8 key tiles): 18.7 -> 20.7 us, hence the 16.
+int fwd_cluster_log2(long long tiles, int key_tiles, const int (&fit)[4]) {
+  int lg = 0;
+  while (lg < 3 && key_tiles >= std::max(16, 4 << (lg + 1)) && tiles <= fit[lg + 1]) ++lg;
+  return lg;
+}
+
 // Dense call: plan == nullptr, one sequence [0, N) per head.  Packed call: B = 1, N = total tokens, plan = device tile
-// list (query order) with n_plan_tiles entries.
+// list (query order) with n_plan_tiles entries, longest_keys = most keys of one sequence.
 int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE, int B, int H, int Hkv, int N, int Nk, int d,
-               float softmax_scale, int causal, unsigned fwd_flags, const int4 *plan, int n_plan_tiles, void *stream) {
+               float softmax_scale, int causal, unsigned fwd_flags, const int4 *plan, int n_plan_tiles, int longest_keys, void *stream) {
   if (!Q || !K || !V || !O || !LSE) return GPROJ_ERR_NULL;
   if (fwd_flags & ~GPROJ_FWD_FLAG_FMA_SOFTMAX) return GPROJ_ERR_FLAGS;
   const bool fma = (fwd_flags & GPROJ_FWD_FLAG_FMA_SOFTMAX) != 0;
   if (int rc = check_shape(B, H, N, d)) return rc;
   if (Hkv <= 0 || H % Hkv != 0 || check_shape(B, Hkv, Nk, d) != GPROJ_OK) return GPROJ_ERR_SHAPE;
-  const int G = H / Hkv;
+  int G = H / Hkv;
   if (!aligned16(Q) || !aligned16(K) || !aligned16(V) || !aligned16(O) || (reinterpret_cast<uintptr_t>(LSE) & 3u))
     return GPROJ_ERR_ALIGN;
   if (!std::isfinite(softmax_scale) || !(softmax_scale > 0.f)) return GPROJ_ERR_SCALE;
   DeviceState *st = nullptr;
   if (int rc = device_state(&st)) return rc;
 
+  // Grouped queries with fewer rows than a tile, or without a mask: the G query heads of a KV head lie end to end in Q, O and
+  // LSE, so they are one head of G N rows; K and V are then read once per KV head and the tiles are full (16 x (32 query, 8
+  // KV heads) x 1 query behind 1000 keys, d = 64: 56.0 -> 18.6 us).
+  int fold = 0;
+  if (!plan && G > 1 && (!causal || (N < 128 && !fma))) {
+    if (causal) fold = N;
+    H = Hkv;
+    N *= G;
+    G = 1;
+  }
   const int BH = B * H;
   const int BHkv = B * Hkv;
   CUtensorMap mQ, mK, mV, mO;
@@ -349,16 +416,28 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
   // that leaves too few items to balance the SMs, items are single tiles.
   const int n_qt = plan ? n_plan_tiles : (N + 127) / 128;
   int tiles_per_item = (!plan && static_cast<long long>(BH) * ((n_qt + 1) / 2) * 2 >= 3LL * st->sm_count) ? 2 : 1;
+  if (fold > 0) tiles_per_item = 1;
   if (tiles_per_item == 2 && d == 64 && causal && N == Nk && fwd_prefers_single_tiles(BH, n_qt, st->sm_count)) tiles_per_item = 1;
   const int total_items = BH * ((n_qt + tiles_per_item - 1) / tiles_per_item);
   if (total_items <= 0) return GPROJ_OK;   // nothing but empty sequences
   const ItemOrder fwd_order = item_order(BH, total_items / BH, tile_group_of(plan != nullptr, causal != 0, BH, total_items / BH, 2 * static_cast<size_t>(BHkv) * Nk * d * 2, st->sm_count,
                                                             tiles_per_item == 2 ? 1.45 : 6.8));
-  const dim3 grid(static_cast<unsigned>(total_items < st->sm_count ? total_items : st->sm_count));   // persistent
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  const int lg = (tiles_per_item == 1 && !fma) ? fwd_cluster_log2(total_items, ((plan ? longest_keys : Nk) + 127) / 128, st->fwd_clusters[d == 128]) : 0;
+  if (lg > 0 || fold > 0) {
+    auto kernel = d == 64 ? (causal ? attn_fwd_kernel<64, true, false, 3> : attn_fwd_kernel<64, false, false, 3>)
+                          : (causal ? attn_fwd_kernel<128, true, false, 3> : attn_fwd_kernel<128, false, false, 3>);
+    launch_cluster(kernel, total_items << lg, 1 << lg, FwdCfg<64>::kThreads, d == 64 ? FwdCfg<64>::kSmemBytes : FwdCfg<128>::kSmemBytes, s,
+                   mQ, mK, mV, mO, static_cast<__nv_bfloat16 *>(O), plan, LSE, N, Nk, BH, H, G, fold, tiles_per_item, total_items, fwd_order, scale_log2,
+                   softmax_scale, st->status_ptr);
+    if (cudaGetLastError() != cudaSuccess) return GPROJ_ERR_CUDA;
+    tl_launch_count = 1;
+    return GPROJ_OK;
+  }
+  const dim3 grid(static_cast<unsigned>(total_items < st->sm_count ? total_items : st->sm_count));   // persistent
 #define GPROJ_LAUNCH_FWD(DD, CC, FF, MM)                                                                            \
   attn_fwd_kernel<DD, CC, FF, MM><<<grid, FwdCfg<DD>::kThreads, FwdCfg<DD>::kSmemBytes, s>>>(                         \
-      mQ, mK, mV, mO, static_cast<__nv_bfloat16 *>(O), plan, LSE, N, Nk, BH, H, G, tiles_per_item, total_items, fwd_order, scale_log2, \
+      mQ, mK, mV, mO, static_cast<__nv_bfloat16 *>(O), plan, LSE, N, Nk, BH, H, G, fold, tiles_per_item, total_items, fwd_order, scale_log2, \
       softmax_scale, st->status_ptr)
 #define GPROJ_LAUNCH_FWD_C(DD, FF, MM)                                                                              \
   do { if (causal) GPROJ_LAUNCH_FWD(DD, true, FF, MM); else GPROJ_LAUNCH_FWD(DD, false, FF, MM); } while (0)
@@ -500,7 +579,7 @@ extern "C" {
 // ---- unequal query and key lengths ------------------------------------------------------------------
 int gproj_attn_fwd_rect(const void *Q, const void *K, const void *V, void *O, float *LSE, int B, int H, int Hkv, int Nq,
                         int Nk, int d, float softmax_scale, int causal, unsigned fwd_flags, void *stream) {
-  return launch_fwd(Q, K, V, O, LSE, B, H, Hkv, Nq, Nk, d, softmax_scale, causal, fwd_flags, nullptr, 0, stream);
+  return launch_fwd(Q, K, V, O, LSE, B, H, Hkv, Nq, Nk, d, softmax_scale, causal, fwd_flags, nullptr, 0, 0, stream);
 }
 
 int gproj_attn_bwd_rect(const void *Q, const void *K, const void *V, const void *O, const float *LSE, const void *dO,
@@ -585,8 +664,10 @@ int fwd_packed(const void *Q, const void *K, const void *V, void *O, float *LSE,
   if (!packed_shape(cu_q, cu_k, num_seqs, &ps)) return GPROJ_ERR_SHAPE;
   if (!plan_device) return GPROJ_ERR_NULL;
   if (reinterpret_cast<uintptr_t>(plan_device) & 15u) return GPROJ_ERR_ALIGN;
+  int longest_keys = 0;
+  for (int q = 0; q < num_seqs; ++q) longest_keys = std::max(longest_keys, cu_k[q + 1] - cu_k[q]);
   return launch_fwd(Q, K, V, O, LSE, 1, H, Hkv, ps.total_q, ps.total_k, d, softmax_scale, causal, fwd_flags,
-                    static_cast<const int4 *>(plan_device), ps.q_tiles, stream);
+                    static_cast<const int4 *>(plan_device), ps.q_tiles, longest_keys, stream);
 }
 
 int bwd_packed(const void *Q, const void *K, const void *V, const void *O, const float *LSE, const void *dO, void *dQ, void *dK,

@@ -393,6 +393,8 @@ __device__ __forceinline__ float bf16_hi_to_f32(uint32_t packed) { return __uint
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
+__device__ __forceinline__ int cluster_size() { uint32_t n; asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(n)); return static_cast<int>(n); }
+__device__ __forceinline__ int cluster_rank() { uint32_t r; asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return static_cast<int>(r); }
 // address of the same shared-memory location in CTA `rank` of the cluster
 __device__ __forceinline__ uint32_t cluster_map_shared(uint32_t addr, int rank) {
   uint32_t out;
@@ -401,6 +403,14 @@ __device__ __forceinline__ uint32_t cluster_map_shared(uint32_t addr, int rank) 
 }
 __device__ __forceinline__ void cluster_load_f4(uint32_t addr, float *v) {
   asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ float cluster_load_f32(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void cluster_store_f4(uint32_t addr, float a, float b, float c, float d) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
 
 // Move registers between warpgroups: every warp of a warpgroup gives back (dec) or takes (inc) registers so that each of its

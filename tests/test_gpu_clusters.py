@@ -1,10 +1,74 @@
-"""Kernels that run as thread-block clusters, at the edges of their dispatch rules (through the C ABI)."""
+"""Kernels that run as thread-block clusters, at the edges of their dispatch rules (through the C ABI, against the oracle).
+
+Tolerances as in the other parity tests: 1 % relative L2 against FP64 (BF16 operands leave 0.2 %), LSE to 1e-4 + 1e-5 |LSE|.
+"""
+import numpy as np
 import pytest
 import torch
 
+import oracle
 import paper_2609_34272_b200 as g
 
 pytestmark = pytest.mark.gpu
+
+
+def tobits(t):
+    return t.contiguous().view(torch.int16).numpy().view(np.uint16)
+
+
+# The forward splits a query tile's key range over 2, 4 or 8 CTAs from 16, 16 and 32 key tiles on, when the tiles are few;
+# grouped queries of fewer than 128 rows (or without a mask) are folded into one head first.
+FWD = [  # B, H, Hkv, Nq, Nk, causal
+    (1, 2, 2, 128, 1921, True), (1, 2, 2, 130, 2048, False), (13, 3, 3, 1, 2047, True), (1, 2, 2, 257, 4100, True),
+    (1, 1, 1, 64, 5000, False), (1, 8, 2, 16, 4096, True), (9, 6, 2, 127, 2500, True), (1, 4, 1, 33, 300, True),
+    (1, 4, 2, 100, 40, True), (1, 6, 2, 200, 2100, False), (1, 8, 1, 1, 1, True), (3, 4, 1, 96, 2049, True),
+]
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("shape", FWD)
+def test_forward_with_the_key_range_split_over_a_cluster(shape, d):
+    B, H, Hkv, Nq, Nk, causal = shape
+    gen = torch.Generator().manual_seed(Nq * 7 + Nk + d)
+    Q = torch.randn(B, H, Nq, d, generator=gen).to(torch.bfloat16)
+    K = (torch.randn(B, Hkv, Nk, d, generator=gen) + 0.5).to(torch.bfloat16)
+    V = torch.randn(B, Hkv, Nk, d, generator=gen).to(torch.bfloat16)
+    ex = oracle.attn_rect_f64(tobits(Q), tobits(K), tobits(V), tobits(torch.zeros_like(Q)), d ** -0.5, causal)
+    q, k, v = Q.cuda(), K.cuda(), V.cuda()
+    O, LSE = torch.full_like(q, float("nan")), torch.full(q.shape[:3], float("nan"), device="cuda")
+    g.gproj_attn_fwd_rect(q, k, v, d ** -0.5, causal, O=O, LSE=LSE)
+    rc, detail = g.gproj_last_device_status()
+    assert rc == 0, hex(detail)
+    O, LSE = O.float().cpu().numpy().astype(np.float64), LSE.cpu().numpy().astype(np.float64)
+    empty = np.isinf(ex["LSE"])
+    assert np.array_equal(np.isposinf(LSE), empty) and np.all(O[empty] == 0.0) and np.all(np.isfinite(O))
+    assert np.all(np.abs(LSE[~empty] - ex["LSE"][~empty]) <= 1e-4 + 1e-5 * np.abs(ex["LSE"][~empty]))
+    assert oracle.rel_l2_percent(O, ex["O"]) <= 1.0
+    assert np.abs(O - ex["O"]).max() <= 0.03 * np.abs(ex["O"]).max()
+
+
+@pytest.mark.parametrize("causal", [True, False])
+def test_packed_forward_with_split_keys_repeats_bitwise(causal):
+    # one long and some short sequences: parts of a tile without any key tile, tiles of different length in one launch
+    lens, H, Hkv, d = [2500, 3, 200, 0, 129], 2, 1, 64
+    gen = torch.Generator().manual_seed(5)
+    T = sum(lens)
+    Q = torch.randn(H, T, d, generator=gen).to(torch.bfloat16)
+    K, V = (torch.randn(Hkv, T, d, generator=gen).to(torch.bfloat16) for _ in range(2))
+    cu = np.concatenate([[0], np.cumsum(lens)])
+    plan = g.VarlenPlan(cu, causal)
+    q, k, v = Q.cuda(), K.cuda(), V.cuda()
+    O, LSE = g.gproj_attn_fwd_varlen(q, k, v, plan, 0.125)
+    for _ in range(5):
+        O2, LSE2 = g.gproj_attn_fwd_varlen(q, k, v, plan, 0.125)
+        assert torch.equal(O, O2) and torch.equal(LSE, LSE2)
+    rc, detail = g.gproj_last_device_status()
+    assert rc == 0, hex(detail)
+    for a, b in zip(cu, cu[1:]):
+        if b > a:
+            part = lambda t: tobits(t[None, :, a:b])
+            ex = oracle.attn_rect_f64(part(Q), part(K), part(V), part(torch.zeros_like(Q)), 0.125, causal)
+            assert oracle.rel_l2_percent(O[:, a:b].float().cpu().numpy()[None], ex["O"]) <= 1.0
 
 
 @pytest.mark.parametrize("rows,d", [(1, 64), (7, 128), (8, 64), (513, 64), (4095, 64), (4097, 64), (2049, 128), (9000, 64)])
