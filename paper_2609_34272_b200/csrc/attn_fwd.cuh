@@ -102,6 +102,12 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   using C = FwdCfg<D>;
   constexpr int S = C::kStages;
   constexpr bool kCluster = (MODE == 3);
+  // Separate K and V rings where the ring is short (two stages at d = 128) and both stages are in use at once (the
+  // warpgroups work on two key tiles): with one ring the next K waited for the whole softmax and P~V of its stage.
+  // Measured, one ring -> two: 8 heads x 4096 x 128, causal: 51.6 -> 44.0 us; 12 packed pairs (4000 queries, 9000 keys, 12
+  // heads): 62.2 -> 51.5 us.  Elsewhere the second commit per key tile and the polling cost more than they give (16 heads
+  // x 4096 x 64: 60.5 -> 62.5 us; pairs at d = 128: 306 us either way; clusters at d = 64: 33.0 -> 38 us).
+  constexpr bool kSepRings = (D == 128 && MODE == 2);
   const int fold = kCluster ? fold_rows : 0;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -109,7 +115,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   uint8_t *sKV = sQ + 2 * C::kTileBytes;            // stage s: K tile, then V tile
 
   __shared__ int s_item[4][2];
-  __shared__ uint64_t bar_q_full[2], bar_q_free[2], bar_k_full[S], bar_v_full[S], bar_kv_empty[S];
+  __shared__ uint64_t bar_q_full[2], bar_q_free[2], bar_k_full[S], bar_v_full[S], bar_k_empty[S], bar_v_empty[S];
   __shared__ uint64_t bar_s_full[2], bar_s_free[2], bar_p_ready[2], bar_pv_done[2], bar_o_free[2], bar_turn[2], bar_merge, bar_drain[2];
   __shared__ float s_m1[2][128], s_l1[2][128];   // split mode: running maximum and normaliser of the second warpgroup, by item parity (with a cluster: of both)
   __shared__ uint32_t tmem_base_smem;
@@ -138,7 +144,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       mbar_init(&bar_q_full[b], 1);
       mbar_init(&bar_q_free[b], tiles_per_item);    // one arrival per query tile slot: its O store has left shared memory
     }
-    for (int s = 0; s < S; ++s) { mbar_init(&bar_k_full[s], 1); mbar_init(&bar_v_full[s], 1); mbar_init(&bar_kv_empty[s], 1); }
+    for (int s = 0; s < S; ++s) { mbar_init(&bar_k_full[s], 1); mbar_init(&bar_v_full[s], 1); mbar_init(&bar_k_empty[s], 1); mbar_init(&bar_v_empty[s], 1); }
     for (int t = 0; t < 2; ++t) {
       mbar_init(&bar_drain[t], 1);
       mbar_init(&bar_s_full[t], 1); mbar_init(&bar_s_free[t], 128); mbar_init(&bar_p_ready[t], 128); mbar_init(&bar_pv_done[t], 1); mbar_init(&bar_o_free[t], 128); mbar_init(&bar_turn[t], 128);
@@ -191,7 +197,57 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer of K_j, V_j
-    if (lane == 0) {
+    // With separate rings a K tile is free as soon as its scores are complete, a V tile only when the probabilities of its
+    // key tile have been multiplied, a whole softmax later.  One thread feeds both rings and takes whichever has a free
+    // slot, so the next K is on its way while a V slot is still busy.
+    if (kSepRings && lane == 0) {
+      struct Cursor {
+        TileSched sched;
+        Item it;
+        int j, kvh, g;
+        bool more;
+      };
+      auto next_item = [&](Cursor &c) {
+        const int lin = c.sched.next();
+        c.more = lin >= 0;
+        if (!c.more) return;
+        c.it = decode(lin);
+        c.kvh = kv_head_of(hix(lin), Hq, G);                 // grouped-query: the group's shared K / V head
+        c.j = 0;
+      };
+      auto settle = [&](Cursor &c) {                         // on to the next key tile of this CTA's
+        while (c.more && !(c.j < c.it.n_kt && mine(c.j))) { if (c.j + 1 < c.it.n_kt) ++c.j; else next_item(c); }
+      };
+      auto feed = [&](Cursor &c, uint64_t *full, uint64_t *empty, const CUtensorMap *map, uint8_t *ring) {
+        const int st = c.g % S;
+        if (!c.more || (c.g >= S && !mbar_test_wait(&empty[st], ((c.g / S) - 1) & 1))) return false;
+        mbar_expect_tx(&full[st], C::kTileBytes);
+        for (int s = 0; s < C::kSlabs; ++s)
+          tma_load_3d(ring + st * 2 * C::kTileBytes + s * C::kSlabBytes, map, &full[st], s * 64, c.it.kseq0 + c.j * C::kBlockN, c.kvh);
+        ++c.g;
+        ++c.j;
+        settle(c);
+        return true;
+      };
+      Cursor ck{sched, Item{}, 0, 0, 0, true}, cv = ck;
+      next_item(ck); settle(ck);
+      cv = ck;
+      BoundedIdle idle;
+      while (ck.more || cv.more) {
+        const bool fed_k = feed(ck, bar_k_full, bar_k_empty, &tmK, sKV);
+        const bool fed_v = feed(cv, bar_v_full, bar_v_empty, &tmV, sKV + C::kTileBytes);
+        if (!idle.go_on(fed_k || fed_v, ab, kFwdWaitKVEmpty)) break;
+      }
+      // Every load is consumed by an MMA the epilogue waits for, so nothing is in flight at exit unless the
+      // CTA aborted; then give the copies a bounded chance to land before shared memory is released.
+      if (cta_abort) {
+        for (int q = (ck.g > S ? ck.g - S : 0); q < ck.g; ++q)
+          for (int spin = 0; spin < 100000 && !mbar_try_wait(&bar_k_full[q % S], (q / S) & 1); ++spin) {}
+        for (int q = (cv.g > S ? cv.g - S : 0); q < cv.g; ++q)
+          for (int spin = 0; spin < 100000 && !mbar_try_wait(&bar_v_full[q % S], (q / S) & 1); ++spin) {}
+      }
+    }
+    if (!kSepRings && lane == 0) {
       int g = 0;
       for (int lin = sched.next(); lin >= 0; lin = sched.next()) {
         const Item it = decode(lin);
@@ -199,7 +255,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         for (int j = 0; j < T; ++j) {
           if (!mine(j)) continue;
           const int st = g % S;
-          if (g >= S) mbar_wait(&bar_kv_empty[st], ((g / S) - 1) & 1, ab, kFwdWaitKVEmpty);
+          if (g >= S) mbar_wait(&bar_v_empty[st], ((g / S) - 1) & 1, ab, kFwdWaitKVEmpty);
           uint8_t *dK = sKV + st * 2 * C::kTileBytes, *dV = dK + C::kTileBytes;
           const int kvh = kv_head_of(bh, Hq, G), krow = it.kseq0 + j * C::kBlockN;   // grouped-query: the group's shared K / V head
           mbar_expect_tx(&bar_k_full[st], C::kTileBytes);
@@ -209,8 +265,6 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           ++g;
         }
       }
-      // Every load is consumed by an MMA the epilogue waits for, so nothing is in flight at exit unless the
-      // CTA aborted; then give the copies a bounded chance to land before shared memory is released.
       if (cta_abort) {
         for (int q = (g > S ? g - S : 0); q < g; ++q) {
           for (int spin = 0; spin < 100000 && !mbar_try_wait(&bar_k_full[q % S], (q / S) & 1); ++spin) {}
@@ -281,6 +335,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           __syncwarp();
           ++cnt[t];
         }
+        if (kSepRings) {
+          if (elect_one_sync()) umma_commit(&bar_k_empty[st]);   // every score product that reads this K tile has been issued
+          __syncwarp();
+        }
         ++g;
       }
     }
@@ -316,7 +374,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           __syncwarp();
           ++cnt[t];
         }
-        if (elect_one_sync()) umma_commit(&bar_kv_empty[st]);    // every MMA that reads this K / V stage has been issued
+        if (elect_one_sync()) umma_commit(&bar_v_empty[st]);     // every product that reads this V tile has been issued
         __syncwarp();
         ++g;
       }

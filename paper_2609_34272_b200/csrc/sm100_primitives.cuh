@@ -127,6 +127,40 @@ __device__ __forceinline__ void mbar_wait(uint64_t *bar, uint32_t parity, const 
   }
 }
 
+// Has the phase completed?  Never suspends the thread (try_wait may), for a thread that watches several barriers.
+__device__ __forceinline__ bool mbar_test_wait(uint64_t *bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred P;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 P, [%1], %2;\n\t"
+      "selp.b32 %0, 1, 0, P;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
+// The bound of mbar_wait for a thread that polls several barriers: go_on() returns false when the CTA has aborted or
+// nothing has progressed for the whole budget (then it raises the abort itself).
+struct BoundedIdle {
+  long long since = 0;
+  uint32_t spins = 0;
+  __device__ __forceinline__ bool go_on(bool progressed, const AbortState &ab, int code) {
+    if (progressed) { spins = 0; return true; }
+    if (++spins == 1) since = clock64();
+    __nanosleep(40);                 // leave the issue slots to the warps that compute
+    if ((spins & 0x3ff) == 0) {
+      if (*ab.cta_abort) return false;
+      if (clock64() - since > kWaitBudgetCycles) {
+        *ab.cta_abort = 1;
+        atomicCAS(ab.global_status, 0, kDevTimeout | (code << 8));
+        return false;
+      }
+    }
+    return true;
+  }
+};
+
 // ------------------------------------------------------------------------------------------
 // TMA: 2-D tiled load global -> shared, completion on an mbarrier
 // ------------------------------------------------------------------------------------------
