@@ -966,7 +966,7 @@ int gproj_fp32_attn_fwd(const void *Q, const void *K, const void *V, void *O, vo
   if (int rc = device_state(&st)) return rc;
   const size_t rows = static_cast<size_t>(B) * H * N;
   float *O32 = static_cast<float *>(saved), *stats = O32 + rows * d;
-  const dim3 grid(static_cast<unsigned>((N + 63) / 64), static_cast<unsigned>(B * H));
+  const dim3 grid(static_cast<unsigned>((N + 31) / 32) * static_cast<unsigned>(B * H));   // 32-row tiles x heads, below 2^31 with B H N
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   auto q = static_cast<const __nv_bfloat16 *>(Q); auto k = static_cast<const __nv_bfloat16 *>(K); auto v = static_cast<const __nv_bfloat16 *>(V);
   auto o = static_cast<__nv_bfloat16 *>(O);
@@ -974,7 +974,7 @@ int gproj_fp32_attn_fwd(const void *Q, const void *K, const void *V, void *O, vo
   do {                                                                                                             \
     if (cudaFuncSetAttribute(fp32_attn_fwd_kernel<DD, CC>, cudaFuncAttributeMaxDynamicSharedMemorySize, Fp32Cfg<DD>::kFwdSmem) != cudaSuccess) \
       return GPROJ_ERR_CUDA;                                                                                       \
-    fp32_attn_fwd_kernel<DD, CC><<<grid, 128, Fp32Cfg<DD>::kFwdSmem, s>>>(q, k, v, o, O32, stats, N, softmax_scale); \
+    fp32_attn_fwd_kernel<DD, CC><<<grid, Fp32Cfg<DD>::kThreads, Fp32Cfg<DD>::kFwdSmem, s>>>(q, k, v, o, O32, stats, N, B * H, softmax_scale); \
   } while (0)
   if (d == 64) { if (causal) GPROJ_FP32_FWD(64, true); else GPROJ_FP32_FWD(64, false); }
   else         { if (causal) GPROJ_FP32_FWD(128, true); else GPROJ_FP32_FWD(128, false); }
@@ -992,17 +992,17 @@ int gproj_fp32_attn_bwd(const void *Q, const void *K, const void *V, const void 
   if (int rc = device_state(&st)) return rc;
   const size_t rows = static_cast<size_t>(B) * H * N;
   float *O32 = static_cast<float *>(saved), *stats = O32 + rows * d, *Drow = stats + 3 * rows;
-  const dim3 grid(static_cast<unsigned>((N + 63) / 64), static_cast<unsigned>(B * H));
+  const dim3 grid(static_cast<unsigned>((N + 31) / 32) * static_cast<unsigned>(B * H));   // 32-row tiles x heads, below 2^31 with B H N
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   auto q = static_cast<const __nv_bfloat16 *>(Q); auto k = static_cast<const __nv_bfloat16 *>(K); auto v = static_cast<const __nv_bfloat16 *>(V);
   auto u = static_cast<const __nv_bfloat16 *>(dO);
 #define GPROJ_FP32_BWD(DD, CC)                                                                                     \
   do {                                                                                                             \
-    if (cudaFuncSetAttribute(fp32_attn_dq_kernel<DD, CC>, cudaFuncAttributeMaxDynamicSharedMemorySize, Fp32Cfg<DD>::kBwdSmem) != cudaSuccess || \
-        cudaFuncSetAttribute(fp32_attn_dkv_kernel<DD, CC>, cudaFuncAttributeMaxDynamicSharedMemorySize, Fp32Cfg<DD>::kBwdSmem) != cudaSuccess) \
+    if (cudaFuncSetAttribute(fp32_attn_dq_kernel<DD, CC>, cudaFuncAttributeMaxDynamicSharedMemorySize, Fp32Cfg<DD>::kDqSmem) != cudaSuccess || \
+        cudaFuncSetAttribute(fp32_attn_dkv_kernel<DD, CC>, cudaFuncAttributeMaxDynamicSharedMemorySize, Fp32Cfg<DD>::kDkvSmem) != cudaSuccess) \
       return GPROJ_ERR_CUDA;                                                                                       \
-    fp32_attn_dq_kernel<DD, CC><<<grid, 128, Fp32Cfg<DD>::kBwdSmem, s>>>(q, k, v, u, O32, stats, Drow, static_cast<__nv_bfloat16 *>(dQ), N, softmax_scale); \
-    fp32_attn_dkv_kernel<DD, CC><<<grid, 128, Fp32Cfg<DD>::kBwdSmem, s>>>(q, k, v, u, stats, Drow, static_cast<__nv_bfloat16 *>(dK), static_cast<__nv_bfloat16 *>(dV), N, softmax_scale); \
+    fp32_attn_dq_kernel<DD, CC><<<grid, Fp32Cfg<DD>::kThreads, Fp32Cfg<DD>::kDqSmem, s>>>(q, k, v, u, O32, stats, Drow, static_cast<__nv_bfloat16 *>(dQ), N, B * H, softmax_scale); \
+    fp32_attn_dkv_kernel<DD, CC><<<grid, Fp32Cfg<DD>::kThreads, Fp32Cfg<DD>::kDkvSmem, s>>>(q, k, v, u, stats, Drow, static_cast<__nv_bfloat16 *>(dK), static_cast<__nv_bfloat16 *>(dV), N, B * H, softmax_scale); \
   } while (0)
   if (d == 64) { if (causal) GPROJ_FP32_BWD(64, true); else GPROJ_FP32_BWD(64, false); }
   else         { if (causal) GPROJ_FP32_BWD(128, true); else GPROJ_FP32_BWD(128, false); }
