@@ -413,8 +413,10 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
   tc_fence_after();
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, tmem_base_smem, 0);   // the shuffle marks it warp-uniform
 
-  // The dK/dV-side kernel that follows in the stream may be scheduled on SMs this kernel has left: its set-up and its
+  // Everything so far may have run beside the kernel before this one in the stream; its memory is visible from here on.
+  // The dK/dV-side kernel that follows may then be scheduled on SMs this kernel has left: its set-up and its
   // stationary-tile loads need nothing from here, and it waits (griddep_wait) before it reads the statistics and Z.
+  griddep_wait();
   griddep_launch_dependents();
 
   TileSched sched(total_tiles);
@@ -800,6 +802,7 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 rows
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, tmem_base_smem, 0);
+  griddep_launch_dependents();   // the next kernel in the stream may set itself up beside this one
 
   TileSched sched(total_tiles);
   // tile decode: causal -> key tile 0 has the most query steps and comes first

@@ -179,6 +179,7 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, tmem_base_smem, 0);
+  griddep_launch_dependents();   // the next kernel in the stream may set itself up beside this one
 
   TileSched sched(total_tiles);
   // A step may reach past the end of the sequence: those query columns are zero fill or the next packed sequence's rows,

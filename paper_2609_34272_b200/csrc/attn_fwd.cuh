@@ -158,6 +158,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   tc_fence_after();
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, tmem_base_smem, 0);   // the shuffle marks it warp-uniform
 
+  // Everything so far may have run beside the kernel before this one in the stream; its memory is visible from here on.
+  griddep_wait();
+  griddep_launch_dependents();
+
   // Work items ordered by decreasing work (causal: last pair first).  Item -> (sequence, first query tile, tiles) and head.
   // Dense calls: one sequence [0, N) per head, items are pairs (or single tiles); packed calls: single tiles from the plan.
   // qt0: index of the first query tile inside its sequence; nq: query tiles; n_kt: key tiles walked; kseq0, klen: the keys.
