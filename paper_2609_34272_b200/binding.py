@@ -116,22 +116,62 @@ def status_string(status: int) -> str:
     return load().gproj_status_string(int(status)).decode()
 
 
+_BF16, _F32, _U8 = torch.bfloat16, torch.float32, torch.uint8
+
+
 def _check_bf16(name, t, shape=None):
-    if not (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype == torch.bfloat16 and t.is_contiguous()):
+    if not (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype is _BF16 and t.is_contiguous()):
         raise TypeError(f"{name} must be a contiguous CUDA bfloat16 tensor")
-    if shape is not None and tuple(t.shape) != tuple(shape):
+    if shape is not None and t.shape != shape:
         raise ValueError(f"{name} has shape {tuple(t.shape)}, expected {tuple(shape)}")
 
 
-def _kv_heads(Q, K):
-    B, H, N, d = Q.shape
-    if K.dim() != 4 or K.shape[0] != B or K.shape[2] != N or K.shape[3] != d or H % K.shape[1] != 0:
-        raise ValueError(f"K/V shape {tuple(K.shape)} does not match Q {tuple(Q.shape)} (need [B, Hkv, N, d], H % Hkv == 0)")
-    return K.shape[1]
+def _kv_heads(q_shape, K):
+    B, H, N, d = q_shape
+    k = K.shape
+    if len(k) != 4 or k[0] != B or k[2] != N or k[3] != d or H % k[1] != 0:
+        raise ValueError(f"K/V shape {tuple(k)} does not match Q {tuple(q_shape)} (need [B, Hkv, N, d], H % Hkv == 0)")
+    return k[1]
+
+
+def _output(name, t, like):
+    """The caller's output tensor, checked (a wrong one would be overwritten out of bounds), or a new one."""
+    if t is None:
+        return torch.empty_like(like)
+    _check_bf16(name, t, like.shape)
+    return t
+
+
+class _Here:
+    """Stands in for torch.cuda.device() where the tensors' device is the current one already."""
+
+    def __enter__(self):
+        return None
+
+    def __exit__(self, *exc):
+        return False
+
+
+_HERE = _Here()
+
+
+def _on_device(index):
+    """Context in which the CUDA device `index` is current; entering it costs nothing when it is."""
+    return _HERE if torch.cuda.current_device() == index else torch.cuda.device(index)
 
 
 def _stream(device):
     return ctypes.c_void_p(torch.cuda.current_stream(device).cuda_stream)
+
+
+def _raw_stream(index):
+    """Handle of the current stream of device `index`, without a torch.cuda.Stream object around it (2.3 -> 0.1 us)."""
+    return torch._C._cuda_getCurrentRawStream(index)
+
+
+def _check_lse(LSE, shape, what):
+    if not (LSE.is_cuda and LSE.dtype is _F32 and LSE.is_contiguous() and LSE.shape == shape):
+        raise TypeError(f"LSE must be a contiguous CUDA float32 tensor [{what}]")
 
 
 def gproj_attn_bwd_workspace_bytes(B, H, N, d) -> int:
@@ -142,24 +182,20 @@ def gproj_attn_fwd(Q, K, V, softmax_scale, causal, O=None, LSE=None, fwd_flags=0
     """O, LSE = attention forward.  Q: CUDA bfloat16 [B, H, N, d]; K, V: [B, Hkv, N, d] with H a multiple of Hkv
     (Hkv < H = grouped-query attention)."""
     _check_bf16("Q", Q)
-    B, H, N, d = Q.shape
+    shape = Q.shape
+    B, H, N, d = shape
     _check_bf16("K", K); _check_bf16("V", V, K.shape)
-    Hkv = _kv_heads(Q, K)
+    Hkv = _kv_heads(shape, K)
     if O is None:
         O = torch.empty_like(Q)
+    else:
+        _check_bf16("O", O, shape)
     if LSE is None:
-        LSE = torch.empty((B, H, N), dtype=torch.float32, device=Q.device)
-    _check_bf16("O", O, Q.shape)
-    with torch.cuda.device(Q.device):
-        if fwd_flags:
-            rc = load().gproj_attn_fwd_ex(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), LSE.data_ptr(), B, H, Hkv, N, d,
-                                          float(softmax_scale), int(bool(causal)), int(fwd_flags), _stream(Q.device))
-        elif Hkv == H:
-            rc = load().gproj_attn_fwd(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), LSE.data_ptr(),
-                                       B, H, N, d, float(softmax_scale), int(bool(causal)), _stream(Q.device))
-        else:
-            rc = load().gproj_attn_fwd_gqa(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), LSE.data_ptr(),
-                                           B, H, Hkv, N, d, float(softmax_scale), int(bool(causal)), _stream(Q.device))
+        LSE = Q.new_empty((B, H, N), dtype=_F32)
+    index = Q.get_device()
+    with _on_device(index):
+        rc = (_lib or load()).gproj_attn_fwd_ex(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), LSE.data_ptr(), B, H, Hkv, N, d,
+                                                float(softmax_scale), bool(causal), int(fwd_flags), _raw_stream(index))
     if rc != GPROJ_OK:
         raise GprojError(rc, "gproj_attn_fwd")
     return O, LSE
@@ -169,31 +205,23 @@ def gproj_attn_bwd(Q, K, V, O, LSE, dO, softmax_scale, causal, flags=0, workspac
     """dQ, dK, dV = attention backward with the GProj correction (flags: FLAG_NO_*_CORRECTION).
     K, V (and dK, dV) may have fewer heads than Q (grouped-query attention)."""
     _check_bf16("Q", Q)
-    B, H, N, d = Q.shape
-    _check_bf16("K", K); _check_bf16("V", V, K.shape)
-    Hkv = _kv_heads(Q, K)
-    for name, t in (("O", O), ("dO", dO)):
-        _check_bf16(name, t, Q.shape)
-    if not (LSE.is_cuda and LSE.dtype == torch.float32 and LSE.is_contiguous() and tuple(LSE.shape) == (B, H, N)):
-        raise TypeError("LSE must be a contiguous CUDA float32 tensor [B, H, N]")
-    need = gproj_attn_bwd_workspace_bytes(B, H, N, d)
+    shape, kv_shape = Q.shape, K.shape
+    B, H, N, d = shape
+    _check_bf16("K", K); _check_bf16("V", V, kv_shape); _check_bf16("O", O, shape); _check_bf16("dO", dO, shape)
+    Hkv = _kv_heads(shape, K)
+    _check_lse(LSE, (B, H, N), "B, H, N")
+    lib = _lib or load()
     if workspace is None:
-        workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=Q.device)
-    dQ = torch.empty_like(Q) if dQ is None else dQ
-    dK = torch.empty_like(K) if dK is None else dK
-    dV = torch.empty_like(K) if dV is None else dV
-    _check_bf16("dQ", dQ, Q.shape); _check_bf16("dK", dK, K.shape); _check_bf16("dV", dV, K.shape)
-    with torch.cuda.device(Q.device):
-        if Hkv == H:
-            rc = load().gproj_attn_bwd(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), LSE.data_ptr(), dO.data_ptr(),
-                                       dQ.data_ptr(), dK.data_ptr(), dV.data_ptr(), B, H, N, d, float(softmax_scale),
-                                       int(bool(causal)), workspace.data_ptr(), workspace.numel() * workspace.element_size(),
-                                       int(flags), _stream(Q.device))
-        else:
-            rc = load().gproj_attn_bwd_gqa(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), LSE.data_ptr(),
-                                           dO.data_ptr(), dQ.data_ptr(), dK.data_ptr(), dV.data_ptr(), B, H, Hkv, N, d,
-                                           float(softmax_scale), int(bool(causal)), workspace.data_ptr(),
-                                           workspace.numel() * workspace.element_size(), int(flags), _stream(Q.device))
+        nbytes = max(lib.gproj_attn_bwd_workspace_bytes(B, H, N, d), 256)
+        workspace = Q.new_empty(nbytes, dtype=_U8)
+    else:
+        nbytes = workspace.numel() * workspace.element_size()
+    dQ = _output("dQ", dQ, Q); dK = _output("dK", dK, K); dV = _output("dV", dV, K)
+    index = Q.get_device()
+    with _on_device(index):
+        rc = lib.gproj_attn_bwd_gqa(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), LSE.data_ptr(), dO.data_ptr(), dQ.data_ptr(),
+                                    dK.data_ptr(), dV.data_ptr(), B, H, Hkv, N, d, float(softmax_scale), bool(causal),
+                                    workspace.data_ptr(), nbytes, int(flags), _raw_stream(index))
     if rc != GPROJ_OK:
         raise GprojError(rc, "gproj_attn_bwd")
     return dQ, dK, dV
@@ -213,11 +241,11 @@ def gproj_attn_fwd_rect(Q, K, V, softmax_scale, causal, O=None, LSE=None, fwd_fl
     j <= i + (Nk - Nq); a query that sees none gets O = 0 and LSE = +inf."""
     B, H, Hkv, Nq, Nk, d = _rect_shapes(Q, K, V)
     O = torch.empty_like(Q) if O is None else O
-    LSE = torch.empty((B, H, Nq), dtype=torch.float32, device=Q.device) if LSE is None else LSE
+    LSE = Q.new_empty((B, H, Nq), dtype=_F32) if LSE is None else LSE
     _check_bf16("O", O, Q.shape)
-    with torch.cuda.device(Q.device):
+    with _on_device(Q.get_device()):
         rc = load().gproj_attn_fwd_rect(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), LSE.data_ptr(), B, H, Hkv, Nq, Nk, d,
-                                        float(softmax_scale), int(bool(causal)), int(fwd_flags), _stream(Q.device))
+                                        float(softmax_scale), int(bool(causal)), int(fwd_flags), _raw_stream(Q.get_device()))
     if rc != GPROJ_OK:
         raise GprojError(rc, "gproj_attn_fwd_rect")
     return O, LSE
@@ -228,19 +256,15 @@ def gproj_attn_bwd_rect(Q, K, V, O, LSE, dO, softmax_scale, causal, flags=0, wor
     B, H, Hkv, Nq, Nk, d = _rect_shapes(Q, K, V)
     for name, t in (("O", O), ("dO", dO)):
         _check_bf16(name, t, Q.shape)
-    if not (LSE.is_cuda and LSE.dtype == torch.float32 and LSE.is_contiguous() and tuple(LSE.shape) == (B, H, Nq)):
-        raise TypeError("LSE must be a contiguous CUDA float32 tensor [B, H, Nq]")
+    _check_lse(LSE, (B, H, Nq), "B, H, Nq")
     if workspace is None:
-        workspace = torch.empty(max(gproj_attn_bwd_workspace_bytes(B, H, Nq, d), 256), dtype=torch.uint8, device=Q.device)
-    dQ = torch.empty_like(Q) if dQ is None else dQ
-    dK = torch.empty_like(K) if dK is None else dK
-    dV = torch.empty_like(K) if dV is None else dV
-    _check_bf16("dQ", dQ, Q.shape); _check_bf16("dK", dK, K.shape); _check_bf16("dV", dV, K.shape)
-    with torch.cuda.device(Q.device):
+        workspace = Q.new_empty(max(gproj_attn_bwd_workspace_bytes(B, H, Nq, d), 256), dtype=_U8)
+    dQ = _output("dQ", dQ, Q); dK = _output("dK", dK, K); dV = _output("dV", dV, K)
+    with _on_device(Q.get_device()):
         rc = load().gproj_attn_bwd_rect(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), LSE.data_ptr(), dO.data_ptr(),
                                         dQ.data_ptr(), dK.data_ptr(), dV.data_ptr(), B, H, Hkv, Nq, Nk, d, float(softmax_scale),
                                         int(bool(causal)), workspace.data_ptr(), workspace.numel() * workspace.element_size(),
-                                        int(flags), _stream(Q.device))
+                                        int(flags), _raw_stream(Q.get_device()))
     if rc != GPROJ_OK:
         raise GprojError(rc, "gproj_attn_bwd_rect")
     return dQ, dK, dV
@@ -258,17 +282,12 @@ def gproj_attn_bwd_static_scratch(Q, K, V, O, LSE, dO, softmax_scale, causal, fl
     B, H, N, d = Q.shape
     for name, t in (("K", K), ("V", V), ("O", O), ("dO", dO)):
         _check_bf16(name, t, Q.shape)
-    if not (LSE.is_cuda and LSE.dtype == torch.float32 and LSE.is_contiguous() and tuple(LSE.shape) == (B, H, N)):
-        raise TypeError("LSE must be a contiguous CUDA float32 tensor [B, H, N]")
-    dQ = torch.empty_like(Q) if dQ is None else dQ
-    dK = torch.empty_like(Q) if dK is None else dK
-    dV = torch.empty_like(Q) if dV is None else dV
-    for name, t in (("dQ", dQ), ("dK", dK), ("dV", dV)):      # a wrong output tensor would be overwritten out of bounds
-        _check_bf16(name, t, Q.shape)
-    with torch.cuda.device(Q.device):
+    _check_lse(LSE, (B, H, N), "B, H, N")
+    dQ = _output("dQ", dQ, Q); dK = _output("dK", dK, Q); dV = _output("dV", dV, Q)
+    with _on_device(Q.get_device()):
         rc = load().gproj_attn_bwd_static_scratch(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), LSE.data_ptr(),
                                                   dO.data_ptr(), dQ.data_ptr(), dK.data_ptr(), dV.data_ptr(), B, H, N, d,
-                                                  float(softmax_scale), int(bool(causal)), int(flags), _stream(Q.device))
+                                                  float(softmax_scale), int(bool(causal)), int(flags), _raw_stream(Q.get_device()))
     if rc != GPROJ_OK:
         raise GprojError(rc, "gproj_attn_bwd_static_scratch")
     return dQ, dK, dV
@@ -281,11 +300,11 @@ def gproj_fp32_attn_fwd(Q, K, V, softmax_scale, causal, saved=None):
     _check_bf16("K", K, Q.shape); _check_bf16("V", V, Q.shape)
     need = int(load().gproj_fp32_attn_saved_bytes(B, H, N, d))
     if saved is None:
-        saved = torch.empty(max(need, 256), dtype=torch.uint8, device=Q.device)
+        saved = Q.new_empty(max(need, 256), dtype=_U8)
     O = torch.empty_like(Q)
-    with torch.cuda.device(Q.device):
+    with _on_device(Q.get_device()):
         rc = load().gproj_fp32_attn_fwd(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), saved.data_ptr(), saved.numel(),
-                                        B, H, N, d, float(softmax_scale), int(bool(causal)), _stream(Q.device))
+                                        B, H, N, d, float(softmax_scale), int(bool(causal)), _raw_stream(Q.get_device()))
     if rc != GPROJ_OK:
         raise GprojError(rc, "gproj_fp32_attn_fwd")
     return O, saved
@@ -298,10 +317,10 @@ def gproj_fp32_attn_bwd(Q, K, V, dO, saved, softmax_scale, causal):
     for name, t in (("K", K), ("V", V), ("dO", dO)):
         _check_bf16(name, t, Q.shape)
     dQ, dK, dV = torch.empty_like(Q), torch.empty_like(Q), torch.empty_like(Q)
-    with torch.cuda.device(Q.device):
+    with _on_device(Q.get_device()):
         rc = load().gproj_fp32_attn_bwd(Q.data_ptr(), K.data_ptr(), V.data_ptr(), dO.data_ptr(), saved.data_ptr(), saved.numel(),
                                         dQ.data_ptr(), dK.data_ptr(), dV.data_ptr(), B, H, N, d, float(softmax_scale),
-                                        int(bool(causal)), _stream(Q.device))
+                                        int(bool(causal)), _raw_stream(Q.get_device()))
     if rc != GPROJ_OK:
         raise GprojError(rc, "gproj_fp32_attn_bwd")
     return dQ, dK, dV
@@ -313,14 +332,14 @@ def gproj_key_smooth(X, Y=None, cu_seqlens=None):
     _check_bf16("X", X)
     Y = torch.empty_like(X) if Y is None else Y
     _check_bf16("Y", Y, X.shape)
-    with torch.cuda.device(X.device):
+    with _on_device(X.get_device()):
         if cu_seqlens is None:
             B, Hkv, N, d = X.shape
-            rc = load().gproj_key_smooth(X.data_ptr(), Y.data_ptr(), B, Hkv, N, d, _stream(X.device))
+            rc = load().gproj_key_smooth(X.data_ptr(), Y.data_ptr(), B, Hkv, N, d, _raw_stream(X.get_device()))
         else:
             Hkv, T, d = X.shape
             cu = (ctypes.c_int * len(cu_seqlens))(*[int(v) for v in cu_seqlens])
-            rc = load().gproj_key_smooth_varlen(X.data_ptr(), Y.data_ptr(), cu, len(cu_seqlens) - 1, Hkv, d, _stream(X.device))
+            rc = load().gproj_key_smooth_varlen(X.data_ptr(), Y.data_ptr(), cu, len(cu_seqlens) - 1, Hkv, d, _raw_stream(X.get_device()))
     if rc != GPROJ_OK:
         raise GprojError(rc, "gproj_key_smooth")
     return Y
@@ -390,11 +409,11 @@ def gproj_attn_fwd_varlen(Q, K, V, plan, softmax_scale, fwd_flags=0):
     if K.dim() != 3 or K.shape[1] != T or K.shape[2] != d or H % K.shape[0] != 0 or T != plan.total:
         raise ValueError("packed K/V must be [Hkv, T, d] with T = cu_seqlens[-1] and H a multiple of Hkv")
     O = torch.empty_like(Q)
-    LSE = torch.empty((H, T), dtype=torch.float32, device=Q.device)
-    with torch.cuda.device(Q.device):
+    LSE = Q.new_empty((H, T), dtype=_F32)
+    with _on_device(Q.get_device()):
         rc = load().gproj_attn_fwd_varlen(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), LSE.data_ptr(), plan.cu,
                                           plan.num_seqs, plan.device.data_ptr(), H, K.shape[0], d, float(softmax_scale),
-                                          int(plan.causal), int(fwd_flags), _stream(Q.device))
+                                          int(plan.causal), int(fwd_flags), _raw_stream(Q.get_device()))
     if rc != GPROJ_OK:
         raise GprojError(rc, "gproj_attn_fwd_varlen")
     return O, LSE
@@ -407,17 +426,16 @@ def gproj_attn_bwd_varlen(Q, K, V, O, LSE, dO, plan, softmax_scale, flags=0, wor
     for name, t in (("O", O), ("dO", dO)):
         _check_bf16(name, t, Q.shape)
     _check_bf16("K", K); _check_bf16("V", V, K.shape)
-    if not (LSE.is_cuda and LSE.dtype == torch.float32 and LSE.is_contiguous() and tuple(LSE.shape) == (H, T)):
-        raise TypeError("LSE must be a contiguous CUDA float32 tensor [H, T]")
+    _check_lse(LSE, (H, T), "H, T")
     need = int(load().gproj_attn_bwd_varlen_workspace_bytes(plan.cu, plan.num_seqs, H, d))
     if workspace is None:
-        workspace = torch.empty(need, dtype=torch.uint8, device=Q.device)
+        workspace = Q.new_empty(need, dtype=_U8)
     dQ, dK, dV = torch.empty_like(Q), torch.empty_like(K), torch.empty_like(V)
-    with torch.cuda.device(Q.device):
+    with _on_device(Q.get_device()):
         rc = load().gproj_attn_bwd_varlen(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), LSE.data_ptr(), dO.data_ptr(),
                                           dQ.data_ptr(), dK.data_ptr(), dV.data_ptr(), plan.cu, plan.num_seqs,
                                           plan.device.data_ptr(), H, K.shape[0], d, float(softmax_scale), int(plan.causal),
-                                          workspace.data_ptr(), workspace.numel(), int(flags), _stream(Q.device))
+                                          workspace.data_ptr(), workspace.numel(), int(flags), _raw_stream(Q.get_device()))
     if rc != GPROJ_OK:
         raise GprojError(rc, "gproj_attn_bwd_varlen")
     return dQ, dK, dV
@@ -438,10 +456,10 @@ def gproj_attn_fwd_bwd_host(Q, K, V, dO, dQ, dK, dV, softmax_scale, causal, stag
     if not (staging.is_cuda and staging.dtype == torch.uint8 and staging.is_contiguous()):
         raise TypeError("staging must be a contiguous CUDA uint8 tensor")
     ptr = lambda t: ctypes.c_void_p(t.data_ptr()) if t is not None else None
-    with torch.cuda.device(staging.device):
+    with _on_device(staging.get_device()):
         rc = load().gproj_attn_fwd_bwd_host(ptr(Q), ptr(K), ptr(V), ptr(dO), ptr(O), ptr(LSE), ptr(dQ), ptr(dK), ptr(dV), B, H, Hkv, N, d,
                                             float(softmax_scale), int(bool(causal)), ptr(staging), staging.numel(), int(flags),
-                                            _stream(staging.device))
+                                            _raw_stream(staging.get_device()))
     if rc != GPROJ_OK:
         raise GprojError(rc, "gproj_attn_fwd_bwd_host")
 
@@ -461,11 +479,11 @@ def gproj_attn_fwd_varlen_qk(Q, K, V, plan, softmax_scale, fwd_flags=0):
     """O, LSE = forward over packed sequences with their own query and key lengths.  Q: [H, Tq, d]; K, V: [Hkv, Tk, d]."""
     H, Hkv, Tq, d = _packed_qk_shapes(Q, K, V, plan)
     O = torch.empty_like(Q)
-    LSE = torch.empty((H, Tq), dtype=torch.float32, device=Q.device)
-    with torch.cuda.device(Q.device):
+    LSE = Q.new_empty((H, Tq), dtype=_F32)
+    with _on_device(Q.get_device()):
         rc = load().gproj_attn_fwd_varlen_qk(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), LSE.data_ptr(), plan.cu, plan.cu_k,
                                              plan.num_seqs, plan.device.data_ptr(), H, Hkv, d, float(softmax_scale),
-                                             int(plan.causal), int(fwd_flags), _stream(Q.device))
+                                             int(plan.causal), int(fwd_flags), _raw_stream(Q.get_device()))
     if rc != GPROJ_OK:
         raise GprojError(rc, "gproj_attn_fwd_varlen_qk")
     return O, LSE
@@ -476,17 +494,16 @@ def gproj_attn_bwd_varlen_qk(Q, K, V, O, LSE, dO, plan, softmax_scale, flags=0, 
     H, Hkv, Tq, d = _packed_qk_shapes(Q, K, V, plan)
     for name, t in (("O", O), ("dO", dO)):
         _check_bf16(name, t, Q.shape)
-    if not (LSE.is_cuda and LSE.dtype == torch.float32 and LSE.is_contiguous() and tuple(LSE.shape) == (H, Tq)):
-        raise TypeError("LSE must be a contiguous CUDA float32 tensor [H, Tq]")
+    _check_lse(LSE, (H, Tq), "H, Tq")
     need = int(load().gproj_attn_bwd_varlen_workspace_bytes(plan.cu, plan.num_seqs, H, d))
     if workspace is None:
-        workspace = torch.empty(need, dtype=torch.uint8, device=Q.device)
+        workspace = Q.new_empty(need, dtype=_U8)
     dQ, dK, dV = torch.empty_like(Q), torch.empty_like(K), torch.empty_like(V)
-    with torch.cuda.device(Q.device):
+    with _on_device(Q.get_device()):
         rc = load().gproj_attn_bwd_varlen_qk(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), LSE.data_ptr(), dO.data_ptr(),
                                              dQ.data_ptr(), dK.data_ptr(), dV.data_ptr(), plan.cu, plan.cu_k, plan.num_seqs,
                                              plan.device.data_ptr(), H, Hkv, d, float(softmax_scale), int(plan.causal),
-                                             workspace.data_ptr(), workspace.numel(), int(flags), _stream(Q.device))
+                                             workspace.data_ptr(), workspace.numel(), int(flags), _raw_stream(Q.get_device()))
     if rc != GPROJ_OK:
         raise GprojError(rc, "gproj_attn_bwd_varlen_qk")
     return dQ, dK, dV

@@ -509,12 +509,14 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
   float *stats = static_cast<float *>(workspace);   // per 64-row block: the row-constant tile (see stats_blocks_bytes)
   __nv_bfloat16 *Zneg = reinterpret_cast<__nv_bfloat16 *>(static_cast<uint8_t *>(workspace) + stats_sz);
 
-  CUtensorMap mQ128, mdO128, mK64, mV64, mK128, mV128, mQ64, mdO64, mZ64, mZst, mdKst, mdVst;
+  // An encoded map costs the host about 0.15 us, so only those the head dimension's kernels use.  mQs, mdOs, mZs: the boxes the
+  // dK/dV side streams, 64 rows high at d = 128 (at d = 64 it streams 128 rows, by mQ128 and mdO128); mdKst, mdVst: its output tiles at d = 64.
+  CUtensorMap mQ128, mdO128, mK64, mV64, mK128, mV128, mQs, mdOs, mZs, mdKst, mdVst;
   bool ok = make_map(&mQ128, Q, BH, N, d, 128) && make_map(&mdO128, dO, BH, N, d, 128) && make_map(&mK64, K, BHkv, Nk, d, 64) &&
             make_map(&mV64, V, BHkv, Nk, d, 64) && make_map(&mK128, K, BHkv, Nk, d, 128) && make_map(&mV128, V, BHkv, Nk, d, 128) &&
-            make_map(&mQ64, Q, BH, N, d, 64) && make_map(&mdO64, dO, BH, N, d, 64) && make_map(&mZ64, Zneg, BH, N, d, 64) &&
-            make_map(&mZst, Zneg, BH, N, d, 128) && make_map(&mdKst, dK, BHkv, Nk, d, 128) &&
-            make_map(&mdVst, dV, BHkv, Nk, d, 128);
+            make_map(&mZs, Zneg, BH, N, d, d == 64 ? 128 : 64);
+  if (d == 64) ok = ok && make_map(&mdKst, dK, BHkv, Nk, d, 128) && make_map(&mdVst, dV, BHkv, Nk, d, 128);
+  else         ok = ok && make_map(&mQs, Q, BH, N, d, 64) && make_map(&mdOs, dO, BH, N, d, 64);
   if (!ok) return GPROJ_ERR_CUDA;
 
   const float scale_log2 = static_cast<float>(static_cast<double>(softmax_scale) * 1.4426950408889634);
@@ -538,7 +540,7 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
           st->status_ptr);                                                                                              \
     if (run_dkv)                                                                                                        \
       launch_after(bwd_dkv_kernel<DD, CC>, grid_kv, 1, BwdCfg<DD>::kDkvThreads, BwdCfg<DD>::kDkvSmemBytes, s, run_dq,            \
-          mK128, mV128, mQ64, mdO64, mZ64, stats, static_cast<__nv_bfloat16 *>(dK),                        \
+          mK128, mV128, mQs, mdOs, mZs, stats, static_cast<__nv_bfloat16 *>(dK),                        \
           static_cast<__nv_bfloat16 *>(dV), plan_kv, nblk, Nk, N, BHkv, Hkv, G, total_kv_tiles, group_kv, scale_log2, softmax_scale, \
           flags,                                                                                                        \
           st->status_ptr);                                                                                              \
@@ -553,7 +555,7 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
           nblk, N, Nk, BH, H, G, total_tiles, group_q, scale_log2, softmax_scale, flags, st->status_ptr);                 \
     if (run_dkv)                                                                                                        \
       launch_after(bwd_dkv_w128_kernel<CC>, grid_kv, 1, BwdW128::kThreads, BwdW128::kDkvSmemBytes, s, run_dq,               \
-          mK128, mV128, mQ128, mdO128, mZst, mdKst, mdVst, stats, static_cast<__nv_bfloat16 *>(dK),                       \
+          mK128, mV128, mQ128, mdO128, mZs, mdKst, mdVst, stats, static_cast<__nv_bfloat16 *>(dK),                       \
           static_cast<__nv_bfloat16 *>(dV), plan_kv, nblk, Nk, N, BHkv, Hkv, G, total_kv_tiles, group_kv, scale_log2, softmax_scale,\
           flags, st->status_ptr);                                                                                       \
   } while (0)
