@@ -60,7 +60,7 @@ struct BwdW128 {
 
 enum BwdW128WaitCode {
   kWkRes = 0x51, kWkQ = 0x52, kWkQEmpty = 0x53, kWkS = 0x54, kWkDP = 0x55, kWkR = 0x56, kWkT = 0x57, kWkSFree = 0x58, kWkYFree = 0x59,
-  kWkAcc = 0x5a, kWkAccFree = 0x5b, kWkResFree = 0x5c
+  kWkAcc = 0x5a, kWkAccFree = 0x5b, kWkResFree = 0x5c, kWkPeerFull = 0x5d, kWkPeerFree = 0x5e
 };
 
 // Arithmetic of one 16-column chunk of the dK/dV side (thread <-> key row, columns = queries), Algorithm 1 lines 5-8:
@@ -106,7 +106,10 @@ __device__ __forceinline__ void dkv_chunk(uint32_t tS, const uint32_t (&xs)[16],
 // ============================================================================================
 // dK / dV side, d = 64, 128-query steps
 // ============================================================================================
-template <bool CAUSAL>
+// CL = 2: a cluster of two CTAs shares every tile: CTA r takes its steps r, r + 2, ... (over all query heads of the group),
+// then CTA 0 gets both parts of dV, CTA 1 both parts of dK, added in FP32 before the cast.  Used where whole tiles cannot be
+// dealt evenly (few KV heads, grouped queries).
+template <bool CAUSAL, int CL>
 __global__ void __launch_bounds__(BwdW128::kThreads, 1)
 bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 rows
                     const __grid_constant__ CUtensorMap tmV,    // box 64 x 128 rows
@@ -132,7 +135,7 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
 
   __shared__ uint64_t bar_res_full, bar_res_free, bar_q_full[S], bar_q_empty[S];
   __shared__ uint64_t bar_s_full[2], bar_rt_ready[2][2], bar_dp_full, bar_y_free;
-  __shared__ uint64_t bar_acc_done, bar_acc_free, bar_drain[3];
+  __shared__ uint64_t bar_acc_done, bar_acc_free, bar_drain[3], bar_peer_full, bar_peer_free;
   __shared__ uint32_t tmem_base_smem;
   __shared__ int cta_abort, cta_skip;
   // Constant operand of the extra K = 16 slice: three eight-row core matrices (zeros, rows of (1, 1, 1, 0, 0, 0, 0, 0), zeros).
@@ -142,7 +145,7 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) cta_skip = *reinterpret_cast<volatile int *>(status);
   __syncthreads();
-  if (cta_skip != 0) return;
+  if (CL == 1 && cta_skip != 0) return;   // a cluster runs on with every wait falling through: its CTAs exchange results
 
   const bool use_z = (flags & kFlagNoKCorrection) == 0;
   const uint32_t stage_tx = (use_z ? 3 : 2) * C::kTileBytes + C::kExtBytes;
@@ -153,7 +156,7 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
 
   AbortState ab{status, &cta_abort};
   if (threadIdx.x == 0) {
-    cta_abort = 0;
+    cta_abort = CL > 1 ? cta_skip : 0;
     mbar_init(&bar_res_full, 1);
     mbar_init(&bar_res_free, 2);   // the last S^T product (issuer 1) and the last dP^T product (issuer 2): the epilogue never touches K / V
     for (int s = 0; s < S; ++s) { mbar_init(&bar_q_full[s], 1); mbar_init(&bar_q_empty[s], 1); }
@@ -165,6 +168,8 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
     mbar_init(&bar_y_free, C::kCompute);
     mbar_init(&bar_acc_done, 1);
     mbar_init(&bar_acc_free, 128);
+    mbar_init(&bar_peer_full, 128);
+    mbar_init(&bar_peer_free, 128);
     mbar_init(&bar_drain[0], 1);
     mbar_init(&bar_drain[1], 1);
     mbar_init(&bar_drain[2], 1);
@@ -176,12 +181,14 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
     tma_prefetch_desc(&tmdK); tma_prefetch_desc(&tmdV);
   }
   tc_fence_before();
-  __syncthreads();
+  if (CL > 1) cluster_sync(); else __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, tmem_base_smem, 0);
   griddep_launch_dependents();   // the next kernel in the stream may set itself up beside this one
 
   TileSched sched(total_tiles);
+  const int rank = CL > 1 ? cluster_rank() : 0;
+  if (CL > 1) { sched.G /= CL; sched.c /= CL; }
   // A step may reach past the end of the sequence: those query columns are zero fill or the next packed sequence's rows,
   // and are masked.
   // N: key rows per head (own operand), Nq: query rows per head.  A key j is seen by the queries i >= j - (L_k - L_q).
@@ -196,6 +203,10 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
     return min(first, ((Lq - 1) >> 6) << 6);
   };
   auto steps_of = [&](const TileInfo &t) { return max(1, (t.oseq_end - t.oseq0 - q_start_of(t) + C::kStepRows - 1) / C::kStepRows); };
+  // This CTA's steps of a tile whose heads have T steps each, and the n-th of them; a CTA that gets none runs step 0 fully
+  // masked.
+  auto own_steps = [&](int T) { return CL == 1 ? G * T : max(1, (G * T - rank + CL - 1) / CL); };
+  auto own_step = [&](int n, int T) { return CL == 1 ? n : (rank < G * T ? CL * n + rank : 0); };
 
   if (warp < 4) {
   setmaxnreg_dec<C::kRegsAux>();
@@ -220,8 +231,8 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
           // launch); nothing this CTA did so far needed it.
           griddep_wait();
         }
-        for (int n = 0; n < G * T; ++n, ++g) {
-          const int st = g % S;
+        for (int m = 0; m < own_steps(T); ++m, ++g) {
+          const int st = g % S, n = own_step(m, T);
           if (g >= S) mbar_wait(&bar_q_empty[st], ((g / S) - 1) & 1, ab, kWkQEmpty);
           mbar_expect_tx(&bar_q_full[st], stage_tx);
           uint8_t *dst = sStage + st * C::kDkvStageBytes;
@@ -232,7 +243,7 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
           // two 64-row blocks of the row-constant tile (the second may lie past the sequence's last block: its columns are masked)
           bulk_load_1d(dst + 3 * C::kTileBytes, reinterpret_cast<const uint8_t *>(stats) + (static_cast<size_t>(qh) * nblk + tl.blk0 + (qrel >> 6)) * kExtBlockBytes,
                        C::kExtBytes, &bar_q_full[st]);
-          if (n == 0 && ti > 0) load_kv(tl.row0, bh);
+          if (m == 0 && ti > 0) load_kv(tl.row0, bh);
         }
       }
       if (cta_abort) {
@@ -251,7 +262,7 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
     const SmemDesc dscExt0 = make_smem_desc_noswizzle(smem_u32(sStage + 3 * C::kTileBytes), 128, 256);
     int g = 0, ti = 0;
     for (int lin = sched.next(); lin >= 0; lin = sched.next(), ++ti) {
-      const int T = G * steps_of(tile_of(lin));
+      const int T = own_steps(steps_of(tile_of(lin)));
       mbar_wait(&bar_res_full, ti & 1, ab, kWkRes);
       for (int n = 0; n < T; ++n, ++g) {
         const int st = g % S, sb = g & 1;
@@ -287,7 +298,7 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
     const SmemDesc dscExt0 = make_smem_desc_noswizzle(smem_u32(sStage + 3 * C::kTileBytes), 128, 256);
     int g = 0, ti = 0;
     for (int lin = sched.next(); lin >= 0; lin = sched.next(), ++ti) {
-      const int T = G * steps_of(tile_of(lin));
+      const int T = own_steps(steps_of(tile_of(lin)));
       mbar_wait(&bar_res_full, ti & 1, ab, kWkRes);
       for (int n = 0; n < T; ++n, ++g) {
         const int st = g % S;
@@ -313,7 +324,7 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
     const SmemDesc dscQ0mn = make_smem_desc(smem_u32(sStage), C::kTileBytes, 1024);        // MN-major view of stage 0
     int g = 0, ti = 0;
     for (int lin = sched.next(); lin >= 0; lin = sched.next(), ++ti) {
-      const int T = G * steps_of(tile_of(lin));
+      const int T = own_steps(steps_of(tile_of(lin)));
       if (ti > 0) mbar_wait(&bar_acc_free, (ti - 1) & 1, ab, kWkAccFree);   // the previous epilogue has read dV, dK
       for (int p = 0; p < T; ++p, ++g) {
         const int st = g % S, sb = g & 1;
@@ -364,7 +375,7 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
     int g0 = 0;
     for (int lin = sched.next(); lin >= 0; lin = sched.next()) {
       const TileInfo tl = tile_of(lin);
-      const int Th = steps_of(tl), T = G * Th, q_start = q_start_of(tl);
+      const int Th = steps_of(tl), T = own_steps(Th), q_start = q_start_of(tl);
 #ifdef GPROJ_TRACE
       const unsigned long long ev_n0 = global_ns(); const long long ev_c0 = clock64(); unsigned long long ev_n1 = 0;
 #endif
@@ -376,12 +387,13 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
         const uint32_t tS0 = tmem_base + lane_addr + (sb ? C::kColZ : C::kColX) + 16 * wg, tS1 = tS0 + 64;
         const uint32_t tdP0 = tmem_base + lane_addr + C::kColY + 16 * wg, tdP1 = tdP0 + 64;
         constexpr int kChunk1 = 64;
-        const int nh = n % Th;                                              // step within the current query head
+        const int nh = own_step(n, Th) % Th;                                // step within the current query head
+        const bool none = CL > 1 && rank >= G * Th;                         // a step of another CTA, run to keep the pipeline in step
         const int Lq = tl.oseq_end - tl.oseq0, off = (tl.seq_end - tl.seq0) - Lq, krel0 = tl.row0 - tl.seq0;
         const int qs = q_start + nh * C::kStepRows;                         // first query (inside its sequence) of the step
         const int q0 = qs + cb;                                             // ... of this thread's first chunk
-        const bool masked = (CAUSAL && qs < krel0 + 128 - off) || qs + C::kStepRows > Lq;
-        const int lim = CAUSAL ? krel0 + row - off - q0 : 0, hi = Lq - 1 - q0;
+        const bool masked = (CAUSAL && qs < krel0 + 128 - off) || qs + C::kStepRows > Lq || none;
+        const int lim = CAUSAL ? krel0 + row - off - q0 : 0, hi = none ? -1 : Lq - 1 - q0;
         // dP^T of both chunks and S^T of the first go to registers at the start of the step; dP^T (single-buffered) is then
         // released to the tensor core.
         mbar_wait(&bar_s_full[sb], (g >> 1) & 1, ab, kWkS);
@@ -426,6 +438,56 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
     for (int lin = sched.next(); lin >= 0; lin = sched.next(), ++ti) {
       const TileInfo tl = tile_of(lin);
       const int bh = hix(lin);
+      if (CL > 1) {
+        // The staging buffer holds the other CTA's part of this CTA's output, [4 chunks of 16 columns][128 rows] x 64 bytes of
+        // FP32, the 16-byte pieces of a row swizzled; the BF16 result goes over each thread's own pieces and out by rows.
+        auto piece = [&](int cc, int r, int v) { return static_cast<uint32_t>(cc * 8192 + r * 64 + ((v ^ ((r >> 1) & 3)) << 4)); };
+        const uint32_t peer_buf = cluster_map_shared(smem_u32(sOut), rank ^ 1);
+        const uint32_t t_own = tmem_base + (rank == 0 ? C::kColAcc0 : C::kColAcc1) + lane_addr, t_send = tmem_base + (rank == 0 ? C::kColAcc1 : C::kColAcc0) + lane_addr;
+        const float scale = rank == 0 ? 1.0f : alpha;
+        mbar_wait(&bar_acc_done, ti & 1, ab, kWkAcc);
+        tc_fence_after();
+        if (ti > 0) mbar_wait_cluster(&bar_peer_free, (ti - 1) & 1, ab, kWkPeerFree);   // the other CTA has taken the previous tile's part
+#pragma unroll
+        for (int cc = 0; cc < D / 16; ++cc) {
+          uint32_t a[16];
+          tmem_ld16(t_send + 16 * cc, a);
+          tmem_wait_ld();
+#pragma unroll
+          for (int v = 0; v < 4; ++v)
+            cluster_store_f4(peer_buf + piece(cc, row, v), __uint_as_float(a[4 * v]), __uint_as_float(a[4 * v + 1]), __uint_as_float(a[4 * v + 2]), __uint_as_float(a[4 * v + 3]));
+        }
+        cluster_mbar_arrive(cluster_map_shared(smem_u32(&bar_peer_full), rank ^ 1));
+        mbar_wait_cluster(&bar_peer_full, ti & 1, ab, kWkPeerFull);
+#pragma unroll
+        for (int cc = 0; cc < D / 16; ++cc) {
+          uint32_t a[16];
+          tmem_ld16(t_own + 16 * cc, a);
+          float b[16];
+#pragma unroll
+          for (int v = 0; v < 4; ++v) *reinterpret_cast<float4 *>(&b[4 * v]) = *reinterpret_cast<const float4 *>(sOut + piece(cc, row, v));
+          tmem_wait_ld();
+          if (cc == D / 16 - 1) { tc_fence_before(); mbar_arrive(&bar_acc_free); }   // the accumulators may be overwritten by the next tile
+          uint32_t w[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            w[i] = pack_bf16x2(__fmul_rn(scale, __fadd_rn(__uint_as_float(a[2 * i]), b[2 * i])), __fmul_rn(scale, __fadd_rn(__uint_as_float(a[2 * i + 1]), b[2 * i + 1])));
+          *reinterpret_cast<uint4 *>(sOut + piece(cc, row, 0)) = make_uint4(w[0], w[1], w[2], w[3]);
+          *reinterpret_cast<uint4 *>(sOut + piece(cc, row, 1)) = make_uint4(w[4], w[5], w[6], w[7]);
+        }
+        __syncwarp();
+        const int wrows = tl.seq_end - tl.row0 - 32 * ew;
+        uint4 *dst = reinterpret_cast<uint4 *>((rank == 0 ? dVg : dKg) + (static_cast<size_t>(bh) * N + tl.row0 + 32 * ew) * D);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const int r = 4 * k + (lane >> 3), p = lane & 7;
+          const uint4 v = *reinterpret_cast<const uint4 *>(sOut + piece(p >> 1, 32 * ew + r, p & 1));
+          if (r < wrows) dst[r * (D / 8) + p] = v;
+        }
+        __syncwarp();
+        cluster_mbar_arrive(cluster_map_shared(smem_u32(&bar_peer_free), rank ^ 1));
+        continue;
+      }
       if (row == 0) bulk_wait_group_read0();                 // the previous tile's stores have left the staging buffer
       named_bar_sync(1, 128);
       mbar_wait(&bar_acc_done, ti & 1, ab, kWkAcc);
@@ -470,7 +532,7 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
   }
 
   tc_fence_before();
-  __syncthreads();
+  if (CL > 1) cluster_sync(); else __syncthreads();   // no CTA leaves while the other one may still write to it
   if (warp == 1) tmem_dealloc(tmem_base, C::kTmemCols);
 }
 

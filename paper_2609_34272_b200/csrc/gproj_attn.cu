@@ -53,6 +53,7 @@ struct DeviceState {
   int *status_ptr = nullptr;
   int sm_count = 0;
   int fwd_clusters[2][4] = {};   // forward with clusters of 2, 4, 8 CTAs (entries 1, 2, 3) at d = 64 and d = 128: how many run at once
+  int dkv_clusters = 0;          // dK/dV side at d = 64 with clusters of two CTAs: how many run at once
   // host-buffer entry point only: copy-in and copy-out streams and the events that order them against the caller's stream
   bool pipe_ready = false;
   cudaStream_t in_stream = nullptr, out_stream = nullptr;
@@ -132,8 +133,11 @@ int device_state(DeviceState **out) {
       ok &= allow_smem(attn_fwd_kernel<128, false, false, 2>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, false, true, 0>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, false, true, 2>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
-      ok &= allow_smem(bwd_dkv_w128_kernel<true>, BwdW128::kDkvSmemBytes) == cudaSuccess;
-      ok &= allow_smem(bwd_dkv_w128_kernel<false>, BwdW128::kDkvSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dkv_w128_kernel<true, 1>, BwdW128::kDkvSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dkv_w128_kernel<false, 1>, BwdW128::kDkvSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dkv_w128_kernel<true, 2>, BwdW128::kDkvSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dkv_w128_kernel<false, 2>, BwdW128::kDkvSmemBytes) == cudaSuccess;
+      ok = ok && max_clusters(bwd_dkv_w128_kernel<true, 2>, 2, BwdW128::kThreads, BwdW128::kDkvSmemBytes, &st.dkv_clusters) == cudaSuccess;
       ok &= allow_smem(bwd_dq_kernel<64, true>, BwdCfg<64>::kDqSmemBytes) == cudaSuccess;
       ok &= allow_smem(bwd_dq_kernel<64, false>, BwdCfg<64>::kDqSmemBytes) == cudaSuccess;
       ok &= allow_smem(bwd_dq_kernel<128, true>, BwdCfg<128>::kDqSmemBytes) == cudaSuccess;
@@ -479,6 +483,35 @@ int gproj_attn_bwd_gqa(const void *Q, const void *K, const void *V, const void *
 
 namespace {
 
+// dK/dV side at d = 64, dense calls: share every key tile between the two CTAs of a cluster?  This replays the static deal of
+// both forms in units of one 128-query step (2.3 per item, the kernel's measured overhead, and 1.5 more for the exchange of
+// the two parts) and takes the pairs where their longest CTA is 3 % shorter.
+// Measured, this kernel alone, whole tiles -> pairs: 16 query / 4 KV heads x 4096, causal: 121 -> 77 us; 8 / 2 heads x 8000,
+// causal: 229 -> 140; 32 / 4 heads x 2000: 121 -> 78; 4 heads x 4096, causal: 43.5 -> 37.2; 1 head x 8192: 62.0 -> 43.5;
+// 16 heads x 4096, causal (stays with whole tiles): 68.
+bool dkv_prefers_pairs(int BHkv, int n_kt, int G, int Nq, int Nk, bool causal, int sms, int pairs) {
+  const long long items = static_cast<long long>(BHkv) * n_kt;
+  if (pairs < 1 || items > 8LL * sms) return false;      // many items per CTA: they balance as they are
+  static std::mutex memo_mutex;
+  static std::map<std::tuple<int, int, int, int, int, bool, int>, bool> memo;
+  const auto key = std::make_tuple(BHkv, n_kt, G, Nq, Nk, causal, sms);
+  {
+    std::lock_guard<std::mutex> lock(memo_mutex);
+    const auto hit = memo.find(key);
+    if (hit != memo.end()) return hit->second;
+  }
+  auto steps = [&](long long lin) {                      // longest tiles first, as the kernel orders them
+    const long long row0 = 128 * (lin / BHkv), off = static_cast<long long>(Nk) - Nq;
+    const long long first = causal ? std::min<long long>(std::max(0LL, row0 - off) & ~63LL, ((Nq - 1) >> 6) << 6) : 0;
+    return static_cast<double>(G * std::max(1LL, (Nq - first + 127) / 128));
+  };
+  const double whole = deal_makespan(items, sms, [&](long long lin) { return steps(lin) + 2.3; });
+  const double split = deal_makespan(items, pairs, [&](long long lin) { return std::ceil(0.5 * steps(lin)) + 3.8; });
+  std::lock_guard<std::mutex> lock(memo_mutex);
+  if (memo.size() < 4096) memo[key] = split < 0.97 * whole;
+  return split < 0.97 * whole;
+}
+
 // Dense call: plans == nullptr.  Packed call: B = 1, N / Nk = total query / key rows, plan_q / plan_kv = device tile lists
 // in the order of the dQ-side and the dK/dV-side kernel, nblk = 64-row statistic blocks per head.
 int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const float *LSE, const void *dO,
@@ -547,6 +580,8 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
   } while (0)
   // At d = 64 the dK/dV side runs with 128-wide steps (every score product an N = 128 instruction); it streams 128-row
   // boxes, which the stationary-tile maps of the dQ side already are.
+  const bool pairs = d == 64 && run_dkv && !plan_q && dkv_prefers_pairs(BHkv, n_kt, G, N, Nk, causal != 0, st->sm_count, st->dkv_clusters);
+  const dim3 grid_dkv(pairs ? 2u * static_cast<unsigned>(std::min(total_kv_tiles, st->dkv_clusters)) : grid_kv.x);
 #define GPROJ_LAUNCH_BWD_W128(CC)                                                                                       \
   do {                                                                                                                  \
     if (run_dq)                                                                                                         \
@@ -554,8 +589,8 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
           mQ128, mdO128, mK64, mV64, static_cast<const __nv_bfloat16 *>(Q), Ob, dOb, LSE, stats, static_cast<__nv_bfloat16 *>(dQ), Zneg, plan_q,    \
           nblk, N, Nk, BH, H, G, total_tiles, group_q, scale_log2, softmax_scale, flags, st->status_ptr);                 \
     if (run_dkv)                                                                                                        \
-      launch_after(bwd_dkv_w128_kernel<CC>, grid_kv, 1, BwdW128::kThreads, BwdW128::kDkvSmemBytes, s, run_dq,               \
-          mK128, mV128, mQ128, mdO128, mZs, mdKst, mdVst, stats, static_cast<__nv_bfloat16 *>(dK),                       \
+      launch_after(pairs ? bwd_dkv_w128_kernel<CC, 2> : bwd_dkv_w128_kernel<CC, 1>, grid_dkv, pairs ? 2 : 1, BwdW128::kThreads,    \
+          BwdW128::kDkvSmemBytes, s, run_dq, mK128, mV128, mQ128, mdO128, mZs, mdKst, mdVst, stats, static_cast<__nv_bfloat16 *>(dK), \
           static_cast<__nv_bfloat16 *>(dV), plan_kv, nblk, Nk, N, BHkv, Hkv, G, total_kv_tiles, group_kv, scale_log2, softmax_scale,\
           flags, st->status_ptr);                                                                                       \
   } while (0)

@@ -446,6 +446,23 @@ __device__ __forceinline__ float cluster_load_f32(uint32_t addr) {
 __device__ __forceinline__ void cluster_store_f4(uint32_t addr, float a, float b, float c, float d) {
   asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
+// arrive on an mbarrier of another CTA of the cluster (its address from cluster_map_shared); this thread's earlier writes to
+// that CTA's shared memory are visible to whoever then waits on it with mbar_wait_cluster
+__device__ __forceinline__ void cluster_mbar_arrive(uint32_t addr) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+// mbar_wait for a phase that another CTA's arrivals complete (acquires at cluster scope)
+__device__ __forceinline__ void mbar_wait_cluster(uint64_t *bar, uint32_t parity, const AbortState &ab, int code) {
+  mbar_wait(bar, parity, ab, code);
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred P;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 P, [%1], %2;\n\t"
+      "selp.b32 %0, 1, 0, P;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+}
 
 // Move registers between warpgroups: every warp of a warpgroup gives back (dec) or takes (inc) registers so that each of its
 // threads holds N.  N is a multiple of 8; the shares of all warpgroups must add up to at most what the launch allocated.
