@@ -188,8 +188,7 @@ size_t align256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
 // the stream still runs (programmatic dependent launch): every kernel launched so waits, by griddep_wait, before it touches
 // memory that an earlier kernel may read or write, so only its set-up (barriers, TMEM, descriptors) and, on the dK/dV
 // side, the loads of K and V overlap.  Measured with calls back to back (with the attribute on the dK/dV side alone -> on
-// all three kernels): forward, 16 heads x 4096 x 64: 62.0 -> 60.3 us; backward, 8 heads x 4096 x 128: 145.1 -> 141.8 us;
-// forward of 16 queries behind 8192 keys: 33.9 -> 31.2 us.
+// the dQ side too): backward, 8 heads x 4096 x 128: 145.1 -> 141.8 us.
 template <typename... Params, typename... Args>
 void launch_after(void (*kernel)(Params...), dim3 grid, int cluster, int threads, size_t smem, cudaStream_t s, bool overlap_previous,
                   Args... args) {
@@ -433,8 +432,14 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
     return GPROJ_OK;
   }
   const dim3 grid(static_cast<unsigned>(total_items < st->sm_count ? total_items : st->sm_count));   // persistent
+  // Start beside the previous kernel only with at most two items per CTA.  CTAs that start early take the SMs in the order in
+  // which the previous kernel leaves them; launched normally, neighbouring CTAs sit side by side in a TPC and walk
+  // neighbouring items, whose K / V requests meet on the way to L2.  Measured, forward + backward back to back, normal ->
+  // early: 2 heads x 256: 23.4 -> 21.7 us; 8 heads x 4096 x 128 (1.7 items per CTA): 185 -> 180; but 96 heads x 1000 x 128
+  // (2.6): 202 -> 211; 16 packed documents of 16384 rows (15): 393 -> 408, its items of 16 key tiles 15.1 -> 20.1 us each.
+  const bool early = total_items <= 2 * st->sm_count;
 #define GPROJ_LAUNCH_FWD(DD, CC, FF, MM)                                                                            \
-  launch_after(attn_fwd_kernel<DD, CC, FF, MM>, grid, 1, FwdCfg<DD>::kThreads, FwdCfg<DD>::kSmemBytes, s, true,                         \
+  launch_after(attn_fwd_kernel<DD, CC, FF, MM>, grid, 1, FwdCfg<DD>::kThreads, FwdCfg<DD>::kSmemBytes, s, early,                        \
       mQ, mK, mV, mO, static_cast<__nv_bfloat16 *>(O), plan, LSE, N, Nk, BH, H, G, fold, tiles_per_item, total_items, fwd_order, scale_log2, \
       softmax_scale, st->status_ptr)
 #define GPROJ_LAUNCH_FWD_C(DD, FF, MM)                                                                              \
