@@ -100,18 +100,22 @@ struct BwdCfg {
 };
 
 // Static persistent schedule: work items are numbered by decreasing work; round r hands item r G + c to CTA c
-// on even rounds and item r G + (G - 1 - c) on odd rounds (G = number of CTAs).
+// on even rounds and item r G + (G - 1 - c) on odd rounds (G = number of CTAs).  With solo > 0 the first `solo` CTAs, whose
+// first item is longer than an even share, get nothing after round 0 and the others share the rest in the same way.
+// With clusters a whole cluster counts as one CTA here.
 struct TileSched {
-  int total, G, c, round;
-  __device__ __forceinline__ explicit TileSched(int total_tiles)
-      : total(total_tiles), G(static_cast<int>(gridDim.x)), c(static_cast<int>(blockIdx.x)), round(0) {}
-  __device__ __forceinline__ int next() {
-    const int idx = round * G + ((round & 1) ? (G - 1 - c) : c);
-    ++round;
-    return idx < total ? idx : -1;
+  int total, W, c, back, round;     // W: CTAs that share the rounds after the first; back: c counted from the other end of them
+  __device__ __forceinline__ TileSched(int total_tiles, int solo, int cluster = 1) {
+    const int G = static_cast<int>(gridDim.x) / cluster;
+    c = static_cast<int>(blockIdx.x) / cluster;
+    W = G - solo;
+    back = solo + G - 1 - c;
+    total = c < solo ? min(total_tiles, G) : total_tiles;
+    round = 0;
   }
-  __device__ __forceinline__ int peek() const {     // the item next() would return, without taking it
-    const int idx = round * G + ((round & 1) ? (G - 1 - c) : c);
+  __device__ __forceinline__ int next() {
+    const int idx = round * W + ((round & 1) ? back : c);
+    ++round;
     return idx < total ? idx : -1;
   }
 };
@@ -136,6 +140,7 @@ struct FastDiv {
 };
 struct ItemOrder {
   int gk, n_full;                   // ranks per group, full groups
+  int solo;                         // CTAs with one item only (TileSched)
   FastDiv per_group, by_gk, by_rem; // items per group (heads x gk); ranks per group; ranks of the short last group
 #ifdef __CUDACC__
   __device__ __forceinline__ void decode(int lin, int &rank, int &head) const {
@@ -419,7 +424,7 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
   griddep_wait();
   griddep_launch_dependents();
 
-  TileSched sched(total_tiles);
+  TileSched sched(total_tiles, order.solo);
   // tile decode: causal -> longest rows first
   auto tix = [&](int lin) { return order.rank(lin); };
   auto hix = [&](int lin) { return order.head(lin); };
@@ -804,7 +809,7 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 rows
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, tmem_base_smem, 0);
   griddep_launch_dependents();   // the next kernel in the stream may set itself up beside this one
 
-  TileSched sched(total_tiles);
+  TileSched sched(total_tiles, order.solo);
   // tile decode: causal -> key tile 0 has the most query steps and comes first
   // Ragged N: query steps round up.  A zero-filled query column past N contributes exactly nothing (its dO, Q and Z rows
   // are zero and its padded statistics are zero, so t = 0 and r multiplies zero rows); key rows past N are clipped on store.

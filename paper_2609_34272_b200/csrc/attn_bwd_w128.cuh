@@ -186,9 +186,8 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, tmem_base_smem, 0);
   griddep_launch_dependents();   // the next kernel in the stream may set itself up beside this one
 
-  TileSched sched(total_tiles);
+  TileSched sched(total_tiles, order.solo, CL);
   const int rank = CL > 1 ? cluster_rank() : 0;
-  if (CL > 1) { sched.G /= CL; sched.c /= CL; }
   // A step may reach past the end of the sequence: those query columns are zero fill or the next packed sequence's rows,
   // and are masked.
   // N: key rows per head (own operand), Nq: query rows per head.  A key j is seen by the queries i >= j - (L_k - L_q).

@@ -169,8 +169,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   struct Item { int seq0, len, qt0, nq, n_kt, kseq0, klen, off; };
   auto tix = [&](int lin) { return order.rank(lin); };
   auto hix = [&](int lin) { return order.head(lin); };
-  TileSched sched(total_items);
-  if (kCluster) { sched.G /= ncta; sched.c /= ncta; }
+  TileSched sched(total_items, order.solo, ncta);
   auto decode_rank = [&](int rank) {       // rank: position of the item's tile (pair) in its head's list, longest first
     Item it;
     if (plan != nullptr) {

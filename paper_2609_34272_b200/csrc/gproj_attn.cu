@@ -209,12 +209,15 @@ void launch_after(void (*kernel)(Params...), dim3 grid, int cluster, int threads
   (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);   // the caller reads cudaGetLastError()
 }
 
+// The row offsets of a packed call (host), for the host's scheduling decisions.
+struct PackedSeqs { const int *cu_q, *cu_k; int num; bool causal; };
+
 int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE, int B, int H, int Hkv, int N, int Nk, int d,
-               float softmax_scale, int causal, unsigned fwd_flags, const int4 *plan, int n_plan_tiles, int longest_keys, void *stream);
+               float softmax_scale, int causal, unsigned fwd_flags, const int4 *plan, int n_plan_tiles, const PackedSeqs *seqs, void *stream);
 int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const float *LSE, const void *dO,
                void *dQ, void *dK, void *dV, int B, int H, int Hkv, int N, int Nk, int d, float softmax_scale, int causal,
                void *workspace, size_t workspace_bytes, unsigned flags, const int4 *plan_q, const int4 *plan_kv,
-               int n_plan_q_tiles, int n_plan_kv_tiles, int nblk, void *stream);
+               int n_plan_q_tiles, int n_plan_kv_tiles, int nblk, const PackedSeqs *seqs, void *stream);
 
 // Row constants (-LSE / alpha, -D) for the dK/dV side: per 64 rows one K-major operand tile of 16 BF16 columns (2048 B;
 // per head ceil(N / 64) of them, the last one zero-padded), plus one spare block: the 128-wide steps fetch two blocks at
@@ -238,7 +241,7 @@ int gproj_attn_fwd_gqa(const void *Q, const void *K, const void *V, void *O, flo
 
 int gproj_attn_fwd_ex(const void *Q, const void *K, const void *V, void *O, float *LSE, int B, int H, int Hkv, int N,
                       int d, float softmax_scale, int causal, unsigned fwd_flags, void *stream) {
-  return launch_fwd(Q, K, V, O, LSE, B, H, Hkv, N, N, d, softmax_scale, causal, fwd_flags, nullptr, 0, 0, stream);
+  return launch_fwd(Q, K, V, O, LSE, B, H, Hkv, N, N, d, softmax_scale, causal, fwd_flags, nullptr, 0, nullptr, stream);
 }
 
 }  // extern "C"
@@ -263,6 +266,7 @@ FastDiv fast_div(unsigned d) {
 
 ItemOrder item_order(int heads, int n_per_head, int group) {
   ItemOrder o;
+  o.solo = 0;
   o.gk = std::max(1, std::min(group, n_per_head));
   o.n_full = n_per_head / o.gk;
   o.per_group = fast_div(static_cast<unsigned>(heads) * static_cast<unsigned>(o.gk));
@@ -273,14 +277,63 @@ ItemOrder item_order(int heads, int n_per_head, int group) {
 
 // Longest CTA of the static boustrophedon deal (TileSched) of `items` items with the given costs.
 template <typename WorkOf>
-double deal_makespan(long long items, int sms, WorkOf work_of) {
-  const int G = static_cast<int>(std::min<long long>(items, sms));
+double deal_makespan(long long items, int sms, WorkOf work_of, int solo = 0) {
+  const int G = static_cast<int>(std::min<long long>(items, sms)), W = G - solo;
   std::vector<double> load(static_cast<size_t>(G), 0.0);
   for (long long lin = 0; lin < items; ++lin) {
-    const long long r = lin / G, pos = lin % G;
-    load[static_cast<size_t>((r & 1) ? G - 1 - pos : pos)] += work_of(lin);
+    int cta = static_cast<int>(lin);
+    if (lin >= G) {
+      const long long r = 1 + (lin - G) / W, pos = (lin - G) % W;
+      cta = static_cast<int>((r & 1) ? G - 1 - pos : solo + pos);
+    }
+    load[static_cast<size_t>(cta)] += work_of(lin);
   }
   return *std::max_element(load.begin(), load.end());
+}
+
+// Work of every tile of a packed call, in the plan's order (decreasing): keys of each query tile (key_side: queries of each
+// key tile, whose walk starts at a 64-row block).
+std::vector<int> packed_work(const PackedSeqs &ps, bool key_side) {
+  std::vector<int> work;
+  for (int s = 0; s < ps.num; ++s) {
+    const int lq = ps.cu_q[s + 1] - ps.cu_q[s], lk = ps.cu_k[s + 1] - ps.cu_k[s], off = lk - lq;
+    if (!key_side)
+      for (int r = 0; r < lq; r += 128) work.push_back(ps.causal ? std::max(0, std::min(lk, std::min(r + 128, lq) + off)) : lk);
+    else if (lq > 0)
+      for (int r = 0; r < lk; r += 128) work.push_back(std::max(0, lq - (ps.causal ? std::max(0, r - off) & ~63 : 0)));
+  }
+  std::sort(work.begin(), work.end(), [](int a, int b) { return a > b; });
+  return work;
+}
+
+int longest_keys(const PackedSeqs &ps) {
+  int most = 0;
+  for (int s = 0; s < ps.num; ++s) most = std::max(most, ps.cu_k[s + 1] - ps.cu_k[s]);
+  return most;
+}
+
+// TileSched's solo CTAs for `heads` copies of tiles with the given costs (decreasing): those whose first item is longer than
+// what an even share of the rest would be.  The boustrophedon rounds would give each of them a second item all the same.
+// Measured, 12 packed pairs (4000 queries, 9000 keys, 12 heads, d = 128; 60 of 456 query tiles twice as long as an even
+// share): forward 53.6 -> 45.5 us, dQ side 76.5 -> 64.0 us.
+int solo_ctas(const std::vector<double> &cost, int heads, int sms) {
+  const long long items = static_cast<long long>(cost.size()) * heads;
+  if (items <= sms || items > 16LL * sms) return 0;
+  double total = 0.0;
+  for (double c : cost) total += c * heads;
+  int solo = 0;
+  double rest = total;
+  while (solo < sms / 2 && cost[static_cast<size_t>(solo / heads)] > rest / (sms - solo)) rest -= cost[static_cast<size_t>(solo++ / heads)];
+  if (solo == 0) return 0;
+  auto work_of = [&](long long lin) { return cost[static_cast<size_t>(lin / heads)]; };
+  return deal_makespan(items, sms, work_of, solo) < 0.99 * deal_makespan(items, sms, work_of) ? solo : 0;
+}
+
+template <typename CostOf>
+int packed_solo(const PackedSeqs &ps, bool key_side, int heads, int sms, CostOf cost_of) {
+  std::vector<double> cost;
+  for (int w : packed_work(ps, key_side)) cost.push_back(cost_of(w));
+  return solo_ctas(cost, heads, sms);
 }
 
 // How many adjacent tile ranks of one head the kernels deal consecutively (see ItemOrder).  Packed calls: 1 (their plan is
@@ -379,7 +432,7 @@ int fwd_cluster_log2(long long tiles, int key_tiles, const int (&fit)[4]) {
 // Dense call: plan == nullptr, one sequence [0, N) per head.  Packed call: B = 1, N = total tokens, plan = device tile
 // list (query order) with n_plan_tiles entries, longest_keys = most keys of one sequence.
 int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE, int B, int H, int Hkv, int N, int Nk, int d,
-               float softmax_scale, int causal, unsigned fwd_flags, const int4 *plan, int n_plan_tiles, int longest_keys, void *stream) {
+               float softmax_scale, int causal, unsigned fwd_flags, const int4 *plan, int n_plan_tiles, const PackedSeqs *seqs, void *stream) {
   if (!Q || !K || !V || !O || !LSE) return GPROJ_ERR_NULL;
   if (fwd_flags & ~GPROJ_FWD_FLAG_FMA_SOFTMAX) return GPROJ_ERR_FLAGS;
   const bool fma = (fwd_flags & GPROJ_FWD_FLAG_FMA_SOFTMAX) != 0;
@@ -417,10 +470,10 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
   if (tiles_per_item == 2 && d == 64 && causal && N == Nk && fwd_prefers_single_tiles(BH, n_qt, st->sm_count)) tiles_per_item = 1;
   const int total_items = BH * ((n_qt + tiles_per_item - 1) / tiles_per_item);
   if (total_items <= 0) return GPROJ_OK;   // nothing but empty sequences
-  const ItemOrder fwd_order = item_order(BH, total_items / BH, tile_group_of(plan != nullptr, causal != 0, BH, total_items / BH, 2 * static_cast<size_t>(BHkv) * Nk * d * 2, st->sm_count,
+  ItemOrder fwd_order = item_order(BH, total_items / BH, tile_group_of(plan != nullptr, causal != 0, BH, total_items / BH, 2 * static_cast<size_t>(BHkv) * Nk * d * 2, st->sm_count,
                                                             tiles_per_item == 2 ? 1.45 : 6.8));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const int lg = (tiles_per_item == 1 && !fma) ? fwd_cluster_log2(total_items, ((plan ? longest_keys : Nk) + 127) / 128, st->fwd_clusters[d == 128]) : 0;
+  const int lg = (tiles_per_item == 1 && !fma) ? fwd_cluster_log2(total_items, ((seqs ? longest_keys(*seqs) : Nk) + 127) / 128, st->fwd_clusters[d == 128]) : 0;
   if (lg > 0 || fold > 0) {
     auto kernel = d == 64 ? (causal ? attn_fwd_kernel<64, true, false, 3> : attn_fwd_kernel<64, false, false, 3>)
                           : (causal ? attn_fwd_kernel<128, true, false, 3> : attn_fwd_kernel<128, false, false, 3>);
@@ -431,6 +484,7 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
     tl_launch_count = 1;
     return GPROJ_OK;
   }
+  if (seqs) fwd_order.solo = packed_solo(*seqs, false, BH, st->sm_count, [](int keys) { return std::max(1, (keys + 127) / 128) + 2.1; });
   const dim3 grid(static_cast<unsigned>(total_items < st->sm_count ? total_items : st->sm_count));   // persistent
   // Start beside the previous kernel only with at most two items per CTA.  CTAs that start early take the SMs in the order in
   // which the previous kernel leaves them; launched normally, neighbouring CTAs sit side by side in a TPC and walk
@@ -481,40 +535,34 @@ int gproj_attn_bwd_gqa(const void *Q, const void *K, const void *V, const void *
                        void *dQ, void *dK, void *dV, int B, int H, int Hkv, int N, int d, float softmax_scale, int causal,
                        void *workspace, size_t workspace_bytes, unsigned flags, void *stream) {
   return launch_bwd(Q, K, V, O, LSE, dO, dQ, dK, dV, B, H, Hkv, N, N, d, softmax_scale, causal, workspace, workspace_bytes, flags,
-                    nullptr, nullptr, 0, 0, (N + 63) / 64, stream);
+                    nullptr, nullptr, 0, 0, (N + 63) / 64, nullptr, stream);
 }
 
 }  // extern "C"
 
 namespace {
 
-// dK/dV side at d = 64, dense calls: share every key tile between the two CTAs of a cluster?  This replays the static deal of
-// both forms in units of one 128-query step (2.3 per item, the kernel's measured overhead, and 1.5 more for the exchange of
-// the two parts) and takes the pairs where their longest CTA is 3 % shorter.
+// dK/dV side at d = 64: share every key tile between the two CTAs of a cluster?  This replays the static deal of both forms
+// in units of one 128-query step (2.3 per item, the kernel's measured overhead, and 1.5 more for the exchange of the two
+// parts) and takes the pairs where their longest CTA is 3 % shorter.  steps: per tile over all heads of a group, decreasing.
 // Measured, this kernel alone, whole tiles -> pairs: 16 query / 4 KV heads x 4096, causal: 121 -> 77 us; 8 / 2 heads x 8000,
 // causal: 229 -> 140; 32 / 4 heads x 2000: 121 -> 78; 4 heads x 4096, causal: 43.5 -> 37.2; 1 head x 8192: 62.0 -> 43.5;
-// 16 heads x 4096, causal (stays with whole tiles): 68.
-bool dkv_prefers_pairs(int BHkv, int n_kt, int G, int Nq, int Nk, bool causal, int sms, int pairs) {
-  const long long items = static_cast<long long>(BHkv) * n_kt;
+// 16 heads x 4096, causal (stays with whole tiles): 68; 16 packed documents of 8192 rows, 16 / 4 heads: 78.6 -> 73.0.
+bool dkv_prefers_pairs(const std::vector<int> &steps, int BHkv, int sms, int pairs) {
+  const long long items = static_cast<long long>(BHkv) * static_cast<long long>(steps.size());
   if (pairs < 1 || items > 8LL * sms) return false;      // many items per CTA: they balance as they are
-  static std::mutex memo_mutex;
-  static std::map<std::tuple<int, int, int, int, int, bool, int>, bool> memo;
-  const auto key = std::make_tuple(BHkv, n_kt, G, Nq, Nk, causal, sms);
-  {
-    std::lock_guard<std::mutex> lock(memo_mutex);
-    const auto hit = memo.find(key);
-    if (hit != memo.end()) return hit->second;
-  }
-  auto steps = [&](long long lin) {                      // longest tiles first, as the kernel orders them
-    const long long row0 = 128 * (lin / BHkv), off = static_cast<long long>(Nk) - Nq;
-    const long long first = causal ? std::min<long long>(std::max(0LL, row0 - off) & ~63LL, ((Nq - 1) >> 6) << 6) : 0;
-    return static_cast<double>(G * std::max(1LL, (Nq - first + 127) / 128));
-  };
-  const double whole = deal_makespan(items, sms, [&](long long lin) { return steps(lin) + 2.3; });
-  const double split = deal_makespan(items, pairs, [&](long long lin) { return std::ceil(0.5 * steps(lin)) + 3.8; });
-  std::lock_guard<std::mutex> lock(memo_mutex);
-  if (memo.size() < 4096) memo[key] = split < 0.97 * whole;
+  const double whole = deal_makespan(items, sms, [&](long long lin) { return steps[static_cast<size_t>(lin / BHkv)] + 2.3; });
+  const double split = deal_makespan(items, pairs, [&](long long lin) { return (steps[static_cast<size_t>(lin / BHkv)] + 1) / 2 + 3.8; });
   return split < 0.97 * whole;
+}
+
+// 128-query steps of the key tiles of a call, over the G heads of a group, decreasing.
+std::vector<int> dkv_steps(const PackedSeqs *seqs, int G, int Nq, int Nk, bool causal) {
+  const int cu_q[2] = {0, Nq}, cu_k[2] = {0, Nk};
+  const PackedSeqs one{cu_q, cu_k, 1, causal};
+  std::vector<int> steps = packed_work(seqs ? *seqs : one, true);
+  for (int &w : steps) w = G * std::max(1, (w + 127) / 128);
+  return steps;
 }
 
 // Dense call: plans == nullptr.  Packed call: B = 1, N / Nk = total query / key rows, plan_q / plan_kv = device tile lists
@@ -522,7 +570,7 @@ bool dkv_prefers_pairs(int BHkv, int n_kt, int G, int Nq, int Nk, bool causal, i
 int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const float *LSE, const void *dO,
                void *dQ, void *dK, void *dV, int B, int H, int Hkv, int N, int Nk, int d, float softmax_scale, int causal,
                void *workspace, size_t workspace_bytes, unsigned flags, const int4 *plan_q, const int4 *plan_kv,
-               int n_plan_q_tiles, int n_plan_kv_tiles, int nblk, void *stream) {
+               int n_plan_q_tiles, int n_plan_kv_tiles, int nblk, const PackedSeqs *seqs, void *stream) {
   if (!Q || !K || !V || !O || !LSE || !dO || !dQ || !dK || !dV) return GPROJ_ERR_NULL;
   if (int rc = check_shape(B, H, N, d)) return rc;
   if (Hkv <= 0 || H % Hkv != 0 || check_shape(B, Hkv, Nk, d) != GPROJ_OK) return GPROJ_ERR_SHAPE;
@@ -562,8 +610,12 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
   const int total_tiles = BH * n_qt, total_kv_tiles = BHkv * n_kt;
   if (total_tiles <= 0) return GPROJ_OK;   // nothing but empty sequences
   if (total_kv_tiles <= 0) run_dkv = false;   // packed call in which no sequence has both queries and keys
-  const ItemOrder group_q = item_order(BH, n_qt, tile_group_of(plan_q != nullptr, causal != 0, BH, n_qt, 2 * static_cast<size_t>(BHkv) * Nk * d * 2, st->sm_count, 3.25));    // streams K, V
-  const ItemOrder group_kv = item_order(BHkv, std::max(n_kt, 1), tile_group_of(plan_q != nullptr, causal != 0, BHkv, n_kt, 3 * static_cast<size_t>(BH) * N * d * 2, st->sm_count, 2.3));   // streams Q, dO, Z
+  ItemOrder group_q = item_order(BH, n_qt, tile_group_of(plan_q != nullptr, causal != 0, BH, n_qt, 2 * static_cast<size_t>(BHkv) * Nk * d * 2, st->sm_count, 3.25));    // streams K, V
+  ItemOrder group_kv = item_order(BHkv, std::max(n_kt, 1), tile_group_of(plan_q != nullptr, causal != 0, BHkv, n_kt, 3 * static_cast<size_t>(BH) * N * d * 2, st->sm_count, 2.3));   // streams Q, dO, Z
+  if (seqs) {
+    group_q.solo = packed_solo(*seqs, false, BH, st->sm_count, [&](int keys) { return std::max(1, (keys + 63) / 64) + (d == 64 ? 3.8 : 3.0); });
+    if (d == 128) group_kv.solo = packed_solo(*seqs, true, BHkv, st->sm_count, [&](int rows) { return G * std::max(1, (rows + 63) / 64) + 3.0; });
+  }
   const dim3 grid(static_cast<unsigned>(total_tiles < st->sm_count ? total_tiles : st->sm_count));   // persistent: one CTA per SM
   const dim3 grid_kv(static_cast<unsigned>(total_kv_tiles < st->sm_count ? total_kv_tiles : st->sm_count));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -585,7 +637,9 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
   } while (0)
   // At d = 64 the dK/dV side runs with 128-wide steps (every score product an N = 128 instruction); it streams 128-row
   // boxes, which the stationary-tile maps of the dQ side already are.
-  const bool pairs = d == 64 && run_dkv && !plan_q && dkv_prefers_pairs(BHkv, n_kt, G, N, Nk, causal != 0, st->sm_count, st->dkv_clusters);
+  const bool few_tiles = static_cast<long long>(total_kv_tiles) <= 8LL * st->sm_count;
+  const bool pairs = d == 64 && run_dkv && few_tiles && dkv_prefers_pairs(dkv_steps(seqs, G, N, Nk, causal != 0), BHkv, st->sm_count, st->dkv_clusters);
+  if (seqs && d == 64 && !pairs) group_kv.solo = packed_solo(*seqs, true, BHkv, st->sm_count, [&](int rows) { return G * std::max(1, (rows + 127) / 128) + 2.3; });
   const dim3 grid_dkv(pairs ? 2u * static_cast<unsigned>(std::min(total_kv_tiles, st->dkv_clusters)) : grid_kv.x);
 #define GPROJ_LAUNCH_BWD_W128(CC)                                                                                       \
   do {                                                                                                                  \
@@ -615,14 +669,14 @@ extern "C" {
 // ---- unequal query and key lengths ------------------------------------------------------------------
 int gproj_attn_fwd_rect(const void *Q, const void *K, const void *V, void *O, float *LSE, int B, int H, int Hkv, int Nq,
                         int Nk, int d, float softmax_scale, int causal, unsigned fwd_flags, void *stream) {
-  return launch_fwd(Q, K, V, O, LSE, B, H, Hkv, Nq, Nk, d, softmax_scale, causal, fwd_flags, nullptr, 0, 0, stream);
+  return launch_fwd(Q, K, V, O, LSE, B, H, Hkv, Nq, Nk, d, softmax_scale, causal, fwd_flags, nullptr, 0, nullptr, stream);
 }
 
 int gproj_attn_bwd_rect(const void *Q, const void *K, const void *V, const void *O, const float *LSE, const void *dO,
                         void *dQ, void *dK, void *dV, int B, int H, int Hkv, int Nq, int Nk, int d, float softmax_scale,
                         int causal, void *workspace, size_t workspace_bytes, unsigned flags, void *stream) {
   return launch_bwd(Q, K, V, O, LSE, dO, dQ, dK, dV, B, H, Hkv, Nq, Nk, d, softmax_scale, causal, workspace, workspace_bytes,
-                    flags, nullptr, nullptr, 0, 0, (Nq + 63) / 64, stream);
+                    flags, nullptr, nullptr, 0, 0, (Nq + 63) / 64, nullptr, stream);
 }
 
 // ---- packed (variable-length) sequences ------------------------------------------------------------
@@ -700,10 +754,9 @@ int fwd_packed(const void *Q, const void *K, const void *V, void *O, float *LSE,
   if (!packed_shape(cu_q, cu_k, num_seqs, &ps)) return GPROJ_ERR_SHAPE;
   if (!plan_device) return GPROJ_ERR_NULL;
   if (reinterpret_cast<uintptr_t>(plan_device) & 15u) return GPROJ_ERR_ALIGN;
-  int longest_keys = 0;
-  for (int q = 0; q < num_seqs; ++q) longest_keys = std::max(longest_keys, cu_k[q + 1] - cu_k[q]);
+  const PackedSeqs seqs{cu_q, cu_k, num_seqs, causal != 0};
   return launch_fwd(Q, K, V, O, LSE, 1, H, Hkv, ps.total_q, ps.total_k, d, softmax_scale, causal, fwd_flags,
-                    static_cast<const int4 *>(plan_device), ps.q_tiles, longest_keys, stream);
+                    static_cast<const int4 *>(plan_device), ps.q_tiles, &seqs, stream);
 }
 
 int bwd_packed(const void *Q, const void *K, const void *V, const void *O, const float *LSE, const void *dO, void *dQ, void *dK,
@@ -714,9 +767,10 @@ int bwd_packed(const void *Q, const void *K, const void *V, const void *O, const
   if (!plan_device) return GPROJ_ERR_NULL;
   if (reinterpret_cast<uintptr_t>(plan_device) & 15u) return GPROJ_ERR_ALIGN;
   const int4 *plan = static_cast<const int4 *>(plan_device);
+  const PackedSeqs seqs{cu_q, cu_k, num_seqs, causal != 0};
   const int rc = launch_bwd(Q, K, V, O, LSE, dO, dQ, dK, dV, 1, H, Hkv, ps.total_q, ps.total_k, d, softmax_scale, causal, workspace,
                             workspace_bytes, flags, plan, plan + 2 * static_cast<size_t>(ps.q_tiles), ps.q_tiles, ps.kv_tiles,
-                            ps.nblk, stream);
+                            ps.nblk, &seqs, stream);
   if (rc != GPROJ_OK || (flags & GPROJ_FLAG_ONLY_DQ_PASS)) return rc;
   // Keys of a sequence without queries are in no tile: their gradient rows are zero.
   const int launches = tl_launch_count;

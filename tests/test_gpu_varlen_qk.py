@@ -149,3 +149,19 @@ def test_random_packings(seed):
     inp = make(Hkv * G, Hkv, lq, lk, d, seed=seed)
     ex = oracle_packed(inp, lq, lk, d ** -0.5, causal)
     print("packing", lq, lk, d, Hkv * G, Hkv, causal, check(run_gpu(inp, lq, lk, d ** -0.5, causal), ex))
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("causal", [True, False])
+def test_few_tiles_longer_than_an_even_share(d, causal):
+    # one long sequence and many short ones over enough heads that CTAs walk several tiles: the CTAs that start with a long
+    # tile get no second one, the others share the rest in rounds of fewer CTAs.  Every row must still be written once.
+    lq, lk = [300] + [90, 130] * 6, [2500] + [70, 40] * 6
+    H = 16
+    inp = make(H, H, lq, lk, d, seed=77 + d)
+    got = run_gpu(inp, lq, lk, d ** -0.5, causal)
+    heads = [0, 7, 15]
+    some = {n: t[heads].contiguous() for n, t in inp.items()}
+    ex = oracle_packed(some, lq, lk, d ** -0.5, causal)
+    check({n: got[n][heads] for n in ex}, ex)
+    assert all(np.all(np.isfinite(got[n])) for n in ("O", "dQ", "dK", "dV"))
