@@ -419,10 +419,10 @@ bool fwd_prefers_single_tiles(int BH, int n_qt, int sms) {
 // CTAs per query tile of the forward (its base-two logarithm): with few tiles and long key ranges a tile's key range is
 // split over a cluster of 2, 4 or 8 CTAs, as many as leave each of their two warpgroups at least two 128-key tiles and let
 // all clusters run at once (`fit`: how many clusters of 2^lg CTAs do).  Beyond one wave the split only adds its merge, and
-// below 16 key tiles the launch and the merge of a cluster (about 6 us) cost what they save.  Measured, one CTA per tile ->
-// cluster: 8 x (16 query, 4 KV heads) x 16 queries behind 16384 keys, d = 64: 109.7 -> 51.8 us (with the query heads
-// folded, see launch_fwd), behind 8192: 58.5 -> 33.0, behind 4096: 33.2 -> 22.9, behind 2048: 20.6 -> 18.6; 4 x 8 heads x 1
-// query behind 16384 keys, d = 128: 201 -> 72 us; 4 heads x 1000 x 128 (8 key tiles): 18.7 -> 20.7 us, hence the 16.
+// below 16 key tiles the launch and the merge of a cluster cost what they save.  Measured, one CTA per tile -> cluster: 8 x (16
+// query, 4 KV heads) x 16 queries behind 16384 keys, d = 64: 109.7 -> 45.7 us (with the query heads folded, see
+// launch_fwd), behind 8192: 58.5 -> 27.2, behind 2048: 20.6 -> 13.6; 4 x 8 heads x 1 query behind 16384 keys, d = 128: 201 ->
+// 63 us; 4 heads x 1000 x 128 (8 key tiles, with a merge by scattered stores): 18.7 -> 20.7 us, hence the 16.
 int fwd_cluster_log2(long long tiles, int key_tiles, const int (&fit)[4]) {
   int lg = 0;
   while (lg < 3 && key_tiles >= std::max(16, 4 << (lg + 1)) && tiles <= fit[lg + 1]) ++lg;
