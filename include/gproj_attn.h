@@ -203,7 +203,7 @@ int gproj_attn_bwd_varlen_qk(const void *Q, const void *K, const void *V, const 
  * Forward and backward in one call from HOST buffers (a convenience around the entry points above; the paper's
  * Algorithm 1 starts from tensors already on the device).  Q, K, V, dO are copied to the device, the forward
  * (Eq. "gproj-forward") and the backward (Algorithm 1) run, and dQ, dK, dV (and O, LSE when those pointers are not NULL)
- * are copied back.  Large problems are cut into up to 16 slabs of whole KV heads (about 2 MiB of Q each) that are pipelined:
+ * are copied back.  Large problems are cut into up to 16 slabs of whole KV heads (about 2.75 MiB of Q each) that are pipelined:
  * the kernels run on `stream`, the copies in and out on two internal streams, ordered by events so that nothing of the call
  * starts before the work already queued on `stream` and `stream` reaches the end of the call only after the last copy-out.
  *   - Q, K, V, dO, O, LSE, dQ, dK, dV are HOST pointers with the layouts of gproj_attn_fwd_gqa / gproj_attn_bwd_gqa.  Page-locked
@@ -211,7 +211,7 @@ int gproj_attn_bwd_varlen_qk(const void *Q, const void *K, const void *V, const 
  *     valid until the stream has reached the end of the call's work.
  *   - `staging` is DEVICE memory owned by the caller, 256-byte aligned, at least gproj_attn_host_staging_bytes() bytes (copies
  *     of the eight tensors, LSE and the backward workspace); GPROJ_ERR_WORKSPACE otherwise.  No device memory is allocated;
- *     the first pipelined call on a device creates the two streams and 34 events, which live until the process exits.
+ *     the first pipelined call on a device creates the two streams and 66 events, which live until the process exits.
  *   - flags: those of gproj_attn_bwd without the ONLY_* bits (GPROJ_ERR_FLAGS for those).
  *   - Calls from several host threads on one device are serialised while they enqueue.
  *   - If the call returns an error after it has begun to enqueue work, `stream` has been made to wait for everything

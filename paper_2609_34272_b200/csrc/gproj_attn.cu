@@ -41,10 +41,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-#ifndef GPROJ_HOST_SLAB_LOG2
-#define GPROJ_HOST_SLAB_LOG2 21
-#endif
-constexpr int kHostSlabLog2 = GPROJ_HOST_SLAB_LOG2;   // log2 of the Q bytes per slab of the host-buffer entry point
+constexpr size_t kHostSlabBytes = 11u << 18;   // Q bytes per slab of the host-buffer entry point: 2.75 MiB
 constexpr int kMaxSlabs = 16;   // the host-buffer entry point pipelines at most this many slabs of heads
 
 struct DeviceState {
@@ -57,7 +54,7 @@ struct DeviceState {
   // host-buffer entry point only: copy-in and copy-out streams and the events that order them against the caller's stream
   bool pipe_ready = false;
   cudaStream_t in_stream = nullptr, out_stream = nullptr;
-  cudaEvent_t ev_start = nullptr, ev_end = nullptr, ev_in[kMaxSlabs] = {}, ev_done[kMaxSlabs] = {};
+  cudaEvent_t ev_start = nullptr, ev_end = nullptr, ev_in[kMaxSlabs] = {}, ev_in_dO[kMaxSlabs] = {}, ev_dq[kMaxSlabs] = {}, ev_done[kMaxSlabs] = {};
 };
 
 std::mutex g_mutex;
@@ -876,10 +873,14 @@ int gproj_attn_fwd_bwd_host(const void *Q, const void *K, const void *V, const v
 
   // The (batch, KV head) axis is cut into slabs of whole KV heads with their query heads (contiguous in every tensor), and
   // the slabs are pipelined: copy-in of slab c + 1 and copy-out of slab c - 1 run on two internal streams while the
-  // caller's stream computes slab c.  About 2 MiB of Q and at least 128 key tiles per slab: smaller slabs leave the
-  // persistent kernels too few tiles (measured: slower than no pipeline at all), larger ones leave the copies exposed.
+  // caller's stream computes slab c.  About 2.75 MiB of Q and at least 128 key tiles per slab: every copy costs some 4 us of
+  // its direction beyond its bytes and the two directions share about 80 GB/s, so many small slabs are slower than few
+  // large ones, while the last slab's kernels and copy-out stay exposed.  The forward starts without dO, and dQ leaves while
+  // dK and dV are computed.  Measured, before (2 MiB slabs, all inputs first, all gradients together) -> now: 16 heads x 4096
+  // x 64: 1020 -> 919 us; 2 x (16 query, 4 KV heads) x 6000 x 64: 1960 -> 1800; 64 heads x 4000 x 128: 6640 -> 6100; 16 / 8
+  // heads x 7000 x 64, not causal: 1930 -> 1608.
   const int kv_heads = B * Hkv, G = H / Hkv;
-  int slabs = static_cast<int>((qb + (size_t(1) << (kHostSlabLog2 - 1))) >> kHostSlabLog2);
+  int slabs = static_cast<int>((qb + kHostSlabBytes / 2) / kHostSlabBytes);
   const long long kv_tiles = static_cast<long long>(kv_heads) * ((N + 127) / 128);
   slabs = std::min(slabs, static_cast<int>(std::min<long long>(kv_tiles / 128, kMaxSlabs)));   // >= 128 key tiles per slab
   slabs = std::max(1, std::min(slabs, kv_heads));
@@ -893,6 +894,8 @@ int gproj_attn_fwd_bwd_host(const void *Q, const void *K, const void *V, const v
               cudaEventCreateWithFlags(&st->ev_end, cudaEventDisableTiming) == cudaSuccess;
     for (int i = 0; ok && i < kMaxSlabs; ++i)
       ok = cudaEventCreateWithFlags(&st->ev_in[i], cudaEventDisableTiming) == cudaSuccess &&
+           cudaEventCreateWithFlags(&st->ev_in_dO[i], cudaEventDisableTiming) == cudaSuccess &&
+           cudaEventCreateWithFlags(&st->ev_dq[i], cudaEventDisableTiming) == cudaSuccess &&
            cudaEventCreateWithFlags(&st->ev_done[i], cudaEventDisableTiming) == cudaSuccess;
     if (!ok) { (void)cudaGetLastError(); return GPROJ_ERR_CUDA; }
     st->pipe_ready = true;
@@ -910,15 +913,23 @@ int gproj_attn_fwd_bwd_host(const void *Q, const void *K, const void *V, const v
   auto slab_begin = [&](int c) {
     if (c >= slabs) return kv_heads;
     if (slabs == 1 || kv_heads < 2 * slabs) return static_cast<int>(static_cast<long long>(kv_heads) * c / slabs);
-    return static_cast<int>((2LL * kv_heads * c + (2 * slabs - 1) / 2) / (2 * slabs - 1));
+    return static_cast<int>((2LL * kv_heads * c + (2 * slabs - 2)) / (2 * slabs - 1));
   };
+  // Queue a copy between `at` bytes into a host and a device buffer.
+  auto copy_in = [&](uint8_t *dev, const void *host, size_t at, size_t bytes) {
+    return cudaMemcpyAsync(dev + at, static_cast<const uint8_t *>(host) + at, bytes, cudaMemcpyHostToDevice, s_in) == cudaSuccess;
+  };
+  auto copy_out = [&](void *host, const uint8_t *dev, size_t at, size_t bytes) {
+    return cudaMemcpyAsync(static_cast<uint8_t *>(host) + at, dev + at, bytes, cudaMemcpyDeviceToHost, s_out) == cudaSuccess;
+  };
+  auto mark = [&](cudaEvent_t e, cudaStream_t on) { return slabs == 1 || cudaEventRecord(e, on) == cudaSuccess; };
+  auto after = [&](cudaStream_t on, cudaEvent_t e) { return slabs == 1 || cudaStreamWaitEvent(on, e, 0) == cudaSuccess; };
   for (int c = 0; ok && c < slabs; ++c) {
     const size_t k0 = slab_begin(c), kn = slab_begin(c + 1) - k0, q0 = k0 * G, qn = kn * G;
-    ok = cudaMemcpyAsync(dQin + q0 * row_bytes, static_cast<const uint8_t *>(Q) + q0 * row_bytes, qn * row_bytes, cudaMemcpyHostToDevice, s_in) == cudaSuccess &&
-         cudaMemcpyAsync(dKin + k0 * row_bytes, static_cast<const uint8_t *>(K) + k0 * row_bytes, kn * row_bytes, cudaMemcpyHostToDevice, s_in) == cudaSuccess &&
-         cudaMemcpyAsync(dVin + k0 * row_bytes, static_cast<const uint8_t *>(V) + k0 * row_bytes, kn * row_bytes, cudaMemcpyHostToDevice, s_in) == cudaSuccess &&
-         cudaMemcpyAsync(dOin + q0 * row_bytes, static_cast<const uint8_t *>(dO) + q0 * row_bytes, qn * row_bytes, cudaMemcpyHostToDevice, s_in) == cudaSuccess;
-    if (ok && slabs > 1) ok = cudaEventRecord(st->ev_in[c], s_in) == cudaSuccess;
+    // the forward starts without dO
+    ok = copy_in(dQin, Q, q0 * row_bytes, qn * row_bytes) && copy_in(dKin, K, k0 * row_bytes, kn * row_bytes) &&
+         copy_in(dVin, V, k0 * row_bytes, kn * row_bytes) && mark(st->ev_in[c], s_in) &&
+         copy_in(dOin, dO, q0 * row_bytes, qn * row_bytes) && mark(st->ev_in_dO[c], s_in);
   }
   // After the first copy has been queued, an error return first makes the caller's stream wait for whatever the call
   // put on its internal streams, so that synchronising `stream` tells the caller its host buffers are free again.
@@ -935,24 +946,36 @@ int gproj_attn_fwd_bwd_host(const void *Q, const void *K, const void *V, const v
   int launches = 0;
   for (int c = 0; c < slabs; ++c) {
     const size_t k0 = slab_begin(c), kn = slab_begin(c + 1) - k0, q0 = k0 * G, qn = kn * G;
-    if (slabs > 1 && cudaStreamWaitEvent(s, st->ev_in[c], 0) != cudaSuccess) return fail(GPROJ_ERR_CUDA);
+    if (!after(s, st->ev_in[c])) return fail(GPROJ_ERR_CUDA);
     float *lse_c = reinterpret_cast<float *>(dLSE + q0 * N * sizeof(float));
     // a slab is a problem with batch 1, kn KV heads and qn query heads; the slabs share the backward workspace in turn
     if (int rc = gproj_attn_fwd_gqa(dQin + q0 * row_bytes, dKin + k0 * row_bytes, dVin + k0 * row_bytes, dOout + q0 * row_bytes, lse_c, 1,
                                     static_cast<int>(qn), static_cast<int>(kn), N, d, softmax_scale, causal, stream))
       return fail(rc);
     launches += tl_launch_count;
-    if (int rc = gproj_attn_bwd_gqa(dQin + q0 * row_bytes, dKin + k0 * row_bytes, dVin + k0 * row_bytes, dOout + q0 * row_bytes, lse_c,
-                                    dOin + q0 * row_bytes, dQout + q0 * row_bytes, dKout + k0 * row_bytes, dVout + k0 * row_bytes, 1,
-                                    static_cast<int>(qn), static_cast<int>(kn), N, d, softmax_scale, causal, ws, ws_bytes, flags, stream))
-      return fail(rc);
-    launches += tl_launch_count;
-    ok = slabs == 1 || (cudaEventRecord(st->ev_done[c], s) == cudaSuccess && cudaStreamWaitEvent(s_out, st->ev_done[c], 0) == cudaSuccess);
-    ok = ok && cudaMemcpyAsync(static_cast<uint8_t *>(dQ) + q0 * row_bytes, dQout + q0 * row_bytes, qn * row_bytes, cudaMemcpyDeviceToHost, s_out) == cudaSuccess &&
-         cudaMemcpyAsync(static_cast<uint8_t *>(dK) + k0 * row_bytes, dKout + k0 * row_bytes, kn * row_bytes, cudaMemcpyDeviceToHost, s_out) == cudaSuccess &&
-         cudaMemcpyAsync(static_cast<uint8_t *>(dV) + k0 * row_bytes, dVout + k0 * row_bytes, kn * row_bytes, cudaMemcpyDeviceToHost, s_out) == cudaSuccess;
-    if (ok && O) ok = cudaMemcpyAsync(static_cast<uint8_t *>(O) + q0 * row_bytes, dOout + q0 * row_bytes, qn * row_bytes, cudaMemcpyDeviceToHost, s_out) == cudaSuccess;
+    if (!after(s, st->ev_in_dO[c])) return fail(GPROJ_ERR_CUDA);
+    auto backward = [&](unsigned only) {
+      const int rc = gproj_attn_bwd_gqa(dQin + q0 * row_bytes, dKin + k0 * row_bytes, dVin + k0 * row_bytes, dOout + q0 * row_bytes, lse_c,
+                                        dOin + q0 * row_bytes, dQout + q0 * row_bytes, dKout + k0 * row_bytes, dVout + k0 * row_bytes, 1,
+                                        static_cast<int>(qn), static_cast<int>(kn), N, d, softmax_scale, causal, ws, ws_bytes, flags | only, stream);
+      launches += tl_launch_count;
+      return rc;
+    };
+    if (slabs == 1) {
+      if (int rc = backward(0u)) return fail(rc);
+    } else {
+      // the two backward kernels one by one, so that dQ is on its way out while dK and dV are computed
+      if (int rc = backward(GPROJ_FLAG_ONLY_DQ_PASS)) return fail(rc);
+      if (!mark(st->ev_dq[c], s) || !after(s_out, st->ev_dq[c])) return fail(GPROJ_ERR_CUDA);
+    }
+    ok = copy_out(dQ, dQout, q0 * row_bytes, qn * row_bytes);
+    if (ok && O) ok = copy_out(O, dOout, q0 * row_bytes, qn * row_bytes);
     if (ok && LSE) ok = cudaMemcpyAsync(LSE + q0 * N, lse_c, qn * N * sizeof(float), cudaMemcpyDeviceToHost, s_out) == cudaSuccess;
+    if (!ok) return fail(GPROJ_ERR_CUDA);
+    if (slabs > 1)
+      if (int rc = backward(GPROJ_FLAG_ONLY_DKV_PASS)) return fail(rc);
+    ok = mark(st->ev_done[c], s) && after(s_out, st->ev_done[c]) && copy_out(dK, dKout, k0 * row_bytes, kn * row_bytes) &&
+         copy_out(dV, dVout, k0 * row_bytes, kn * row_bytes);
     if (!ok) return fail(GPROJ_ERR_CUDA);
   }
   // the caller's stream reaches the end of the call only when the last copy-out has landed
