@@ -41,7 +41,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-constexpr size_t kHostSlabBytes = 11u << 18;   // Q bytes per slab of the host-buffer entry point: 2.75 MiB
+constexpr size_t kHostSlabBytes = 4u << 20;   // the host-buffer entry point cuts one more slab for every so many bytes of Q
 constexpr int kMaxSlabs = 16;   // the host-buffer entry point pipelines at most this many slabs of heads
 
 struct DeviceState {
@@ -873,14 +873,14 @@ int gproj_attn_fwd_bwd_host(const void *Q, const void *K, const void *V, const v
 
   // The (batch, KV head) axis is cut into slabs of whole KV heads with their query heads (contiguous in every tensor), and
   // the slabs are pipelined: copy-in of slab c + 1 and copy-out of slab c - 1 run on two internal streams while the
-  // caller's stream computes slab c.  About 2.75 MiB of Q and at least 128 key tiles per slab: every copy costs some 4 us of
+  // caller's stream computes slab c.  2 to 4 MiB of Q and at least 128 key tiles per slab: every copy costs some 4 us of
   // its direction beyond its bytes and the two directions share about 80 GB/s, so many small slabs are slower than few
   // large ones, while the last slab's kernels and copy-out stay exposed.  The forward starts without dO, and dQ leaves while
   // dK and dV are computed.  Measured, before (2 MiB slabs, all inputs first, all gradients together) -> now: 16 heads x 4096
   // x 64: 1020 -> 919 us; 2 x (16 query, 4 KV heads) x 6000 x 64: 1960 -> 1800; 64 heads x 4000 x 128: 6640 -> 6100; 16 / 8
   // heads x 7000 x 64, not causal: 1930 -> 1608.
   const int kv_heads = B * Hkv, G = H / Hkv;
-  int slabs = static_cast<int>((qb + kHostSlabBytes / 2) / kHostSlabBytes);
+  int slabs = static_cast<int>(1 + qb / kHostSlabBytes);
   const long long kv_tiles = static_cast<long long>(kv_heads) * ((N + 127) / 128);
   slabs = std::min(slabs, static_cast<int>(std::min<long long>(kv_tiles / 128, kMaxSlabs)));   // >= 128 key tiles per slab
   slabs = std::max(1, std::min(slabs, kv_heads));
