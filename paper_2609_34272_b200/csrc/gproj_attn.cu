@@ -1154,11 +1154,11 @@ static int smooth_rows(const void *X, void *Y, int heads, long long rows_total, 
       ++q;
     }
     if (m == 0) continue;
+    const int cluster = static_cast<long long>(m) * heads * 8 <= st->sm_count * 3LL ? 8 : 4;   // eight while all CTAs run at once
     for (int h0 = 0; h0 < heads; h0 += 65535) {       // heads along y, whose limit is 65535
-      const dim3 grid(static_cast<unsigned>(m * kSmoothCluster), static_cast<unsigned>(std::min(heads - h0, 65535)));
+      const dim3 grid(static_cast<unsigned>(m * cluster), static_cast<unsigned>(std::min(heads - h0, 65535)));
       const long long at = static_cast<long long>(h0) * rows_total * d;
-      if (d == 64) smooth_rows_kernel<64><<<grid, kSmoothThreads, 0, s>>>(x + at, y + at, rows_total * d, off);
-      else         smooth_rows_kernel<128><<<grid, kSmoothThreads, 0, s>>>(x + at, y + at, rows_total * d, off);
+      launch_after(d == 64 ? smooth_rows_kernel<64> : smooth_rows_kernel<128>, grid, cluster, kSmoothThreads, 0, s, true, x + at, y + at, rows_total * d, off);
       ++launches;
     }
   }

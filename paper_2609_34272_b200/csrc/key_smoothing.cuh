@@ -7,13 +7,13 @@
 //                        the vector-Jacobian product of the subtraction (in exact arithmetic sum_j dK~_j = 0,
 //                        Proposition 3.1, so the second call removes only what rounding leaked into that sum).
 //
-// One cluster of eight CTAs per (head, sequence), all sequences of a call in one launch (the offsets travel as a kernel
-// parameter).  A CTA takes an eighth of the rows, keeps as many of them in registers as fit (256 rows at d = 64, so
-// that sequences up to 2048 rows are read once; what is beyond is read a second time, from L2), and the eight column
-// sums are exchanged through distributed shared memory.  Sums are FP32 in a fixed order, so results are reproducible.
-// One CTA per (head, sequence) and one launch per sequence, as it was before, left 4 of 148 SMs busy for a document on
-// four KV heads: 16 documents, 8192 rows, 4 heads, d = 64: 92.6 us a call then, 16.9 us now; 24 documents, 16384 rows:
-// 157.7 us then, 20.5 us now.  (512 threads per CTA, one CTA per SM: 30.7 us on the first.)
+// One cluster of four CTAs (eight where the call has few sequences and heads) per (head, sequence), all sequences of a call in
+// one launch (the offsets travel as a kernel parameter).  A CTA takes its share of the rows, keeps as many of them in
+// registers as fit (256 rows at d = 64, so that sequences up to 1024 rows are read once; what is beyond is read a second
+// time, from L2), and the column sums are exchanged through distributed shared memory.  Sums are FP32 in a fixed order, so
+// results are reproducible.  What a call takes is the latency of one CTA (load, two exchanges, store) times the waves of
+// CTAs.  Measured, 16 documents, 8192 rows, 4 heads, d = 64: 92.6 us a call with one CTA per (head, sequence) and a launch per
+// sequence, 17.2 us with clusters of eight, 10.0 us with clusters of four; 24 documents, 16384 rows: 157.7, 20.5, 10.3 us.
 #pragma once
 #include <cuda_bf16.h>
 #include <stdint.h>
@@ -22,20 +22,22 @@
 
 namespace gproj {
 
-constexpr int kSmoothThreads = 256, kSmoothCluster = 8, kSmoothMaxSeqs = 512;
+constexpr int kSmoothThreads = 256, kSmoothMaxSeqs = 512;
 struct SmoothOffsets { int cu[kSmoothMaxSeqs + 1]; };
 
-// X, Y: [heads][rows_total][d] BF16; sequence blockIdx.x / kSmoothCluster of head blockIdx.y.
+// X, Y: [heads][rows_total][d] BF16; sequence blockIdx.x / (cluster size) of head blockIdx.y.
 template <int D>
-__global__ void __launch_bounds__(kSmoothThreads, 3) __cluster_dims__(kSmoothCluster, 1, 1)
+__global__ void __launch_bounds__(kSmoothThreads, 3)
 smooth_rows_kernel(const __nv_bfloat16 *__restrict__ X, __nv_bfloat16 *__restrict__ Y, long long head_stride, const __grid_constant__ SmoothOffsets off) {
   constexpr int kLanes = D / 8;                       // threads across a row (8 BF16 = 16 bytes each)
   constexpr int kRowsPerPass = kSmoothThreads / kLanes, kWarps = kSmoothThreads / 32, kKeep = 8;
   __shared__ float part[kWarps][D];
   __shared__ __align__(16) float cta_sum[D];
-  const int seq = blockIdx.x / kSmoothCluster, rank = blockIdx.x % kSmoothCluster;
+  griddep_wait();
+  griddep_launch_dependents();
+  const int ncta = cluster_size(), rank = cluster_rank(), seq = blockIdx.x / ncta;
   const int row0 = off.cu[seq], rows = off.cu[seq + 1] - row0;
-  const int per = (rows + kSmoothCluster - 1) / kSmoothCluster, r_begin = min(rows, rank * per), r_end = min(rows, r_begin + per);
+  const int per = (rows + ncta - 1) / ncta, r_begin = min(rows, rank * per), r_end = min(rows, r_begin + per);
   const int lane8 = threadIdx.x % kLanes, rsub = threadIdx.x / kLanes, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long base = static_cast<long long>(blockIdx.y) * head_stride + static_cast<long long>(row0) * D + 8 * lane8;
   const __nv_bfloat16 *x = X + base;
@@ -77,8 +79,8 @@ smooth_rows_kernel(const __nv_bfloat16 *__restrict__ X, __nv_bfloat16 *__restric
   float m[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) m[i] = 0.f;
-#pragma unroll
-  for (int c = 0; c < kSmoothCluster; ++c) {
+#pragma unroll 4
+  for (int c = 0; c < ncta; ++c) {
     const uint32_t remote = cluster_map_shared(smem_u32(&cta_sum[8 * lane8]), c);
     float v[8];
     cluster_load_f4(remote, v);
