@@ -183,7 +183,7 @@ __device__ __forceinline__ void store_rows_clipped(const uint8_t *stage, int sla
 }
 
 enum BwdWaitCode {
-  kDqWaitQ = 0x21, kDqWaitKV = 0x22, kDqWaitKVEmpty = 0x23, kDqWaitSdP = 0x24, kDqWaitTR = 0x25, kDqWaitAcc = 0x26, kDqWaitBuf = 0x27, kDqWaitResFree = 0x28, kDqWaitAccFree = 0x29, kDqWaitStats = 0x2a, kDqWaitMass = 0x2b,
+  kDqWaitQ = 0x21, kDqWaitKV = 0x22, kDqWaitKVEmpty = 0x23, kDqWaitSdP = 0x24, kDqWaitTR = 0x25, kDqWaitAcc = 0x26, kDqWaitBuf = 0x27, kDqWaitResFree = 0x28, kDqWaitAccFree = 0x29, kDqWaitStats = 0x2a, kDqWaitMass = 0x2b, kDqWaitPeer = 0x2c,
   kDkvWaitKV = 0x31, kDkvWaitQ = 0x32, kDkvWaitQEmpty = 0x33, kDkvWaitSdP = 0x34, kDkvWaitTR = 0x35, kDkvWaitAcc = 0x36, kDkvWaitBuf = 0x37, kDkvWaitResFree = 0x38, kDkvWaitAccFree = 0x39
 };
 
@@ -361,7 +361,10 @@ __device__ __forceinline__ void saved_output_dots(const __nv_bfloat16 *O, const 
 // ============================================================================================
 // dQ side
 // ============================================================================================
-template <int D, bool CAUSAL>
+// CL = 2: a cluster of two CTAs shares every tile: CTA r takes the key steps r, r + 2, ...; the row masses are exchanged, and CTA
+// r gets both parts of A and B for its half of the columns (over the consumed Q / dO buffer), of which it writes dQ and Z.
+// Used where whole tiles cannot be dealt evenly.
+template <int D, bool CAUSAL, int CL>
 __global__ void __launch_bounds__(BwdCfg<D>::kDqThreads, 1)
 bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
               const __grid_constant__ CUtensorMap tmdO,   // box 64 x 128 rows
@@ -383,7 +386,8 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
 
   __shared__ uint64_t bar_res_full[R], bar_res_free[R], bar_kv_full[S], bar_kv_empty[S];
   __shared__ uint64_t bar_sdp_full[NB], bar_tr_ready[NB], bar_acc_done, bar_acc_free, bar_drain[2];
-  __shared__ uint64_t bar_stats_ready[2], bar_mass_ready[2], bar_mass_free[2];
+  __shared__ uint64_t bar_stats_ready[2], bar_mass_ready[2], bar_mass_free[2], bar_peer_mass, bar_peer_ready, bar_peer_full;
+  __shared__ float s_peer[CL > 1 ? 4 : 1][128];          // the other CTA's rho and m, by tile parity
   __shared__ uint32_t tmem_base_smem;
   __shared__ int cta_abort, cta_skip;
   // per tile parity: row constants for the compute warpgroups, their row masses for the epilogue
@@ -392,18 +396,19 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) cta_skip = *reinterpret_cast<volatile int *>(status);
   __syncthreads();
-  if (cta_skip != 0) return;   // an earlier wait gave up: drain the rest of the grid quickly
+  if (CL == 1 && cta_skip != 0) return;   // an earlier wait gave up: drain the rest of the grid quickly (a cluster runs on with every wait falling through)
 
   // Ragged N: tiles and steps round up; rows past N load as zero (TMA fill) and are clipped on store.
   const int n_qt = (N + 127) / 128;
   AbortState ab{status, &cta_abort};
   if (threadIdx.x == 0) {
-    cta_abort = 0;
-    for (int r = 0; r < R; ++r) { mbar_init(&bar_res_full[r], 1); mbar_init(&bar_res_free[r], 1); }
+    cta_abort = CL > 1 ? cta_skip : 0;
+    for (int r = 0; r < R; ++r) { mbar_init(&bar_res_full[r], 1); mbar_init(&bar_res_free[r], CL > 1 ? 1 + 128 : 1); }
     for (int p = 0; p < 2; ++p) { mbar_init(&bar_stats_ready[p], 128); mbar_init(&bar_mass_ready[p], C::kCompute); mbar_init(&bar_mass_free[p], 128); }
     for (int s = 0; s < S; ++s) { mbar_init(&bar_kv_full[s], 1); mbar_init(&bar_kv_empty[s], 1); }
     for (int b = 0; b < NB; ++b) { mbar_init(&bar_sdp_full[b], 1); mbar_init(&bar_tr_ready[b], 128 * C::kSlices); }
     mbar_init(&bar_acc_done, 1);
+    mbar_init(&bar_peer_mass, 128); mbar_init(&bar_peer_ready, 1); mbar_init(&bar_peer_full, 128);
     mbar_init(&bar_acc_free, 128);
     mbar_init(&bar_drain[0], 1);
     mbar_init(&bar_drain[1], 1);
@@ -414,7 +419,7 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
     tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmdO); tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV);
   }
   tc_fence_before();
-  __syncthreads();
+  if (CL > 1) cluster_sync(); else __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, tmem_base_smem, 0);   // the shuffle marks it warp-uniform
 
@@ -424,7 +429,8 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
   griddep_wait();
   griddep_launch_dependents();
 
-  TileSched sched(total_tiles, order.solo);
+  TileSched sched(total_tiles, order.solo, CL);
+  const int rank = CL > 1 ? cluster_rank() : 0;
   // tile decode: causal -> longest rows first
   auto tix = [&](int lin) { return order.rank(lin); };
   auto hix = [&](int lin) { return order.head(lin); };
@@ -436,6 +442,9 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
     const int kend = CAUSAL ? min(Lk, t.row0 - t.seq0 + 128 + off) : Lk;
     return max(1, (max(kend, 0) + C::kStepRows - 1) / C::kStepRows);
   };
+  // This CTA's steps of a tile with T steps, and the n-th of them; a CTA that gets none runs step 0 fully masked.
+  auto own_steps = [&](int T) { return CL == 1 ? T : max(1, (T - rank + CL - 1) / CL); };
+  auto own_step = [&](int n, int T) { return CL == 1 ? n : (rank < T ? CL * n + rank : 0); };
 
   if (warp < 4) {
   if constexpr (C::kDqMoveRegs) setmaxnreg_dec<C::kDqRegsAux>();
@@ -446,8 +455,8 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
       for (int lin = sched.next(); lin >= 0; lin = sched.next()) {
         const TileInfo tl = tile_of(lin);
         const int bh = hix(lin), T = steps_of(tl);
-        for (int n = 0; n < T; ++n, ++g) {
-          const int st = g % S;
+        for (int m = 0; m < own_steps(T); ++m, ++g) {
+          const int st = g % S, n = own_step(m, T);
           if (g >= S) mbar_wait(&bar_kv_empty[st], ((g / S) - 1) & 1, ab, kDqWaitKVEmpty);
           mbar_expect_tx(&bar_kv_full[st], C::kDqStageBytes);
           uint8_t *dst = sKV + st * C::kDqStageBytes;
@@ -493,7 +502,7 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
     const SmemDesc dscK0 = make_smem_desc(smem_u32(sKV), 16, 1024);                          // K-major view of stage 0
     int g = 0, ti = 0;
     for (int lin = sched.next(); lin >= 0; lin = sched.next(), ++ti) {
-      const int T = steps_of(tile_of(lin)), rb = ti % R;
+      const int T = own_steps(steps_of(tile_of(lin))), rb = ti % R;
       mbar_wait(&bar_res_full[rb], (ti / R) & 1, ab, kDqWaitQ);
       const SmemDesc dscQ = dscRes0.advanced(rb * 2 * C::kBigTileBytes), dscdO = dscQ.advanced(C::kBigTileBytes);
       for (int n = 0; n < T; ++n, ++g) {
@@ -529,7 +538,7 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
     const SmemDesc dscK0mn = make_smem_desc(smem_u32(sKV), C::kStepSlabBytes, 1024);       // MN-major view of stage 0
     int g = 0, ti = 0;
     for (int lin = sched.next(); lin >= 0; lin = sched.next(), ++ti) {
-      const int T = steps_of(tile_of(lin));
+      const int T = own_steps(steps_of(tile_of(lin)));
       if (ti > 0) mbar_wait(&bar_acc_free, (ti - 1) & 1, ab, kDqWaitAccFree);   // the previous epilogue has read A, B
       for (int p = 0; p < T; ++p, ++g) {
         const int st = g % S, b = g % NB;
@@ -564,7 +573,7 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
     int g0 = 0, ti = 0;
     for (int lin = sched.next(); lin >= 0; lin = sched.next(), ++ti) {
       const TileInfo tl = tile_of(lin);
-      const int T = steps_of(tl), par = ti & 1;
+      const int Tall = steps_of(tl), T = own_steps(Tall), par = ti & 1;
       const int qrow = tl.row0 + row;                  // this thread's query row within the head (past seq_end in a ragged tile)
 #ifdef GPROJ_TRACE
       const unsigned long long ev_n0 = global_ns(); const long long ev_c0 = clock64(); unsigned long long ev_n1 = 0, ev_n2 = 0;
@@ -579,7 +588,7 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
         if (wg == 0) {
           s_lse[0][row] = lse_row;
           const int rel = qrow - tl.seq0;
-          if (rel < ((tl.seq_end - tl.seq0 + 63) / 64) * 64)
+          if (rank == 0 && rel < ((tl.seq_end - tl.seq0 + 63) / 64) * 64)
             write_row_constants(stats, static_cast<size_t>(hix(lin)) * nblk + tl.blk0 + (rel >> 6), rel & 63, -lse_row * 1.4426950408889634f, s_D[0][row], scale_log2);
           mbar_arrive(&bar_stats_ready[0]);
         }
@@ -599,11 +608,13 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
         // Probabilities are zeroed beyond the causal diagonal and, in the ragged last step, for the zero-filled keys
         // past N (which would otherwise enter the row masses).  Rows of a causal tile never reach such keys.
         const int Lk = tl.oseq_end - tl.oseq0, off = Lk - (tl.seq_end - tl.seq0);
-        const int krel0 = n * C::kStepRows + C::kSliceCols * slice;          // key (inside its sequence) of the slice's column 0
-        const bool masked = (CAUSAL && (n + 1) * C::kStepRows - 1 > tl.row0 - tl.seq0 + off) || (n + 1) * C::kStepRows > Lk;
+        const int ns = own_step(n, Tall);
+        const bool none = CL > 1 && rank >= Tall;                            // a step of the other CTA, run to keep the pipeline in step
+        const int krel0 = ns * C::kStepRows + C::kSliceCols * slice;         // key (inside its sequence) of the slice's column 0
+        const bool masked = (CAUSAL && (ns + 1) * C::kStepRows - 1 > tl.row0 - tl.seq0 + off) || (ns + 1) * C::kStepRows > Lk || none;
         if (masked) {
           const int lim_c = CAUSAL ? qrow - tl.seq0 + off - krel0 : (1 << 30);
-          dq_slice<true>(tS16, tdP16, scale_log2, neg_lse2, Dv, min(lim_c, Lk - 1 - krel0), rho2, msum2);
+          dq_slice<true>(tS16, tdP16, scale_log2, neg_lse2, Dv, none ? -1 : min(lim_c, Lk - 1 - krel0), rho2, msum2);
         } else {
           dq_slice<false>(tS16, tdP16, scale_log2, neg_lse2, Dv, 0, rho2, msum2);
         }
@@ -641,7 +652,7 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
       __syncwarp();
       s_lse[par][row] = lse_row;
       const int rel = tl.row0 + row - tl.seq0;             // row inside the sequence; its last 64-row block is padded with zeros
-      if (rel < ((tl.seq_end - tl.seq0 + 63) / 64) * 64)
+      if (rank == 0 && rel < ((tl.seq_end - tl.seq0 + 63) / 64) * 64)
         write_row_constants(stats, static_cast<size_t>(bh) * nblk + tl.blk0 + (rel >> 6), rel & 63, -lse_row * 1.4426950408889634f, s_D[par][row], scale_log2);
       mbar_arrive(&bar_stats_ready[par]);
     };
@@ -654,11 +665,13 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
       // q of this warp's 32 rows, D / 8 lanes to a row (whole lines per load and store; one row per thread touches 32
       // lines with every instruction and took 2.2 us instead of 1 us of the tail at d = 128), the first kQ loads ahead of
       // the wait
-      constexpr int L = D / 8, RPI = 32 / L, kIters = 32 / RPI;
+      constexpr int kCols = D / CL;                        // columns this CTA writes, from col0 on
+      constexpr int L = kCols / 8, RPI = 32 / L, kIters = 32 / RPI;
+      const int col0 = CL == 1 ? 0 : rank * kCols;
       const int sub = lane / L, part = lane % L;
-      const size_t wrow0 = (static_cast<size_t>(hix(lin)) * N + tl.row0 + 32 * ew) * D;
+      const size_t wrow0 = (static_cast<size_t>(hix(lin)) * N + tl.row0 + 32 * ew) * D + col0;
       const int wrows = tl.seq_end - tl.row0 - 32 * ew;    // rows of this warp that exist
-      constexpr int kQ = D == 128 ? 8 : 4;                 // loads in flight (80 registers at d = 64)
+      constexpr int kQ = D / CL == 128 ? 8 : 4;            // loads in flight (80 registers at d = 64)
       uint4 qv[kQ];
       auto fetch_q = [&](int h) {
 #pragma unroll
@@ -674,6 +687,15 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
 #pragma unroll
       for (int w = 1; w < C::kWG; ++w) { rho_t += s_rho[par][w][row]; m_t += s_m[par][w][row]; }
       mbar_arrive(&bar_mass_free[par]);
+      if (CL > 1) {
+        const uint32_t peer = cluster_map_shared(smem_u32(&s_peer[2 * par][row]), rank ^ 1);
+        cluster_store_f32(peer, rho_t);
+        cluster_store_f32(peer + 512, m_t);
+        cluster_mbar_arrive(cluster_map_shared(smem_u32(&bar_peer_mass), rank ^ 1));
+        mbar_wait_cluster(&bar_peer_mass, ti & 1, ab, kDqWaitPeer);
+        rho_t += s_peer[2 * par][row];                     // two terms: the same sum in both CTAs
+        m_t += s_peer[2 * par + 1][row];
+      }
       const float lam = (m_t != 0.f) ? __fdiv_rn(rho_t, m_t) : 0.f;
       const float lam_q = (flags & kFlagNoQCorrection) ? 0.f : lam, lam_k = (flags & kFlagNoKCorrection) ? 0.f : lam;
       // z = BF16(fl32[lambda q]), stored negated (the sign flip is exact), while the last products still run
@@ -695,15 +717,49 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
       mbar_wait(&bar_acc_done, ti & 1, ab, kDqWaitAcc);
       tc_fence_after();
       uint8_t *stg = sStaging + 4096 * ew;
+      // The other CTA's parts land in this tile's Q / dO buffer, whose last reader (the last score product) is done:
+      // [A, B][kCols / 16 chunks of 16 columns][128 rows] x 64 bytes of FP32, the 16-byte pieces of a row swizzled.
+      uint8_t *parts = sRes + (ti % R) * 2 * C::kBigTileBytes;
+      auto piece = [&](int chunk, int v) { return static_cast<uint32_t>(chunk * 8192 + row * 64 + ((v ^ ((row >> 1) & 3)) << 4)); };
+      if (CL > 1) {
+        if (row == 0) cluster_mbar_arrive(cluster_map_shared(smem_u32(&bar_peer_ready), rank ^ 1));
+        mbar_wait_cluster(&bar_peer_ready, ti & 1, ab, kDqWaitPeer);
+        const uint32_t peer = cluster_map_shared(smem_u32(parts), rank ^ 1);
 #pragma unroll
-      for (int hd = 0; hd < D / 64; ++hd) {
-#pragma unroll
-        for (int cc = 0; cc < 4; ++cc) {
-          uint32_t a[16], b[16];
-          tmem_ld16(tmem_base + C::kColAcc0 + lane_addr + 64 * hd + 16 * cc, a);
-          tmem_ld16(tmem_base + C::kColAcc1 + lane_addr + 64 * hd + 16 * cc, b);
+        for (int c = 0; c < 2 * kCols / 16; ++c) {         // A, then B, of the other CTA's columns
+          const int cc = c % (kCols / 16);
+          uint32_t a[16];
+          tmem_ld16(tmem_base + (c < kCols / 16 ? C::kColAcc0 : C::kColAcc1) + lane_addr + (D - kCols - col0) + 16 * cc, a);
           tmem_wait_ld();
-          if (hd == D / 64 - 1 && cc == 3) { tc_fence_before(); mbar_arrive(&bar_acc_free); }   // the accumulators may be overwritten by the next tile
+#pragma unroll
+          for (int v = 0; v < 4; ++v)
+            cluster_store_f4(peer + piece(c, v), __uint_as_float(a[4 * v]), __uint_as_float(a[4 * v + 1]), __uint_as_float(a[4 * v + 2]), __uint_as_float(a[4 * v + 3]));
+        }
+        cluster_mbar_arrive(cluster_map_shared(smem_u32(&bar_peer_full), rank ^ 1));
+        mbar_wait_cluster(&bar_peer_full, ti & 1, ab, kDqWaitPeer);
+      }
+      constexpr int kHd = kCols < 64 ? kCols : 64;         // columns staged at a time
+#pragma unroll
+      for (int hd = 0; hd < kCols / kHd; ++hd) {
+#pragma unroll
+        for (int cc = 0; cc < kHd / 16; ++cc) {
+          uint32_t a[16], b[16];
+          tmem_ld16(tmem_base + C::kColAcc0 + lane_addr + col0 + kHd * hd + 16 * cc, a);
+          tmem_ld16(tmem_base + C::kColAcc1 + lane_addr + col0 + kHd * hd + 16 * cc, b);
+          tmem_wait_ld();
+          if (hd == kCols / kHd - 1 && cc == kHd / 16 - 1) { tc_fence_before(); mbar_arrive(&bar_acc_free); }   // the accumulators may be overwritten by the next tile
+          if (CL > 1) {
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+              const float4 pa = *reinterpret_cast<const float4 *>(parts + piece((kHd / 16) * hd + cc, v)), pb = *reinterpret_cast<const float4 *>(parts + piece(kCols / 16 + (kHd / 16) * hd + cc, v));
+              const float fa[4] = {pa.x, pa.y, pa.z, pa.w}, fb[4] = {pb.x, pb.y, pb.z, pb.w};
+#pragma unroll
+              for (int w = 0; w < 4; ++w) {
+                a[4 * v + w] = __float_as_uint(__fadd_rn(__uint_as_float(a[4 * v + w]), fa[w]));
+                b[4 * v + w] = __float_as_uint(__fadd_rn(__uint_as_float(b[4 * v + w]), fb[w]));
+              }
+            }
+          }
 #pragma unroll
           for (int v = 0; v < 2; ++v) {
             uint32_t dqw[4];
@@ -718,13 +774,18 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
           }
         }
         __syncwarp();
+        constexpr int LS = kHd / 8, RS = 32 / LS;          // lanes per row, rows per warp-wide store
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const int r = 4 * k + (lane >> 3);
-          const uint4 v = *reinterpret_cast<const uint4 *>(stg + swz128_offset(r, lane & 7));
-          if (r < wrows) reinterpret_cast<uint4 *>(dQg + wrow0 + static_cast<size_t>(r) * D + 64 * hd)[lane & 7] = v;
+        for (int k = 0; k < 32 / RS; ++k) {
+          const int r = RS * k + lane / LS;
+          const uint4 v = *reinterpret_cast<const uint4 *>(stg + swz128_offset(r, lane % LS));
+          if (r < wrows) reinterpret_cast<uint4 *>(dQg + wrow0 + static_cast<size_t>(r) * D + kHd * hd)[lane % LS] = v;
         }
         __syncwarp();
+      }
+      if (CL > 1) {
+        fence_proxy_async_smem();
+        mbar_arrive(&bar_res_free[ti % R]);                // the parts have been read: the buffer may be loaded again
       }
       lin = next;
       ++ti;
@@ -732,7 +793,7 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
   }
 
   tc_fence_before();
-  __syncthreads();
+  if (CL > 1) cluster_sync(); else __syncthreads();   // no CTA leaves while the other one may still write to it
   if (warp == 1) tmem_dealloc(tmem_base, C::kTmemCols);
 }
 

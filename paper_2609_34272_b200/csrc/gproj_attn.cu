@@ -50,6 +50,7 @@ struct DeviceState {
   int *status_ptr = nullptr;
   int sm_count = 0;
   int fwd_clusters[2][4] = {};   // forward with clusters of 2, 4, 8 CTAs (entries 1, 2, 3) at d = 64 and d = 128: how many run at once
+  int dq_clusters[2] = {};       // dQ side with clusters of two CTAs at d = 64 and d = 128: how many run at once
   int dkv_clusters = 0;          // dK/dV side at d = 64 with clusters of two CTAs: how many run at once
   // host-buffer entry point only: copy-in and copy-out streams and the events that order them against the caller's stream
   bool pipe_ready = false;
@@ -134,17 +135,23 @@ int device_state(DeviceState **out) {
       ok &= allow_smem(bwd_dkv_w128_kernel<false, 1>, BwdW128::kDkvSmemBytes) == cudaSuccess;
       ok &= allow_smem(bwd_dkv_w128_kernel<true, 2>, BwdW128::kDkvSmemBytes) == cudaSuccess;
       ok &= allow_smem(bwd_dkv_w128_kernel<false, 2>, BwdW128::kDkvSmemBytes) == cudaSuccess;
-      ok = ok && max_clusters(bwd_dkv_w128_kernel<true, 2>, 2, BwdW128::kThreads, BwdW128::kDkvSmemBytes, &st.dkv_clusters) == cudaSuccess;
-      ok &= allow_smem(bwd_dq_kernel<64, true>, BwdCfg<64>::kDqSmemBytes) == cudaSuccess;
-      ok &= allow_smem(bwd_dq_kernel<64, false>, BwdCfg<64>::kDqSmemBytes) == cudaSuccess;
-      ok &= allow_smem(bwd_dq_kernel<128, true>, BwdCfg<128>::kDqSmemBytes) == cudaSuccess;
-      ok &= allow_smem(bwd_dq_kernel<128, false>, BwdCfg<128>::kDqSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dq_kernel<64, true, 1>, BwdCfg<64>::kDqSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dq_kernel<64, true, 2>, BwdCfg<64>::kDqSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dq_kernel<64, false, 1>, BwdCfg<64>::kDqSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dq_kernel<64, false, 2>, BwdCfg<64>::kDqSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dq_kernel<128, true, 1>, BwdCfg<128>::kDqSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dq_kernel<128, true, 2>, BwdCfg<128>::kDqSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dq_kernel<128, false, 1>, BwdCfg<128>::kDqSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dq_kernel<128, false, 2>, BwdCfg<128>::kDqSmemBytes) == cudaSuccess;
       ok &= allow_smem(bwd_dkv_kernel<128, true>, BwdCfg<128>::kDkvSmemBytes) == cudaSuccess;
       ok &= allow_smem(bwd_dkv_kernel<128, false>, BwdCfg<128>::kDkvSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<64, true, false, 3>, FwdCfg<64>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<64, false, false, 3>, FwdCfg<64>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, true, false, 3>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, false, false, 3>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
+      ok = ok && max_clusters(bwd_dq_kernel<64, true, 2>, 2, BwdCfg<64>::kDqThreads, BwdCfg<64>::kDqSmemBytes, &st.dq_clusters[0]) == cudaSuccess;
+      ok = ok && max_clusters(bwd_dq_kernel<128, true, 2>, 2, BwdCfg<128>::kDqThreads, BwdCfg<128>::kDqSmemBytes, &st.dq_clusters[1]) == cudaSuccess;
+      ok = ok && max_clusters(bwd_dkv_w128_kernel<true, 2>, 2, BwdW128::kThreads, BwdW128::kDkvSmemBytes, &st.dkv_clusters) == cudaSuccess;
       for (int lg = 1; ok && lg < 4; ++lg) {
         ok &= max_clusters(attn_fwd_kernel<64, true, false, 3>, 1 << lg, FwdCfg<64>::kThreads, FwdCfg<64>::kSmemBytes, &st.fwd_clusters[0][lg]) == cudaSuccess;
         ok &= max_clusters(attn_fwd_kernel<128, true, false, 3>, 1 << lg, FwdCfg<128>::kThreads, FwdCfg<128>::kSmemBytes, &st.fwd_clusters[1][lg]) == cudaSuccess;
@@ -539,26 +546,29 @@ int gproj_attn_bwd_gqa(const void *Q, const void *K, const void *V, const void *
 
 namespace {
 
-// dK/dV side at d = 64: share every key tile between the two CTAs of a cluster?  This replays the static deal of both forms
-// in units of one 128-query step (2.3 per item, the kernel's measured overhead, and 1.5 more for the exchange of the two
-// parts) and takes the pairs where their longest CTA is 3 % shorter.  steps: per tile over all heads of a group, decreasing.
-// Measured, this kernel alone, whole tiles -> pairs: 16 query / 4 KV heads x 4096, causal: 121 -> 77 us; 8 / 2 heads x 8000,
+// Share every tile of a backward kernel between the two CTAs of a cluster?  This replays the static deal of both forms in
+// units of one step (per_item: the kernel's measured overhead per item; exchange: what the exchange of the two parts adds)
+// and takes the pairs where their longest CTA is 3 % shorter.  steps: of each tile of a head, decreasing.
+// Measured, dK/dV side at d = 64 alone, whole tiles -> pairs: 16 query / 4 KV heads x 4096, causal: 121 -> 77 us; 8 / 2 heads x 8000,
 // causal: 229 -> 140; 32 / 4 heads x 2000: 121 -> 78; 4 heads x 4096, causal: 43.5 -> 37.2; 1 head x 8192: 62.0 -> 43.5;
 // 16 heads x 4096, causal (stays with whole tiles): 68; 16 packed documents of 8192 rows, 16 / 4 heads: 78.6 -> 73.0.
-bool dkv_prefers_pairs(const std::vector<int> &steps, int BHkv, int sms, int pairs) {
-  const long long items = static_cast<long long>(BHkv) * static_cast<long long>(steps.size());
+// dQ side: 1 head x 8192 x 64: 83 -> 52 us; 4 heads x 4096 x 64, causal: 44.7 -> 34.4; 16 heads x 300 queries behind 9000 keys,
+// d = 128: 126 -> 92; 4 heads x 2048 x 128, causal: 36.5 -> 32.8; 4 heads x 1000 x 128 (16 steps): 20.7 -> 21.3, hence the
+// 8 steps the exchange counts at d = 128.
+bool prefers_pairs(const std::vector<int> &steps, int heads, int sms, int pairs, double per_item, double exchange) {
+  const long long items = static_cast<long long>(heads) * static_cast<long long>(steps.size());
   if (pairs < 1 || items > 8LL * sms) return false;      // many items per CTA: they balance as they are
-  const double whole = deal_makespan(items, sms, [&](long long lin) { return steps[static_cast<size_t>(lin / BHkv)] + 2.3; });
-  const double split = deal_makespan(items, pairs, [&](long long lin) { return (steps[static_cast<size_t>(lin / BHkv)] + 1) / 2 + 3.8; });
+  const double whole = deal_makespan(items, sms, [&](long long lin) { return steps[static_cast<size_t>(lin / heads)] + per_item; });
+  const double split = deal_makespan(items, pairs, [&](long long lin) { return (steps[static_cast<size_t>(lin / heads)] + 1) / 2 + per_item + exchange; });
   return split < 0.97 * whole;
 }
 
-// 128-query steps of the key tiles of a call, over the G heads of a group, decreasing.
-std::vector<int> dkv_steps(const PackedSeqs *seqs, int G, int Nq, int Nk, bool causal) {
+// Steps of `rows` rows of the tiles of a call (key_side: of the key tiles, over the G heads of a group), decreasing.
+std::vector<int> tile_steps(const PackedSeqs *seqs, bool key_side, int rows, int G, int Nq, int Nk, bool causal) {
   const int cu_q[2] = {0, Nq}, cu_k[2] = {0, Nk};
   const PackedSeqs one{cu_q, cu_k, 1, causal};
-  std::vector<int> steps = packed_work(seqs ? *seqs : one, true);
-  for (int &w : steps) w = G * std::max(1, (w + 127) / 128);
+  std::vector<int> steps = packed_work(seqs ? *seqs : one, key_side);
+  for (int &w : steps) w = G * std::max(1, (w + rows - 1) / rows);
   return steps;
 }
 
@@ -609,18 +619,21 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
   if (total_kv_tiles <= 0) run_dkv = false;   // packed call in which no sequence has both queries and keys
   ItemOrder group_q = item_order(BH, n_qt, tile_group_of(plan_q != nullptr, causal != 0, BH, n_qt, 2 * static_cast<size_t>(BHkv) * Nk * d * 2, st->sm_count, 3.25));    // streams K, V
   ItemOrder group_kv = item_order(BHkv, std::max(n_kt, 1), tile_group_of(plan_q != nullptr, causal != 0, BHkv, n_kt, 3 * static_cast<size_t>(BH) * N * d * 2, st->sm_count, 2.3));   // streams Q, dO, Z
+  const int dq_fit = st->dq_clusters[d == 128];
+  const bool dq_pairs = run_dq && total_tiles <= 8LL * st->sm_count &&
+                        prefers_pairs(tile_steps(seqs, false, 64, 1, N, Nk, causal != 0), BH, st->sm_count, dq_fit, d == 64 ? 3.8 : 3.0, d == 64 ? 3.0 : 8.0);
   if (seqs) {
-    group_q.solo = packed_solo(*seqs, false, BH, st->sm_count, [&](int keys) { return std::max(1, (keys + 63) / 64) + (d == 64 ? 3.8 : 3.0); });
+    if (!dq_pairs) group_q.solo = packed_solo(*seqs, false, BH, st->sm_count, [&](int keys) { return std::max(1, (keys + 63) / 64) + (d == 64 ? 3.8 : 3.0); });
     if (d == 128) group_kv.solo = packed_solo(*seqs, true, BHkv, st->sm_count, [&](int rows) { return G * std::max(1, (rows + 63) / 64) + 3.0; });
   }
-  const dim3 grid(static_cast<unsigned>(total_tiles < st->sm_count ? total_tiles : st->sm_count));   // persistent: one CTA per SM
+  const dim3 grid(static_cast<unsigned>(dq_pairs ? 2 * std::min(total_tiles, dq_fit) : std::min(total_tiles, st->sm_count)));   // persistent: one CTA per SM
   const dim3 grid_kv(static_cast<unsigned>(total_kv_tiles < st->sm_count ? total_kv_tiles : st->sm_count));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const __nv_bfloat16 *Ob = static_cast<const __nv_bfloat16 *>(O), *dOb = static_cast<const __nv_bfloat16 *>(dO);
 #define GPROJ_LAUNCH_BWD(DD, CC)                                                                                        \
   do {                                                                                                                  \
     if (run_dq)                                                                                                         \
-      launch_after(bwd_dq_kernel<DD, CC>, grid, 1, BwdCfg<DD>::kDqThreads, BwdCfg<DD>::kDqSmemBytes, s, true,                               \
+      launch_after(dq_pairs ? bwd_dq_kernel<DD, CC, 2> : bwd_dq_kernel<DD, CC, 1>, grid, dq_pairs ? 2 : 1, BwdCfg<DD>::kDqThreads, BwdCfg<DD>::kDqSmemBytes, s, true,                               \
           mQ128, mdO128, mK64, mV64, static_cast<const __nv_bfloat16 *>(Q), Ob, dOb, LSE, stats, static_cast<__nv_bfloat16 *>(dQ), Zneg, plan_q, nblk,   \
           N, Nk, BH, H, G, total_tiles, group_q, scale_log2, softmax_scale,                                           \
           flags,                                                                                                        \
@@ -635,13 +648,13 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
   // At d = 64 the dK/dV side runs with 128-wide steps (every score product an N = 128 instruction); it streams 128-row
   // boxes, which the stationary-tile maps of the dQ side already are.
   const bool few_tiles = static_cast<long long>(total_kv_tiles) <= 8LL * st->sm_count;
-  const bool pairs = d == 64 && run_dkv && few_tiles && dkv_prefers_pairs(dkv_steps(seqs, G, N, Nk, causal != 0), BHkv, st->sm_count, st->dkv_clusters);
+  const bool pairs = d == 64 && run_dkv && few_tiles && prefers_pairs(tile_steps(seqs, true, 128, G, N, Nk, causal != 0), BHkv, st->sm_count, st->dkv_clusters, 2.3, 1.5);
   if (seqs && d == 64 && !pairs) group_kv.solo = packed_solo(*seqs, true, BHkv, st->sm_count, [&](int rows) { return G * std::max(1, (rows + 127) / 128) + 2.3; });
   const dim3 grid_dkv(pairs ? 2u * static_cast<unsigned>(std::min(total_kv_tiles, st->dkv_clusters)) : grid_kv.x);
 #define GPROJ_LAUNCH_BWD_W128(CC)                                                                                       \
   do {                                                                                                                  \
     if (run_dq)                                                                                                         \
-      launch_after(bwd_dq_kernel<64, CC>, grid, 1, BwdCfg<64>::kDqThreads, BwdCfg<64>::kDqSmemBytes, s, true,                                \
+      launch_after(dq_pairs ? bwd_dq_kernel<64, CC, 2> : bwd_dq_kernel<64, CC, 1>, grid, dq_pairs ? 2 : 1, BwdCfg<64>::kDqThreads, BwdCfg<64>::kDqSmemBytes, s, true,                                \
           mQ128, mdO128, mK64, mV64, static_cast<const __nv_bfloat16 *>(Q), Ob, dOb, LSE, stats, static_cast<__nv_bfloat16 *>(dQ), Zneg, plan_q,    \
           nblk, N, Nk, BH, H, G, total_tiles, group_q, scale_log2, softmax_scale, flags, st->status_ptr);                 \
     if (run_dkv)                                                                                                        \

@@ -84,18 +84,20 @@ def test_key_smoothing_at_the_edges_of_its_row_split(rows, d):
     assert torch.all((got - want).abs() <= 2.0 ** -8 * want.abs() + 2.0 ** -20 * X.float().abs().max())
 
 
-# The dK/dV side shares key tiles between two CTAs where whole tiles cannot be dealt evenly: one-step tiles (a CTA without a
-# step of its own), odd and even step counts, query heads split between the CTAs, ragged ends, keys no query sees.
+# Both backward kernels share tiles between two CTAs where whole tiles cannot be dealt evenly: one-step tiles (a CTA without a
+# step of its own), odd and even step counts, query heads split between the CTAs, ragged ends, keys no query sees, rows that
+# see no key, several tiles per cluster.
 BWD = [  # B, H, Hkv, Nq, Nk, causal
     (1, 1, 1, 700, 700, True), (1, 3, 1, 333, 333, True), (2, 4, 2, 1000, 1000, False), (1, 2, 1, 900, 130, True),
-    (1, 2, 1, 641, 257, False), (1, 2, 2, 600, 1100, True), (1, 8, 2, 1025, 1025, True),
+    (1, 2, 1, 641, 257, False), (1, 2, 2, 600, 1100, True), (1, 8, 2, 1025, 1025, True), (1, 1, 1, 5, 1700, True),
+    (2, 5, 5, 1290, 1290, True),
 ]
 
 
 @pytest.mark.parametrize("flags", [0, g.FLAG_NO_K_CORRECTION])
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("shape", BWD)
-def test_backward_with_key_tiles_shared_by_two_ctas(shape, d, flags):
+def test_backward_with_tiles_shared_by_two_ctas(shape, d, flags):
     B, H, Hkv, Nq, Nk, causal = shape
     gen = torch.Generator().manual_seed(Nq + 3 * Nk + d)
     Q, dO = (torch.randn(B, H, Nq, d, generator=gen).to(torch.bfloat16) for _ in range(2))
