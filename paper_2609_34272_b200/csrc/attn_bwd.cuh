@@ -184,7 +184,7 @@ __device__ __forceinline__ void store_rows_clipped(const uint8_t *stage, int sla
 
 enum BwdWaitCode {
   kDqWaitQ = 0x21, kDqWaitKV = 0x22, kDqWaitKVEmpty = 0x23, kDqWaitSdP = 0x24, kDqWaitTR = 0x25, kDqWaitAcc = 0x26, kDqWaitBuf = 0x27, kDqWaitResFree = 0x28, kDqWaitAccFree = 0x29, kDqWaitStats = 0x2a, kDqWaitMass = 0x2b, kDqWaitPeer = 0x2c,
-  kDkvWaitKV = 0x31, kDkvWaitQ = 0x32, kDkvWaitQEmpty = 0x33, kDkvWaitSdP = 0x34, kDkvWaitTR = 0x35, kDkvWaitAcc = 0x36, kDkvWaitBuf = 0x37, kDkvWaitResFree = 0x38, kDkvWaitAccFree = 0x39
+  kDkvWaitKV = 0x31, kDkvWaitQ = 0x32, kDkvWaitQEmpty = 0x33, kDkvWaitSdP = 0x34, kDkvWaitTR = 0x35, kDkvWaitAcc = 0x36, kDkvWaitBuf = 0x37, kDkvWaitResFree = 0x38, kDkvWaitAccFree = 0x39, kDkvWaitPeer = 0x3a
 };
 
 // Arithmetic of one pair of adjacent score columns, shared by both kernels (Algorithm 1 lines 5-8):
@@ -800,7 +800,12 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
 // ============================================================================================
 // dK / dV side
 // ============================================================================================
-template <int D, bool CAUSAL>
+// CL = 2: a cluster of two CTAs shares every tile: CTA r takes its steps r, r + 2, ... (over all query heads of the group), then
+// CTA 0 gets both parts of dV, CTA 1 both parts of dK, over the consumed K / V tile (its 64 KB hold one 128 x 128 part in
+// FP32), added in FP32 before the cast.  Bound where whole tiles are used: the CTA with the longest tile, since a causal or
+// grouped call has few tiles of very different length.  This kernel alone, whole tiles -> pairs, d = 128, causal: 16 query / 4 KV
+// heads x 4096: 275 -> 151 us (1136 TFLOP/s); 4 heads x 4000: 72.2 -> 53.0; 4 heads x 2048: 43.1 -> 31.3.
+template <int D, bool CAUSAL, int CL>
 __global__ void __launch_bounds__(BwdCfg<D>::kDkvThreads, 1)
 bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 rows
                const __grid_constant__ CUtensorMap tmV,    // box 64 x 128 rows
@@ -824,14 +829,14 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 rows
   uint8_t *sStaging = sStage + S * C::kDkvStageBytes;   // epilogue warp w: 2048 w
 
   __shared__ uint64_t bar_res_full, bar_res_free, bar_q_full[S], bar_q_empty[S];
-  __shared__ uint64_t bar_s_full[NB], bar_dp_full[NB], bar_r_ready[NB], bar_t_ready[NB], bar_acc_done, bar_acc_free, bar_drain[2];
+  __shared__ uint64_t bar_s_full[NB], bar_dp_full[NB], bar_r_ready[NB], bar_t_ready[NB], bar_acc_done, bar_acc_free, bar_drain[2], bar_peer_ready, bar_peer_full;
   __shared__ uint32_t tmem_base_smem;
   __shared__ int cta_abort, cta_skip;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) cta_skip = *reinterpret_cast<volatile int *>(status);
   __syncthreads();
-  if (cta_skip != 0) return;
+  if (CL == 1 && cta_skip != 0) return;   // a cluster runs on with every wait falling through: its CTAs exchange results
 
   const bool use_z = (flags & kFlagNoKCorrection) == 0;
   const uint32_t stage_tx = (use_z ? 3 : 2) * C::kStepTileBytes + kExtBlockBytes;
@@ -846,15 +851,17 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 rows
 
   AbortState ab{status, &cta_abort};
   if (threadIdx.x == 0) {
-    cta_abort = 0;
+    cta_abort = CL > 1 ? cta_skip : 0;
     mbar_init(&bar_res_full, 1);
-    mbar_init(&bar_res_free, 1);
+    mbar_init(&bar_res_free, CL > 1 ? 1 + 128 : 1);
     for (int s = 0; s < S; ++s) { mbar_init(&bar_q_full[s], 1); mbar_init(&bar_q_empty[s], 1); }
     for (int b = 0; b < NB; ++b) {
       mbar_init(&bar_s_full[b], 1); mbar_init(&bar_dp_full[b], 1);
       mbar_init(&bar_r_ready[b], 128 * C::kSlices); mbar_init(&bar_t_ready[b], 128 * C::kSlices);
     }
     mbar_init(&bar_acc_done, 1);
+    mbar_init(&bar_peer_ready, 1);
+    mbar_init(&bar_peer_full, 128);
     mbar_init(&bar_acc_free, 128);
     mbar_init(&bar_drain[0], 1);
     mbar_init(&bar_drain[1], 1);
@@ -865,12 +872,13 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 rows
     tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV); tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmdO); tma_prefetch_desc(&tmZ);
   }
   tc_fence_before();
-  __syncthreads();
+  if (CL > 1) cluster_sync(); else __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, tmem_base_smem, 0);
   griddep_launch_dependents();   // the next kernel in the stream may set itself up beside this one
 
-  TileSched sched(total_tiles, order.solo);
+  TileSched sched(total_tiles, order.solo, CL);
+  const int rank = CL > 1 ? cluster_rank() : 0;
   // tile decode: causal -> key tile 0 has the most query steps and comes first
   // Ragged N: query steps round up.  A zero-filled query column past N contributes exactly nothing (its dO, Q and Z rows
   // are zero and its padded statistics are zero, so t = 0 and r multiplies zero rows); key rows past N are clipped on store.
@@ -887,6 +895,10 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 rows
     return min(first, ((Lq - 1) >> 6) << 6);
   };
   auto steps_of = [&](const TileInfo &t) { return max(1, (t.oseq_end - t.oseq0 - q_start_of(t) + C::kStepRows - 1) / C::kStepRows); };
+  // This CTA's steps of a tile whose heads have T steps each, and the n-th of them; a CTA that gets none runs step 0 fully
+  // masked.
+  auto own_steps = [&](int T) { return CL == 1 ? G * T : max(1, (G * T - rank + CL - 1) / CL); };
+  auto own_step = [&](int n, int T) { return CL == 1 ? n : (rank < G * T ? CL * n + rank : 0); };
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer of the streamed (Q, dO, Z, stats) step tiles
@@ -899,8 +911,8 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 rows
         const TileInfo tl = tile_of(lin);
         const int bh = hix(lin), T = steps_of(tl), q_start = q_start_of(tl);
         const int q_head0 = (bh / Hkv) * (Hkv * G) + (bh % Hkv) * G;     // first query head of the group (flat index)
-        for (int n = 0; n < G * T; ++n, ++g) {
-          const int st = g % S;
+        for (int m = 0; m < own_steps(T); ++m, ++g) {
+          const int st = g % S, n = own_step(m, T);
           if (g >= S) mbar_wait(&bar_q_empty[st], ((g / S) - 1) & 1, ab, kDkvWaitQEmpty);
           mbar_expect_tx(&bar_q_full[st], stage_tx);
           uint8_t *dst = sStage + st * C::kDkvStageBytes;
@@ -945,7 +957,7 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 rows
     const SmemDesc dscExt0 = make_smem_desc_noswizzle(smem_u32(sStage + 3 * C::kStepTileBytes), 128, 256);
     int g = 0, ti = 0;
     for (int lin = sched.next(); lin >= 0; lin = sched.next(), ++ti) {
-      const int T = G * steps_of(tile_of(lin));
+      const int T = own_steps(steps_of(tile_of(lin)));
       mbar_wait(&bar_res_full, ti & 1, ab, kDkvWaitKV);
       for (int n = 0; n < T; ++n, ++g) {
         const int st = g % S, b = g % NB;
@@ -981,7 +993,7 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 rows
     const SmemDesc dscQ0mn = make_smem_desc(smem_u32(sStage), C::kStepSlabBytes, 1024);    // MN-major view of stage 0
     int g = 0, ti = 0;
     for (int lin = sched.next(); lin >= 0; lin = sched.next(), ++ti) {
-      const int T = G * steps_of(tile_of(lin));
+      const int T = own_steps(steps_of(tile_of(lin)));
       if (ti > 0) mbar_wait(&bar_acc_free, (ti - 1) & 1, ab, kDkvWaitAccFree);   // the previous epilogue has read dV, dK
       for (int p = 0; p < T; ++p, ++g) {
         const int st = g % S, b = g % NB;
@@ -1026,7 +1038,7 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 rows
     int g0 = 0;
     for (int lin = sched.next(); lin >= 0; lin = sched.next()) {
       const TileInfo tl = tile_of(lin);
-      const int Th = steps_of(tl), T = G * Th, q_start = q_start_of(tl);
+      const int Th = steps_of(tl), T = own_steps(Th), q_start = q_start_of(tl);
 #ifdef GPROJ_TRACE
       const unsigned long long tile_t0 = global_ns();
 #endif
@@ -1035,13 +1047,14 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 rows
         mbar_wait(&bar_s_full[b], (g / NB) & 1, ab, kDkvWaitSdP);
         tc_fence_after();
         const uint32_t tS16 = slice_addr + 128 * b, tdP16 = tS16 + 64;
-        const int nh = n % Th;                                      // step within the current query head
+        const int nh = own_step(n, Th) % Th;                        // step within the current query head
+        const bool none = CL > 1 && rank >= G * Th;                 // a step of the other CTA, run to keep the pipeline in step
         const int Lq = tl.oseq_end - tl.oseq0, off = (tl.seq_end - tl.seq0) - Lq, krel0 = tl.row0 - tl.seq0;
         const int qs = q_start + nh * C::kStepRows;                           // first query (inside its sequence) of the step
         const int q0 = qs + C::kSliceCols * slice;                            // ... of the slice's column 0
         float pkeep[32];
-        if ((CAUSAL && qs < krel0 + 128 - off) || qs + C::kStepRows > Lq)
-          dkv_phase1<true>(tS16, scale_log2, CAUSAL ? krel0 + row - off - q0 : 0, Lq - 1 - q0, pkeep);
+        if ((CAUSAL && qs < krel0 + 128 - off) || qs + C::kStepRows > Lq || none)
+          dkv_phase1<true>(tS16, scale_log2, CAUSAL ? krel0 + row - off - q0 : 0, none ? -1 : Lq - 1 - q0, pkeep);
         else
           dkv_phase1<false>(tS16, scale_log2, 0, 0, pkeep);
         tmem_wait_st();
@@ -1077,6 +1090,59 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 rows
       const int wrows = tl.seq_end - tl.row0 - 32 * ew;      // rows of this warp that exist
       mbar_wait(&bar_acc_done, ti & 1, ab, kDkvWaitAcc);
       tc_fence_after();
+      if (CL > 1) {
+        // [D / 16 chunks of 16 columns][128 rows] x 64 bytes of FP32, the 16-byte pieces of a row swizzled
+        const int row = 32 * ew + lane;
+        auto piece = [&](int chunk, int v) { return static_cast<uint32_t>(chunk * 8192 + row * 64 + ((v ^ ((row >> 1) & 3)) << 4)); };
+        const uint32_t t_own = tmem_base + (rank == 0 ? C::kColAcc0 : C::kColAcc1) + lane_addr, t_send = tmem_base + (rank == 0 ? C::kColAcc1 : C::kColAcc0) + lane_addr;
+        const uint32_t peer = cluster_map_shared(smem_u32(sK), rank ^ 1);
+        const float scale = rank == 0 ? 1.0f : alpha;
+        if (row == 0) cluster_mbar_arrive(cluster_map_shared(smem_u32(&bar_peer_ready), rank ^ 1));   // this CTA's K / V tile is consumed
+        mbar_wait_cluster(&bar_peer_ready, ti & 1, ab, kDkvWaitPeer);
+#pragma unroll 2
+        for (int cc = 0; cc < D / 16; ++cc) {
+          uint32_t a[16];
+          tmem_ld16(t_send + 16 * cc, a);
+          tmem_wait_ld();
+#pragma unroll
+          for (int v = 0; v < 4; ++v)
+            cluster_store_f4(peer + piece(cc, v), __uint_as_float(a[4 * v]), __uint_as_float(a[4 * v + 1]), __uint_as_float(a[4 * v + 2]), __uint_as_float(a[4 * v + 3]));
+        }
+        cluster_mbar_arrive(cluster_map_shared(smem_u32(&bar_peer_full), rank ^ 1));
+        mbar_wait_cluster(&bar_peer_full, ti & 1, ab, kDkvWaitPeer);
+#pragma unroll 1
+        for (int c = 0; c < D / 32; ++c) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int cc = 2 * c + h;
+            uint32_t a[16], w8[8];
+            tmem_ld16(t_own + 16 * cc, a);
+            float b[16];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) *reinterpret_cast<float4 *>(&b[4 * v]) = *reinterpret_cast<const float4 *>(sK + piece(cc, v));
+            tmem_wait_ld();
+            if (cc == D / 16 - 1) { tc_fence_before(); mbar_arrive(&bar_acc_free); }   // the accumulators may be overwritten by the next tile
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              w8[i] = pack_bf16x2(__fmul_rn(scale, __fadd_rn(__uint_as_float(a[2 * i]), b[2 * i])), __fmul_rn(scale, __fadd_rn(__uint_as_float(a[2 * i + 1]), b[2 * i + 1])));
+#pragma unroll
+            for (int v = 0; v < 2; ++v)
+              *reinterpret_cast<uint4 *>(stg + lane * 64 + (((2 * h + v) ^ ((lane >> 1) & 3)) << 4)) = make_uint4(w8[4 * v], w8[4 * v + 1], w8[4 * v + 2], w8[4 * v + 3]);
+          }
+          __syncwarp();
+          __nv_bfloat16 *dst = (rank == 0 ? dVg : dKg) + wrow0 + 32 * c;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int r = 8 * k + (lane >> 2), p = lane & 3;
+            const uint4 v = *reinterpret_cast<const uint4 *>(stg + r * 64 + ((p ^ ((r >> 1) & 3)) << 4));
+            if (r < wrows) reinterpret_cast<uint4 *>(dst + static_cast<size_t>(r) * D)[p] = v;
+          }
+          __syncwarp();
+        }
+        fence_proxy_async_smem();
+        mbar_arrive(&bar_res_free);                          // the parts have been read: K and V may be loaded again
+        continue;
+      }
 #pragma unroll 1
       for (int c = 0; c < 2 * D / 32; ++c) {                 // 32-column chunks of dV, then of dK (adjacent accumulator columns)
         const float scale = c < D / 32 ? 1.0f : alpha;
@@ -1109,7 +1175,7 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 rows
   }
 
   tc_fence_before();
-  __syncthreads();
+  if (CL > 1) cluster_sync(); else __syncthreads();   // no CTA leaves while the other one may still write to it
   if (warp == 1) tmem_dealloc(tmem_base, C::kTmemCols);
 }
 

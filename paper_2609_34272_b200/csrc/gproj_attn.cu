@@ -51,7 +51,7 @@ struct DeviceState {
   int sm_count = 0;
   int fwd_clusters[2][4] = {};   // forward with clusters of 2, 4, 8 CTAs (entries 1, 2, 3) at d = 64 and d = 128: how many run at once
   int dq_clusters[2] = {};       // dQ side with clusters of two CTAs at d = 64 and d = 128: how many run at once
-  int dkv_clusters = 0;          // dK/dV side at d = 64 with clusters of two CTAs: how many run at once
+  int dkv_clusters[2] = {};      // the same for the dK/dV side
   // host-buffer entry point only: copy-in and copy-out streams and the events that order them against the caller's stream
   bool pipe_ready = false;
   cudaStream_t in_stream = nullptr, out_stream = nullptr;
@@ -143,15 +143,18 @@ int device_state(DeviceState **out) {
       ok &= allow_smem(bwd_dq_kernel<128, true, 2>, BwdCfg<128>::kDqSmemBytes) == cudaSuccess;
       ok &= allow_smem(bwd_dq_kernel<128, false, 1>, BwdCfg<128>::kDqSmemBytes) == cudaSuccess;
       ok &= allow_smem(bwd_dq_kernel<128, false, 2>, BwdCfg<128>::kDqSmemBytes) == cudaSuccess;
-      ok &= allow_smem(bwd_dkv_kernel<128, true>, BwdCfg<128>::kDkvSmemBytes) == cudaSuccess;
-      ok &= allow_smem(bwd_dkv_kernel<128, false>, BwdCfg<128>::kDkvSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dkv_kernel<128, true, 1>, BwdCfg<128>::kDkvSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dkv_kernel<128, true, 2>, BwdCfg<128>::kDkvSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dkv_kernel<128, false, 1>, BwdCfg<128>::kDkvSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dkv_kernel<128, false, 2>, BwdCfg<128>::kDkvSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<64, true, false, 3>, FwdCfg<64>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<64, false, false, 3>, FwdCfg<64>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, true, false, 3>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, false, false, 3>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok = ok && max_clusters(bwd_dq_kernel<64, true, 2>, 2, BwdCfg<64>::kDqThreads, BwdCfg<64>::kDqSmemBytes, &st.dq_clusters[0]) == cudaSuccess;
       ok = ok && max_clusters(bwd_dq_kernel<128, true, 2>, 2, BwdCfg<128>::kDqThreads, BwdCfg<128>::kDqSmemBytes, &st.dq_clusters[1]) == cudaSuccess;
-      ok = ok && max_clusters(bwd_dkv_w128_kernel<true, 2>, 2, BwdW128::kThreads, BwdW128::kDkvSmemBytes, &st.dkv_clusters) == cudaSuccess;
+      ok = ok && max_clusters(bwd_dkv_w128_kernel<true, 2>, 2, BwdW128::kThreads, BwdW128::kDkvSmemBytes, &st.dkv_clusters[0]) == cudaSuccess;
+      ok = ok && max_clusters(bwd_dkv_kernel<128, true, 2>, 2, BwdCfg<128>::kDkvThreads, BwdCfg<128>::kDkvSmemBytes, &st.dkv_clusters[1]) == cudaSuccess;
       for (int lg = 1; ok && lg < 4; ++lg) {
         ok &= max_clusters(attn_fwd_kernel<64, true, false, 3>, 1 << lg, FwdCfg<64>::kThreads, FwdCfg<64>::kSmemBytes, &st.fwd_clusters[0][lg]) == cudaSuccess;
         ok &= max_clusters(attn_fwd_kernel<128, true, false, 3>, 1 << lg, FwdCfg<128>::kThreads, FwdCfg<128>::kSmemBytes, &st.fwd_clusters[1][lg]) == cudaSuccess;
@@ -552,6 +555,8 @@ namespace {
 // Measured, dK/dV side at d = 64 alone, whole tiles -> pairs: 16 query / 4 KV heads x 4096, causal: 121 -> 77 us; 8 / 2 heads x 8000,
 // causal: 229 -> 140; 32 / 4 heads x 2000: 121 -> 78; 4 heads x 4096, causal: 43.5 -> 37.2; 1 head x 8192: 62.0 -> 43.5;
 // 16 heads x 4096, causal (stays with whole tiles): 68; 16 packed documents of 8192 rows, 16 / 4 heads: 78.6 -> 73.0.
+// dK/dV side at d = 128: 16 / 4 heads x 4096, causal: 275 -> 151; 8 / 1 heads x 3000, causal: 375 -> 200; 16 / 8 heads x 700, causal: 30.9 ->
+// 25.0; 2 heads x 1500, causal: 30.9 -> 24.8; 4 heads x 1000 (16 steps, stays with whole tiles): 25.1.
 // dQ side: 1 head x 8192 x 64: 83 -> 52 us; 4 heads x 4096 x 64, causal: 44.7 -> 34.4; 16 heads x 300 queries behind 9000 keys,
 // d = 128: 126 -> 92; 4 heads x 2048 x 128, causal: 36.5 -> 32.8; 4 heads x 1000 x 128 (16 steps): 20.7 -> 21.3, hence the
 // 8 steps the exchange counts at d = 128.
@@ -622,12 +627,15 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
   const int dq_fit = st->dq_clusters[d == 128];
   const bool dq_pairs = run_dq && total_tiles <= 8LL * st->sm_count &&
                         prefers_pairs(tile_steps(seqs, false, 64, 1, N, Nk, causal != 0), BH, st->sm_count, dq_fit, d == 64 ? 3.8 : 3.0, d == 64 ? 3.0 : 8.0);
-  if (seqs) {
-    if (!dq_pairs) group_q.solo = packed_solo(*seqs, false, BH, st->sm_count, [&](int keys) { return std::max(1, (keys + 63) / 64) + (d == 64 ? 3.8 : 3.0); });
-    if (d == 128) group_kv.solo = packed_solo(*seqs, true, BHkv, st->sm_count, [&](int rows) { return G * std::max(1, (rows + 63) / 64) + 3.0; });
-  }
+  if (seqs && !dq_pairs)
+    group_q.solo = packed_solo(*seqs, false, BH, st->sm_count, [&](int keys) { return std::max(1, (keys + 63) / 64) + (d == 64 ? 3.8 : 3.0); });
+  const int dkv_fit = st->dkv_clusters[d == 128], dkv_rows = d == 64 ? 128 : 64;   // rows of a step
+  const bool dkv_pairs = run_dkv && total_kv_tiles <= 8LL * st->sm_count &&
+                         prefers_pairs(tile_steps(seqs, true, dkv_rows, G, N, Nk, causal != 0), BHkv, st->sm_count, dkv_fit, d == 64 ? 2.3 : 3.0, d == 64 ? 1.5 : 8.0);
+  if (seqs && !dkv_pairs)
+    group_kv.solo = packed_solo(*seqs, true, BHkv, st->sm_count, [&](int rows) { return G * std::max(1, (rows + dkv_rows - 1) / dkv_rows) + (d == 64 ? 2.3 : 3.0); });
   const dim3 grid(static_cast<unsigned>(dq_pairs ? 2 * std::min(total_tiles, dq_fit) : std::min(total_tiles, st->sm_count)));   // persistent: one CTA per SM
-  const dim3 grid_kv(static_cast<unsigned>(total_kv_tiles < st->sm_count ? total_kv_tiles : st->sm_count));
+  const dim3 grid_kv(static_cast<unsigned>(dkv_pairs ? 2 * std::min(total_kv_tiles, dkv_fit) : std::min(total_kv_tiles, st->sm_count)));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const __nv_bfloat16 *Ob = static_cast<const __nv_bfloat16 *>(O), *dOb = static_cast<const __nv_bfloat16 *>(dO);
 #define GPROJ_LAUNCH_BWD(DD, CC)                                                                                        \
@@ -639,7 +647,7 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
           flags,                                                                                                        \
           st->status_ptr);                                                                                              \
     if (run_dkv)                                                                                                        \
-      launch_after(bwd_dkv_kernel<DD, CC>, grid_kv, 1, BwdCfg<DD>::kDkvThreads, BwdCfg<DD>::kDkvSmemBytes, s, run_dq,            \
+      launch_after(dkv_pairs ? bwd_dkv_kernel<DD, CC, 2> : bwd_dkv_kernel<DD, CC, 1>, grid_kv, dkv_pairs ? 2 : 1, BwdCfg<DD>::kDkvThreads, BwdCfg<DD>::kDkvSmemBytes, s, run_dq,            \
           mK128, mV128, mQs, mdOs, mZs, stats, static_cast<__nv_bfloat16 *>(dK),                        \
           static_cast<__nv_bfloat16 *>(dV), plan_kv, nblk, Nk, N, BHkv, Hkv, G, total_kv_tiles, group_kv, scale_log2, softmax_scale, \
           flags,                                                                                                        \
@@ -647,10 +655,6 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
   } while (0)
   // At d = 64 the dK/dV side runs with 128-wide steps (every score product an N = 128 instruction); it streams 128-row
   // boxes, which the stationary-tile maps of the dQ side already are.
-  const bool few_tiles = static_cast<long long>(total_kv_tiles) <= 8LL * st->sm_count;
-  const bool pairs = d == 64 && run_dkv && few_tiles && prefers_pairs(tile_steps(seqs, true, 128, G, N, Nk, causal != 0), BHkv, st->sm_count, st->dkv_clusters, 2.3, 1.5);
-  if (seqs && d == 64 && !pairs) group_kv.solo = packed_solo(*seqs, true, BHkv, st->sm_count, [&](int rows) { return G * std::max(1, (rows + 127) / 128) + 2.3; });
-  const dim3 grid_dkv(pairs ? 2u * static_cast<unsigned>(std::min(total_kv_tiles, st->dkv_clusters)) : grid_kv.x);
 #define GPROJ_LAUNCH_BWD_W128(CC)                                                                                       \
   do {                                                                                                                  \
     if (run_dq)                                                                                                         \
@@ -658,7 +662,7 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
           mQ128, mdO128, mK64, mV64, static_cast<const __nv_bfloat16 *>(Q), Ob, dOb, LSE, stats, static_cast<__nv_bfloat16 *>(dQ), Zneg, plan_q,    \
           nblk, N, Nk, BH, H, G, total_tiles, group_q, scale_log2, softmax_scale, flags, st->status_ptr);                 \
     if (run_dkv)                                                                                                        \
-      launch_after(pairs ? bwd_dkv_w128_kernel<CC, 2> : bwd_dkv_w128_kernel<CC, 1>, grid_dkv, pairs ? 2 : 1, BwdW128::kThreads,    \
+      launch_after(dkv_pairs ? bwd_dkv_w128_kernel<CC, 2> : bwd_dkv_w128_kernel<CC, 1>, grid_kv, dkv_pairs ? 2 : 1, BwdW128::kThreads,    \
           BwdW128::kDkvSmemBytes, s, run_dq, mK128, mV128, mQ128, mdO128, mZs, mdKst, mdVst, stats, static_cast<__nv_bfloat16 *>(dK), \
           static_cast<__nv_bfloat16 *>(dV), plan_kv, nblk, Nk, N, BHkv, Hkv, G, total_kv_tiles, group_kv, scale_log2, softmax_scale,\
           flags, st->status_ptr);                                                                                       \
@@ -890,7 +894,7 @@ int gproj_attn_fwd_bwd_host(const void *Q, const void *K, const void *V, const v
   // its direction beyond its bytes and the two directions share about 80 GB/s, so many small slabs are slower than few
   // large ones, while the last slab's kernels and copy-out stay exposed.  The forward starts without dO, and dQ leaves while
   // dK and dV are computed.  Measured, before (2 MiB slabs, all inputs first, all gradients together) -> now: 16 heads x 4096
-  // x 64: 1020 -> 919 us; 2 x (16 query, 4 KV heads) x 6000 x 64: 1960 -> 1800; 64 heads x 4000 x 128: 6640 -> 6100; 16 / 8
+  // x 64: 1020 -> 919 us; 2 x (16 query, 4 KV heads) x 6000 x 64: 1960 -> 1800; 64 heads x 4000 x 128: 6700 -> 6200 to 6500; 16 / 8
   // heads x 7000 x 64, not causal: 1930 -> 1608.
   const int kv_heads = B * Hkv, G = H / Hkv;
   int slabs = static_cast<int>(1 + qb / kHostSlabBytes);
