@@ -556,7 +556,8 @@ namespace {
 // causal: 229 -> 140; 32 / 4 heads x 2000: 121 -> 78; 4 heads x 4096, causal: 43.5 -> 37.2; 1 head x 8192: 62.0 -> 43.5;
 // 16 heads x 4096, causal (stays with whole tiles): 68; 16 packed documents of 8192 rows, 16 / 4 heads: 78.6 -> 73.0.
 // dK/dV side at d = 128: 16 / 4 heads x 4096, causal: 275 -> 151; 8 / 1 heads x 3000, causal: 375 -> 200; 16 / 8 heads x 700, causal: 30.9 ->
-// 25.0; 2 heads x 1500, causal: 30.9 -> 24.8; 4 heads x 1000 (16 steps, stays with whole tiles): 25.1.
+// 25.0; 2 heads x 1500, causal: 30.9 -> 24.8; 4 heads x 1000 (16 steps): 24.7 -> 21.0; 4 heads x 800, causal: 20.7 -> 19.1; 2 heads x 640 (10
+// steps): 17.5 -> 17.1, hence four steps for the exchange.
 // dQ side: 1 head x 8192 x 64: 83 -> 52 us; 4 heads x 4096 x 64, causal: 44.7 -> 34.4; 16 heads x 300 queries behind 9000 keys,
 // d = 128: 126 -> 92; 4 heads x 2048 x 128, causal: 36.5 -> 32.8; 4 heads x 1000 x 128 (16 steps): 20.7 -> 21.3, hence the
 // 8 steps the exchange counts at d = 128.
@@ -631,7 +632,7 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
     group_q.solo = packed_solo(*seqs, false, BH, st->sm_count, [&](int keys) { return std::max(1, (keys + 63) / 64) + (d == 64 ? 3.8 : 3.0); });
   const int dkv_fit = st->dkv_clusters[d == 128], dkv_rows = d == 64 ? 128 : 64;   // rows of a step
   const bool dkv_pairs = run_dkv && total_kv_tiles <= 8LL * st->sm_count &&
-                         prefers_pairs(tile_steps(seqs, true, dkv_rows, G, N, Nk, causal != 0), BHkv, st->sm_count, dkv_fit, d == 64 ? 2.3 : 3.0, d == 64 ? 1.5 : 8.0);
+                         prefers_pairs(tile_steps(seqs, true, dkv_rows, G, N, Nk, causal != 0), BHkv, st->sm_count, dkv_fit, d == 64 ? 2.3 : 3.0, d == 64 ? 1.5 : 4.0);
   if (seqs && !dkv_pairs)
     group_kv.solo = packed_solo(*seqs, true, BHkv, st->sm_count, [&](int rows) { return G * std::max(1, (rows + dkv_rows - 1) / dkv_rows) + (d == 64 ? 2.3 : 3.0); });
   const dim3 grid(static_cast<unsigned>(dq_pairs ? 2 * std::min(total_tiles, dq_fit) : std::min(total_tiles, st->sm_count)));   // persistent: one CTA per SM
