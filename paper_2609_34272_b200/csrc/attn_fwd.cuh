@@ -538,7 +538,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             uint32_t o[16];
             tmem_ld16(tO + 16 * c, o);
             tmem_wait_ld();
-            const bool has = l_run > 0.f;          // otherwise the accumulator may never have been written
+            const bool has = l_run != 0.f;         // otherwise the accumulator may never have been written; a NaN goes on to the output
 #pragma unroll
             for (int v = 0; v < 4; ++v)
               *reinterpret_cast<uint4 *>(part + 16 * c + 4 * v) = has ? make_uint4(o[4 * v], o[4 * v + 1], o[4 * v + 2], o[4 * v + 3]) : make_uint4(0u, 0u, 0u, 0u);

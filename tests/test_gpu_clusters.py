@@ -47,6 +47,34 @@ def test_forward_with_the_key_range_split_over_a_cluster(shape, d):
     assert np.abs(O - ex["O"]).max() <= 0.03 * np.abs(ex["O"]).max()
 
 
+# query heads folded on one CTA per tile; clusters with and without folding; the last without either, for comparison
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("shape", [(1, 8, 1, 4, 40, True), (2, 8, 2, 16, 4096, True), (1, 2, 2, 128, 4100, False), (1, 2, 2, 600, 600, True)])
+def test_a_nan_reaches_every_output_row_that_sees_it(shape, d):
+    B, H, Hkv, Nq, Nk, causal = shape
+    gen = torch.Generator().manual_seed(Nq + Nk + d)
+    rand = lambda h, n: torch.randn(B, h, n, d, generator=gen).to(torch.bfloat16).cuda()
+    for name in ("Q", "K", "V"):
+        x = {"Q": rand(H, Nq), "K": rand(Hkv, Nk), "V": rand(Hkv, Nk)}
+        at = 1 if name == "Q" else Nk // 3
+        x[name][0, 0, at, 3] = float("nan")
+        O, _ = g.gproj_attn_fwd_rect(x["Q"], x["K"], x["V"], d ** -0.5, causal)
+        want = torch.zeros(B, H, Nq, dtype=torch.bool)
+        if name == "Q":
+            want[0, 0, at] = True
+        else:                                     # the queries of the KV head's group that see key `at`
+            want[0, :H // Hkv] = (torch.arange(Nq) + Nk - Nq >= at) if causal else True
+        nan = O.isnan().cpu()
+        if name == "V":                           # one column of those rows; elsewhere 0 x NaN of a masked key may appear
+            assert nan[..., 3][want].all()
+        else:
+            assert nan[want].all()
+            if name == "Q":
+                assert not nan[~want].any()
+    rc, detail = g.gproj_last_device_status()
+    assert rc == 0, hex(detail)
+
+
 @pytest.mark.parametrize("causal", [True, False])
 def test_packed_forward_with_split_keys_repeats_bitwise(causal):
     # one long and some short sequences: parts of a tile without any key tile, tiles of different length in one launch
