@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(256, 1) fp32_attn_fwd_kernel(const __nv_bfloat
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int g = 0; g < SG; ++g) {
       const float mg = mm[g * 32 + r];
-      L += (mg == -INFINITY) ? 0.f : ml[g * 32 + r] * __expf(mg - M);
+      L += ml[g * 32 + r] * ((mg == -INFINITY) ? 0.f : __expf(mg - M));     // l is 0 without a key, and NaN where all scores were
       const float4 v = *reinterpret_cast<const float4 *>(mo + g * C::kMergeF + r * (D + 4) + 4 * c4);
       s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
     }

@@ -28,3 +28,15 @@ def test_fp32_arm_at_tile_edges(N, d, causal):
         assert np.all(np.isfinite(t)), n
         assert oracle.rel_l2_percent(t, ex[n]) <= 0.3, n
         assert np.abs(t - ex[n]).max() <= 0.01 * np.abs(ex[n]).max(), n
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_fp32_arm_keeps_a_nan_in_the_normaliser(d):
+    # Keys 0..3 go to one share of the streamed rows and are all that it sees of rows 0..5: its maximum stays -inf while its
+    # normaliser is NaN.  Every row sees such a key, so all probabilities and with them all gradients are NaN.
+    gen = torch.Generator().manual_seed(d)
+    Q, K, V, dO = (torch.randn(1, 1, 6, d, generator=gen).to(torch.bfloat16).cuda() for _ in range(4))
+    K[0, 0, :4] = float("nan")
+    O, saved = g.gproj_fp32_attn_fwd(Q, K, V, d ** -0.5, True)
+    for t in (O,) + tuple(g.gproj_fp32_attn_bwd(Q, K, V, dO, saved, d ** -0.5, True)):
+        assert t.isnan().all()
