@@ -47,6 +47,8 @@ namespace gproj {
 constexpr unsigned kFlagNoQCorrection = 1u;
 constexpr unsigned kFlagNoKCorrection = 2u;
 
+constexpr int kMaxSeqRows = 1 << 24;   // rows of a head (the entry points check it)
+
 // Bytes of one 64-row block of the row-constant tile (64 rows x 16 BF16 columns).
 constexpr int kExtBlockBytes = 2048;
 
@@ -378,6 +380,7 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
   // N: query rows per head (own operand), Nk: key rows per head.  Causal support of query i: keys j <= i + (L_k - L_q).
   using C = BwdCfg<D>;
   constexpr int NB = C::kNB, R = C::kDqResBufs, S = C::kDqStages;
+  constexpr long long kTileBudget = tile_wait_budget(kMaxSeqRows / C::kStepRows + 1);   // of a wait that may span a tile
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t *sRes = smem;                                        // buffer rb: Q tile, then dO tile
@@ -481,7 +484,7 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
       for (int lin = sched.next(); lin >= 0; lin = sched.next(), ++ti) {
         const int rb = ti % R, bh = hix(lin);
         const TileInfo tl = tile_of(lin);
-        if (ti >= R) mbar_wait(&bar_res_free[rb], ((ti / R) - 1) & 1, ab, kDqWaitResFree);
+        if (ti >= R) mbar_wait(&bar_res_free[rb], ((ti / R) - 1) & 1, ab, kDqWaitResFree, kTileBudget);
         mbar_expect_tx(&bar_res_full[rb], 2 * C::kBigTileBytes);
         uint8_t *dst = sRes + rb * 2 * C::kBigTileBytes;
         for (int s = 0; s < C::kSlabs; ++s) {
@@ -682,7 +685,7 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
       };
       fetch_q(0);
       // row masses of all warpgroups (fixed order), lambda = rho / m with the zero-mass rule (Algorithm 1 line 14)
-      mbar_wait(&bar_mass_ready[par], (ti >> 1) & 1, ab, kDqWaitMass);
+      mbar_wait(&bar_mass_ready[par], (ti >> 1) & 1, ab, kDqWaitMass, kTileBudget);
       float rho_t = s_rho[par][0][row], m_t = s_m[par][0][row];
 #pragma unroll
       for (int w = 1; w < C::kWG; ++w) { rho_t += s_rho[par][w][row]; m_t += s_m[par][w][row]; }
@@ -692,7 +695,7 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
         cluster_store_f32(peer, rho_t);
         cluster_store_f32(peer + 512, m_t);
         cluster_mbar_arrive(cluster_map_shared(smem_u32(&bar_peer_mass), rank ^ 1));
-        mbar_wait_cluster(&bar_peer_mass, ti & 1, ab, kDqWaitPeer);
+        mbar_wait_cluster(&bar_peer_mass, ti & 1, ab, kDqWaitPeer, kTileBudget);
         rho_t += s_peer[2 * par][row];                     // two terms: the same sum in both CTAs
         m_t += s_peer[2 * par + 1][row];
       }
@@ -714,7 +717,7 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
         }
         if (h + 1 < kIters / kQ) fetch_q(h + 1);
       }
-      mbar_wait(&bar_acc_done, ti & 1, ab, kDqWaitAcc);
+      mbar_wait(&bar_acc_done, ti & 1, ab, kDqWaitAcc, kTileBudget);
       tc_fence_after();
       uint8_t *stg = sStaging + 4096 * ew;
       // The other CTA's parts land in this tile's Q / dO buffer, whose last reader (the last score product) is done:
@@ -723,7 +726,7 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
       auto piece = [&](int chunk, int v) { return static_cast<uint32_t>(chunk * 8192 + row * 64 + ((v ^ ((row >> 1) & 3)) << 4)); };
       if (CL > 1) {
         if (row == 0) cluster_mbar_arrive(cluster_map_shared(smem_u32(&bar_peer_ready), rank ^ 1));
-        mbar_wait_cluster(&bar_peer_ready, ti & 1, ab, kDqWaitPeer);
+        mbar_wait_cluster(&bar_peer_ready, ti & 1, ab, kDqWaitPeer, kTileBudget);
         const uint32_t peer = cluster_map_shared(smem_u32(parts), rank ^ 1);
 #pragma unroll
         for (int c = 0; c < 2 * kCols / 16; ++c) {         // A, then B, of the other CTA's columns
@@ -736,7 +739,7 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
             cluster_store_f4(peer + piece(c, v), __uint_as_float(a[4 * v]), __uint_as_float(a[4 * v + 1]), __uint_as_float(a[4 * v + 2]), __uint_as_float(a[4 * v + 3]));
         }
         cluster_mbar_arrive(cluster_map_shared(smem_u32(&bar_peer_full), rank ^ 1));
-        mbar_wait_cluster(&bar_peer_full, ti & 1, ab, kDqWaitPeer);
+        mbar_wait_cluster(&bar_peer_full, ti & 1, ab, kDqWaitPeer, kTileBudget);
       }
       constexpr int kHd = kCols < 64 ? kCols : 64;         // columns staged at a time
 #pragma unroll
@@ -899,6 +902,7 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 rows
   // masked.
   auto own_steps = [&](int T) { return CL == 1 ? G * T : max(1, (G * T - rank + CL - 1) / CL); };
   auto own_step = [&](int n, int T) { return CL == 1 ? n : (rank < G * T ? CL * n + rank : 0); };
+  auto tile_budget = [&]() { return tile_wait_budget(static_cast<long long>(G) * (Nq / C::kStepRows + 1)); };   // of a wait that may span a tile
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer of the streamed (Q, dO, Z, stats) step tiles
@@ -937,7 +941,7 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 rows
       int ti = 0;
       for (int lin = sched.next(); lin >= 0; lin = sched.next(), ++ti) {
         const int bh = hix(lin), krow0 = tile_of(lin).row0;
-        if (ti >= 1) mbar_wait(&bar_res_free, (ti - 1) & 1, ab, kDkvWaitResFree);
+        if (ti >= 1) mbar_wait(&bar_res_free, (ti - 1) & 1, ab, kDkvWaitResFree, tile_budget());
         mbar_expect_tx(&bar_res_full, 2 * C::kBigTileBytes);
         for (int s = 0; s < C::kSlabs; ++s) {
           tma_load_3d(sK + s * C::kBigSlabBytes, &tmK, &bar_res_full, s * 64, krow0, bh);
@@ -994,7 +998,7 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 rows
     int g = 0, ti = 0;
     for (int lin = sched.next(); lin >= 0; lin = sched.next(), ++ti) {
       const int T = own_steps(steps_of(tile_of(lin)));
-      if (ti > 0) mbar_wait(&bar_acc_free, (ti - 1) & 1, ab, kDkvWaitAccFree);   // the previous epilogue has read dV, dK
+      if (ti > 0) mbar_wait(&bar_acc_free, (ti - 1) & 1, ab, kDkvWaitAccFree, tile_budget());   // the previous epilogue has read dV, dK
       for (int p = 0; p < T; ++p, ++g) {
         const int st = g % S, b = g % NB;
         const SmemDesc dscQ = dscQ0mn.advanced(st * C::kDkvStageBytes), dscdO = dscQ.advanced(C::kStepTileBytes),
@@ -1088,7 +1092,7 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 rows
       const TileInfo tl = tile_of(lin);
       const size_t wrow0 = (static_cast<size_t>(hix(lin)) * N + tl.row0 + 32 * ew) * D;
       const int wrows = tl.seq_end - tl.row0 - 32 * ew;      // rows of this warp that exist
-      mbar_wait(&bar_acc_done, ti & 1, ab, kDkvWaitAcc);
+      mbar_wait(&bar_acc_done, ti & 1, ab, kDkvWaitAcc, tile_budget());
       tc_fence_after();
       if (CL > 1) {
         // [D / 16 chunks of 16 columns][128 rows] x 64 bytes of FP32, the 16-byte pieces of a row swizzled
@@ -1098,7 +1102,7 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 rows
         const uint32_t peer = cluster_map_shared(smem_u32(sK), rank ^ 1);
         const float scale = rank == 0 ? 1.0f : alpha;
         if (row == 0) cluster_mbar_arrive(cluster_map_shared(smem_u32(&bar_peer_ready), rank ^ 1));   // this CTA's K / V tile is consumed
-        mbar_wait_cluster(&bar_peer_ready, ti & 1, ab, kDkvWaitPeer);
+        mbar_wait_cluster(&bar_peer_ready, ti & 1, ab, kDkvWaitPeer, tile_budget());
 #pragma unroll 2
         for (int cc = 0; cc < D / 16; ++cc) {
           uint32_t a[16];
@@ -1109,7 +1113,7 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 rows
             cluster_store_f4(peer + piece(cc, v), __uint_as_float(a[4 * v]), __uint_as_float(a[4 * v + 1]), __uint_as_float(a[4 * v + 2]), __uint_as_float(a[4 * v + 3]));
         }
         cluster_mbar_arrive(cluster_map_shared(smem_u32(&bar_peer_full), rank ^ 1));
-        mbar_wait_cluster(&bar_peer_full, ti & 1, ab, kDkvWaitPeer);
+        mbar_wait_cluster(&bar_peer_full, ti & 1, ab, kDkvWaitPeer, tile_budget());
 #pragma unroll 1
         for (int c = 0; c < D / 32; ++c) {
 #pragma unroll

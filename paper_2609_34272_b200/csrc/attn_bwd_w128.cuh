@@ -206,6 +206,7 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
   // masked.
   auto own_steps = [&](int T) { return CL == 1 ? G * T : max(1, (G * T - rank + CL - 1) / CL); };
   auto own_step = [&](int n, int T) { return CL == 1 ? n : (rank < G * T ? CL * n + rank : 0); };
+  auto tile_budget = [&]() { return tile_wait_budget(static_cast<long long>(G) * (Nq / C::kStepRows + 1)); };   // of a wait that may span a tile
 
   if (warp < 4) {
   setmaxnreg_dec<C::kRegsAux>();
@@ -215,7 +216,7 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
     if (lane == 0) {
       int g = 0, ti = 0;
       auto load_kv = [&](int krow0, int bh) {
-        if (ti >= 1) mbar_wait(&bar_res_free, (ti - 1) & 1, ab, kWkResFree);
+        if (ti >= 1) mbar_wait(&bar_res_free, (ti - 1) & 1, ab, kWkResFree, tile_budget());
         mbar_expect_tx(&bar_res_full, 2 * C::kTileBytes);
         tma_load_3d(sK, &tmK, &bar_res_full, 0, krow0, bh);
         tma_load_3d(sV, &tmV, &bar_res_full, 0, krow0, bh);
@@ -324,7 +325,7 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
     int g = 0, ti = 0;
     for (int lin = sched.next(); lin >= 0; lin = sched.next(), ++ti) {
       const int T = own_steps(steps_of(tile_of(lin)));
-      if (ti > 0) mbar_wait(&bar_acc_free, (ti - 1) & 1, ab, kWkAccFree);   // the previous epilogue has read dV, dK
+      if (ti > 0) mbar_wait(&bar_acc_free, (ti - 1) & 1, ab, kWkAccFree, tile_budget());   // the previous epilogue has read dV, dK
       for (int p = 0; p < T; ++p, ++g) {
         const int st = g % S, sb = g & 1;
         const SmemDesc dscQ = dscQ0mn.advanced(st * C::kDkvStageBytes), dscdO = dscQ.advanced(C::kTileBytes);
@@ -444,9 +445,9 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
         const uint32_t peer_buf = cluster_map_shared(smem_u32(sOut), rank ^ 1);
         const uint32_t t_own = tmem_base + (rank == 0 ? C::kColAcc0 : C::kColAcc1) + lane_addr, t_send = tmem_base + (rank == 0 ? C::kColAcc1 : C::kColAcc0) + lane_addr;
         const float scale = rank == 0 ? 1.0f : alpha;
-        mbar_wait(&bar_acc_done, ti & 1, ab, kWkAcc);
+        mbar_wait(&bar_acc_done, ti & 1, ab, kWkAcc, tile_budget());
         tc_fence_after();
-        if (ti > 0) mbar_wait_cluster(&bar_peer_free, (ti - 1) & 1, ab, kWkPeerFree);   // the other CTA has taken the previous tile's part
+        if (ti > 0) mbar_wait_cluster(&bar_peer_free, (ti - 1) & 1, ab, kWkPeerFree, tile_budget());   // the other CTA has taken the previous tile's part
 #pragma unroll
         for (int cc = 0; cc < D / 16; ++cc) {
           uint32_t a[16];
@@ -457,7 +458,7 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
             cluster_store_f4(peer_buf + piece(cc, row, v), __uint_as_float(a[4 * v]), __uint_as_float(a[4 * v + 1]), __uint_as_float(a[4 * v + 2]), __uint_as_float(a[4 * v + 3]));
         }
         cluster_mbar_arrive(cluster_map_shared(smem_u32(&bar_peer_full), rank ^ 1));
-        mbar_wait_cluster(&bar_peer_full, ti & 1, ab, kWkPeerFull);
+        mbar_wait_cluster(&bar_peer_full, ti & 1, ab, kWkPeerFull, tile_budget());
 #pragma unroll
         for (int cc = 0; cc < D / 16; ++cc) {
           uint32_t a[16];
@@ -489,7 +490,7 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
       }
       if (row == 0) bulk_wait_group_read0();                 // the previous tile's stores have left the staging buffer
       named_bar_sync(1, 128);
-      mbar_wait(&bar_acc_done, ti & 1, ab, kWkAcc);
+      mbar_wait(&bar_acc_done, ti & 1, ab, kWkAcc, tile_budget());
       tc_fence_after();
 #pragma unroll
       for (int cc = 0; cc < D / 16; ++cc) {

@@ -291,7 +291,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         const Item it = decode(lin);
         const int bh = hix(lin), tiles = it.nq;
         const int qb = q_buf(ti), use = q_use(ti);
-        if (use >= 1) mbar_wait(&bar_q_free[qb], (use - 1) & 1, ab, kFwdWaitQFree);
+        if (use >= 1) mbar_wait(&bar_q_free[qb], (use - 1) & 1, ab, kFwdWaitQFree, tile_wait_budget(2LL * (Nk / C::kBlockN + 1)));   // up to two tiles
         // The softmax warps (168 registers, the kernel's tightest code) take the item's rank and head from here instead
         // of decoding the item number themselves; the barrier's completion publishes the two words.  The loader is at
         // most two items ahead of them, the ring has four entries.

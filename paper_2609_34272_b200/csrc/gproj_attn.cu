@@ -185,7 +185,7 @@ int check_shape(int B, int H, int N, int d) {
   if (B <= 0 || H <= 0 || N <= 0) return GPROJ_ERR_SHAPE;
   if (d != 64 && d != 128) return GPROJ_ERR_SHAPE;
   const long long rows = static_cast<long long>(B) * H * N;
-  if (rows >= (1LL << 31) || static_cast<long long>(B) * H >= (1LL << 20) || N > (1 << 24)) return GPROJ_ERR_SHAPE;
+  if (rows >= (1LL << 31) || static_cast<long long>(B) * H >= (1LL << 20) || N > kMaxSeqRows) return GPROJ_ERR_SHAPE;
   return GPROJ_OK;
 }
 

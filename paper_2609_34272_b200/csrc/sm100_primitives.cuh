@@ -8,6 +8,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "wait_budget.h"
+
 namespace gproj {
 
 // ------------------------------------------------------------------------------------------
@@ -104,13 +106,11 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
   return ok != 0;
 }
 
-// Bounded wait.  Gives up after ~kWaitBudgetCycles SM clocks (a fraction of a second), records
+// Bounded wait.  Gives up after `budget` SM clocks (a fraction of a second unless the wait spans a tile), records
 // `code` in the launch's status word and raises the CTA's abort flag; once the flag is up every
 // later wait of the CTA returns at once, so all roles run to the end of their loops and the CTA
 // exits through its normal epilogue (TMEM freed, no thread left behind).
-constexpr long long kWaitBudgetCycles = 400LL * 1000 * 1000;
-
-__device__ __forceinline__ void mbar_wait(uint64_t *bar, uint32_t parity, const AbortState &ab, int code) {
+__device__ __forceinline__ void mbar_wait(uint64_t *bar, uint32_t parity, const AbortState &ab, int code, long long budget = kWaitBudgetCycles) {
   if (mbar_try_wait(bar, parity)) return;
   if (*ab.cta_abort) return;
   long long t0 = clock64();
@@ -118,7 +118,7 @@ __device__ __forceinline__ void mbar_wait(uint64_t *bar, uint32_t parity, const 
   while (!mbar_try_wait(bar, parity)) {
     if ((++spins & 0x3ff) == 0) {
       if (*ab.cta_abort) return;
-      if (clock64() - t0 > kWaitBudgetCycles) {
+      if (clock64() - t0 > budget) {
         *ab.cta_abort = 1;
         atomicCAS(ab.global_status, 0, kDevTimeout | (code << 8));
         return;
@@ -455,8 +455,8 @@ __device__ __forceinline__ void cluster_mbar_arrive(uint32_t addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
 // mbar_wait for a phase that another CTA's arrivals complete (acquires at cluster scope)
-__device__ __forceinline__ void mbar_wait_cluster(uint64_t *bar, uint32_t parity, const AbortState &ab, int code) {
-  mbar_wait(bar, parity, ab, code);
+__device__ __forceinline__ void mbar_wait_cluster(uint64_t *bar, uint32_t parity, const AbortState &ab, int code, long long budget) {
+  mbar_wait(bar, parity, ab, code, budget);
   uint32_t ok;
   asm volatile(
       "{\n\t.reg .pred P;\n\t"

@@ -1,0 +1,39 @@
+"""Limits of the kernels' waits, checked without a GPU: by arithmetic, and by which wait has which limit."""
+import ctypes
+import os
+import re
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2609_34272_b200", "csrc")
+CLOCKS_PER_STEP = 2000          # upper end of what a step of any kernel takes
+
+
+@pytest.fixture(scope="module")
+def budget(tmp_path_factory):
+    d = tmp_path_factory.mktemp("wait_budget")
+    (d / "b.cpp").write_text('#include "wait_budget.h"\nextern "C" long long budget(long long s) { return gproj::tile_wait_budget(s); }\n')
+    subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, "-o", str(d / "b.so"), str(d / "b.cpp")], check=True)
+    f = ctypes.CDLL(str(d / "b.so")).budget
+    f.restype, f.argtypes = ctypes.c_longlong, [ctypes.c_longlong]
+    return f
+
+
+# (query heads per KV head, queries): a single key tile's steps of 64 queries; the last is the largest that the entry points take
+@pytest.mark.parametrize("G,Nq", [(1, 128), (64, 1 << 18), (16, 1 << 20), (64, 1 << 20), (127, 1 << 24)])
+def test_a_wait_for_a_whole_tile_outlasts_the_tile(budget, G, Nq):
+    steps = G * (Nq // 64 + 1)
+    assert budget(steps) >= 4 * steps * CLOCKS_PER_STEP and budget(steps) >= budget(0) > 0
+
+
+def test_every_wait_that_may_span_a_tile_has_the_tile_limit():
+    # loaders of a stationary tile, epilogues, parts of another CTA (what waits for an epilogue waits for its last microseconds)
+    bars = "res_free|acc_done|mass_ready|peer_mass|peer_ready|peer_full|peer_free|q_free"
+    found = 0
+    for name in ("attn_fwd.cuh", "attn_bwd.cuh", "attn_bwd_w128.cuh"):
+        for line in open(os.path.join(CSRC, name)):
+            for call in re.findall(r"mbar_wait(?:_cluster)?\(&bar_(?:%s)\b[^;]*;" % bars, line):
+                found += 1
+                assert any(b in call for b in ("tile_budget()", "kTileBudget", "tile_wait_budget(")), (name, call)
+    assert found >= 16
