@@ -399,7 +399,7 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) cta_skip = *reinterpret_cast<volatile int *>(status);
   __syncthreads();
-  if (CL == 1 && cta_skip != 0) return;   // an earlier wait gave up: drain the rest of the grid quickly (a cluster runs on with every wait falling through)
+  if (CL == 1 && cta_skip != 0) { griddep_wait(); return; }   // an earlier wait gave up: drain the rest of the grid quickly (a cluster runs on with every wait falling through)
 
   // Ragged N: tiles and steps round up; rows past N load as zero (TMA fill) and are clipped on store.
   const int n_qt = (N + 127) / 128;
@@ -839,7 +839,7 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 rows
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) cta_skip = *reinterpret_cast<volatile int *>(status);
   __syncthreads();
-  if (CL == 1 && cta_skip != 0) return;   // a cluster runs on with every wait falling through: its CTAs exchange results
+  if (CL == 1 && cta_skip != 0) { griddep_wait(); return; }   // a cluster runs on with every wait falling through: its CTAs exchange results
 
   const bool use_z = (flags & kFlagNoKCorrection) == 0;
   const uint32_t stage_tx = (use_z ? 3 : 2) * C::kStepTileBytes + kExtBlockBytes;

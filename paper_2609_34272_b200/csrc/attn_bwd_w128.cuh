@@ -145,7 +145,7 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) cta_skip = *reinterpret_cast<volatile int *>(status);
   __syncthreads();
-  if (CL == 1 && cta_skip != 0) return;   // a cluster runs on with every wait falling through: its CTAs exchange results
+  if (CL == 1 && cta_skip != 0) { griddep_wait(); return; }   // a cluster runs on with every wait falling through: its CTAs exchange results
 
   const bool use_z = (flags & kFlagNoKCorrection) == 0;
   const uint32_t stage_tx = (use_z ? 3 : 2) * C::kTileBytes + C::kExtBytes;

@@ -125,9 +125,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) cta_skip = *reinterpret_cast<volatile int *>(status);
   __syncthreads();
-  // An earlier wait gave up: drain the rest of the grid quickly.  The CTAs of a cluster wait for one another at the end, so
-  // they run on with every wait falling through instead.
-  if (!kCluster && cta_skip != 0) return;
+  // An earlier wait gave up: drain the rest of the grid quickly, but not past the kernel before this one, for whose end the
+  // next kernel in the stream relies on this one.  The CTAs of a cluster wait for one another at the end, so they run on with
+  // every wait falling through instead.
+  if (!kCluster && cta_skip != 0) { griddep_wait(); return; }
 
   const int n_qt = (N + C::kBlockM - 1) / C::kBlockM;   // the last tile may be ragged: rows past N load as zero, stores clip
   const int TPI = tiles_per_item;                  // 2: a pair of query tiles per work item; 1: single tiles, key range split

@@ -37,3 +37,15 @@ def test_every_wait_that_may_span_a_tile_has_the_tile_limit():
                 found += 1
                 assert any(b in call for b in ("tile_budget()", "kTileBudget", "tile_wait_budget(")), (name, call)
     assert found >= 16
+
+
+def test_a_cta_that_skips_its_work_still_waits_for_the_previous_kernel():
+    # after a wait has given up, the CTAs of later launches return at once; one that was launched early (programmatic
+    # dependent launch) must not let its grid end before the one in front of it, which may still be writing
+    found = 0
+    for name in ("attn_fwd.cuh", "attn_bwd.cuh", "attn_bwd_w128.cuh"):
+        for line in open(os.path.join(CSRC, name)):
+            if "cta_skip != 0" in line and "return" in line:
+                found += 1
+                assert line.index("griddep_wait();") < line.index("return"), (name, line)
+    assert found == 4
