@@ -9,8 +9,10 @@
 
 namespace gproj {
 
-// A wait for the next stage of a pipeline: a fraction of a second.
-constexpr long long kWaitBudgetCycles = 400LL * 1000 * 1000;
+// A wait for the next stage of a pipeline: about half a second.  The dK/dV side starts beside the end of the dQ side, and its
+// first waits last until that has ended: up to one tile of it, 2^24 / 64 steps of at most 2000 clocks.  (Letting all its
+// warps pass griddepcontrol.wait first instead cost 0.1 to 0.9 us a call.)
+constexpr long long kWaitBudgetCycles = 1000LL * 1000 * 1000;
 
 // A wait from one tile to the next (a tile loader, an epilogue, another CTA's part) lasts as long as the tile: 700 to 2000
 // clocks for each of its steps, and a long tile has a million of them (64 query heads on one KV head at 2^20 queries walk

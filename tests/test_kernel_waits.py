@@ -27,6 +27,11 @@ def test_a_wait_for_a_whole_tile_outlasts_the_tile(budget, G, Nq):
     assert budget(steps) >= 4 * steps * CLOCKS_PER_STEP and budget(steps) >= budget(0) > 0
 
 
+def test_a_stage_wait_outlasts_a_tile_of_the_kernel_in_front(budget):
+    # the dK/dV side starts beside the dQ side's last tiles; a tile of that has at most 2^24 / 64 steps
+    assert budget(0) >= (2 ** 24 // 64 + 1) * CLOCKS_PER_STEP
+
+
 def test_every_wait_that_may_span_a_tile_has_the_tile_limit():
     # loaders of a stationary tile, epilogues, parts of another CTA (what waits for an epilogue waits for its last microseconds)
     bars = "res_free|acc_done|mass_ready|peer_mass|peer_ready|peer_full|peer_free|q_free"
