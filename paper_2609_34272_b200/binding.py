@@ -5,6 +5,7 @@ memory and the stream.  There is no CPU fallback: if the library is missing or t
 device is not sm_100a the calls raise.
 """
 import ctypes
+import math
 import os
 
 import torch
@@ -174,6 +175,30 @@ def _check_lse(LSE, shape, what):
         raise TypeError(f"LSE must be a contiguous CUDA float32 tensor [{what}]")
 
 
+def _check_buffer(name, t, index, dtype=None, count=0):
+    """A caller's buffer that the kernels write: on the call's device, contiguous, and with room for `count` elements."""
+    if not (isinstance(t, torch.Tensor) and t.is_cuda and t.get_device() == index and t.is_contiguous() and (dtype is None or t.dtype is dtype)):
+        raise TypeError(f"{name} must be a contiguous {dtype or ''} tensor on the inputs' CUDA device")
+    if t.numel() < count:
+        raise ValueError(f"{name} has {t.numel()} elements, needs {count}")
+
+
+def _lse_out(LSE, Q, shape):
+    """The caller's LSE output, checked, or a new one."""
+    if LSE is None:
+        return Q.new_empty(shape, dtype=_F32)
+    _check_buffer("LSE", LSE, Q.get_device(), _F32, math.prod(shape))
+    return LSE
+
+
+def _scratch(name, t, Q, nbytes):
+    """The caller's scratch or saved state (the library checks its size), or a new one of at least 256 bytes."""
+    if t is None:
+        return Q.new_empty(max(nbytes, 256), dtype=_U8)
+    _check_buffer(name, t, Q.get_device())
+    return t
+
+
 def gproj_attn_bwd_workspace_bytes(B, H, N, d) -> int:
     return int(load().gproj_attn_bwd_workspace_bytes(B, H, N, d))
 
@@ -190,8 +215,7 @@ def gproj_attn_fwd(Q, K, V, softmax_scale, causal, O=None, LSE=None, fwd_flags=0
         O = torch.empty_like(Q)
     else:
         _check_bf16("O", O, shape)
-    if LSE is None:
-        LSE = Q.new_empty((B, H, N), dtype=_F32)
+    LSE = _lse_out(LSE, Q, (B, H, N))
     index = Q.get_device()
     with _on_device(index):
         rc = (_lib or load()).gproj_attn_fwd_ex(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), LSE.data_ptr(), B, H, Hkv, N, d,
@@ -211,11 +235,8 @@ def gproj_attn_bwd(Q, K, V, O, LSE, dO, softmax_scale, causal, flags=0, workspac
     Hkv = _kv_heads(shape, K)
     _check_lse(LSE, (B, H, N), "B, H, N")
     lib = _lib or load()
-    if workspace is None:
-        nbytes = max(lib.gproj_attn_bwd_workspace_bytes(B, H, N, d), 256)
-        workspace = Q.new_empty(nbytes, dtype=_U8)
-    else:
-        nbytes = workspace.numel() * workspace.element_size()
+    workspace = _scratch("workspace", workspace, Q, lib.gproj_attn_bwd_workspace_bytes(B, H, N, d))
+    nbytes = workspace.numel() * workspace.element_size()
     dQ = _output("dQ", dQ, Q); dK = _output("dK", dK, K); dV = _output("dV", dV, K)
     index = Q.get_device()
     with _on_device(index):
@@ -241,7 +262,7 @@ def gproj_attn_fwd_rect(Q, K, V, softmax_scale, causal, O=None, LSE=None, fwd_fl
     j <= i + (Nk - Nq); a query that sees none gets O = 0 and LSE = +inf."""
     B, H, Hkv, Nq, Nk, d = _rect_shapes(Q, K, V)
     O = torch.empty_like(Q) if O is None else O
-    LSE = Q.new_empty((B, H, Nq), dtype=_F32) if LSE is None else LSE
+    LSE = _lse_out(LSE, Q, (B, H, Nq))
     _check_bf16("O", O, Q.shape)
     with _on_device(Q.get_device()):
         rc = load().gproj_attn_fwd_rect(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), LSE.data_ptr(), B, H, Hkv, Nq, Nk, d,
@@ -257,8 +278,7 @@ def gproj_attn_bwd_rect(Q, K, V, O, LSE, dO, softmax_scale, causal, flags=0, wor
     for name, t in (("O", O), ("dO", dO)):
         _check_bf16(name, t, Q.shape)
     _check_lse(LSE, (B, H, Nq), "B, H, Nq")
-    if workspace is None:
-        workspace = Q.new_empty(max(gproj_attn_bwd_workspace_bytes(B, H, Nq, d), 256), dtype=_U8)
+    workspace = _scratch("workspace", workspace, Q, gproj_attn_bwd_workspace_bytes(B, H, Nq, d))
     dQ = _output("dQ", dQ, Q); dK = _output("dK", dK, K); dV = _output("dV", dV, K)
     with _on_device(Q.get_device()):
         rc = load().gproj_attn_bwd_rect(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), LSE.data_ptr(), dO.data_ptr(),
@@ -299,8 +319,7 @@ def gproj_fp32_attn_fwd(Q, K, V, softmax_scale, causal, saved=None):
     B, H, N, d = Q.shape
     _check_bf16("K", K, Q.shape); _check_bf16("V", V, Q.shape)
     need = int(load().gproj_fp32_attn_saved_bytes(B, H, N, d))
-    if saved is None:
-        saved = Q.new_empty(max(need, 256), dtype=_U8)
+    saved = _scratch("saved", saved, Q, need)
     O = torch.empty_like(Q)
     with _on_device(Q.get_device()):
         rc = load().gproj_fp32_attn_fwd(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), saved.data_ptr(), saved.numel(),
@@ -316,6 +335,7 @@ def gproj_fp32_attn_bwd(Q, K, V, dO, saved, softmax_scale, causal):
     B, H, N, d = Q.shape
     for name, t in (("K", K), ("V", V), ("dO", dO)):
         _check_bf16(name, t, Q.shape)
+    _check_buffer("saved", saved, Q.get_device())
     dQ, dK, dV = torch.empty_like(Q), torch.empty_like(Q), torch.empty_like(Q)
     with _on_device(Q.get_device()):
         rc = load().gproj_fp32_attn_bwd(Q.data_ptr(), K.data_ptr(), V.data_ptr(), dO.data_ptr(), saved.data_ptr(), saved.numel(),
@@ -401,13 +421,19 @@ class VarlenPlan:
         self.device = host.to(device)
 
 
-def gproj_attn_fwd_varlen(Q, K, V, plan, softmax_scale, fwd_flags=0):
-    """O, LSE = forward over packed sequences.  Q: CUDA bfloat16 [H, T, d]; K, V: [Hkv, T, d]; plan: VarlenPlan."""
+def _packed_shapes(Q, K, V, plan):
     _check_bf16("Q", Q)
     H, T, d = Q.shape
     _check_bf16("K", K); _check_bf16("V", V, K.shape)
-    if K.dim() != 3 or K.shape[1] != T or K.shape[2] != d or H % K.shape[0] != 0 or T != plan.total:
+    # the kernels take every extent from the plan
+    if K.dim() != 3 or K.shape[1] != T or K.shape[2] != d or H % K.shape[0] != 0 or T != plan.total or T != plan.total_k:
         raise ValueError("packed K/V must be [Hkv, T, d] with T = cu_seqlens[-1] and H a multiple of Hkv")
+    return H, T, d
+
+
+def gproj_attn_fwd_varlen(Q, K, V, plan, softmax_scale, fwd_flags=0):
+    """O, LSE = forward over packed sequences.  Q: CUDA bfloat16 [H, T, d]; K, V: [Hkv, T, d]; plan: VarlenPlan."""
+    H, T, d = _packed_shapes(Q, K, V, plan)
     O = torch.empty_like(Q)
     LSE = Q.new_empty((H, T), dtype=_F32)
     with _on_device(Q.get_device()):
@@ -421,15 +447,12 @@ def gproj_attn_fwd_varlen(Q, K, V, plan, softmax_scale, fwd_flags=0):
 
 def gproj_attn_bwd_varlen(Q, K, V, O, LSE, dO, plan, softmax_scale, flags=0, workspace=None):
     """dQ, dK, dV = backward over packed sequences (same layout as gproj_attn_fwd_varlen)."""
-    _check_bf16("Q", Q)
-    H, T, d = Q.shape
+    H, T, d = _packed_shapes(Q, K, V, plan)
     for name, t in (("O", O), ("dO", dO)):
         _check_bf16(name, t, Q.shape)
-    _check_bf16("K", K); _check_bf16("V", V, K.shape)
     _check_lse(LSE, (H, T), "H, T")
     need = int(load().gproj_attn_bwd_varlen_workspace_bytes(plan.cu, plan.num_seqs, H, d))
-    if workspace is None:
-        workspace = Q.new_empty(need, dtype=_U8)
+    workspace = _scratch("workspace", workspace, Q, need)
     dQ, dK, dV = torch.empty_like(Q), torch.empty_like(K), torch.empty_like(V)
     with _on_device(Q.get_device()):
         rc = load().gproj_attn_bwd_varlen(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), LSE.data_ptr(), dO.data_ptr(),
@@ -496,8 +519,7 @@ def gproj_attn_bwd_varlen_qk(Q, K, V, O, LSE, dO, plan, softmax_scale, flags=0, 
         _check_bf16(name, t, Q.shape)
     _check_lse(LSE, (H, Tq), "H, Tq")
     need = int(load().gproj_attn_bwd_varlen_workspace_bytes(plan.cu, plan.num_seqs, H, d))
-    if workspace is None:
-        workspace = Q.new_empty(need, dtype=_U8)
+    workspace = _scratch("workspace", workspace, Q, need)
     dQ, dK, dV = torch.empty_like(Q), torch.empty_like(K), torch.empty_like(V)
     with _on_device(Q.get_device()):
         rc = load().gproj_attn_bwd_varlen_qk(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), LSE.data_ptr(), dO.data_ptr(),
