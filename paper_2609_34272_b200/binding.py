@@ -359,6 +359,8 @@ def gproj_key_smooth(X, Y=None, cu_seqlens=None):
         else:
             Hkv, T, d = X.shape
             cu = (ctypes.c_int * len(cu_seqlens))(*[int(v) for v in cu_seqlens])
+            if cu[len(cu) - 1] > T or (cu[len(cu) - 1] != T and Hkv > 1):        # the last offset is the heads' stride
+                raise ValueError(f"cu_seqlens ends at {cu[len(cu) - 1]}, X has {T} rows per head")
             rc = load().gproj_key_smooth_varlen(X.data_ptr(), Y.data_ptr(), cu, len(cu_seqlens) - 1, Hkv, d, _raw_stream(X.get_device()))
     if rc != GPROJ_OK:
         raise GprojError(rc, "gproj_key_smooth")
@@ -476,6 +478,15 @@ def gproj_attn_fwd_bwd_host(Q, K, V, dO, dQ, dK, dV, softmax_scale, causal, stag
             raise TypeError(f"{name} must be a contiguous CPU bfloat16 tensor")
     B, H, N, d = Q.shape
     Hkv = K.shape[1]
+    rows = {"Q": H, "K": Hkv, "V": Hkv, "dO": H, "dQ": H, "dK": Hkv, "dV": Hkv, "O": H}
+    for name, t in (("Q", Q), ("K", K), ("V", V), ("dO", dO), ("dQ", dQ), ("dK", dK), ("dV", dV), ("O", O)):
+        if t is not None and t.numel() < B * rows[name] * N * d:
+            raise ValueError(f"{name} has shape {tuple(t.shape)}, needs {B} x {rows[name]} x {N} x {d} elements")
+    for name, t, dtype in (("O", O, _BF16), ("LSE", LSE, _F32)):
+        if t is not None and not (not t.is_cuda and t.dtype is dtype and t.is_contiguous()):
+            raise TypeError(f"{name} must be a contiguous CPU {dtype} tensor")
+    if LSE is not None and LSE.numel() < B * H * N:
+        raise ValueError(f"LSE has {LSE.numel()} elements, needs {B * H * N}")
     if not (staging.is_cuda and staging.dtype == torch.uint8 and staging.is_contiguous()):
         raise TypeError("staging must be a contiguous CUDA uint8 tensor")
     ptr = lambda t: ctypes.c_void_p(t.data_ptr()) if t is not None else None

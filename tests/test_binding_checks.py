@@ -103,3 +103,26 @@ def test_packed_shapes_are_checked_against_the_plan(calls, plan, kv):
     with pytest.raises(ValueError):
         binding.gproj_attn_bwd_varlen(q, k, k, q, lse, q, plan, 0.1)
     assert calls == []
+
+
+def test_offsets_of_key_smoothing_are_checked(calls):
+    for heads, cu in ((1, [0, 33]), (2, [0, 10, 40]), (2, [0, 31])):
+        with pytest.raises(ValueError):
+            binding.gproj_key_smooth(bf16(heads, 32, D), cu_seqlens=cu)
+    assert calls == []
+    binding.gproj_key_smooth(bf16(1, 32, D), cu_seqlens=[0, 31])                 # one head: the leading rows, as before
+    binding.gproj_key_smooth(bf16(2, 32, D), cu_seqlens=[0, 5, 32])
+    assert len(calls) == 2
+
+
+@pytest.mark.parametrize("name", ["K", "V", "dO", "dQ", "dK", "dV", "O", "LSE"])
+def test_host_tensors_of_the_host_call_are_checked(calls, name):
+    t = {n: host(*(X if n in ("Q", "dO", "dQ", "O") else KV)) for n in ("Q", "K", "V", "dO", "dQ", "dK", "dV", "O")}
+    t["LSE"] = host(*L, dtype=torch.float32)
+    staging = host(1 << 16, **U8).as_subclass(Cuda)
+    run = lambda: binding.gproj_attn_fwd_bwd_host(t["Q"], t["K"], t["V"], t["dO"], t["dQ"], t["dK"], t["dV"], 0.1, True, staging, O=t["O"], LSE=t["LSE"])
+    run()
+    t[name] = t[name][:, :, :31].contiguous()
+    with pytest.raises(ValueError):
+        run()
+    assert len(calls) == 1
