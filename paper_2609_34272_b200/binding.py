@@ -229,9 +229,9 @@ def gproj_attn_bwd(Q, K, V, O, LSE, dO, softmax_scale, causal, flags=0, workspac
     """dQ, dK, dV = attention backward with the GProj correction (flags: FLAG_NO_*_CORRECTION).
     K, V (and dK, dV) may have fewer heads than Q (grouped-query attention)."""
     _check_bf16("Q", Q)
-    shape, kv_shape = Q.shape, K.shape
+    shape = Q.shape
     B, H, N, d = shape
-    _check_bf16("K", K); _check_bf16("V", V, kv_shape); _check_bf16("O", O, shape); _check_bf16("dO", dO, shape)
+    _check_bf16("K", K); _check_bf16("V", V, K.shape); _check_bf16("O", O, shape); _check_bf16("dO", dO, shape)
     Hkv = _kv_heads(shape, K)
     _check_lse(LSE, (B, H, N), "B, H, N")
     lib = _lib or load()

@@ -126,3 +126,13 @@ def test_host_tensors_of_the_host_call_are_checked(calls, name):
     with pytest.raises(ValueError):
         run()
     assert len(calls) == 1
+
+
+def test_a_missing_tensor_is_a_type_error(calls):
+    q, k, lse = bf16(*X), bf16(*KV), f32(*L)
+    for at in range(4):
+        args = [q, k, k, q]
+        args[at] = None
+        with pytest.raises(TypeError):
+            binding.gproj_attn_bwd(*args, lse, q, 0.1, True)
+    assert calls == []
