@@ -15,6 +15,7 @@
 #include "attn_fwd.cuh"
 #include "key_smoothing.cuh"
 #include "attn_fp32.cuh"
+#include "host_rules.h"
 
 namespace {
 
@@ -77,9 +78,9 @@ cudaLaunchAttribute cluster_attr(int size) {
   return a;
 }
 
-// How many clusters of `size` CTAs of `kernel` the device runs at once.
+// How many clusters of `size` CTAs of `kernel` the device runs at once; none where it cannot say.
 template <typename... Params>
-cudaError_t max_clusters(void (*kernel)(Params...), int size, int threads, int smem, int *out) {
+int max_clusters(void (*kernel)(Params...), int size, int threads, int smem) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(size));
   cfg.blockDim = dim3(static_cast<unsigned>(threads));
@@ -87,7 +88,11 @@ cudaError_t max_clusters(void (*kernel)(Params...), int size, int threads, int s
   cudaLaunchAttribute attr = cluster_attr(size);
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  return cudaOccupancyMaxActiveClusters(out, kernel, &cfg);
+  return count_or_none([&](int *n) {
+    const bool ok = cudaOccupancyMaxActiveClusters(n, kernel, &cfg) == cudaSuccess;
+    if (!ok) (void)cudaGetLastError();
+    return ok;
+  });
 }
 
 // One-time, per-device set-up: capability check, status word address, shared-memory opt-in.
@@ -151,15 +156,15 @@ int device_state(DeviceState **out) {
       ok &= allow_smem(attn_fwd_kernel<64, false, false, 3>, FwdCfg<64>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, true, false, 3>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, false, false, 3>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
-      ok = ok && max_clusters(bwd_dq_kernel<64, true, 2>, 2, BwdCfg<64>::kDqThreads, BwdCfg<64>::kDqSmemBytes, &st.dq_clusters[0]) == cudaSuccess;
-      ok = ok && max_clusters(bwd_dq_kernel<128, true, 2>, 2, BwdCfg<128>::kDqThreads, BwdCfg<128>::kDqSmemBytes, &st.dq_clusters[1]) == cudaSuccess;
-      ok = ok && max_clusters(bwd_dkv_w128_kernel<true, 2>, 2, BwdW128::kThreads, BwdW128::kDkvSmemBytes, &st.dkv_clusters[0]) == cudaSuccess;
-      ok = ok && max_clusters(bwd_dkv_kernel<128, true, 2>, 2, BwdCfg<128>::kDkvThreads, BwdCfg<128>::kDkvSmemBytes, &st.dkv_clusters[1]) == cudaSuccess;
-      for (int lg = 1; ok && lg < 4; ++lg) {
-        ok &= max_clusters(attn_fwd_kernel<64, true, false, 3>, 1 << lg, FwdCfg<64>::kThreads, FwdCfg<64>::kSmemBytes, &st.fwd_clusters[0][lg]) == cudaSuccess;
-        ok &= max_clusters(attn_fwd_kernel<128, true, false, 3>, 1 << lg, FwdCfg<128>::kThreads, FwdCfg<128>::kSmemBytes, &st.fwd_clusters[1][lg]) == cudaSuccess;
-      }
       if (!ok) { (void)cudaGetLastError(); return GPROJ_ERR_CUDA; }
+      st.dq_clusters[0] = max_clusters(bwd_dq_kernel<64, true, 2>, 2, BwdCfg<64>::kDqThreads, BwdCfg<64>::kDqSmemBytes);
+      st.dq_clusters[1] = max_clusters(bwd_dq_kernel<128, true, 2>, 2, BwdCfg<128>::kDqThreads, BwdCfg<128>::kDqSmemBytes);
+      st.dkv_clusters[0] = max_clusters(bwd_dkv_w128_kernel<true, 2>, 2, BwdW128::kThreads, BwdW128::kDkvSmemBytes);
+      st.dkv_clusters[1] = max_clusters(bwd_dkv_kernel<128, true, 2>, 2, BwdCfg<128>::kDkvThreads, BwdCfg<128>::kDkvSmemBytes);
+      for (int lg = 1; lg < 4; ++lg) {
+        st.fwd_clusters[0][lg] = max_clusters(attn_fwd_kernel<64, true, false, 3>, 1 << lg, FwdCfg<64>::kThreads, FwdCfg<64>::kSmemBytes);
+        st.fwd_clusters[1][lg] = max_clusters(attn_fwd_kernel<128, true, false, 3>, 1 << lg, FwdCfg<128>::kThreads, FwdCfg<128>::kSmemBytes);
+      }
     }
     st.ready = true;
   }
