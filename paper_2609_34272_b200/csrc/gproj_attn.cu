@@ -428,19 +428,6 @@ bool fwd_prefers_single_tiles(int BH, int n_qt, int sms) {
   return t_single < t_pairs;
 }
 
-// CTAs per query tile of the forward (its base-two logarithm): with few tiles and long key ranges a tile's key range is
-// split over a cluster of 2, 4 or 8 CTAs, as many as leave each of their two warpgroups at least two 128-key tiles and let
-// all clusters run at once (`fit`: how many clusters of 2^lg CTAs do).  Beyond one wave the split only adds its merge, and
-// below 16 key tiles the launch and the merge of a cluster cost what they save.  Measured, one CTA per tile -> cluster: 8 x (16
-// query, 4 KV heads) x 16 queries behind 16384 keys, d = 64: 109.7 -> 45.7 us (with the query heads folded, see
-// launch_fwd), behind 8192: 58.5 -> 27.2, behind 2048: 20.6 -> 13.6; 4 x 8 heads x 1 query behind 16384 keys, d = 128: 201 ->
-// 63 us; 4 heads x 1000 x 128 (8 key tiles, with a merge by scattered stores): 18.7 -> 20.7 us, hence the 16.
-int fwd_cluster_log2(long long tiles, int key_tiles, const int (&fit)[4]) {
-  int lg = 0;
-  while (lg < 3 && key_tiles >= std::max(16, 4 << (lg + 1)) && tiles <= fit[lg + 1]) ++lg;
-  return lg;
-}
-
 // Dense call: plan == nullptr, one sequence [0, N) per head.  Packed call: B = 1, N = total tokens, plan = device tile
 // list (query order) with n_plan_tiles entries, longest_keys = most keys of one sequence.
 int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE, int B, int H, int Hkv, int N, int Nk, int d,
@@ -457,11 +444,10 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
   DeviceState *st = nullptr;
   if (int rc = device_state(&st)) return rc;
 
-  // Grouped queries with fewer rows than a tile, or without a mask: the G query heads of a KV head lie end to end in Q, O and
-  // LSE, so they are one head of G N rows; K and V are then read once per KV head and the tiles are full (16 x (32 query, 8
-  // KV heads) x 1 query behind 1000 keys, d = 64: 56.0 -> 18.6 us).
+  // Grouped queries: the G query heads of a KV head lie end to end in Q, O and LSE, so they may be one head of G N rows; K and
+  // V are then read once per KV head and the tiles are full.  Without a mask always; with one where the rule finds it faster.
   int fold = 0;
-  if (!plan && G > 1 && (!causal || (N < 128 && !fma))) {
+  if (!plan && G > 1 && (!causal || (!fma && fwd_folds_heads(B * Hkv, G, N, Nk, d, st->sm_count, st->fwd_clusters[d == 128])))) {
     if (causal) fold = N;
     H = Hkv;
     N *= G;

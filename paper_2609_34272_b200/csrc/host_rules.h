@@ -13,4 +13,46 @@ int count_or_none(Query query) {
   return query(&n) ? std::max(n, 0) : 0;
 }
 
+// CTAs per query tile of the forward (its base-two logarithm): with few tiles and long key ranges a tile's key range is
+// split over a cluster of 2, 4 or 8 CTAs, as many as leave each of their two warpgroups at least two 128-key tiles and let
+// all clusters run at once (`fit`: how many clusters of 2^lg CTAs do).  Beyond one wave the split only adds its merge, and
+// below 16 key tiles the launch and the merge of a cluster cost what they save.  Measured, one CTA per tile -> cluster: 8 x (16
+// query, 4 KV heads) x 16 queries behind 16384 keys, d = 64: 109.7 -> 45.7 us (with the query heads folded, see
+// fwd_folds_heads), behind 8192: 58.5 -> 27.2, behind 2048: 20.6 -> 13.6; 4 x 8 heads x 1 query behind 16384 keys, d = 128: 201 ->
+// 63 us; 4 heads x 1000 x 128 (8 key tiles, with a merge by scattered stores): 18.7 -> 20.7 us, hence the 16.
+inline int fwd_cluster_log2(long long tiles, int key_tiles, const int (&fit)[4]) {
+  int lg = 0;
+  while (lg < 3 && key_tiles >= std::max(16, 4 << (lg + 1)) && tiles <= fit[lg + 1]) ++lg;
+  return lg;
+}
+
+// Causal forward of grouped queries shorter than a tile: is it faster with the G query heads of a KV head folded into one head
+// of G N rows?  Folded, the kernel runs one tile per CTA (or cluster) and merges its parts through shared memory, which costs
+// more per tile than the persistent form; unfolded, every head is a tile of its own with N of its 128 rows in use.  The two
+// times are estimated in microseconds from what was measured (148 CTAs at once):
+//   folded          per round 6.3 + 6.5 x (share of the tile's rows in use) + 1.55 per key tile at d = 128; 5.9, 2.8, 0.83 at d = 64
+//   unfolded        3 + per round 4.2 + 1.05 per key tile (4.0, 0.72) while the key range of a tile is split between the
+//                   warpgroups; beyond 1.5 tiles per SM, where it is not, 3.5 + 2.0 (2.95, 1.32)
+// Measured, unfolded -> folded, d = 64: 16 x (32 query, 8 KV heads) x 1 query behind 1000 keys: 56.5 -> 12.8 us; 64 x (32, 8) x 64
+// behind 2048: 341 -> 160; 32 x (64, 4) x 64 behind 600: 131 -> 93; but 32 x (64, 4) x 120 behind 600: 139 -> 174; 64 x (16, 4) x 100
+// on as many keys: 32.8 -> 65.4; 2 x (64, 8) x 100 behind 1000: 12.5 -> 16.5.  d = 128: 79.7 -> 18.5, 502 -> 265, 191 -> 138; 199 ->
+// 257, 41.0 -> 88.7, 15.9 -> 23.9.  Over 100 such shapes the choice costs at most 3 % against the better of the two.
+inline bool fwd_folds_heads(int kv_heads, int G, int N, int Nk, int d, int sms, const int (&fit)[4]) {
+  if (N >= 128) return false;
+  const bool wide = d == 128;
+  const int key_tiles = (Nk + 127) / 128;
+  const long long whole = static_cast<long long>(kv_heads) * G, folded = static_cast<long long>(kv_heads) * ((static_cast<long long>(G) * N + 127) / 128);
+  auto rounds = [&](long long tiles) { return static_cast<double>((tiles + sms - 1) / sms); };
+  auto merged = [&](long long tiles, long long rows) {
+    const int lg = fwd_cluster_log2(tiles, key_tiles, fit);
+    const double used = static_cast<double>(std::min<long long>(128, rows)) / 128;
+    return (lg > 0 ? 1.0 : rounds(tiles)) * ((wide ? 6.3 + 6.5 * used : 5.9 + 2.8 * used) + (wide ? 1.55 : 0.83) * ((key_tiles + (1 << lg) - 1) >> lg));
+  };
+  double t_whole;
+  if (fwd_cluster_log2(whole, key_tiles, fit) > 0) t_whole = merged(whole, N);
+  else if (2 * whole < 3LL * sms) t_whole = 3.0 + rounds(whole) * (wide ? 4.2 + 1.05 * key_tiles : 4.0 + 0.72 * key_tiles);
+  else t_whole = 3.0 + rounds(whole) * (wide ? 3.5 + 2.0 * key_tiles : 2.95 + 1.32 * key_tiles);
+  return merged(folded, static_cast<long long>(G) * N) < t_whole;
+}
+
 }  // namespace gproj

@@ -17,11 +17,13 @@ def tobits(t):
 
 
 # The forward splits a query tile's key range over 2, 4 or 8 CTAs from 16, 16 and 32 key tiles on, when the tiles are few;
-# grouped queries of fewer than 128 rows (or without a mask) are folded into one head first.
+# grouped queries without a mask are folded into one head first, with one those of the second half of the list.
 FWD = [  # B, H, Hkv, Nq, Nk, causal
     (1, 2, 2, 128, 1921, True), (1, 2, 2, 130, 2048, False), (13, 3, 3, 1, 2047, True), (1, 2, 2, 257, 4100, True),
     (1, 1, 1, 64, 5000, False), (1, 8, 2, 16, 4096, True), (9, 6, 2, 127, 2500, True), (1, 4, 1, 33, 300, True),
     (1, 4, 2, 100, 40, True), (1, 6, 2, 200, 2100, False), (1, 8, 1, 1, 1, True), (3, 4, 1, 96, 2049, True),
+    (40, 8, 2, 1, 300, True), (50, 8, 2, 20, 130, True), (70, 8, 1, 33, 300, True), (3, 64, 8, 5, 2300, True), (20, 12, 3, 60, 2100, True),
+    (8, 16, 4, 16, 8192, True), (60, 8, 1, 3, 2, True),
 ]
 
 
@@ -49,7 +51,7 @@ def test_forward_with_the_key_range_split_over_a_cluster(shape, d):
 
 # query heads folded on one CTA per tile; clusters with and without folding; the last without either, for comparison
 @pytest.mark.parametrize("d", [64, 128])
-@pytest.mark.parametrize("shape", [(1, 8, 1, 4, 40, True), (2, 8, 2, 16, 4096, True), (1, 2, 2, 128, 4100, False), (1, 2, 2, 600, 600, True)])
+@pytest.mark.parametrize("shape", [(50, 8, 2, 20, 130, True), (8, 16, 4, 16, 8192, True), (1, 2, 2, 128, 4100, False), (1, 2, 2, 600, 600, True)])
 def test_a_nan_reaches_every_output_row_that_sees_it(shape, d):
     B, H, Hkv, Nq, Nk, causal = shape
     gen = torch.Generator().manual_seed(Nq + Nk + d)

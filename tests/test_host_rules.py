@@ -12,6 +12,7 @@ HARNESS = r"""
 using namespace gproj;
 extern "C" {
 int count(int ok, int n) { return count_or_none([&](int *out) { *out = n; return ok != 0; }); }
+int folds(int kv_heads, int G, int N, int Nk, int d) { const int fit[4] = {0, 74, 36, 16}; return fwd_folds_heads(kv_heads, G, N, Nk, d, 148, fit); }
 }
 """
 
@@ -30,3 +31,17 @@ def test_a_failed_cluster_query_means_no_clusters(rules):
     # ... and does not fail the set-up of a device, which calls without clusters need as well
     text = open(os.path.join(CSRC, "gproj_attn.cu")).read()
     assert "count_or_none" in text and not re.search(r"ok[^;]*=[^;]*max_clusters\(", text)
+
+
+# batch x KV heads, group, queries, keys, and which form measured faster by 5 % or more at both head dimensions (folded, else whole)
+FOLD = [(256, 4, 100, 100, 0), (64, 4, 100, 100, 0), (32, 4, 100, 100, 0), (256, 4, 64, 64, 0), (256, 4, 32, 32, 1), (2048, 4, 1, 1000, 1),
+        (512, 4, 16, 2048, 1), (512, 4, 64, 2048, 1), (128, 16, 120, 600, 0), (128, 16, 64, 600, 1), (128, 2, 64, 600, 1), (512, 2, 100, 256, 0),
+        (512, 2, 16, 256, 1), (8, 8, 100, 1000, 0), (16, 8, 100, 1000, 0), (1024, 8, 1, 64, 1), (128, 4, 1, 1000, 1), (64, 4, 1, 1900, 1),
+        (64, 2, 64, 300, 0), (64, 2, 100, 1900, 0), (400, 2, 64, 300, 1), (60, 2, 90, 2000, 0), (32, 8, 127, 1000, 0)]
+
+
+@pytest.mark.parametrize("kv_heads,G,N,Nk,folded", FOLD)
+def test_query_heads_are_folded_where_that_is_faster(rules, kv_heads, G, N, Nk, folded):
+    for d in (64, 128):
+        assert rules.folds(kv_heads, G, N, Nk, d) == folded
+    assert rules.folds(kv_heads, G, 128, Nk, 64) == 0
