@@ -1163,7 +1163,9 @@ static int smooth_rows(const void *X, void *Y, int heads, long long rows_total, 
       ++q;
     }
     if (m == 0) continue;
-    const int cluster = static_cast<long long>(m) * heads * 8 <= st->sm_count * 3LL ? 8 : 4;   // eight while all CTAs run at once
+    int longest = 0;
+    for (int i = 0; i < m; ++i) longest = std::max(longest, off.cu[i + 1] - off.cu[i]);
+    const int cluster = smooth_cluster(static_cast<long long>(m) * heads, static_cast<long long>(off.cu[m] - off.cu[0]) * heads, longest, d, st->sm_count);
     for (int h0 = 0; h0 < heads; h0 += 65535) {       // heads along y, whose limit is 65535
       const dim3 grid(static_cast<unsigned>(m * cluster), static_cast<unsigned>(std::min(heads - h0, 65535)));
       const long long at = static_cast<long long>(h0) * rows_total * d;

@@ -55,4 +55,26 @@ inline bool fwd_folds_heads(int kv_heads, int G, int N, int Nk, int d, int sms, 
   return merged(folded, static_cast<long long>(G) * N) < t_whole;
 }
 
+// CTAs per (head, sequence) of key smoothing: 1, 2, 4 or 8.  pairs: (head, sequence) pairs of the launch; rows: their rows
+// together; longest: rows of the longest one.  A pair is split further
+//   - while all CTAs still run at once (three per SM: the fourth is there for uneven sequences), or
+//   - while what the running pairs read is more than L2 holds until the second pass, or while a CTA of the longest sequence has
+//     more than 1024 rows, which it alone would be busy with at the end;
+// but not below 32 KB of a CTA's rows, nor beyond four unless few long sequences are all there is.
+// Measured, CTAs per pair 8, 4, 2, 1 [taken], d = 64: 64 x 32 heads x 200: 249, 78, 37, [21] us; x 1000: 265, 118, [98], 113; x 2048: 308,
+// [201], 231, 244; 4 x 32 x 4096: 39, [30], 32, 44; 16 x 4096: 9.5, [8.7], 13, 21; 4 x 8000: [9.1], 12.8, 22, 38.  d = 128: 64 x 32 x 512: 437, 135, [101],
+// 116; 16 x 16 x 1000: 72, 35, 28, [30]; 24 documents, 19446 rows, 4 heads: 31, [19], 24, 30.
+constexpr int kSmoothCtasPerSm = 4;
+inline int smooth_cluster(long long pairs, long long rows, int longest, int d, int sms) {
+  const int least = 32 * 1024 / (2 * d);               // rows of a CTA
+  const double bytes = 2.0 * d * static_cast<double>(rows);
+  int c = 1;
+  while (c < 4 && longest >= 2 * c * least) {
+    const double running = std::min(1.0, static_cast<double>(kSmoothCtasPerSm) * sms / c / static_cast<double>(pairs));
+    if (pairs * 2 * c > 3LL * sms && running * bytes <= 70e6 && longest <= 1024 * c) break;
+    c *= 2;
+  }
+  return c == 4 && longest > 4096 && pairs * 8 <= 3LL * sms ? 8 : c;
+}
+
 }  // namespace gproj

@@ -7,30 +7,32 @@
 //                        the vector-Jacobian product of the subtraction (in exact arithmetic sum_j dK~_j = 0,
 //                        Proposition 3.1, so the second call removes only what rounding leaked into that sum).
 //
-// One cluster of four CTAs (eight where the call has few sequences and heads) per (head, sequence), all sequences of a call in
-// one launch (the offsets travel as a kernel parameter).  A CTA takes its share of the rows, keeps as many of them in
-// registers as fit (256 rows at d = 64, so that sequences up to 1024 rows are read once; what is beyond is read a second
-// time, from L2), and the column sums are exchanged through distributed shared memory.  Sums are FP32 in a fixed order, so
-// results are reproducible.  What a call takes is the latency of one CTA (load, two exchanges, store) times the waves of
-// CTAs.  Measured, 16 documents, 8192 rows, 4 heads, d = 64: 92.6 us a call with one CTA per (head, sequence) and a launch per
-// sequence, 17.2 us with clusters of eight, 10.0 us with clusters of four; 24 documents, 16384 rows: 157.7, 20.5, 10.3 us.
+// One CTA, or a cluster of 2, 4 or 8 (smooth_cluster in host_rules.h), per (head, sequence); all sequences of a call in one launch
+// (the offsets travel as a kernel parameter).  A CTA reads its share of the rows twice, the second time from L2, with eight
+// 16-byte loads per thread in flight, and the column sums of a cluster are exchanged through distributed shared memory.  Sums
+// are FP32 in a fixed order, so results are reproducible.  Small calls are bound by the latency of one CTA (load, two
+// exchanges, store), large ones by memory.  Keeping eight rows per thread in registers between the two passes instead needs
+// 80 registers, with three CTAs on an SM instead of four, and loads the rows beyond them two at a time: measured, that -> this, in
+// clusters of the same size, 64 x 32 heads x 1000 x 64: 149 -> 113 us; 4 x 32 x 4096 x 128: 122 -> 69; 24 documents, 19446 rows, 4 heads, d = 64:
+// 12.8 -> 11.3; 8 heads x 300: the same.
 #pragma once
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include "host_rules.h"
 #include "sm100_primitives.cuh"
 
 namespace gproj {
 
-constexpr int kSmoothThreads = 256, kSmoothMaxSeqs = 512;
+constexpr int kSmoothThreads = 256, kSmoothMaxSeqs = 512;   // at most kSmoothCtasPerSm CTAs run on an SM (host_rules.h)
 struct SmoothOffsets { int cu[kSmoothMaxSeqs + 1]; };
 
 // X, Y: [heads][rows_total][d] BF16; sequence blockIdx.x / (cluster size) of head blockIdx.y.
 template <int D>
-__global__ void __launch_bounds__(kSmoothThreads, 3)
+__global__ void __launch_bounds__(kSmoothThreads, kSmoothCtasPerSm)
 smooth_rows_kernel(const __nv_bfloat16 *__restrict__ X, __nv_bfloat16 *__restrict__ Y, long long head_stride, const __grid_constant__ SmoothOffsets off) {
   constexpr int kLanes = D / 8;                       // threads across a row (8 BF16 = 16 bytes each)
-  constexpr int kRowsPerPass = kSmoothThreads / kLanes, kWarps = kSmoothThreads / 32, kKeep = 8;
+  constexpr int kRowsPerPass = kSmoothThreads / kLanes, kWarps = kSmoothThreads / 32, kBatch = 8;
   __shared__ float part[kWarps][D];
   __shared__ __align__(16) float cta_sum[D];
   griddep_wait();
@@ -50,16 +52,19 @@ smooth_rows_kernel(const __nv_bfloat16 *__restrict__ X, __nv_bfloat16 *__restric
 #pragma unroll
     for (int i = 0; i < 4; ++i) { acc[2 * i] += bf16_lo_to_f32(w[i]); acc[2 * i + 1] += bf16_hi_to_f32(w[i]); }
   };
-  uint4 keep[kKeep];
+  uint4 batch[kBatch];
+  auto fetch = [&](int r0) {
 #pragma unroll
-  for (int k = 0; k < kKeep; ++k) {
-    const int r = r_begin + rsub + k * kRowsPerPass;
-    keep[k] = r < r_end ? *reinterpret_cast<const uint4 *>(x + static_cast<long long>(r) * D) : make_uint4(0u, 0u, 0u, 0u);
+    for (int k = 0; k < kBatch; ++k) {
+      const int r = r0 + k * kRowsPerPass;
+      batch[k] = r < r_end ? *reinterpret_cast<const uint4 *>(x + static_cast<long long>(r) * D) : make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  for (int r = r_begin + rsub; r < r_end; r += kBatch * kRowsPerPass) {
+    fetch(r);
+#pragma unroll
+    for (int k = 0; k < kBatch; ++k) add(batch[k]);
   }
-#pragma unroll
-  for (int k = 0; k < kKeep; ++k) add(keep[k]);
-#pragma unroll 2
-  for (int r = r_begin + rsub + kKeep * kRowsPerPass; r < r_end; r += kRowsPerPass) add(*reinterpret_cast<const uint4 *>(x + static_cast<long long>(r) * D));
   // column sums: over the rows of a warp, over the warps, over the cluster
 #pragma unroll
   for (int o = kLanes; o < 32; o <<= 1)
@@ -97,13 +102,14 @@ smooth_rows_kernel(const __nv_bfloat16 *__restrict__ X, __nv_bfloat16 *__restric
     for (int i = 0; i < 4; ++i) o[i] = pack_bf16x2(__fsub_rn(bf16_lo_to_f32(w[i]), m[2 * i]), __fsub_rn(bf16_hi_to_f32(w[i]), m[2 * i + 1]));
     *reinterpret_cast<uint4 *>(y + static_cast<long long>(r) * D) = make_uint4(o[0], o[1], o[2], o[3]);
   };
+  for (int r0 = r_begin + rsub; r0 < r_end; r0 += kBatch * kRowsPerPass) {
+    fetch(r0);
 #pragma unroll
-  for (int k = 0; k < kKeep; ++k) {
-    const int r = r_begin + rsub + k * kRowsPerPass;
-    if (r < r_end) put(r, keep[k]);
+    for (int k = 0; k < kBatch; ++k) {
+      const int r = r0 + k * kRowsPerPass;
+      if (r < r_end) put(r, batch[k]);
+    }
   }
-#pragma unroll 2
-  for (int r = r_begin + rsub + kKeep * kRowsPerPass; r < r_end; r += kRowsPerPass) put(r, *reinterpret_cast<const uint4 *>(x + static_cast<long long>(r) * D));
   cluster_sync();                                     // no CTA leaves while another one may still read its sums
 }
 

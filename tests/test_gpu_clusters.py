@@ -101,9 +101,9 @@ def test_packed_forward_with_split_keys_repeats_bitwise(causal):
             assert oracle.rel_l2_percent(O[:, a:b].float().cpu().numpy()[None], ex["O"]) <= 1.0
 
 
-@pytest.mark.parametrize("rows,d", [(1, 64), (7, 128), (8, 64), (513, 64), (4095, 64), (4097, 64), (2049, 128), (9000, 64)])
+@pytest.mark.parametrize("rows,d", [(1, 64), (7, 128), (8, 64), (255, 64), (257, 64), (129, 128), (513, 64), (2047, 64), (4097, 64), (2049, 128), (9000, 64)])
 def test_key_smoothing_at_the_edges_of_its_row_split(rows, d):
-    # one row, fewer rows than CTAs, the last row kept in registers, the first rows read twice.  FP32 sums of n values in
+    # one row, fewer rows than a pass, the edges of a batch of eight passes, one to eight CTAs.  FP32 sums of n values in
     # any order lie within n 2^-24 of each other relative to the sum of magnitudes; one BF16 step of the output covers it.
     gen = torch.Generator().manual_seed(rows + d)
     X = (torch.randn(3, rows, d, generator=gen) + 4.0 * torch.randn(3, 1, d, generator=gen)).to(torch.bfloat16)

@@ -13,6 +13,7 @@ using namespace gproj;
 extern "C" {
 int count(int ok, int n) { return count_or_none([&](int *out) { *out = n; return ok != 0; }); }
 int folds(int kv_heads, int G, int N, int Nk, int d) { const int fit[4] = {0, 74, 36, 16}; return fwd_folds_heads(kv_heads, G, N, Nk, d, 148, fit); }
+int smooth(long long pairs, long long rows, int longest, int d) { return smooth_cluster(pairs, rows, longest, d, 148); }
 }
 """
 
@@ -45,3 +46,17 @@ def test_query_heads_are_folded_where_that_is_faster(rules, kv_heads, G, N, Nk, 
     for d in (64, 128):
         assert rules.folds(kv_heads, G, N, Nk, d) == folded
     assert rules.folds(kv_heads, G, 128, Nk, 64) == 0
+
+
+# pairs, rows of each (dense), head dimension, CTAs per pair that measured fastest or within 10 % of it
+SMOOTH = [(2048, 200, 64, 1), (2048, 20, 64, 1), (2048, 1000, 64, 2), (2048, 2048, 64, 4), (512, 512, 64, 1), (256, 200, 64, 1), (256, 4000, 64, 4),
+          (100, 300, 64, 1), (100, 3000, 64, 4), (128, 4096, 64, 4), (16, 4096, 64, 4), (4, 8000, 64, 8), (1, 32768, 64, 8), (16, 32768, 64, 8),
+          (2048, 200, 128, 1), (2048, 512, 128, 2), (2048, 1000, 128, 4), (2048, 2048, 128, 4), (512, 512, 128, 1), (128, 1000, 128, 2),
+          (128, 4096, 128, 4), (64, 3000, 128, 4), (4, 8000, 128, 8), (1000, 100, 128, 1)]
+
+
+@pytest.mark.parametrize("pairs,N,d,ctas", SMOOTH)
+def test_key_smoothing_splits_a_sequence_where_that_is_faster(rules, pairs, N, d, ctas):
+    f = rules.smooth
+    f.argtypes = [ctypes.c_longlong, ctypes.c_longlong, ctypes.c_int, ctypes.c_int]
+    assert f(pairs, pairs * N, N, d) == ctas
