@@ -15,6 +15,7 @@
 //   split (2)     one item = one query tile; warpgroup t takes the key tiles j = t (mod 2) with its own running
 //                 maximum, normaliser and accumulator, and warpgroup 0 merges the two halves at the end.  Used when
 //                 pairs would leave SMs idle and for packed sequences.
+//   split (4)     the same with separate rings for K and V (d = 128, long key ranges).
 //   cluster (3)   one item = one query tile on a cluster of 2, 4 or 8 CTAs that share its key tiles in the same way and
 //                 merge 4, 8 or 16 parts through distributed shared memory.  Used when even single tiles leave SMs
 //                 idle: a block of new queries behind a key history, a short batch.
@@ -90,7 +91,8 @@ __device__ __forceinline__ float softmax_exp_store(const uint32_t (&xr)[4][32], 
 
 // MODE: 0 = pairs of query tiles, 1 = pairs whose warpgroups take turns in the exponential phase, 2 = single tiles with
 // the key range split between the warpgroups, 3 = single tiles with the key range split over the warpgroups of a cluster of
-// CTAs (one tile per cluster; the parts of all CTAs are merged through distributed shared memory).
+// CTAs (one tile per cluster; the parts of all CTAs are merged through distributed shared memory), 4 = as 2, with separate rings
+// for K and V.
 template <int D, bool CAUSAL, bool FMA_SOFTMAX, int MODE>
 __global__ void __launch_bounds__(384, 1)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
@@ -102,12 +104,13 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   using C = FwdCfg<D>;
   constexpr int S = C::kStages;
   constexpr bool kCluster = (MODE == 3);
-  // Separate K and V rings where the ring is short (two stages at d = 128) and both stages are in use at once (the
-  // warpgroups work on two key tiles): with one ring the next K waited for the whole softmax and P~V of its stage.
-  // Measured, one ring -> two: 8 heads x 4096 x 128, causal: 51.6 -> 44.0 us; 12 packed pairs (4000 queries, 9000 keys, 12
-  // heads): 62.2 -> 51.5 us.  Elsewhere the second commit per key tile and the polling cost more than they give (16 heads
-  // x 4096 x 64: 60.5 -> 62.5 us; pairs at d = 128: 306 us either way; clusters at d = 64: 33.0 -> 38 us).
-  constexpr bool kSepRings = (D == 128 && MODE == 2);
+  // Separate K and V rings: with one ring the next K waits for the whole softmax and P~V of its stage, which is what a ring of
+  // two stages (d = 128) is bound by while the warpgroups work on two key tiles.  Measured, one ring -> two: 8 heads x 4096 x 128, causal:
+  // 49.1 -> 41.4 us; 12 packed pairs (4000 queries, 9000 keys, 12 heads): 62.2 -> 51.5.  With few key tiles to an item (fwd_separate_rings
+  // in host_rules.h), with more stages or where both stages hold one tile's work, the second commit per key tile and the
+  // thread that polls both rings cost more than they give (200 packed documents of 30 to 300 rows, 16 heads, d = 128: 230 -> 270 us;
+  // 16 heads x 4096 x 64: 60.5 -> 62.5; pairs at d = 128: 306 either way; clusters at d = 64: 33.0 -> 38).
+  constexpr bool kSepRings = (MODE == 4);
   const int fold = kCluster ? fold_rows : 0;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));

@@ -136,6 +136,10 @@ int device_state(DeviceState **out) {
       ok &= allow_smem(attn_fwd_kernel<128, false, false, 2>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, false, true, 0>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, false, true, 2>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
+      ok &= allow_smem(attn_fwd_kernel<128, true, false, 4>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
+      ok &= allow_smem(attn_fwd_kernel<128, true, true, 4>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
+      ok &= allow_smem(attn_fwd_kernel<128, false, false, 4>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
+      ok &= allow_smem(attn_fwd_kernel<128, false, true, 4>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(bwd_dkv_w128_kernel<true, 1>, BwdW128::kDkvSmemBytes) == cudaSuccess;
       ok &= allow_smem(bwd_dkv_w128_kernel<false, 1>, BwdW128::kDkvSmemBytes) == cudaSuccess;
       ok &= allow_smem(bwd_dkv_w128_kernel<true, 2>, BwdW128::kDkvSmemBytes) == cudaSuccess;
@@ -316,6 +320,13 @@ std::vector<int> packed_work(const PackedSeqs &ps, bool key_side) {
   }
   std::sort(work.begin(), work.end(), [](int a, int b) { return a > b; });
   return work;
+}
+
+// Key tiles that a head's query tiles walk over all sequences.
+long long walked_key_tiles(const PackedSeqs &ps) {
+  long long sum = 0;
+  for (int s = 0; s < ps.num; ++s) sum += fwd_key_tiles(ps.cu_q[s + 1] - ps.cu_q[s], ps.cu_k[s + 1] - ps.cu_k[s], ps.causal);
+  return sum;
 }
 
 int longest_keys(const PackedSeqs &ps) {
@@ -502,6 +513,7 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
   // they alternate in the exponential phase (measured to pay there only).
   const bool split = (tiles_per_item == 1), turns = (d == 128) && !split && !fma;
   if (d == 64) { if (split) GPROJ_LAUNCH_FWD_F(64, 2); else GPROJ_LAUNCH_FWD_F(64, 0); }
+  else if (split && fwd_separate_rings(total_items, st->sm_count, seqs ? walked_key_tiles(*seqs) : fwd_key_tiles(N, Nk, causal != 0), n_qt)) GPROJ_LAUNCH_FWD_F(128, 4);
   else if (split) GPROJ_LAUNCH_FWD_F(128, 2);
   else if (turns) GPROJ_LAUNCH_FWD_C(128, false, 1);
   else GPROJ_LAUNCH_FWD_F(128, 0);

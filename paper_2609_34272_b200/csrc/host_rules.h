@@ -13,6 +13,23 @@ int count_or_none(Query query) {
   return query(&n) ? std::max(n, 0) : 0;
 }
 
+// Key tiles that the query tiles of one sequence walk: all of them, or those up to the diagonal that ends at the last query and
+// key; one where a tile sees no key.
+inline long long fwd_key_tiles(int lq, int lk, bool causal) {
+  const long long tq = (lq + 127LL) / 128, tk = std::max<long long>(1, (lk + 127LL) / 128);
+  if (!causal || tq == 0) return tq * tk;
+  const long long off = static_cast<long long>(lk) - lq, e = off >= 0 ? (off + 127) / 128 : -(-off / 128);   // off / 128, rounded up
+  const long long ones = std::max<long long>(0, std::min(tq, -e));      // tiles before the diagonal reaches key 0, beside the next
+  const long long n = tq - ones;                                        // the others: ones + 1 + e, ones + 2 + e, ... tq + e
+  return ones + n * (ones + 1 + e + tq + e) / 2 - (n > 0 ? std::max<long long>(0, tq + e - tk) : 0);
+}
+
+// Forward at d = 128 with the key range of a tile split between the warpgroups: separate rings for K and V (see attn_fwd.cuh)?
+// With one item per CTA, or from three key tiles per item on.  items: over all heads; key_tiles, tiles: of one head.  Measured, one
+// ring -> two, 16 query / 4 KV heads, 40000 rows in sequences of one length, causal: 512 rows (2.5 key tiles per item) 228 -> 239 us, 640
+// (3.0) 256 -> 256, 1024 (4.5) 332 -> 312; not causal: 256 (2) 177 -> 190, 384 (3) 240 -> 234; 16 heads x 500 (64 items): 11.0 -> 10.4.
+inline bool fwd_separate_rings(long long items, int sms, long long key_tiles, long long tiles) { return items <= sms || key_tiles >= 3 * tiles; }
+
 // CTAs per query tile of the forward (its base-two logarithm): with few tiles and long key ranges a tile's key range is
 // split over a cluster of 2, 4 or 8 CTAs, as many as leave each of their two warpgroups at least two 128-key tiles and let
 // all clusters run at once (`fit`: how many clusters of 2^lg CTAs do).  Beyond one wave the split only adds its merge, and

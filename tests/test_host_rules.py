@@ -14,6 +14,8 @@ extern "C" {
 int count(int ok, int n) { return count_or_none([&](int *out) { *out = n; return ok != 0; }); }
 int folds(int kv_heads, int G, int N, int Nk, int d) { const int fit[4] = {0, 74, 36, 16}; return fwd_folds_heads(kv_heads, G, N, Nk, d, 148, fit); }
 int smooth(long long pairs, long long rows, int longest, int d) { return smooth_cluster(pairs, rows, longest, d, 148); }
+long long key_tiles(int lq, int lk, int causal) { return fwd_key_tiles(lq, lk, causal != 0); }
+int rings(long long items, long long key_tiles, long long tiles) { return fwd_separate_rings(items, 148, key_tiles, tiles); }
 }
 """
 
@@ -60,3 +62,26 @@ def test_key_smoothing_splits_a_sequence_where_that_is_faster(rules, pairs, N, d
     f = rules.smooth
     f.argtypes = [ctypes.c_longlong, ctypes.c_longlong, ctypes.c_int, ctypes.c_int]
     assert f(pairs, pairs * N, N, d) == ctas
+
+
+def walked(lq, lk, causal):
+    """Key tiles of every query tile, as the forward's decode_rank counts them."""
+    off = lk - lq
+    return sum(max(1, -(-max(min(lk, r + 128 + off) if causal else lk, 0) // 128)) for r in range(0, lq, 128))
+
+
+def test_key_tiles_of_a_sequence(rules):
+    f = rules.key_tiles
+    f.restype = ctypes.c_longlong
+    for causal in (0, 1):
+        for lq in (0, 1, 127, 128, 129, 256, 300, 1000, 1024):
+            for lk in (0, 1, 100, 128, 129, 255, 256, 257, 640, 1000, 1024, 3000):
+                # the closed form takes the tile in which the diagonal passes key 0 and the last, ragged one as whole tiles
+                assert abs(f(lq, lk, causal) - walked(lq, lk, causal)) <= (1 if causal and lq > 0 else 0), (lq, lk, causal)
+
+
+@pytest.mark.parametrize("rows,causal,two", [(128, 1, 0), (200, 0, 0), (256, 1, 0), (256, 0, 0), (512, 1, 0), (384, 0, 1), (640, 1, 1), (1500, 1, 1), (4096, 1, 1)])
+def test_separate_rings_from_three_key_tiles_on(rules, rows, causal, two):
+    key_tiles, tiles = ctypes.c_longlong(walked(rows, rows, causal)), ctypes.c_longlong(-(-rows // 128))
+    assert rules.rings(ctypes.c_longlong(149), key_tiles, tiles) == two
+    assert rules.rings(ctypes.c_longlong(148), key_tiles, tiles) == 1
