@@ -5,7 +5,6 @@ memory and the stream.  There is no CPU fallback: if the library is missing or t
 device is not sm_100a the calls raise.
 """
 import ctypes
-import math
 import os
 
 import torch
@@ -177,7 +176,7 @@ def _check_lse(LSE, shape, what):
 
 def _check_buffer(name, t, index, dtype=None, count=0):
     """A caller's buffer that the kernels write: on the call's device, contiguous, and with room for `count` elements."""
-    if not (isinstance(t, torch.Tensor) and t.is_cuda and t.get_device() == index and t.is_contiguous() and (dtype is None or t.dtype is dtype)):
+    if not (isinstance(t, torch.Tensor) and t.get_device() == index and t.is_contiguous() and (dtype is None or t.dtype is dtype)):
         raise TypeError(f"{name} must be a contiguous {dtype or ''} tensor on the inputs' CUDA device")
     if t.numel() < count:
         raise ValueError(f"{name} has {t.numel()} elements, needs {count}")
@@ -187,7 +186,7 @@ def _lse_out(LSE, Q, shape):
     """The caller's LSE output, checked, or a new one."""
     if LSE is None:
         return Q.new_empty(shape, dtype=_F32)
-    _check_buffer("LSE", LSE, Q.get_device(), _F32, math.prod(shape))
+    _check_buffer("LSE", LSE, Q.get_device(), _F32, shape[0] * shape[1] * shape[2])
     return LSE
 
 
