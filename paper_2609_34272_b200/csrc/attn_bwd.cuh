@@ -366,7 +366,13 @@ __device__ __forceinline__ void saved_output_dots(const __nv_bfloat16 *O, const 
 // CL = 2: a cluster of two CTAs shares every tile: CTA r takes the key steps r, r + 2, ...; the row masses are exchanged, and CTA
 // r gets both parts of A and B for its half of the columns (over the consumed Q / dO buffer), of which it writes dQ and Z.
 // Used where whole tiles cannot be dealt evenly.
-template <int D, bool CAUSAL, int CL>
+// SHORT: the compute warpgroups prepare the row constants of every tile, not of their first one only.  At d = 128 the extra
+// warpgroup needs 4 us for those of one tile and 5 us for the epilogue of another, one after the other, and a tile of few steps is
+// through the step loop sooner; the compute warps meanwhile wait for its Q and dO, which have a single buffer.  Measured, d = 128,
+// off -> on (in brackets the kernel in which 512 threads did both): 64 x 16 heads x 128, causal: 80.3 -> 59.1 us (63.6); 64 x 16 x 500,
+// causal: 371 -> 293 (302); 200 packed documents of 30 to 300 rows, 16 heads: 484 -> 302 (351); 8000 of 20 rows, 2 heads: 887 -> 628
+// (535); but 16 x 16 x 700, not causal (11 steps a tile): 167 -> 182 (207).
+template <int D, bool CAUSAL, int CL, bool SHORT>
 __global__ void __launch_bounds__(BwdCfg<D>::kDqThreads, 1)
 bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
               const __grid_constant__ CUtensorMap tmdO,   // box 64 x 128 rows
@@ -581,19 +587,22 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
 #ifdef GPROJ_TRACE
       const unsigned long long ev_n0 = global_ns(); const long long ev_c0 = clock64(); unsigned long long ev_n1 = 0, ev_n2 = 0;
 #endif
-      if (ti == 0) {
-        // The first tile's constants come from these warps, which have nothing else to do yet.
+      if (SHORT || ti == 0) {
+        // The first tile's constants come from these warps, which have nothing else to do yet, and so do a short one's.  They
+        // overwrite those of tile ti - 2, whose readers have all handed in their row masses.
+        if (SHORT && ti >= 2) mbar_wait(&bar_mass_ready[par], ((ti >> 1) - 1) & 1, ab, kDqWaitMass, kTileBudget);
         constexpr int kRows = 128 / (4 * C::kWG);
+        const int cp = SHORT ? par : 0;
         const size_t row0 = static_cast<size_t>(hix(lin)) * N + tl.row0;
         const float lse_row = (qrow < tl.seq_end) ? LSE[row0 + row] : 0.f;
-        saved_output_dots<D, kRows>(Og + row0 * D, dOg + row0 * D, kRows * (warp - 4), tl.seq_end - tl.row0, s_D[0]);
+        saved_output_dots<D, kRows>(Og + row0 * D, dOg + row0 * D, kRows * (warp - 4), tl.seq_end - tl.row0, s_D[cp]);
         named_bar_sync(1, C::kCompute);
         if (wg == 0) {
-          s_lse[0][row] = lse_row;
+          s_lse[cp][row] = lse_row;
           const int rel = qrow - tl.seq0;
           if (rank == 0 && rel < ((tl.seq_end - tl.seq0 + 63) / 64) * 64)
-            write_row_constants(stats, static_cast<size_t>(hix(lin)) * nblk + tl.blk0 + (rel >> 6), rel & 63, -lse_row * 1.4426950408889634f, s_D[0][row], scale_log2);
-          mbar_arrive(&bar_stats_ready[0]);
+            write_row_constants(stats, static_cast<size_t>(hix(lin)) * nblk + tl.blk0 + (rel >> 6), rel & 63, -lse_row * 1.4426950408889634f, s_D[cp][row], scale_log2);
+          mbar_arrive(&bar_stats_ready[cp]);
         }
       }
       mbar_wait(&bar_stats_ready[par], (ti >> 1) & 1, ab, kDqWaitStats);
@@ -663,7 +672,7 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 rows
     while (lin >= 0) {
       const int next = sched.next(), par = ti & 1;
       // The constants of tile ti + 1 overwrite those of tile ti - 1, whose readers have all handed in their row masses.
-      if (next >= 0) row_constants(next, par ^ 1);
+      if (!SHORT && next >= 0) row_constants(next, par ^ 1);
       const TileInfo tl = tile_of(lin);
       // q of this warp's 32 rows, D / 8 lanes to a row (whole lines per load and store; one row per thread touches 32
       // lines with every instruction and took 2.2 us instead of 1 us of the tail at d = 128), the first kQ loads ahead of

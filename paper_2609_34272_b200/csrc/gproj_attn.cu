@@ -144,14 +144,16 @@ int device_state(DeviceState **out) {
       ok &= allow_smem(bwd_dkv_w128_kernel<false, 1>, BwdW128::kDkvSmemBytes) == cudaSuccess;
       ok &= allow_smem(bwd_dkv_w128_kernel<true, 2>, BwdW128::kDkvSmemBytes) == cudaSuccess;
       ok &= allow_smem(bwd_dkv_w128_kernel<false, 2>, BwdW128::kDkvSmemBytes) == cudaSuccess;
-      ok &= allow_smem(bwd_dq_kernel<64, true, 1>, BwdCfg<64>::kDqSmemBytes) == cudaSuccess;
-      ok &= allow_smem(bwd_dq_kernel<64, true, 2>, BwdCfg<64>::kDqSmemBytes) == cudaSuccess;
-      ok &= allow_smem(bwd_dq_kernel<64, false, 1>, BwdCfg<64>::kDqSmemBytes) == cudaSuccess;
-      ok &= allow_smem(bwd_dq_kernel<64, false, 2>, BwdCfg<64>::kDqSmemBytes) == cudaSuccess;
-      ok &= allow_smem(bwd_dq_kernel<128, true, 1>, BwdCfg<128>::kDqSmemBytes) == cudaSuccess;
-      ok &= allow_smem(bwd_dq_kernel<128, true, 2>, BwdCfg<128>::kDqSmemBytes) == cudaSuccess;
-      ok &= allow_smem(bwd_dq_kernel<128, false, 1>, BwdCfg<128>::kDqSmemBytes) == cudaSuccess;
-      ok &= allow_smem(bwd_dq_kernel<128, false, 2>, BwdCfg<128>::kDqSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dq_kernel<64, true, 1, false>, BwdCfg<64>::kDqSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dq_kernel<64, true, 2, false>, BwdCfg<64>::kDqSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dq_kernel<64, false, 1, false>, BwdCfg<64>::kDqSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dq_kernel<64, false, 2, false>, BwdCfg<64>::kDqSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dq_kernel<128, true, 1, false>, BwdCfg<128>::kDqSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dq_kernel<128, true, 2, false>, BwdCfg<128>::kDqSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dq_kernel<128, false, 1, false>, BwdCfg<128>::kDqSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dq_kernel<128, false, 2, false>, BwdCfg<128>::kDqSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dq_kernel<128, true, 1, true>, BwdCfg<128>::kDqSmemBytes) == cudaSuccess;
+      ok &= allow_smem(bwd_dq_kernel<128, false, 1, true>, BwdCfg<128>::kDqSmemBytes) == cudaSuccess;
       ok &= allow_smem(bwd_dkv_kernel<128, true, 1>, BwdCfg<128>::kDkvSmemBytes) == cudaSuccess;
       ok &= allow_smem(bwd_dkv_kernel<128, true, 2>, BwdCfg<128>::kDkvSmemBytes) == cudaSuccess;
       ok &= allow_smem(bwd_dkv_kernel<128, false, 1>, BwdCfg<128>::kDkvSmemBytes) == cudaSuccess;
@@ -161,8 +163,8 @@ int device_state(DeviceState **out) {
       ok &= allow_smem(attn_fwd_kernel<128, true, false, 3>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, false, false, 3>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       if (!ok) { (void)cudaGetLastError(); return GPROJ_ERR_CUDA; }
-      st.dq_clusters[0] = max_clusters(bwd_dq_kernel<64, true, 2>, 2, BwdCfg<64>::kDqThreads, BwdCfg<64>::kDqSmemBytes);
-      st.dq_clusters[1] = max_clusters(bwd_dq_kernel<128, true, 2>, 2, BwdCfg<128>::kDqThreads, BwdCfg<128>::kDqSmemBytes);
+      st.dq_clusters[0] = max_clusters(bwd_dq_kernel<64, true, 2, false>, 2, BwdCfg<64>::kDqThreads, BwdCfg<64>::kDqSmemBytes);
+      st.dq_clusters[1] = max_clusters(bwd_dq_kernel<128, true, 2, false>, 2, BwdCfg<128>::kDqThreads, BwdCfg<128>::kDqSmemBytes);
       st.dkv_clusters[0] = max_clusters(bwd_dkv_w128_kernel<true, 2>, 2, BwdW128::kThreads, BwdW128::kDkvSmemBytes);
       st.dkv_clusters[1] = max_clusters(bwd_dkv_kernel<128, true, 2>, 2, BwdCfg<128>::kDkvThreads, BwdCfg<128>::kDkvSmemBytes);
       for (int lg = 1; lg < 4; ++lg) {
@@ -633,6 +635,7 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
                         prefers_pairs(tile_steps(seqs, false, 64, 1, N, Nk, causal != 0), BH, st->sm_count, dq_fit, d == 64 ? 3.8 : 3.0, d == 64 ? 3.0 : 8.0);
   if (seqs && !dq_pairs)
     group_q.solo = packed_solo(*seqs, false, BH, st->sm_count, [&](int keys) { return std::max(1, (keys + 63) / 64) + (d == 64 ? 3.8 : 3.0); });
+  const bool dq_short = d == 128 && !dq_pairs && dq_short_tiles(seqs ? walked_key_tiles(*seqs) : fwd_key_tiles(N, Nk, causal != 0), n_qt, causal != 0);
   const int dkv_fit = st->dkv_clusters[d == 128], dkv_rows = d == 64 ? 128 : 64;   // rows of a step
   const bool dkv_pairs = run_dkv && total_kv_tiles <= 8LL * st->sm_count &&
                          prefers_pairs(tile_steps(seqs, true, dkv_rows, G, N, Nk, causal != 0), BHkv, st->sm_count, dkv_fit, d == 64 ? 2.3 : 3.0, d == 64 ? 1.5 : 4.0);
@@ -645,7 +648,7 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
 #define GPROJ_LAUNCH_BWD(DD, CC)                                                                                        \
   do {                                                                                                                  \
     if (run_dq)                                                                                                         \
-      launch_after(dq_pairs ? bwd_dq_kernel<DD, CC, 2> : bwd_dq_kernel<DD, CC, 1>, grid, dq_pairs ? 2 : 1, BwdCfg<DD>::kDqThreads, BwdCfg<DD>::kDqSmemBytes, s, true,                               \
+      launch_after(dq_pairs ? bwd_dq_kernel<DD, CC, 2, false> : dq_short ? bwd_dq_kernel<DD, CC, 1, DD == 128> : bwd_dq_kernel<DD, CC, 1, false>, grid, dq_pairs ? 2 : 1, BwdCfg<DD>::kDqThreads, BwdCfg<DD>::kDqSmemBytes, s, true,                               \
           mQ128, mdO128, mK64, mV64, static_cast<const __nv_bfloat16 *>(Q), Ob, dOb, LSE, stats, static_cast<__nv_bfloat16 *>(dQ), Zneg, plan_q, nblk,   \
           N, Nk, BH, H, G, total_tiles, group_q, scale_log2, softmax_scale,                                           \
           flags,                                                                                                        \
@@ -662,7 +665,7 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
 #define GPROJ_LAUNCH_BWD_W128(CC)                                                                                       \
   do {                                                                                                                  \
     if (run_dq)                                                                                                         \
-      launch_after(dq_pairs ? bwd_dq_kernel<64, CC, 2> : bwd_dq_kernel<64, CC, 1>, grid, dq_pairs ? 2 : 1, BwdCfg<64>::kDqThreads, BwdCfg<64>::kDqSmemBytes, s, true,                                \
+      launch_after(dq_pairs ? bwd_dq_kernel<64, CC, 2, false> : bwd_dq_kernel<64, CC, 1, false>, grid, dq_pairs ? 2 : 1, BwdCfg<64>::kDqThreads, BwdCfg<64>::kDqSmemBytes, s, true,                                \
           mQ128, mdO128, mK64, mV64, static_cast<const __nv_bfloat16 *>(Q), Ob, dOb, LSE, stats, static_cast<__nv_bfloat16 *>(dQ), Zneg, plan_q,    \
           nblk, N, Nk, BH, H, G, total_tiles, group_q, scale_log2, softmax_scale, flags, st->status_ptr);                 \
     if (run_dkv)                                                                                                        \

@@ -30,6 +30,11 @@ inline long long fwd_key_tiles(int lq, int lk, bool causal) {
 // (3.0) 256 -> 256, 1024 (4.5) 332 -> 312; not causal: 256 (2) 177 -> 190, 384 (3) 240 -> 234; 16 heads x 500 (64 items): 11.0 -> 10.4.
 inline bool fwd_separate_rings(long long items, int sms, long long key_tiles, long long tiles) { return items <= sms || key_tiles >= 3 * tiles; }
 
+// dQ side at d = 128: are the tiles so short that the compute warpgroups should prepare the row constants (SHORT in attn_bwd.cuh)?
+// key_tiles, tiles: of one head.  Measured, off -> on, causal, rows (key tiles per tile): 256 (1.5) 162 -> 124 us, 500 (2.5) 371 -> 293, 700
+// (3.5) 147 -> 133, 1000 (4.5) 83.3 -> 83.3, 2300 (9.5) 212 -> 219; not causal: 256 (2) 142 -> 125, 384 (3) 123 -> 125, 500 (4) 181 -> 192.
+inline bool dq_short_tiles(long long key_tiles, long long tiles, bool causal) { return 2 * key_tiles <= (causal ? 7 : 5) * tiles; }
+
 // CTAs per query tile of the forward (its base-two logarithm): with few tiles and long key ranges a tile's key range is
 // split over a cluster of 2, 4 or 8 CTAs, as many as leave each of their two warpgroups at least two 128-key tiles and let
 // all clusters run at once (`fit`: how many clusters of 2^lg CTAs do).  Beyond one wave the split only adds its merge, and

@@ -191,11 +191,13 @@ def test_head_shards_give_the_bits_of_the_whole_call(d, causal):
     assert rc == 0, hex(detail)
 
 
-@pytest.mark.parametrize("B,H,N,d,causal", [(2, 24, 1000, 64, True), (1, 160, 300, 64, False), (2, 80, 257, 128, True), (1, 300, 65, 64, True)])
+@pytest.mark.parametrize("B,H,N,d,causal", [(2, 24, 1000, 64, True), (1, 160, 300, 64, False), (2, 80, 257, 128, True), (1, 300, 65, 64, True),
+                                              (1, 500, 100, 128, False), (3, 110, 129, 128, True), (1, 60, 1000, 128, False)])
 def test_ragged_lengths_with_several_tiles_per_cta(B, H, N, d, causal):
     # More tiles than twice the SM count, with a ragged last tile in every head: a CTA walks three or more tiles, so the
     # per-tile hand-overs that only start at a CTA's second and third tile (row constants prepared one tile ahead in the
-    # other stationary buffer, buffers reused across tiles) are exercised on ragged data.  The oracle runs on eight heads.
+    # other stationary buffer, buffers reused across tiles) are exercised on ragged data, at d = 128 with the row constants
+    # from the compute warps (short tiles) and from the extra warpgroup.  The oracle runs on eight heads.
     w = Workload("ragged_many", B, H, N, d, causal, k_offset=8.0, seed=900 + N + H)
     inp = make_inputs(w)
     dev = {k: v.cuda() for k, v in inp.items()}

@@ -15,6 +15,7 @@ int count(int ok, int n) { return count_or_none([&](int *out) { *out = n; return
 int folds(int kv_heads, int G, int N, int Nk, int d) { const int fit[4] = {0, 74, 36, 16}; return fwd_folds_heads(kv_heads, G, N, Nk, d, 148, fit); }
 int smooth(long long pairs, long long rows, int longest, int d) { return smooth_cluster(pairs, rows, longest, d, 148); }
 long long key_tiles(int lq, int lk, int causal) { return fwd_key_tiles(lq, lk, causal != 0); }
+int short_tiles(long long key_tiles, long long tiles, int causal) { return dq_short_tiles(key_tiles, tiles, causal != 0); }
 int rings(long long items, long long key_tiles, long long tiles) { return fwd_separate_rings(items, 148, key_tiles, tiles); }
 }
 """
@@ -85,3 +86,8 @@ def test_separate_rings_from_three_key_tiles_on(rules, rows, causal, two):
     key_tiles, tiles = ctypes.c_longlong(walked(rows, rows, causal)), ctypes.c_longlong(-(-rows // 128))
     assert rules.rings(ctypes.c_longlong(149), key_tiles, tiles) == two
     assert rules.rings(ctypes.c_longlong(148), key_tiles, tiles) == 1
+
+
+@pytest.mark.parametrize("rows,causal,short", [(1, 1, 1), (128, 1, 1), (500, 1, 1), (700, 1, 1), (1000, 1, 0), (4096, 1, 0), (128, 0, 1), (256, 0, 1), (384, 0, 0), (700, 0, 0)])
+def test_row_constants_of_short_tiles_by_the_compute_warps(rules, rows, causal, short):
+    assert rules.short_tiles(ctypes.c_longlong(walked(rows, rows, causal)), ctypes.c_longlong(-(-rows // 128)), causal) == short
