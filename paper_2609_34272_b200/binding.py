@@ -190,10 +190,10 @@ def _lse_out(LSE, Q, shape):
     return LSE
 
 
-def _scratch(name, t, Q, nbytes):
-    """The caller's scratch or saved state (the library checks its size), or a new one of at least 256 bytes."""
+def _scratch(name, t, Q, bytes_of, *sizes):
+    """The caller's scratch or saved state (the library checks its size), or a new one of bytes_of(*sizes), at least 256, bytes."""
     if t is None:
-        return Q.new_empty(max(nbytes, 256), dtype=_U8)
+        return Q.new_empty(max(bytes_of(*sizes), 256), dtype=_U8)
     _check_buffer(name, t, Q.get_device())
     return t
 
@@ -234,7 +234,7 @@ def gproj_attn_bwd(Q, K, V, O, LSE, dO, softmax_scale, causal, flags=0, workspac
     Hkv = _kv_heads(shape, K)
     _check_lse(LSE, (B, H, N), "B, H, N")
     lib = _lib or load()
-    workspace = _scratch("workspace", workspace, Q, lib.gproj_attn_bwd_workspace_bytes(B, H, N, d))
+    workspace = _scratch("workspace", workspace, Q, lib.gproj_attn_bwd_workspace_bytes, B, H, N, d)
     nbytes = workspace.numel() * workspace.element_size()
     dQ = _output("dQ", dQ, Q); dK = _output("dK", dK, K); dV = _output("dV", dV, K)
     index = Q.get_device()
@@ -277,7 +277,7 @@ def gproj_attn_bwd_rect(Q, K, V, O, LSE, dO, softmax_scale, causal, flags=0, wor
     for name, t in (("O", O), ("dO", dO)):
         _check_bf16(name, t, Q.shape)
     _check_lse(LSE, (B, H, Nq), "B, H, Nq")
-    workspace = _scratch("workspace", workspace, Q, gproj_attn_bwd_workspace_bytes(B, H, Nq, d))
+    workspace = _scratch("workspace", workspace, Q, gproj_attn_bwd_workspace_bytes, B, H, Nq, d)
     dQ = _output("dQ", dQ, Q); dK = _output("dK", dK, K); dV = _output("dV", dV, K)
     with _on_device(Q.get_device()):
         rc = load().gproj_attn_bwd_rect(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), LSE.data_ptr(), dO.data_ptr(),
@@ -317,8 +317,7 @@ def gproj_fp32_attn_fwd(Q, K, V, softmax_scale, causal, saved=None):
     _check_bf16("Q", Q)
     B, H, N, d = Q.shape
     _check_bf16("K", K, Q.shape); _check_bf16("V", V, Q.shape)
-    need = int(load().gproj_fp32_attn_saved_bytes(B, H, N, d))
-    saved = _scratch("saved", saved, Q, need)
+    saved = _scratch("saved", saved, Q, load().gproj_fp32_attn_saved_bytes, B, H, N, d)
     O = torch.empty_like(Q)
     with _on_device(Q.get_device()):
         rc = load().gproj_fp32_attn_fwd(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), saved.data_ptr(), saved.numel(),
@@ -452,8 +451,7 @@ def gproj_attn_bwd_varlen(Q, K, V, O, LSE, dO, plan, softmax_scale, flags=0, wor
     for name, t in (("O", O), ("dO", dO)):
         _check_bf16(name, t, Q.shape)
     _check_lse(LSE, (H, T), "H, T")
-    need = int(load().gproj_attn_bwd_varlen_workspace_bytes(plan.cu, plan.num_seqs, H, d))
-    workspace = _scratch("workspace", workspace, Q, need)
+    workspace = _scratch("workspace", workspace, Q, load().gproj_attn_bwd_varlen_workspace_bytes, plan.cu, plan.num_seqs, H, d)
     dQ, dK, dV = torch.empty_like(Q), torch.empty_like(K), torch.empty_like(V)
     with _on_device(Q.get_device()):
         rc = load().gproj_attn_bwd_varlen(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), LSE.data_ptr(), dO.data_ptr(),
@@ -528,8 +526,7 @@ def gproj_attn_bwd_varlen_qk(Q, K, V, O, LSE, dO, plan, softmax_scale, flags=0, 
     for name, t in (("O", O), ("dO", dO)):
         _check_bf16(name, t, Q.shape)
     _check_lse(LSE, (H, Tq), "H, Tq")
-    need = int(load().gproj_attn_bwd_varlen_workspace_bytes(plan.cu, plan.num_seqs, H, d))
-    workspace = _scratch("workspace", workspace, Q, need)
+    workspace = _scratch("workspace", workspace, Q, load().gproj_attn_bwd_varlen_workspace_bytes, plan.cu, plan.num_seqs, H, d)
     dQ, dK, dV = torch.empty_like(Q), torch.empty_like(K), torch.empty_like(V)
     with _on_device(Q.get_device()):
         rc = load().gproj_attn_bwd_varlen_qk(Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), LSE.data_ptr(), dO.data_ptr(),
