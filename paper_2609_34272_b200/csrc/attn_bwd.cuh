@@ -41,6 +41,7 @@
 // next.
 #pragma once
 #include "sm100_primitives.cuh"
+#include "tile_schedule.h"
 
 namespace gproj {
 
@@ -99,27 +100,6 @@ struct BwdCfg {
   static constexpr int kDkvStagingBytes = 4 * 32 * 64;             // each epilogue warp: 32 rows x 32 columns of dK or dV
   static constexpr int kDkvSmemBytes = 2 * kBigTileBytes + kDkvStages * kDkvStageBytes + kDkvStagingBytes + 1024;
   static_assert(kDqStages >= kNB + 1 && kDkvStages >= kNB + 1, "a stage stays busy until its second-stage MMAs finish");
-};
-
-// Static persistent schedule: work items are numbered by decreasing work; round r hands item r G + c to CTA c
-// on even rounds and item r G + (G - 1 - c) on odd rounds (G = number of CTAs).  With solo > 0 the first `solo` CTAs, whose
-// first item is longer than an even share, get nothing after round 0 and the others share the rest in the same way.
-// With clusters a whole cluster counts as one CTA here.
-struct TileSched {
-  int total, W, c, back, round;     // W: CTAs that share the rounds after the first; back: c counted from the other end of them
-  __device__ __forceinline__ TileSched(int total_tiles, int solo, int cluster = 1) {
-    const int G = static_cast<int>(gridDim.x) / cluster;
-    c = static_cast<int>(blockIdx.x) / cluster;
-    W = G - solo;
-    back = solo + G - 1 - c;
-    total = c < solo ? min(total_tiles, G) : total_tiles;
-    round = 0;
-  }
-  __device__ __forceinline__ int next() {
-    const int idx = round * W + ((round & 1) ? back : c);
-    ++round;
-    return idx < total ? idx : -1;
-  }
 };
 
 // Item number -> (rank of the tile in decreasing work, head).  Items are dealt in groups of `group` consecutive ranks of

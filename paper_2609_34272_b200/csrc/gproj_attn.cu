@@ -5,6 +5,7 @@
 #include <cmath>
 #include <cstdint>
 #include <algorithm>
+#include <array>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -227,9 +228,6 @@ void launch_after(void (*kernel)(Params...), dim3 grid, int cluster, int threads
   (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);   // the caller reads cudaGetLastError()
 }
 
-// The row offsets of a packed call (host), for the host's scheduling decisions.
-struct PackedSeqs { const int *cu_q, *cu_k; int num; bool causal; };
-
 int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE, int B, int H, int Hkv, int N, int Nk, int d,
                float softmax_scale, int causal, unsigned fwd_flags, const int4 *plan, int n_plan_tiles, const PackedSeqs *seqs, void *stream);
 int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const float *LSE, const void *dO,
@@ -291,74 +289,6 @@ ItemOrder item_order(int heads, int n_per_head, int group) {
   o.by_gk = fast_div(static_cast<unsigned>(o.gk));
   o.by_rem = fast_div(static_cast<unsigned>(std::max(1, n_per_head - o.n_full * o.gk)));
   return o;
-}
-
-// Longest CTA of the static boustrophedon deal (TileSched) of `items` items with the given costs.
-template <typename WorkOf>
-double deal_makespan(long long items, int sms, WorkOf work_of, int solo = 0) {
-  const int G = static_cast<int>(std::min<long long>(items, sms)), W = G - solo;
-  std::vector<double> load(static_cast<size_t>(G), 0.0);
-  for (long long lin = 0; lin < items; ++lin) {
-    int cta = static_cast<int>(lin);
-    if (lin >= G) {
-      const long long r = 1 + (lin - G) / W, pos = (lin - G) % W;
-      cta = static_cast<int>((r & 1) ? G - 1 - pos : solo + pos);
-    }
-    load[static_cast<size_t>(cta)] += work_of(lin);
-  }
-  return *std::max_element(load.begin(), load.end());
-}
-
-// Work of every tile of a packed call, in the plan's order (decreasing): keys of each query tile (key_side: queries of each
-// key tile, whose walk starts at a 64-row block).
-std::vector<int> packed_work(const PackedSeqs &ps, bool key_side) {
-  std::vector<int> work;
-  for (int s = 0; s < ps.num; ++s) {
-    const int lq = ps.cu_q[s + 1] - ps.cu_q[s], lk = ps.cu_k[s + 1] - ps.cu_k[s], off = lk - lq;
-    if (!key_side)
-      for (int r = 0; r < lq; r += 128) work.push_back(ps.causal ? std::max(0, std::min(lk, std::min(r + 128, lq) + off)) : lk);
-    else if (lq > 0)
-      for (int r = 0; r < lk; r += 128) work.push_back(std::max(0, lq - (ps.causal ? std::max(0, r - off) & ~63 : 0)));
-  }
-  std::sort(work.begin(), work.end(), [](int a, int b) { return a > b; });
-  return work;
-}
-
-// Key tiles that a head's query tiles walk over all sequences.
-long long walked_key_tiles(const PackedSeqs &ps) {
-  long long sum = 0;
-  for (int s = 0; s < ps.num; ++s) sum += fwd_key_tiles(ps.cu_q[s + 1] - ps.cu_q[s], ps.cu_k[s + 1] - ps.cu_k[s], ps.causal);
-  return sum;
-}
-
-int longest_keys(const PackedSeqs &ps) {
-  int most = 0;
-  for (int s = 0; s < ps.num; ++s) most = std::max(most, ps.cu_k[s + 1] - ps.cu_k[s]);
-  return most;
-}
-
-// TileSched's solo CTAs for `heads` copies of tiles with the given costs (decreasing): those whose first item is longer than
-// what an even share of the rest would be.  The boustrophedon rounds would give each of them a second item all the same.
-// Measured, 12 packed pairs (4000 queries, 9000 keys, 12 heads, d = 128; 60 of 456 query tiles twice as long as an even
-// share): forward 53.6 -> 45.5 us, dQ side 76.5 -> 64.0 us.
-int solo_ctas(const std::vector<double> &cost, int heads, int sms) {
-  const long long items = static_cast<long long>(cost.size()) * heads;
-  if (items <= sms || items > 16LL * sms) return 0;
-  double total = 0.0;
-  for (double c : cost) total += c * heads;
-  int solo = 0;
-  double rest = total;
-  while (solo < sms / 2 && cost[static_cast<size_t>(solo / heads)] > rest / (sms - solo)) rest -= cost[static_cast<size_t>(solo++ / heads)];
-  if (solo == 0) return 0;
-  auto work_of = [&](long long lin) { return cost[static_cast<size_t>(lin / heads)]; };
-  return deal_makespan(items, sms, work_of, solo) < 0.99 * deal_makespan(items, sms, work_of) ? solo : 0;
-}
-
-template <typename CostOf>
-int packed_solo(const PackedSeqs &ps, bool key_side, int heads, int sms, CostOf cost_of) {
-  std::vector<double> cost;
-  for (int w : packed_work(ps, key_side)) cost.push_back(cost_of(w));
-  return solo_ctas(cost, heads, sms);
 }
 
 // How many adjacent tile ranks of one head the kernels deal consecutively (see ItemOrder).  Packed calls: 1 (their plan is
@@ -484,7 +414,8 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
   ItemOrder fwd_order = item_order(BH, total_items / BH, tile_group_of(plan != nullptr, causal != 0, BH, total_items / BH, 2 * static_cast<size_t>(BHkv) * Nk * d * 2, st->sm_count,
                                                             tiles_per_item == 2 ? 1.45 : 6.8));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const int lg = (tiles_per_item == 1 && !fma) ? fwd_cluster_log2(total_items, ((seqs ? longest_keys(*seqs) : Nk) + 127) / 128, st->fwd_clusters[d == 128]) : 0;
+  const int (&fit)[4] = st->fwd_clusters[d == 128];
+  const int lg = (tiles_per_item == 1 && !fma && total_items <= fit[1]) ? fwd_cluster_log2(total_items, ((seqs ? longest_keys(*seqs) : Nk) + 127) / 128, fit) : 0;
   if (lg > 0 || fold > 0) {
     auto kernel = d == 64 ? (causal ? attn_fwd_kernel<64, true, false, 3> : attn_fwd_kernel<64, false, false, 3>)
                           : (causal ? attn_fwd_kernel<128, true, false, 3> : attn_fwd_kernel<128, false, false, 3>);
@@ -495,7 +426,8 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
     tl_launch_count = 1;
     return GPROJ_OK;
   }
-  if (seqs) fwd_order.solo = packed_solo(*seqs, false, BH, st->sm_count, [](int keys) { return std::max(1, (keys + 127) / 128) + 2.1; });
+  if (seqs && total_items > st->sm_count && total_items <= 16LL * st->sm_count)
+    fwd_order.solo = solo_ctas(tile_steps(*seqs, false, 128, 1), BH, st->sm_count, 2.1);
   const dim3 grid(static_cast<unsigned>(total_items < st->sm_count ? total_items : st->sm_count));   // persistent
   // Start beside the previous kernel only with at most two items per CTA.  CTAs that start early take the SMs in the order in
   // which the previous kernel leaves them; launched normally, neighbouring CTAs sit side by side in a TPC and walk
@@ -515,7 +447,7 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
   // they alternate in the exponential phase (measured to pay there only).
   const bool split = (tiles_per_item == 1), turns = (d == 128) && !split && !fma;
   if (d == 64) { if (split) GPROJ_LAUNCH_FWD_F(64, 2); else GPROJ_LAUNCH_FWD_F(64, 0); }
-  else if (split && fwd_separate_rings(total_items, st->sm_count, seqs ? walked_key_tiles(*seqs) : fwd_key_tiles(N, Nk, causal != 0), n_qt)) GPROJ_LAUNCH_FWD_F(128, 4);
+  else if (split && (total_items <= st->sm_count || fwd_separate_rings(seqs ? walked_key_tiles(*seqs) : fwd_key_tiles(N, Nk, causal != 0), n_qt))) GPROJ_LAUNCH_FWD_F(128, 4);
   else if (split) GPROJ_LAUNCH_FWD_F(128, 2);
   else if (turns) GPROJ_LAUNCH_FWD_C(128, false, 1);
   else GPROJ_LAUNCH_FWD_F(128, 0);
@@ -554,33 +486,23 @@ int gproj_attn_bwd_gqa(const void *Q, const void *K, const void *V, const void *
 
 namespace {
 
-// Share every tile of a backward kernel between the two CTAs of a cluster?  This replays the static deal of both forms in
-// units of one step (per_item: the kernel's measured overhead per item; exchange: what the exchange of the two parts adds)
-// and takes the pairs where their longest CTA is 3 % shorter.  steps: of each tile of a head, decreasing.
-// Measured, dK/dV side at d = 64 alone, whole tiles -> pairs: 16 query / 4 KV heads x 4096, causal: 121 -> 77 us; 8 / 2 heads x 8000,
-// causal: 229 -> 140; 32 / 4 heads x 2000: 121 -> 78; 4 heads x 4096, causal: 43.5 -> 37.2; 1 head x 8192: 62.0 -> 43.5;
-// 16 heads x 4096, causal (stays with whole tiles): 68; 16 packed documents of 8192 rows, 16 / 4 heads: 78.6 -> 73.0.
-// dK/dV side at d = 128: 16 / 4 heads x 4096, causal: 275 -> 151; 8 / 1 heads x 3000, causal: 375 -> 200; 16 / 8 heads x 700, causal: 30.9 ->
-// 25.0; 2 heads x 1500, causal: 30.9 -> 24.8; 4 heads x 1000 (16 steps): 24.7 -> 21.0; 4 heads x 800, causal: 20.7 -> 19.1; 2 heads x 640 (10
-// steps): 17.5 -> 17.1, hence four steps for the exchange.
-// dQ side: 1 head x 8192 x 64: 83 -> 52 us; 4 heads x 4096 x 64, causal: 44.7 -> 34.4; 16 heads x 300 queries behind 9000 keys,
-// d = 128: 126 -> 92; 4 heads x 2048 x 128, causal: 36.5 -> 32.8; 4 heads x 1000 x 128 (16 steps): 20.7 -> 21.3, hence the
-// 8 steps the exchange counts at d = 128.
-bool prefers_pairs(const std::vector<int> &steps, int heads, int sms, int pairs, double per_item, double exchange) {
-  const long long items = static_cast<long long>(heads) * static_cast<long long>(steps.size());
-  if (pairs < 1 || items > 8LL * sms) return false;      // many items per CTA: they balance as they are
-  const double whole = deal_makespan(items, sms, [&](long long lin) { return steps[static_cast<size_t>(lin / heads)] + per_item; });
-  const double split = deal_makespan(items, pairs, [&](long long lin) { return (steps[static_cast<size_t>(lin / heads)] + 1) / 2 + per_item + exchange; });
-  return split < 0.97 * whole;
-}
-
-// Steps of `rows` rows of the tiles of a call (key_side: of the key tiles, over the G heads of a group), decreasing.
-std::vector<int> tile_steps(const PackedSeqs *seqs, bool key_side, int rows, int G, int Nq, int Nk, bool causal) {
+// deal_form (host_rules.h) of one kernel of a call.  The answer for a dense call is remembered by its sizes (the replays take 4 to 15 us).
+DealForm deal_form_of(const PackedSeqs *seqs, bool key_side, int Nq, int Nk, bool causal, int G, int heads, int tiles, int sms, int fit, const DealCosts &c) {
+  if (seqs) return deal_form(*seqs, true, key_side, G, heads, tiles, sms, fit, c);
+  if (static_cast<long long>(heads) * tiles > 8LL * sms) return DealForm{false, 0};
+  static std::mutex memo_mutex;
+  static std::map<std::array<int, 11>, DealForm> memo;
+  const std::array<int, 11> key = {key_side, Nq, Nk, causal, G, heads, sms, fit, c.rows, static_cast<int>(c.per_item * 100.0), static_cast<int>(c.exchange * 100.0)};
+  {
+    std::lock_guard<std::mutex> lock(memo_mutex);
+    const auto hit = memo.find(key);
+    if (hit != memo.end()) return hit->second;
+  }
   const int cu_q[2] = {0, Nq}, cu_k[2] = {0, Nk};
-  const PackedSeqs one{cu_q, cu_k, 1, causal};
-  std::vector<int> steps = packed_work(seqs ? *seqs : one, key_side);
-  for (int &w : steps) w = G * std::max(1, (w + rows - 1) / rows);
-  return steps;
+  const DealForm form = deal_form(PackedSeqs{cu_q, cu_k, 1, causal}, false, key_side, G, heads, tiles, sms, fit, c);
+  std::lock_guard<std::mutex> lock(memo_mutex);
+  if (memo.size() < 4096) memo[key] = form;
+  return form;
 }
 
 // Dense call: plans == nullptr.  Packed call: B = 1, N / Nk = total query / key rows, plan_q / plan_kv = device tile lists
@@ -630,17 +552,14 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
   if (total_kv_tiles <= 0) run_dkv = false;   // packed call in which no sequence has both queries and keys
   ItemOrder group_q = item_order(BH, n_qt, tile_group_of(plan_q != nullptr, causal != 0, BH, n_qt, 2 * static_cast<size_t>(BHkv) * Nk * d * 2, st->sm_count, 3.25));    // streams K, V
   ItemOrder group_kv = item_order(BHkv, std::max(n_kt, 1), tile_group_of(plan_q != nullptr, causal != 0, BHkv, n_kt, 3 * static_cast<size_t>(BH) * N * d * 2, st->sm_count, 2.3));   // streams Q, dO, Z
-  const int dq_fit = st->dq_clusters[d == 128];
-  const bool dq_pairs = run_dq && total_tiles <= 8LL * st->sm_count &&
-                        prefers_pairs(tile_steps(seqs, false, 64, 1, N, Nk, causal != 0), BH, st->sm_count, dq_fit, d == 64 ? 3.8 : 3.0, d == 64 ? 3.0 : 8.0);
-  if (seqs && !dq_pairs)
-    group_q.solo = packed_solo(*seqs, false, BH, st->sm_count, [&](int keys) { return std::max(1, (keys + 63) / 64) + (d == 64 ? 3.8 : 3.0); });
-  const bool dq_short = d == 128 && !dq_pairs && dq_short_tiles(seqs ? walked_key_tiles(*seqs) : fwd_key_tiles(N, Nk, causal != 0), n_qt, causal != 0);
-  const int dkv_fit = st->dkv_clusters[d == 128], dkv_rows = d == 64 ? 128 : 64;   // rows of a step
-  const bool dkv_pairs = run_dkv && total_kv_tiles <= 8LL * st->sm_count &&
-                         prefers_pairs(tile_steps(seqs, true, dkv_rows, G, N, Nk, causal != 0), BHkv, st->sm_count, dkv_fit, d == 64 ? 2.3 : 3.0, d == 64 ? 1.5 : 4.0);
-  if (seqs && !dkv_pairs)
-    group_kv.solo = packed_solo(*seqs, true, BHkv, st->sm_count, [&](int rows) { return G * std::max(1, (rows + dkv_rows - 1) / dkv_rows) + (d == 64 ? 2.3 : 3.0); });
+  const int dq_fit = st->dq_clusters[d == 128], dkv_fit = st->dkv_clusters[d == 128];
+  const DealForm none{false, 0};
+  const DealForm dq_form = run_dq ? deal_form_of(seqs, false, N, Nk, causal != 0, 1, BH, n_qt, st->sm_count, dq_fit, d == 64 ? DealCosts{64, 3.8, 3.0} : DealCosts{64, 3.0, 8.0}) : none;
+  const DealForm dkv_form = run_dkv ? deal_form_of(seqs, true, N, Nk, causal != 0, G, BHkv, n_kt, st->sm_count, dkv_fit, d == 64 ? DealCosts{128, 2.3, 1.5} : DealCosts{64, 3.0, 4.0}) : none;
+  const bool dq_pairs = dq_form.pairs, dkv_pairs = dkv_form.pairs;
+  group_q.solo = dq_form.solo;
+  group_kv.solo = dkv_form.solo;
+  const bool dq_short = run_dq && d == 128 && !dq_pairs && dq_short_tiles(seqs ? walked_key_tiles(*seqs) : fwd_key_tiles(N, Nk, causal != 0), n_qt, causal != 0);
   const dim3 grid(static_cast<unsigned>(dq_pairs ? 2 * std::min(total_tiles, dq_fit) : std::min(total_tiles, st->sm_count)));   // persistent: one CTA per SM
   const dim3 grid_kv(static_cast<unsigned>(dkv_pairs ? 2 * std::min(total_kv_tiles, dkv_fit) : std::min(total_kv_tiles, st->sm_count)));
   cudaStream_t s = static_cast<cudaStream_t>(stream);

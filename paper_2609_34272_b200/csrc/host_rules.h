@@ -2,6 +2,7 @@
 #pragma once
 
 #include <algorithm>
+#include <vector>
 
 namespace gproj {
 
@@ -25,10 +26,10 @@ inline long long fwd_key_tiles(int lq, int lk, bool causal) {
 }
 
 // Forward at d = 128 with the key range of a tile split between the warpgroups: separate rings for K and V (see attn_fwd.cuh)?
-// With one item per CTA, or from three key tiles per item on.  items: over all heads; key_tiles, tiles: of one head.  Measured, one
+// From three key tiles per item on (key_tiles, tiles: of one head), and always with one item per CTA.  Measured, one
 // ring -> two, 16 query / 4 KV heads, 40000 rows in sequences of one length, causal: 512 rows (2.5 key tiles per item) 228 -> 239 us, 640
 // (3.0) 256 -> 256, 1024 (4.5) 332 -> 312; not causal: 256 (2) 177 -> 190, 384 (3) 240 -> 234; 16 heads x 500 (64 items): 11.0 -> 10.4.
-inline bool fwd_separate_rings(long long items, int sms, long long key_tiles, long long tiles) { return items <= sms || key_tiles >= 3 * tiles; }
+inline bool fwd_separate_rings(long long key_tiles, long long tiles) { return key_tiles >= 3 * tiles; }
 
 // dQ side at d = 128: are the tiles so short that the compute warpgroups should prepare the row constants (SHORT in attn_bwd.cuh)?
 // key_tiles, tiles: of one head.  Measured, off -> on, causal, rows (key tiles per tile): 256 (1.5) 162 -> 124 us, 500 (2.5) 371 -> 293, 700
@@ -97,6 +98,122 @@ inline int smooth_cluster(long long pairs, long long rows, int longest, int d, i
     c *= 2;
   }
   return c == 4 && longest > 4096 && pairs * 8 <= 3LL * sms ? 8 : c;
+}
+
+// The row offsets of a packed call (host).
+struct PackedSeqs { const int *cu_q, *cu_k; int num; bool causal; };
+
+// Work of every tile of a packed call, in the plan's order (decreasing): keys of each query tile (key_side: queries of each
+// key tile, whose walk starts at a 64-row block).
+inline std::vector<int> packed_work(const PackedSeqs &ps, bool key_side) {
+  std::vector<int> work;
+  for (int s = 0; s < ps.num; ++s) {
+    const int lq = ps.cu_q[s + 1] - ps.cu_q[s], lk = ps.cu_k[s + 1] - ps.cu_k[s], off = lk - lq;
+    if (!key_side)
+      for (int r = 0; r < lq; r += 128) work.push_back(ps.causal ? std::max(0, std::min(lk, std::min(r + 128, lq) + off)) : lk);
+    else if (lq > 0)
+      for (int r = 0; r < lk; r += 128) work.push_back(std::max(0, lq - (ps.causal ? std::max(0, r - off) & ~63 : 0)));
+  }
+  std::sort(work.begin(), work.end(), [](int a, int b) { return a > b; });
+  return work;
+}
+
+// Key tiles that a head's query tiles walk over all sequences.
+inline long long walked_key_tiles(const PackedSeqs &ps) {
+  long long sum = 0;
+  for (int s = 0; s < ps.num; ++s) sum += fwd_key_tiles(ps.cu_q[s + 1] - ps.cu_q[s], ps.cu_k[s + 1] - ps.cu_k[s], ps.causal);
+  return sum;
+}
+
+inline int longest_keys(const PackedSeqs &ps) {
+  int most = 0;
+  for (int s = 0; s < ps.num; ++s) most = std::max(most, ps.cu_k[s + 1] - ps.cu_k[s]);
+  return most;
+}
+
+// Longest CTA of the static deal (TileSched, walked item by item) of `items` items.  work_of is called once for every item, in order.
+template <typename WorkOf>
+double deal_makespan(long long items, int ctas, WorkOf work_of, int solo = 0) {
+  const int G = static_cast<int>(std::min<long long>(items, ctas)), W = G - solo;
+  std::vector<double> load(static_cast<size_t>(G));
+  long long lin = 0;
+  for (int c = 0; c < G; ++c) load[static_cast<size_t>(c)] = work_of(lin++);
+  for (bool odd = true; lin < items; odd = !odd) {
+    const int n = static_cast<int>(std::min<long long>(W, items - lin));
+    if (odd) for (int c = 0; c < n; ++c) load[static_cast<size_t>(G - 1 - c)] += work_of(lin++);
+    else     for (int c = 0; c < n; ++c) load[static_cast<size_t>(solo + c)] += work_of(lin++);
+  }
+  return *std::max_element(load.begin(), load.end());
+}
+
+// ... of `heads` copies of every tile, with the cost that cost_of gives for its steps.
+template <typename CostOf>
+double deal_tiles(const std::vector<int> &steps, int heads, int ctas, CostOf cost_of, int solo = 0) {
+  size_t k = 0;
+  int left = 0;
+  double cost = 0.0;
+  return deal_makespan(static_cast<long long>(steps.size()) * heads, ctas, [&](long long) {
+    if (left == 0) { cost = cost_of(steps[k++]); left = heads; }
+    --left;
+    return cost;
+  }, solo);
+}
+
+// TileSched's solo CTAs for `heads` copies of tiles with the given costs (decreasing): those whose first item is longer than
+// what an even share of the rest would be.  The boustrophedon rounds would give each of them a second item all the same.
+// Measured, 12 packed pairs (4000 queries, 9000 keys, 12 heads, d = 128; 60 of 456 query tiles twice as long as an even
+// share): forward 53.6 -> 45.5 us, dQ side 76.5 -> 64.0 us.
+// per_item: the kernel's measured overhead per item, in steps.
+inline int solo_ctas(const std::vector<int> &steps, int heads, int sms, double per_item) {
+  const long long items = static_cast<long long>(steps.size()) * heads;
+  if (items <= sms || items > 16LL * sms) return 0;
+  auto cost = [&](int n) { return n + per_item; };
+  double rest = 0.0;
+  for (int n : steps) rest += cost(n) * heads;
+  int solo = 0;
+  while (solo < sms / 2 && cost(steps[static_cast<size_t>(solo / heads)]) > rest / (sms - solo)) rest -= cost(steps[static_cast<size_t>(solo++ / heads)]);
+  if (solo == 0) return 0;
+  return deal_tiles(steps, heads, sms, cost, solo) < 0.99 * deal_tiles(steps, heads, sms, cost) ? solo : 0;
+}
+
+// Share every tile of a backward kernel between the two CTAs of a cluster?  This replays the static deal of both forms in
+// units of one step (per_item: the kernel's measured overhead per item; exchange: what the exchange of the two parts adds)
+// and takes the pairs where their longest CTA is 3 % shorter.  steps: of each tile of a head, decreasing.
+// Measured, dK/dV side at d = 64 alone, whole tiles -> pairs: 16 query / 4 KV heads x 4096, causal: 121 -> 77 us; 8 / 2 heads x 8000,
+// causal: 229 -> 140; 32 / 4 heads x 2000: 121 -> 78; 4 heads x 4096, causal: 43.5 -> 37.2; 1 head x 8192: 62.0 -> 43.5;
+// 16 heads x 4096, causal (stays with whole tiles): 68; 16 packed documents of 8192 rows, 16 / 4 heads: 78.6 -> 73.0.
+// dK/dV side at d = 128: 16 / 4 heads x 4096, causal: 275 -> 151; 8 / 1 heads x 3000, causal: 375 -> 200; 16 / 8 heads x 700, causal: 30.9 ->
+// 25.0; 2 heads x 1500, causal: 30.9 -> 24.8; 4 heads x 1000 (16 steps): 24.7 -> 21.0; 4 heads x 800, causal: 20.7 -> 19.1; 2 heads x 640 (10
+// steps): 17.5 -> 17.1, hence four steps for the exchange.
+// dQ side: 1 head x 8192 x 64: 83 -> 52 us; 4 heads x 4096 x 64, causal: 44.7 -> 34.4; 16 heads x 300 queries behind 9000 keys,
+// d = 128: 126 -> 92; 4 heads x 2048 x 128, causal: 36.5 -> 32.8; 4 heads x 1000 x 128 (16 steps): 20.7 -> 21.3, hence the
+// 8 steps the exchange counts at d = 128.
+inline bool prefers_pairs(const std::vector<int> &steps, int heads, int sms, int pairs, double per_item, double exchange) {
+  const long long items = static_cast<long long>(heads) * static_cast<long long>(steps.size());
+  if (pairs < 1 || items < 1 || items > 8LL * sms) return false;      // many items per CTA: they balance as they are
+  const double whole = deal_tiles(steps, heads, sms, [&](int n) { return n + per_item; });
+  const double split = deal_tiles(steps, heads, pairs, [&](int n) { return (n + 1) / 2 + per_item + exchange; });
+  return split < 0.97 * whole;
+}
+
+// Steps of `rows` rows of the tiles of a call (key_side: of the key tiles, over the G heads of a group), decreasing.
+inline std::vector<int> tile_steps(const PackedSeqs &seqs, bool key_side, int rows, int G) {
+  std::vector<int> steps = packed_work(seqs, key_side);
+  for (int &w : steps) w = G * std::max(1, (w + rows - 1) / rows);
+  return steps;
+}
+
+// How the items of a backward kernel are dealt: every tile shared by two CTAs, or else `solo` CTAs with one item only.
+struct DealForm { bool pairs; int solo; };
+struct DealCosts { int rows; double per_item, exchange; };   // rows of a step; prefers_pairs
+// tiles: of a head.  Beyond 16 items per CTA neither matters, and beyond 8 (where dense calls end, whose tiles need no solo CTAs) only
+// solo: the tiles are not even listed (8000 packed sequences: 120 us of host time).
+inline DealForm deal_form(const PackedSeqs &seqs, bool packed, bool key_side, int G, int heads, int tiles, int sms, int fit, const DealCosts &c) {
+  const long long items = static_cast<long long>(heads) * tiles;
+  if (items < 1 || items > (packed ? 16LL : 8LL) * sms) return DealForm{false, 0};
+  const std::vector<int> steps = tile_steps(seqs, key_side, c.rows, G);
+  if (prefers_pairs(steps, heads, sms, fit, c.per_item, c.exchange)) return DealForm{true, 0};
+  return DealForm{false, packed ? solo_ctas(steps, heads, sms, c.per_item) : 0};
 }
 
 }  // namespace gproj

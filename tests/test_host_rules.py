@@ -1,6 +1,7 @@
 """The host's choices between kernels and launch shapes, checked without a GPU (host_rules.h compiled with g++)."""
 import ctypes
 import os
+import random
 import re
 import subprocess
 
@@ -9,6 +10,7 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2609_34272_b200", "csrc")
 HARNESS = r"""
 #include "host_rules.h"
+#include "tile_schedule.h"
 using namespace gproj;
 extern "C" {
 int count(int ok, int n) { return count_or_none([&](int *out) { *out = n; return ok != 0; }); }
@@ -16,7 +18,25 @@ int folds(int kv_heads, int G, int N, int Nk, int d) { const int fit[4] = {0, 74
 int smooth(long long pairs, long long rows, int longest, int d) { return smooth_cluster(pairs, rows, longest, d, 148); }
 long long key_tiles(int lq, int lk, int causal) { return fwd_key_tiles(lq, lk, causal != 0); }
 int short_tiles(long long key_tiles, long long tiles, int causal) { return dq_short_tiles(key_tiles, tiles, causal != 0); }
-int rings(long long items, long long key_tiles, long long tiles) { return fwd_separate_rings(items, 148, key_tiles, tiles); }
+int rings(long long key_tiles, long long tiles) { return fwd_separate_rings(key_tiles, tiles); }
+double deal(const int *steps, int n, int heads, int ctas, int solo, double per_item) {
+  return deal_tiles(std::vector<int>(steps, steps + n), heads, ctas, [&](int s) { return s + per_item; }, solo);
+}
+double walk(const int *steps, int n, int heads, int ctas, int solo, double per_item, int *taken) {
+  const int items = n * heads, G = std::min(items, ctas);
+  double most = 0.0;
+  for (int c = 0; c < G; ++c) {
+    TileSched sched(items, solo, G, c);
+    double sum = 0.0;
+    for (int lin = sched.next(); lin >= 0; lin = sched.next()) { sum += steps[lin / heads] + per_item; ++taken[lin]; }
+    most = std::max(most, sum);
+  }
+  return most;
+}
+int form(const int *cu_q, const int *cu_k, int num, int causal, int packed, int key_side, int G, int heads, int tiles) {
+  const DealForm f = deal_form(PackedSeqs{cu_q, cu_k, num, causal != 0}, packed != 0, key_side != 0, G, heads, tiles, 148, 74, DealCosts{64, 3.0, 8.0});
+  return f.pairs ? -1 : f.solo;
+}
 }
 """
 
@@ -84,10 +104,34 @@ def test_key_tiles_of_a_sequence(rules):
 @pytest.mark.parametrize("rows,causal,two", [(128, 1, 0), (200, 0, 0), (256, 1, 0), (256, 0, 0), (512, 1, 0), (384, 0, 1), (640, 1, 1), (1500, 1, 1), (4096, 1, 1)])
 def test_separate_rings_from_three_key_tiles_on(rules, rows, causal, two):
     key_tiles, tiles = ctypes.c_longlong(walked(rows, rows, causal)), ctypes.c_longlong(-(-rows // 128))
-    assert rules.rings(ctypes.c_longlong(149), key_tiles, tiles) == two
-    assert rules.rings(ctypes.c_longlong(148), key_tiles, tiles) == 1
+    assert rules.rings(key_tiles, tiles) == two
 
 
 @pytest.mark.parametrize("rows,causal,short", [(1, 1, 1), (128, 1, 1), (500, 1, 1), (700, 1, 1), (1000, 1, 0), (4096, 1, 0), (128, 0, 1), (256, 0, 1), (384, 0, 0), (700, 0, 0)])
 def test_row_constants_of_short_tiles_by_the_compute_warps(rules, rows, causal, short):
     assert rules.short_tiles(ctypes.c_longlong(walked(rows, rows, causal)), ctypes.c_longlong(-(-rows // 128)), causal) == short
+
+
+def test_the_weighed_deal_is_the_kernels_deal(rules):
+    rng = random.Random(1)
+    args = [ctypes.POINTER(ctypes.c_int), ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_double]
+    rules.deal.restype = rules.walk.restype = ctypes.c_double
+    rules.deal.argtypes, rules.walk.argtypes = args, args + [ctypes.POINTER(ctypes.c_int)]
+    for _ in range(300):
+        n, heads, ctas = rng.randint(1, 40), rng.randint(1, 30), rng.choice([1, 2, 7, 74, 148])
+        steps = sorted((rng.randint(1, 100) for _ in range(n)), reverse=True)
+        solo = rng.randint(0, ctas // 2) if n * heads > ctas else 0
+        arr, taken = (ctypes.c_int * n)(*steps), (ctypes.c_int * (n * heads))()
+        assert abs(rules.deal(arr, n, heads, ctas, solo, 2.5) - rules.walk(arr, n, heads, ctas, solo, 2.5, taken)) < 1e-6
+        assert set(taken) == {1}
+
+
+def test_tiles_are_not_listed_where_the_deal_does_not_matter(rules):
+    # null offsets: listing the tiles would read them
+    assert rules.form(None, None, 8000, 1, 1, 0, 1, 2, 8000) == 0 and rules.form(None, None, 8000, 1, 1, 1, 1, 2, 8000) == 0
+    assert rules.form(None, None, 1, 1, 0, 0, 1, 100, 12) == 0
+    one = lambda n: (ctypes.c_int * 2)(0, n)
+    assert rules.form(one(4096), one(4096), 1, 1, 0, 0, 1, 4, 32) == -1             # 128 tiles of very different length: pairs
+    short = [128 * i for i in range(101)]
+    cu_q, cu_k = ((ctypes.c_int * 102)(0, *[first + x for x in short]) for first in (300, 9000))
+    assert rules.form(cu_q, cu_k, 101, 0, 1, 0, 1, 12, 103) == 36                   # three long tiles of 12 heads, 1200 short ones
