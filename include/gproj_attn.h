@@ -304,6 +304,18 @@ const char *gproj_status_string(int status);
 /* Number of kernels the most recent successful gproj_attn_fwd / gproj_attn_bwd call on this thread launched. */
 int gproj_last_launch_count(void);
 
+/* The form in which the most recent attention calls of this thread were launched (0 before the first; -1 for an unknown
+ * index).  Which form a call takes follows from its sizes alone; results agree to rounding.
+ *   GPROJ_FORM_FWD_CTAS   CTAs that share a query tile of the forward (1, 2, 4 or 8)
+ *   GPROJ_FORM_FWD_HEADS  query heads of a KV head taken as one head by the forward (1: none)
+ *   GPROJ_FORM_DQ_CTAS    CTAs that share a query tile of the dQ side (0: not run, 1 or 2)
+ *   GPROJ_FORM_DKV_CTAS   CTAs that share a key tile of the dK/dV side (0: not run, 1 or 2) */
+#define GPROJ_FORM_FWD_CTAS 0
+#define GPROJ_FORM_FWD_HEADS 1
+#define GPROJ_FORM_DQ_CTAS 2
+#define GPROJ_FORM_DKV_CTAS 3
+int gproj_last_form(int what);
+
 #ifdef __cplusplus
 }
 #endif

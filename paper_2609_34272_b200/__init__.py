@@ -8,6 +8,10 @@ from .binding import (  # noqa: F401
     FLAG_NO_Q_CORRECTION,
     FLAG_ONLY_DKV_PASS,
     FLAG_ONLY_DQ_PASS,
+    FORM_DKV_CTAS,
+    FORM_DQ_CTAS,
+    FORM_FWD_CTAS,
+    FORM_FWD_HEADS,
     FWD_FLAG_FMA_SOFTMAX,
     GprojError,
     VarlenPlan,
@@ -27,6 +31,7 @@ from .binding import (  # noqa: F401
     gproj_attn_fwd_varlen,
     gproj_attn_fwd_varlen_qk,
     gproj_last_device_status,
+    gproj_last_form,
     gproj_last_launch_count,
     gproj_selftest_wait_timeout,
     status_string,

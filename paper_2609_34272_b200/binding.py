@@ -18,6 +18,7 @@ FLAG_NO_K_CORRECTION = 2
 FLAG_ONLY_DQ_PASS = 4
 FLAG_ONLY_DKV_PASS = 8
 FWD_FLAG_FMA_SOFTMAX = 1
+FORM_FWD_CTAS, FORM_FWD_HEADS, FORM_DQ_CTAS, FORM_DKV_CTAS = range(4)
 
 STATIC_SCRATCH_BYTES = 16 << 20
 
@@ -29,7 +30,7 @@ EXPORTS = ("gproj_attn_fwd", "gproj_attn_bwd_workspace_bytes", "gproj_attn_bwd",
            "gproj_attn_host_staging_bytes", "gproj_attn_fwd_bwd_host", "gproj_key_smooth", "gproj_key_smooth_varlen",
            "gproj_fp32_attn_saved_bytes", "gproj_fp32_attn_fwd", "gproj_fp32_attn_bwd",
            "gproj_last_device_status", "gproj_selftest_wait_timeout",
-           "gproj_status_string", "gproj_last_launch_count")
+           "gproj_status_string", "gproj_last_launch_count", "gproj_last_form")
 
 _lib = None
 
@@ -108,6 +109,8 @@ def load():
         lib.gproj_status_string.argtypes = [i]
         lib.gproj_last_launch_count.restype = i
         lib.gproj_last_launch_count.argtypes = []
+        lib.gproj_last_form.restype = i
+        lib.gproj_last_form.argtypes = [i]
         _lib = lib
     return _lib
 
@@ -385,6 +388,11 @@ def gproj_selftest_wait_timeout(device=None):
 
 def gproj_last_launch_count() -> int:
     return int(load().gproj_last_launch_count())
+
+
+def gproj_last_form(what) -> int:
+    """Form of this thread's most recent launch (``FORM_*``): CTAs that share a tile, query heads taken as one."""
+    return int(load().gproj_last_form(int(what)))
 
 
 class VarlenPlan:

@@ -65,6 +65,7 @@ std::mutex g_pipe_mutex;   // serialises the host-buffer entry point's use of th
 DeviceState g_dev[kMaxDevices];
 EncodeTiledFn g_encode = nullptr;
 thread_local int tl_launch_count = 0;
+thread_local int tl_form[4] = {};   // gproj_last_form
 
 template <typename Kernel>
 cudaError_t allow_smem(Kernel kernel, int bytes) {
@@ -380,6 +381,7 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
   const bool fma = (fwd_flags & GPROJ_FWD_FLAG_FMA_SOFTMAX) != 0;
   if (int rc = check_shape(B, H, N, d)) return rc;
   if (Hkv <= 0 || H % Hkv != 0 || check_shape(B, Hkv, Nk, d) != GPROJ_OK) return GPROJ_ERR_SHAPE;
+  const int Hq = H;
   int G = H / Hkv;
   if (!aligned16(Q) || !aligned16(K) || !aligned16(V) || !aligned16(O) || (reinterpret_cast<uintptr_t>(LSE) & 3u))
     return GPROJ_ERR_ALIGN;
@@ -414,8 +416,10 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
   ItemOrder fwd_order = item_order(BH, total_items / BH, tile_group_of(plan != nullptr, causal != 0, BH, total_items / BH, 2 * static_cast<size_t>(BHkv) * Nk * d * 2, st->sm_count,
                                                             tiles_per_item == 2 ? 1.45 : 6.8));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  tl_form[GPROJ_FORM_FWD_HEADS] = Hkv == H ? Hq / Hkv : 1;
   const int (&fit)[4] = st->fwd_clusters[d == 128];
   const int lg = (tiles_per_item == 1 && !fma && total_items <= fit[1]) ? fwd_cluster_log2(total_items, ((seqs ? longest_keys(*seqs) : Nk) + 127) / 128, fit) : 0;
+  tl_form[GPROJ_FORM_FWD_CTAS] = 1 << lg;
   if (lg > 0 || fold > 0) {
     auto kernel = d == 64 ? (causal ? attn_fwd_kernel<64, true, false, 3> : attn_fwd_kernel<64, false, false, 3>)
                           : (causal ? attn_fwd_kernel<128, true, false, 3> : attn_fwd_kernel<128, false, false, 3>);
@@ -557,6 +561,8 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
   const DealForm dq_form = run_dq ? deal_form_of(seqs, false, N, Nk, causal != 0, 1, BH, n_qt, st->sm_count, dq_fit, d == 64 ? DealCosts{64, 3.8, 3.0} : DealCosts{64, 3.0, 8.0}) : none;
   const DealForm dkv_form = run_dkv ? deal_form_of(seqs, true, N, Nk, causal != 0, G, BHkv, n_kt, st->sm_count, dkv_fit, d == 64 ? DealCosts{128, 2.3, 1.5} : DealCosts{64, 3.0, 4.0}) : none;
   const bool dq_pairs = dq_form.pairs, dkv_pairs = dkv_form.pairs;
+  tl_form[GPROJ_FORM_DQ_CTAS] = run_dq ? (dq_pairs ? 2 : 1) : 0;
+  tl_form[GPROJ_FORM_DKV_CTAS] = run_dkv ? (dkv_pairs ? 2 : 1) : 0;
   group_q.solo = dq_form.solo;
   group_kv.solo = dkv_form.solo;
   const bool dq_short = run_dq && d == 128 && !dq_pairs && dq_short_tiles(seqs ? walked_key_tiles(*seqs) : fwd_key_tiles(N, Nk, causal != 0), n_qt, causal != 0);
@@ -997,6 +1003,8 @@ const char *gproj_status_string(int status) {
 }
 
 int gproj_last_launch_count(void) { return tl_launch_count; }
+
+int gproj_last_form(int what) { return what >= 0 && what < 4 ? tl_form[what] : -1; }
 
 // ---- fused FP32 attention (comparison arm; plain SIMT arithmetic) ------------------------------------------------------
 size_t gproj_fp32_attn_saved_bytes(int B, int H, int N, int d) {

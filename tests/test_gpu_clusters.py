@@ -1,6 +1,8 @@
 """Kernels that run as thread-block clusters, at the edges of their dispatch rules (through the C ABI, against the oracle).
 
-Tolerances as in the other parity tests: 1 % relative L2 against FP64 (BF16 operands leave 0.2 %), LSE to 1e-4 + 1e-5 |LSE|.
+Tolerances: BF16 operands and results leave 0.11 to 0.26 % relative L2 against FP64 at these sizes, and one BF16 step of the largest
+value is 0.4 % of it; 0.3 % and 1 % of the largest value bound them, while one wrong weight among the sixteen parts of a merge
+moves a result by several per cent.  LSE to 1e-4 + 1e-5 |LSE|.
 """
 import numpy as np
 import pytest
@@ -18,19 +20,19 @@ def tobits(t):
 
 # The forward splits a query tile's key range over 2, 4 or 8 CTAs from 16, 16 and 32 key tiles on, when the tiles are few;
 # grouped queries without a mask are folded into one head first, with one those of the second half of the list.
-FWD = [  # B, H, Hkv, Nq, Nk, causal
-    (1, 2, 2, 128, 1921, True), (1, 2, 2, 130, 2048, False), (13, 3, 3, 1, 2047, True), (1, 2, 2, 257, 4100, True),
-    (1, 1, 1, 64, 5000, False), (1, 8, 2, 16, 4096, True), (9, 6, 2, 127, 2500, True), (1, 4, 1, 33, 300, True),
-    (1, 4, 2, 100, 40, True), (1, 6, 2, 200, 2100, False), (1, 8, 1, 1, 1, True), (3, 4, 1, 96, 2049, True),
-    (40, 8, 2, 1, 300, True), (50, 8, 2, 20, 130, True), (70, 8, 1, 33, 300, True), (3, 64, 8, 5, 2300, True), (20, 12, 3, 60, 2100, True),
-    (8, 16, 4, 16, 8192, True), (60, 8, 1, 3, 2, True),
+FWD = [  # B, H, Hkv, Nq, Nk, causal, CTAs per tile, query heads taken as one (at d = 64, at d = 128)
+    (1, 2, 2, 128, 1921, True, 4, 1, 1), (1, 2, 2, 130, 2048, False, 4, 1, 1), (13, 3, 3, 1, 2047, True, 2, 1, 1), (1, 2, 2, 257, 4100, True, 8, 1, 1),
+    (1, 1, 1, 64, 5000, False, 8, 1, 1), (1, 8, 2, 16, 4096, True, 8, 1, 1), (9, 6, 2, 127, 2500, True, 2, 1, 1), (1, 4, 1, 33, 300, True, 1, 1, 1),
+    (1, 4, 2, 100, 40, True, 1, 1, 1), (1, 6, 2, 200, 2100, False, 4, 3, 3), (1, 8, 1, 1, 1, True, 1, 8, 1), (3, 4, 1, 96, 2049, True, 4, 1, 1),
+    (40, 8, 2, 1, 300, True, 1, 4, 4), (50, 8, 2, 20, 130, True, 1, 4, 4), (70, 8, 1, 33, 300, True, 1, 8, 8), (3, 64, 8, 5, 2300, True, 4, 8, 8),
+    (20, 12, 3, 60, 2100, True, 1, 4, 4), (8, 16, 4, 16, 8192, True, 4, 4, 4), (60, 8, 1, 3, 2, True, 1, 8, 8),
 ]
 
 
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("shape", FWD)
 def test_forward_with_the_key_range_split_over_a_cluster(shape, d):
-    B, H, Hkv, Nq, Nk, causal = shape
+    B, H, Hkv, Nq, Nk, causal, ctas, heads64, heads128 = shape
     gen = torch.Generator().manual_seed(Nq * 7 + Nk + d)
     Q = torch.randn(B, H, Nq, d, generator=gen).to(torch.bfloat16)
     K = (torch.randn(B, Hkv, Nk, d, generator=gen) + 0.5).to(torch.bfloat16)
@@ -39,14 +41,15 @@ def test_forward_with_the_key_range_split_over_a_cluster(shape, d):
     q, k, v = Q.cuda(), K.cuda(), V.cuda()
     O, LSE = torch.full_like(q, float("nan")), torch.full(q.shape[:3], float("nan"), device="cuda")
     g.gproj_attn_fwd_rect(q, k, v, d ** -0.5, causal, O=O, LSE=LSE)
+    assert g.gproj_last_form(g.FORM_FWD_CTAS) == ctas and g.gproj_last_form(g.FORM_FWD_HEADS) == (heads64 if d == 64 else heads128)
     rc, detail = g.gproj_last_device_status()
     assert rc == 0, hex(detail)
     O, LSE = O.float().cpu().numpy().astype(np.float64), LSE.cpu().numpy().astype(np.float64)
     empty = np.isinf(ex["LSE"])
     assert np.array_equal(np.isposinf(LSE), empty) and np.all(O[empty] == 0.0) and np.all(np.isfinite(O))
     assert np.all(np.abs(LSE[~empty] - ex["LSE"][~empty]) <= 1e-4 + 1e-5 * np.abs(ex["LSE"][~empty]))
-    assert oracle.rel_l2_percent(O, ex["O"]) <= 1.0
-    assert np.abs(O - ex["O"]).max() <= 0.03 * np.abs(ex["O"]).max()
+    assert oracle.rel_l2_percent(O, ex["O"]) <= 0.3
+    assert np.abs(O - ex["O"]).max() <= 0.01 * np.abs(ex["O"]).max()
 
 
 # query heads folded on one CTA per tile; clusters with and without folding; the last without either, for comparison
@@ -89,6 +92,7 @@ def test_packed_forward_with_split_keys_repeats_bitwise(causal):
     plan = g.VarlenPlan(cu, causal)
     q, k, v = Q.cuda(), K.cuda(), V.cuda()
     O, LSE = g.gproj_attn_fwd_varlen(q, k, v, plan, 0.125)
+    assert g.gproj_last_form(g.FORM_FWD_CTAS) == 2
     for _ in range(5):
         O2, LSE2 = g.gproj_attn_fwd_varlen(q, k, v, plan, 0.125)
         assert torch.equal(O, O2) and torch.equal(LSE, LSE2)
@@ -98,7 +102,7 @@ def test_packed_forward_with_split_keys_repeats_bitwise(causal):
         if b > a:
             part = lambda t: tobits(t[None, :, a:b])
             ex = oracle.attn_rect_f64(part(Q), part(K), part(V), part(torch.zeros_like(Q)), 0.125, causal)
-            assert oracle.rel_l2_percent(O[:, a:b].float().cpu().numpy()[None], ex["O"]) <= 1.0
+            assert oracle.rel_l2_percent(O[:, a:b].float().cpu().numpy()[None], ex["O"]) <= 0.3
 
 
 @pytest.mark.parametrize("rows,d", [(1, 64), (7, 128), (8, 64), (255, 64), (257, 64), (129, 128), (513, 64), (2047, 64), (4097, 64), (2049, 128), (9000, 64)])
@@ -116,11 +120,12 @@ def test_key_smoothing_at_the_edges_of_its_row_split(rows, d):
 
 # Both backward kernels share tiles between two CTAs where whole tiles cannot be dealt evenly: one-step tiles (a CTA without a
 # step of its own), odd and even step counts, query heads split between the CTAs, ragged ends, keys no query sees, rows that
-# see no key, several tiles per cluster.
-BWD = [  # B, H, Hkv, Nq, Nk, causal
-    (1, 1, 1, 700, 700, True), (1, 3, 1, 333, 333, True), (2, 4, 2, 1000, 1000, False), (1, 2, 1, 900, 130, True),
-    (1, 2, 1, 641, 257, False), (1, 2, 2, 600, 1100, True), (1, 8, 2, 1025, 1025, True), (1, 1, 1, 5, 1700, True),
-    (2, 5, 5, 1290, 1290, True),
+# see no key; the last four have more tiles than the 74 clusters that run at once, i.e. two tiles for some of them (three on
+# the dK/dV side of the last one and, at d = 64, on its dQ side).
+BWD = [  # B, H, Hkv, Nq, Nk, causal, CTAs per tile: dQ and dK/dV side at d = 64, the same at d = 128
+    (1, 1, 1, 700, 700, True, 2, 2, 1, 2), (1, 3, 1, 333, 333, True, 1, 2, 1, 2), (2, 4, 2, 1000, 1000, False, 2, 2, 1, 2), (1, 2, 1, 900, 130, True, 1, 2, 1, 1),
+    (1, 2, 1, 641, 257, False, 1, 2, 1, 2), (1, 2, 2, 600, 1100, True, 2, 2, 2, 2), (1, 8, 2, 1025, 1025, True, 2, 2, 1, 2), (1, 1, 1, 5, 1700, True, 2, 1, 2, 1),
+    (2, 5, 5, 1290, 1290, True, 2, 2, 1, 2), (1, 4, 4, 2500, 2500, True, 2, 2, 2, 2), (1, 6, 3, 2500, 2500, True, 2, 2, 2, 2), (1, 6, 6, 3100, 3100, True, 2, 2, 1, 2),
 ]
 
 
@@ -128,7 +133,7 @@ BWD = [  # B, H, Hkv, Nq, Nk, causal
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("shape", BWD)
 def test_backward_with_tiles_shared_by_two_ctas(shape, d, flags):
-    B, H, Hkv, Nq, Nk, causal = shape
+    B, H, Hkv, Nq, Nk, causal, *ctas = shape
     gen = torch.Generator().manual_seed(Nq + 3 * Nk + d)
     Q, dO = (torch.randn(B, H, Nq, d, generator=gen).to(torch.bfloat16) for _ in range(2))
     K = (torch.randn(B, Hkv, Nk, d, generator=gen) + 0.5).to(torch.bfloat16)
@@ -140,11 +145,12 @@ def test_backward_with_tiles_shared_by_two_ctas(shape, d, flags):
     for _ in range(3):
         out = [torch.full_like(t, float("nan")) for t in (q, k, v)]
         runs.append(g.gproj_attn_bwd_rect(q, k, v, O, LSE, u, d ** -0.5, causal, flags=flags, dQ=out[0], dK=out[1], dV=out[2]))
+    assert [g.gproj_last_form(g.FORM_DQ_CTAS), g.gproj_last_form(g.FORM_DKV_CTAS)] == (ctas[:2] if d == 64 else ctas[2:])
     rc, detail = g.gproj_last_device_status()
     assert rc == 0, hex(detail)
     assert all(torch.equal(a, b) for r in runs[1:] for a, b in zip(runs[0], r))
     for n, t in zip(("dQ", "dK", "dV"), runs[0]):
         t = t.float().cpu().numpy().astype(np.float64)
         assert np.all(np.isfinite(t)), n
-        assert oracle.rel_l2_percent(t, ex[n]) <= (1.0 if flags == 0 else 5.0), n     # 5 %: uncorrected, as in test_gpu_rect.py
-        assert np.abs(t - ex[n]).max() <= (0.03 if flags == 0 else 0.15) * np.abs(ex[n]).max(), n
+        assert oracle.rel_l2_percent(t, ex[n]) <= 0.3, n
+        assert np.abs(t - ex[n]).max() <= 0.01 * np.abs(ex[n]).max(), n
