@@ -203,7 +203,8 @@ int gproj_attn_bwd_varlen_qk(const void *Q, const void *K, const void *V, const 
  * Forward and backward in one call from HOST buffers (a convenience around the entry points above; the paper's
  * Algorithm 1 starts from tensors already on the device).  Q, K, V, dO are copied to the device, the forward
  * (Eq. "gproj-forward") and the backward (Algorithm 1) run, and dQ, dK, dV (and O, LSE when those pointers are not NULL)
- * are copied back.  Large problems are cut into up to 16 slabs of whole KV heads (2 to 4 MiB of Q each) that are pipelined:
+ * are copied back.  Large problems are cut into up to 16 slabs of whole KV heads (one, and one more for every 4 MiB of Q,
+ * but no more than leave 128 key tiles to a slab on average; the last one is smaller) that are pipelined:
  * the kernels run on `stream`, the copies in and out on two internal streams, ordered by events so that nothing of the call
  * starts before the work already queued on `stream` and `stream` reaches the end of the call only after the last copy-out.
  *   - Q, K, V, dO, O, LSE, dQ, dK, dV are HOST pointers with the layouts of gproj_attn_fwd_gqa / gproj_attn_bwd_gqa.  Page-locked

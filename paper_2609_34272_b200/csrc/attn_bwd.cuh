@@ -95,11 +95,11 @@ struct BwdCfg {
   static constexpr int kDqStagingBytes = 4 * 32 * 128;             // each epilogue warp: 32 rows x 64 columns of dQ
   static constexpr int kDqSmemBytes = kDqResBufs * 2 * kBigTileBytes + kDqStages * kDqStageBytes + kDqStagingBytes + 1024;
   // dK/dV-side kernel: K, V resident; ring of (Q, dO, Z, stats) step tiles
-  static constexpr int kDkvStages = (D == 64) ? 5 : 3;
+  static constexpr int kDkvStages = 3;                             // (this kernel runs at d = 128 only)
   static constexpr int kDkvStageBytes = 3 * kStepTileBytes + kExtBlockBytes;   // + the step's 64-row block of the row-constant tile
   static constexpr int kDkvStagingBytes = 4 * 32 * 64;             // each epilogue warp: 32 rows x 32 columns of dK or dV
   static constexpr int kDkvSmemBytes = 2 * kBigTileBytes + kDkvStages * kDkvStageBytes + kDkvStagingBytes + 1024;
-  static_assert(kDqStages >= kNB + 1 && kDkvStages >= kNB + 1, "a stage stays busy until its second-stage MMAs finish");
+  static_assert(kDqStages >= kNB + 1 && (D == 64 || kDkvStages >= kNB + 1), "a stage stays busy until its second-stage MMAs finish");
 };
 
 // Item number -> (rank of the tile in decreasing work, head).  Items are dealt in groups of `group` consecutive ranks of
@@ -817,7 +817,7 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 rows
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t *sK = smem;
   uint8_t *sV = sK + C::kBigTileBytes;
-  uint8_t *sStage = sV + C::kBigTileBytes;   // stage s: Q, dO, Z step tiles, then 64 x {-LSE log2 e} and 64 x {-D}
+  uint8_t *sStage = sV + C::kBigTileBytes;   // stage s: Q, dO, Z step tiles, then the 64-row block of the row-constant tile
   uint8_t *sStaging = sStage + S * C::kDkvStageBytes;   // epilogue warp w: 2048 w
 
   __shared__ uint64_t bar_res_full, bar_res_free, bar_q_full[S], bar_q_empty[S];

@@ -254,9 +254,9 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
       }
     }
   } else if (warp == 1) {
-    // ---------------------------------------------------------------- tensor-core issuer 1: S^T = K Q^T, dP^T = V dO^T
+    // ---------------------------------------------------------------- tensor-core issuer 1: S^T = K Q^T
     constexpr uint32_t idesc_s = idesc_bf16_f32(128, 128, 0, 0);   // [128 keys] x [128 queries], contraction over d
-    const SmemDesc dscK = make_smem_desc(smem_u32(sK), 16, 1024), dscV = make_smem_desc(smem_u32(sV), 16, 1024);
+    const SmemDesc dscK = make_smem_desc(smem_u32(sK), 16, 1024);
     const SmemDesc dscQ0 = make_smem_desc(smem_u32(sStage), 16, 1024);
     const SmemDesc dscOnes = make_smem_desc_noswizzle(smem_u32(s_ones) + 128, 128, 0);                 // (ones, zeros), every row group the same
     const SmemDesc dscExt0 = make_smem_desc_noswizzle(smem_u32(sStage + 3 * C::kTileBytes), 128, 256);
@@ -269,7 +269,7 @@ bwd_dkv_w128_kernel(const __grid_constant__ CUtensorMap tmK,    // box 64 x 128 
         mbar_wait(&bar_q_full[st], (g / S) & 1, ab, kWkQ);
         if (g >= 2) mbar_wait(&bar_q_empty[(g - 2) % S], ((g - 2) / S) & 1, ab, kWkSFree);   // step g - 2 done: its r, t are consumed
         tc_fence_after();
-        const SmemDesc dscQ = dscQ0.advanced(st * C::kDkvStageBytes), dscdO = dscQ.advanced(C::kTileBytes);
+        const SmemDesc dscQ = dscQ0.advanced(st * C::kDkvStageBytes);
         const uint32_t tS = tmem_base + (sb ? C::kColZ : C::kColX);
         if (elect_one_sync()) {
 #pragma unroll

@@ -207,8 +207,12 @@ size_t align256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
 // Launch `kernel`, in clusters of `cluster` CTAs.  With overlap_previous it may be scheduled while the kernel before it in
 // the stream still runs (programmatic dependent launch): every kernel launched so waits, by griddep_wait, before it touches
 // memory that an earlier kernel may read or write, so only its set-up (barriers, TMEM, descriptors) and, on the dK/dV
-// side, the loads of K and V overlap.  Measured with calls back to back (with the attribute on the dK/dV side alone -> on
-// the dQ side too): backward, 8 heads x 4096 x 128: 145.1 -> 141.8 us.
+// side, the loads of K and V overlap.  Measured with
+// calls back to back (with the attribute on the dK/dV side alone -> on the dQ side too): backward, 8 heads x 4096 x 128: 145.1 -> 141.8
+// us.  The dQ side and the forward with clusters or folded heads are always launched so, the other forwards where launch_fwd says.
+// dQ side with many items per CTA, normal -> early: 96 heads x 1000 x 128: 83.9 -> 80.8 us; 64 x 16 heads x 256 x 64, causal: 95.8 -> 93.4
+// (backward 150.6 -> 144.4); 200 packed documents of 30 to 300 rows, 16 heads, d = 64: 252.3 -> 250.1; 24 of 19446 rows, d = 128: 376.5 -> 379.8 (backward
+// 821 -> 818).  Folded forward, 32 x (64, 4 heads) x 20 behind 600 keys, d = 64: 41.0 -> 37.9 us, 256 x (32, 8) x 1 behind 1000: 174.9 -> 172.3.
 template <typename... Params, typename... Args>
 void launch_after(void (*kernel)(Params...), dim3 grid, int cluster, int threads, size_t smem, cudaStream_t s, bool overlap_previous,
                   Args... args) {
@@ -573,7 +577,7 @@ int launch_bwd(const void *Q, const void *K, const void *V, const void *O, const
 #define GPROJ_LAUNCH_BWD(DD, CC)                                                                                        \
   do {                                                                                                                  \
     if (run_dq)                                                                                                         \
-      launch_after(dq_pairs ? bwd_dq_kernel<DD, CC, 2, false> : dq_short ? bwd_dq_kernel<DD, CC, 1, DD == 128> : bwd_dq_kernel<DD, CC, 1, false>, grid, dq_pairs ? 2 : 1, BwdCfg<DD>::kDqThreads, BwdCfg<DD>::kDqSmemBytes, s, true,                               \
+      launch_after(dq_pairs ? bwd_dq_kernel<DD, CC, 2, false> : dq_short ? bwd_dq_kernel<DD, CC, 1, true> : bwd_dq_kernel<DD, CC, 1, false>, grid, dq_pairs ? 2 : 1, BwdCfg<DD>::kDqThreads, BwdCfg<DD>::kDqSmemBytes, s, true,                               \
           mQ128, mdO128, mK64, mV64, static_cast<const __nv_bfloat16 *>(Q), Ob, dOb, LSE, stats, static_cast<__nv_bfloat16 *>(dQ), Zneg, plan_q, nblk,   \
           N, Nk, BH, H, G, total_tiles, group_q, scale_log2, softmax_scale,                                           \
           flags,                                                                                                        \
@@ -822,7 +826,8 @@ int gproj_attn_fwd_bwd_host(const void *Q, const void *K, const void *V, const v
 
   // The (batch, KV head) axis is cut into slabs of whole KV heads with their query heads (contiguous in every tensor), and
   // the slabs are pipelined: copy-in of slab c + 1 and copy-out of slab c - 1 run on two internal streams while the
-  // caller's stream computes slab c.  2 to 4 MiB of Q and at least 128 key tiles per slab: every copy costs some 4 us of
+  // caller's stream computes slab c.  One slab and one more for every 4 MiB of Q, but no more than leave 128 key tiles to a slab on
+  // average, than there are KV heads, and than 16; the last one is about half as large as the others.  Every copy costs some 4 us of
   // its direction beyond its bytes and the two directions share about 80 GB/s, so many small slabs are slower than few
   // large ones, while the last slab's kernels and copy-out stay exposed.  The forward starts without dO, and dQ leaves while
   // dK and dV are computed.  Measured, before (2 MiB slabs, all inputs first, all gradients together) -> now: 16 heads x 4096

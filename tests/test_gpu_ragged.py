@@ -168,7 +168,9 @@ def test_many_heads_long_causal_matches_chunks_of_heads(d):
 @pytest.mark.parametrize("d,causal", [(64, True), (128, False)])
 def test_head_shards_give_the_bits_of_the_whole_call(d, causal):
     # The multi-GPU launch cuts the flat (batch, head) axis into contiguous shares (one per rank, no exchange).  Run the
-    # shares one after the other on this GPU: laid side by side they must be the whole call's outputs bit for bit.
+    # shares one after the other on this GPU: laid side by side they must be the whole call's outputs bit for bit, as long
+    # as share and whole take the same form, as here (where two CTAs share a tile in one of them only, its two parts are added
+    # in another order and the results agree to rounding).
     from paper_2609_34272_b200.sharding import shard_heads
     B, H, N = 2, 5, 640
     gen = torch.Generator().manual_seed(606 + d)
