@@ -48,9 +48,11 @@ def test_a_cta_that_skips_its_work_still_waits_for_the_previous_kernel():
     # after a wait has given up, the CTAs of later launches return at once; one that was launched early (programmatic
     # dependent launch) must not let its grid end before the one in front of it, which may still be writing
     found = 0
-    for name in ("attn_fwd.cuh", "attn_bwd.cuh", "attn_bwd_w128.cuh"):
-        for line in open(os.path.join(CSRC, name)):
-            if "cta_skip != 0" in line and "return" in line:
-                found += 1
-                assert line.index("griddep_wait();") < line.index("return"), (name, line)
+    for name, kernels in (("attn_fwd.cuh", 1), ("attn_bwd.cuh", 2), ("attn_bwd_w128.cuh", 1)):
+        for body in open(os.path.join(CSRC, name)).read().split("__global__")[1:]:
+            skip = re.search(r"if \([^()]*cta_skip != 0\)[^;]*", body)
+            found += 1
+            # the wait stands in the branch, in front of the return, or on everybody's way before the branch
+            branch = body[skip.start():body.index("return;", skip.start())]
+            assert "griddep_wait();" in branch or "griddep_wait();" in body[:skip.start()], name
     assert found == 4
