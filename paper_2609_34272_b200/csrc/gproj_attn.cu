@@ -434,8 +434,14 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
     tl_launch_count = 1;
     return GPROJ_OK;
   }
-  if (seqs && total_items > st->sm_count && total_items <= 16LL * st->sm_count)
-    fwd_order.solo = solo_ctas(tile_steps(*seqs, false, 128, 1), BH, st->sm_count, 2.1);
+  bool sep_rings = d == 128 && tiles_per_item == 1 && total_items <= st->sm_count;
+  if (seqs && total_items > st->sm_count && total_items <= 16LL * st->sm_count) {
+    const std::vector<int> key_tiles = tile_steps(*seqs, false, 128, 1);
+    fwd_order.solo = solo_ctas(key_tiles, BH, st->sm_count, 2.1);
+    sep_rings = d == 128 && fwd_separate_rings(key_tiles, BH, st->sm_count, fwd_order.solo);
+  } else if (d == 128 && !sep_rings && tiles_per_item == 1) {
+    sep_rings = fwd_separate_rings(seqs ? walked_key_tiles(*seqs) : fwd_key_tiles(N, Nk, causal != 0), n_qt);
+  }
   const dim3 grid(static_cast<unsigned>(total_items < st->sm_count ? total_items : st->sm_count));   // persistent
   // Start beside the previous kernel only with at most two items per CTA.  CTAs that start early take the SMs in the order in
   // which the previous kernel leaves them; launched normally, neighbouring CTAs sit side by side in a TPC and walk
@@ -455,7 +461,7 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
   // they alternate in the exponential phase (measured to pay there only).
   const bool split = (tiles_per_item == 1), turns = (d == 128) && !split && !fma;
   if (d == 64) { if (split) GPROJ_LAUNCH_FWD_F(64, 2); else GPROJ_LAUNCH_FWD_F(64, 0); }
-  else if (split && (total_items <= st->sm_count || fwd_separate_rings(seqs ? walked_key_tiles(*seqs) : fwd_key_tiles(N, Nk, causal != 0), n_qt))) GPROJ_LAUNCH_FWD_F(128, 4);
+  else if (split && sep_rings) GPROJ_LAUNCH_FWD_F(128, 4);
   else if (split) GPROJ_LAUNCH_FWD_F(128, 2);
   else if (turns) GPROJ_LAUNCH_FWD_C(128, false, 1);
   else GPROJ_LAUNCH_FWD_F(128, 0);

@@ -26,9 +26,10 @@ inline long long fwd_key_tiles(int lq, int lk, bool causal) {
 }
 
 // Forward at d = 128 with the key range of a tile split between the warpgroups: separate rings for K and V (see attn_fwd.cuh)?
-// From three key tiles per item on (key_tiles, tiles: of one head), and always with one item per CTA.  Measured, one
-// ring -> two, 16 query / 4 KV heads, 40000 rows in sequences of one length, causal: 512 rows (2.5 key tiles per item) 228 -> 239 us, 640
-// (3.0) 256 -> 256, 1024 (4.5) 332 -> 312; not causal: 256 (2) 177 -> 190, 384 (3) 240 -> 234; 16 heads x 500 (64 items): 11.0 -> 10.4.
+// From three key tiles per item on (key_tiles, tiles: of one head, or of the items of one CTA), and always with one item per CTA.
+// Measured, one ring -> two, 16 query / 4 KV heads, 40000 rows in sequences of one length, causal: 512 rows (2.5 key tiles per item)
+// 228 -> 239 us, 640 (3.0) 256 -> 256, 1024 (4.5) 332 -> 312; not causal: 256 (2) 177 -> 190, 384 (3) 240 -> 234; 16 heads x 500 (64
+// items): 11.0 -> 10.4.
 inline bool fwd_separate_rings(long long key_tiles, long long tiles) { return key_tiles >= 3 * tiles; }
 
 // dQ side at d = 128: are the tiles so short that the compute warpgroups should prepare the row constants (SHORT in attn_bwd.cuh)?
@@ -131,9 +132,9 @@ inline int longest_keys(const PackedSeqs &ps) {
   return most;
 }
 
-// Longest CTA of the static deal (TileSched, walked item by item) of `items` items.  work_of is called once for every item, in order.
+// What each CTA gets in the static deal (TileSched, walked item by item) of `items` items.  work_of is called once for every item, in order.
 template <typename WorkOf>
-double deal_makespan(long long items, int ctas, WorkOf work_of, int solo = 0) {
+std::vector<double> deal_loads(long long items, int ctas, WorkOf work_of, int solo = 0) {
   const int G = static_cast<int>(std::min<long long>(items, ctas)), W = G - solo;
   std::vector<double> load(static_cast<size_t>(G));
   long long lin = 0;
@@ -143,20 +144,41 @@ double deal_makespan(long long items, int ctas, WorkOf work_of, int solo = 0) {
     if (odd) for (int c = 0; c < n; ++c) load[static_cast<size_t>(G - 1 - c)] += work_of(lin++);
     else     for (int c = 0; c < n; ++c) load[static_cast<size_t>(solo + c)] += work_of(lin++);
   }
+  return load;
+}
+// The longest of them.
+template <typename WorkOf>
+double deal_makespan(long long items, int ctas, WorkOf work_of, int solo = 0) {
+  const std::vector<double> load = deal_loads(items, ctas, work_of, solo);
   return *std::max_element(load.begin(), load.end());
 }
 
 // ... of `heads` copies of every tile, with the cost that cost_of gives for its steps.
 template <typename CostOf>
-double deal_tiles(const std::vector<int> &steps, int heads, int ctas, CostOf cost_of, int solo = 0) {
+std::vector<double> deal_tile_loads(const std::vector<int> &steps, int heads, int ctas, CostOf cost_of, int solo = 0) {
   size_t k = 0;
   int left = 0;
   double cost = 0.0;
-  return deal_makespan(static_cast<long long>(steps.size()) * heads, ctas, [&](long long) {
+  return deal_loads(static_cast<long long>(steps.size()) * heads, ctas, [&](long long) {
     if (left == 0) { cost = cost_of(steps[k++]); left = heads; }
     --left;
     return cost;
   }, solo);
+}
+template <typename CostOf>
+double deal_tiles(const std::vector<int> &steps, int heads, int ctas, CostOf cost_of, int solo = 0) {
+  const std::vector<double> load = deal_tile_loads(steps, heads, ctas, cost_of, solo);
+  return *std::max_element(load.begin(), load.end());
+}
+
+// fwd_separate_rings for a packed call of few items per CTA: what counts is the CTA that takes longest (its items' key tiles, and
+// 2.1 more for each), which has long tiles where the others have many short ones.  48 documents of 6288 rows together, 2 heads, causal: one
+// ring 23.5 us, two 19.8; 49 pairs of 3485 queries and 13379 keys, 4 heads: 26.9, 23.1.
+inline bool fwd_separate_rings(const std::vector<int> &key_tiles, int heads, int sms, int solo) {
+  const std::vector<double> load = deal_tile_loads(key_tiles, heads, sms, [](int n) { return n + 2.1; }, solo);
+  const std::vector<double> items = deal_tile_loads(key_tiles, heads, sms, [](int) { return 1.0; }, solo);
+  const size_t c = static_cast<size_t>(std::max_element(load.begin(), load.end()) - load.begin());
+  return load[c] - 2.1 * items[c] >= 3.0 * items[c] - 1e-6;
 }
 
 // TileSched's solo CTAs for `heads` copies of tiles with the given costs (decreasing): those whose first item is longer than

@@ -18,6 +18,7 @@ int folds(int kv_heads, int G, int N, int Nk, int d) { const int fit[4] = {0, 74
 int smooth(long long pairs, long long rows, int longest, int d) { return smooth_cluster(pairs, rows, longest, d, 148); }
 long long key_tiles(int lq, int lk, int causal) { return fwd_key_tiles(lq, lk, causal != 0); }
 int short_tiles(long long key_tiles, long long tiles, int causal) { return dq_short_tiles(key_tiles, tiles, causal != 0); }
+int packed_rings(const int *key_tiles, int n, int heads, int solo) { return fwd_separate_rings(std::vector<int>(key_tiles, key_tiles + n), heads, 148, solo); }
 int rings(long long key_tiles, long long tiles) { return fwd_separate_rings(key_tiles, tiles); }
 double deal(const int *steps, int n, int heads, int ctas, int solo, double per_item) {
   return deal_tiles(std::vector<int>(steps, steps + n), heads, ctas, [&](int s) { return s + per_item; }, solo);
@@ -135,3 +136,13 @@ def test_tiles_are_not_listed_where_the_deal_does_not_matter(rules):
     short = [128 * i for i in range(101)]
     cu_q, cu_k = ((ctypes.c_int * 102)(0, *[first + x for x in short]) for first in (300, 9000))
     assert rules.form(cu_q, cu_k, 101, 0, 1, 0, 1, 12, 103) == 36                   # three long tiles of 12 heads, 1200 short ones
+
+
+def test_separate_rings_of_a_packed_call_follow_its_longest_cta(rules):
+    def rings(lens, heads, solo=0):
+        tiles = sorted((-(-min(r + 128, n) // 128) for n in lens for r in range(0, n, 128)), reverse=True)
+        return rules.packed_rings((ctypes.c_int * len(tiles))(*tiles), len(tiles), heads, solo)
+    # sequences of one length: as their mean says
+    assert [rings([n] * 60, 16) for n in (128, 256, 512, 1024)] == [0, 0, 0, 1]
+    # a few long ones among many short ones: one CTA with the longest tile, the others with up to three of one key tile
+    assert rings([2000] + [100] * 60, 4) == 1 and rings([100] * 80, 4) == 0
