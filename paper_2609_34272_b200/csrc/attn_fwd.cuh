@@ -128,6 +128,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) cta_skip = *reinterpret_cast<volatile int *>(status);
   __syncthreads();
+  if (MODE == 1 && cta_skip != 0) { griddep_wait(); return; }   // see below
 
   const int n_qt = (N + C::kBlockM - 1) / C::kBlockM;   // the last tile may be ragged: rows past N load as zero, stores clip
   const int TPI = tiles_per_item;                  // 2: a pair of query tiles per work item; 1: single tiles, key range split
@@ -164,9 +165,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   griddep_launch_dependents();
   // An earlier wait gave up: drain the rest of the grid quickly, but not past the kernel before this one, for whose end the
   // next kernel in the stream relies on this one.  The CTAs of a cluster wait for one another at the end, so they run on with
-  // every wait falling through instead.  (With this return above, behind a griddep_wait of its own, calls of one or two key
-  // tiles per item were up to 2.5 % slower: 584 heads x 3 queries x 4 keys, d = 128: 23.2 -> 23.8 us.)
-  if (!kCluster && cta_skip != 0) {
+  // every wait falling through instead.  Where this return stands changes the code of the softmax loop.  Above, behind a
+  // griddep_wait of its own, calls of one or two key tiles per item are up to 3 % slower (64 x 16 heads x 100 x 64: 31.7 -> 32.8 us); here,
+  // long calls with turns are (8 heads x 32768 x 128, causal: 2346 -> 2414 us).
+  if (!kCluster && MODE != 1 && cta_skip != 0) {
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem_base, C::kTmemCols);
     return;

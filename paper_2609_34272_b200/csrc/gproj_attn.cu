@@ -458,8 +458,8 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
 #define GPROJ_LAUNCH_FWD_F(DD, MM)                                                                                  \
   do { if (fma) GPROJ_LAUNCH_FWD_C(DD, true, MM); else GPROJ_LAUNCH_FWD_C(DD, false, MM); } while (0)
   // Single tiles: the two softmax warpgroups split the key range of the tile.  Pairs: one tile each, and at d = 128
-  // they alternate in the exponential phase (measured to pay there only).
-  const bool split = (tiles_per_item == 1), turns = (d == 128) && !split && !fma;
+  // they alternate in the exponential phase (measured to pay there only) unless there is one tile to a head, and no pair.
+  const bool split = (tiles_per_item == 1), turns = (d == 128) && !split && !fma && n_qt > 1;
   if (d == 64) { if (split) GPROJ_LAUNCH_FWD_F(64, 2); else GPROJ_LAUNCH_FWD_F(64, 0); }
   else if (split && sep_rings) GPROJ_LAUNCH_FWD_F(128, 4);
   else if (split) GPROJ_LAUNCH_FWD_F(128, 2);

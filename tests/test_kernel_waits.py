@@ -50,9 +50,9 @@ def test_a_cta_that_skips_its_work_still_waits_for_the_previous_kernel():
     found = 0
     for name, kernels in (("attn_fwd.cuh", 1), ("attn_bwd.cuh", 2), ("attn_bwd_w128.cuh", 1)):
         for body in open(os.path.join(CSRC, name)).read().split("__global__")[1:]:
-            skip = re.search(r"if \([^()]*cta_skip != 0\)[^;]*", body)
-            found += 1
-            # the wait stands in the branch, in front of the return, or on everybody's way before the branch
-            branch = body[skip.start():body.index("return;", skip.start())]
-            assert "griddep_wait();" in branch or "griddep_wait();" in body[:skip.start()], name
-    assert found == 4
+            for skip in re.finditer(r"if \([^()]*cta_skip != 0\)", body):
+                found += 1
+                # the wait stands in the branch, in front of the return, or on everybody's way before the branch
+                branch = body[skip.start():body.index("return;", skip.start())]
+                assert "griddep_wait();" in branch or "griddep_wait();" in body[:skip.start()], name
+    assert found == 5
