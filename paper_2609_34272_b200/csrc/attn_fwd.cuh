@@ -10,8 +10,9 @@
 //                 the other one (the tensor-core queue is only 1-2 instructions deep, hence two issuing warps: each
 //                 one's barrier polls overlap the other's MMAs).
 // Work items (template parameter MODE):
-//   pairs (0, 1)  one item = two 128-row query tiles of one (batch, head), warpgroup t <-> tile t, every K / V tile
-//                 serves both; with MODE 1 the warpgroups also take turns in the exponential phase.
+//   pairs (0)     one item = two 128-row query tiles of one (batch, head), warpgroup t <-> tile t, every K / V tile
+//                 serves both.
+//   pairs (5)     the same with separate rings for K and V (d = 128).
 //   split (2)     one item = one query tile; warpgroup t takes the key tiles j = t (mod 2) with its own running
 //                 maximum, normaliser and accumulator, and warpgroup 0 merges the two halves at the end.  Used when
 //                 pairs would leave SMs idle and for packed sequences.
@@ -25,9 +26,7 @@
 // product uses BF16(z); the running maximum is raised lazily and the accumulator rescaled only then.
 // The saved state is BF16 O (staged in the TMA layout over the consumed Q tile, written by a TMA store) and
 // FP32 LSE = alpha x_max + ln l  (Algorithm 1, "Input").
-// TMEM: S_0, S_1 (128 columns each), O_0, O_1 (d each); at d = 64 the packed P~_t have their own 64 columns, so
-// S_t of the next key tile can be issued as soon as the softmax has copied the current one to registers; at d = 128
-// TMEM is full and P~_t overwrites the first half of S_t.
+// TMEM: see FwdTmem.
 #pragma once
 #include "attn_bwd.cuh"   // TileSched
 #include "sm100_primitives.cuh"
@@ -47,16 +46,38 @@ struct FwdCfg {
   static constexpr int kStages = (D == 64) ? 4 : 2;    // ring of (K, V) tile pairs
   static constexpr int kSmemBytes = 2 * kTileBytes + kStages * 2 * kTileBytes + 1024;
   static constexpr int kTmemCols = 512;
-  static constexpr bool kSepP = (D == 64);             // P~ in its own TMEM columns
-  static constexpr uint32_t kColS = 0, kColO = 256, kColP = 256 + 2 * D;   // S_t at 128 t, O_t at 256 + D t, P_t at kColP + 64 t
+  static constexpr uint32_t kColS = 0, kColO = 256;    // O_t at 256 + D t; S_t and P~_t as in FwdTmem
   static constexpr int kThreads = 384;
+  // MODE 4 and 5 re-deal the 384 x 168 registers of the launch: with 168 the causal pairs spill 156 bytes (32 heads x 4096: 149 us, re-dealt
+  // 138; 8 x 32768: 1960, 1845).  At d = 64 it does not pay (60.4 -> 62 us).
+  static constexpr int kRegsSoftmax = 216, kRegsAux = 72;
+  static_assert(2 * kRegsSoftmax + kRegsAux <= 3 * 168, "register shares");
   static constexpr int kPartF = D + 4;                 // row stride (floats) of a part in the cluster merge
   static_assert(256 * 4 * kPartF <= 2 * kTileBytes + kStages * 2 * kTileBytes, "the cluster merge goes over the Q and K / V tiles");
 };
 
+// TMEM columns of the scores and the probabilities.  At d = 64 there is room for S_0, S_1, P~_0 and P~_1.  At d = 128 there is
+// not.  With P~_t over S_t a warpgroup's key tile is a serial chain of scores (512 clk), softmax (2600) and P~_t V (512), since the
+// next scores have to wait for the last product: 3900 clk for two tiles in flight.  MODE 4 and 5 keep P~_0 and P~_1 apart and
+// one score tile that the warpgroups, half a tile apart, use in turn: it is free again as soon as one of them has copied its
+// scores to registers, and the other's are computed while that one is in its exponentials.  Bound then by the exponentials of
+// two warps per scheduler (2900 clk).  Measured (forward alone, calls back to back in a graph), P~ over S -> one score tile: pairs,
+// causal: 8 heads x 32768: 2260 -> 1845 us; 32 x 4096: 167 -> 138; 96 x 1000: 49.0 -> 42.0; 256 x 500: 50.9 -> 43.6; not causal: 32 x
+// 8192: 1050 -> 912; single tiles, causal: 8 x 4096: 42.6 -> 36; 8 x 2300: 25.3 -> 21.1; 24 packed documents, 16676 rows, 8 heads: 75.5
+// -> 68.6.  Where the second warpgroup would only wait for its first scores the old form is kept: tiles of one or two key tiles
+// (64 heads x 384, causal: 12.3 -> 13.3; 200 documents of 30 to 300 rows, 16 heads: 218 -> 227; 1000 heads x 64: 35.5 -> 37.8)
+// and clusters (8 x (16, 4 heads) x 16 queries behind 8192 keys: 38.5 -> 43).
+template <int D, int MODE>
+struct FwdTmem {
+  static constexpr bool kSepP = (D == 64) || MODE == 4 || MODE == 5;             // P~ in its own columns
+  static constexpr bool kSharedS = kSepP && D == 128;              // one score tile for both warpgroups
+  static constexpr uint32_t kSStride = kSharedS ? 0 : 128;         // S_t at kSStride t
+  static constexpr uint32_t kColP = !kSepP ? 0 : kSharedS ? 128 : 384, kPStride = kSepP ? 64 : 128;   // P~_t at kColP + kPStride t
+};
+
 enum FwdWaitCode {
   kFwdWaitQ = 0x11, kFwdWaitK = 0x12, kFwdWaitV = 0x13, kFwdWaitKVEmpty = 0x14, kFwdWaitS = 0x15, kFwdWaitP = 0x16,
-  kFwdWaitPV = 0x17, kFwdWaitSFree = 0x18, kFwdWaitOFree = 0x19, kFwdWaitQFree = 0x1a, kFwdWaitTurn = 0x1b, kFwdWaitMerge = 0x1c
+  kFwdWaitPV = 0x17, kFwdWaitSFree = 0x18, kFwdWaitOFree = 0x19, kFwdWaitQFree = 0x1a, kFwdWaitMerge = 0x1c
 };
 
 
@@ -89,10 +110,9 @@ __device__ __forceinline__ float softmax_exp_store(const uint32_t (&xr)[4][32], 
   return (r0 + r1) + (r2 + r3);
 }
 
-// MODE: 0 = pairs of query tiles, 1 = pairs whose warpgroups take turns in the exponential phase, 2 = single tiles with
-// the key range split between the warpgroups, 3 = single tiles with the key range split over the warpgroups of a cluster of
-// CTAs (one tile per cluster; the parts of all CTAs are merged through distributed shared memory), 4 = as 2, with separate rings
-// for K and V.
+// MODE: 0 = pairs of query tiles, 2 = single tiles with the key range split between the warpgroups, 3 = single tiles with the key
+// range split over the warpgroups of a cluster of CTAs (one tile per cluster; the parts of all CTAs are merged through
+// distributed shared memory), 4 = as 2, 5 = as 0, with separate rings for K and V and the scores of both warpgroups in one place (d = 128).
 template <int D, bool CAUSAL, bool FMA_SOFTMAX, int MODE>
 __global__ void __launch_bounds__(384, 1)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
@@ -109,8 +129,11 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   // 49.1 -> 41.4 us; 12 packed pairs (4000 queries, 9000 keys, 12 heads): 62.2 -> 51.5.  With few key tiles to an item (fwd_separate_rings
   // in host_rules.h), with more stages or where both stages hold one tile's work, the second commit per key tile and the
   // thread that polls both rings cost more than they give (200 packed documents of 30 to 300 rows, 16 heads, d = 128: 230 -> 270 us;
-  // 16 heads x 4096 x 64: 60.5 -> 62.5; pairs at d = 128: 306 either way; clusters at d = 64: 33.0 -> 38).
-  constexpr bool kSepRings = (MODE == 4);
+  // 16 heads x 4096 x 64: 60.5 -> 62.5; clusters at d = 64: 33.0 -> 38).  With the scores in one place they pay at every length of
+  // pairs: 32 heads x 4096, causal: 159 -> 141; 32 x 2048: 72.5 -> 66.0.
+  constexpr bool kSepRings = (MODE == 4 || MODE == 5);
+  using M = FwdTmem<D, MODE>;
+  constexpr bool kMoveRegs = M::kSharedS;
   const int fold = kCluster ? fold_rows : 0;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -119,7 +142,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 
   __shared__ int s_item[4][2];
   __shared__ uint64_t bar_q_full[2], bar_q_free[2], bar_k_full[S], bar_v_full[S], bar_k_empty[S], bar_v_empty[S];
-  __shared__ uint64_t bar_s_full[2], bar_s_free[2], bar_p_ready[2], bar_pv_done[2], bar_o_free[2], bar_turn[2], bar_merge, bar_drain[2];
+  __shared__ uint64_t bar_s_full[2], bar_s_free[2], bar_p_ready[2], bar_pv_done[2], bar_o_free[2], bar_merge, bar_drain[2];
   __shared__ float s_m1[2][128], s_l1[2][128];   // split mode: running maximum and normaliser of the second warpgroup, by item parity (with a cluster: of both)
   __shared__ float s_pm[kCluster ? 256 : 1], s_pl[kCluster ? 256 : 1];   // cluster merge: every part's maximum and normaliser for this CTA's rows
   __shared__ uint32_t tmem_base_smem;
@@ -128,15 +151,14 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) cta_skip = *reinterpret_cast<volatile int *>(status);
   __syncthreads();
-  if (MODE == 1 && cta_skip != 0) { griddep_wait(); return; }   // see below
+  if (MODE == 5 && cta_skip != 0) { griddep_wait(); return; }   // see below
 
   const int n_qt = (N + C::kBlockM - 1) / C::kBlockM;   // the last tile may be ragged: rows past N load as zero, stores clip
   const int TPI = tiles_per_item;                  // 2: a pair of query tiles per work item; 1: single tiles, key range split
-  constexpr bool split = (MODE >= 2);              // one query tile; warpgroup t takes the key tiles j = t (mod 2), merged at the end
+  constexpr bool split = (MODE >= 2 && MODE <= 4);              // one query tile; warpgroup t takes the key tiles j = t (mod 2), merged at the end
   // Key tile j of the item belongs to CTA (j / 2) mod ncta of the cluster (ncta = 1 without a cluster), warpgroup j mod 2.
   const int ncta = kCluster ? cluster_size() : 1, crank = kCluster ? cluster_rank() : 0;
   auto mine = [&](int j) { return !kCluster || ((j >> 1) % ncta) == crank; };
-  constexpr bool TURNS = (MODE == 1);
   const int n_pairs = (n_qt + TPI - 1) / TPI;
   AbortState ab{status, &cta_abort};
   if (threadIdx.x == 0) {
@@ -149,7 +171,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     for (int s = 0; s < S; ++s) { mbar_init(&bar_k_full[s], 1); mbar_init(&bar_v_full[s], 1); mbar_init(&bar_k_empty[s], 1); mbar_init(&bar_v_empty[s], 1); }
     for (int t = 0; t < 2; ++t) {
       mbar_init(&bar_drain[t], 1);
-      mbar_init(&bar_s_full[t], 1); mbar_init(&bar_s_free[t], 128); mbar_init(&bar_p_ready[t], 128); mbar_init(&bar_pv_done[t], 1); mbar_init(&bar_o_free[t], 128); mbar_init(&bar_turn[t], 128);
+      mbar_init(&bar_s_full[t], 1); mbar_init(&bar_s_free[t], 128); mbar_init(&bar_p_ready[t], 128); mbar_init(&bar_pv_done[t], 1); mbar_init(&bar_o_free[t], 128);
     }
     fence_mbar_init();
   }
@@ -167,8 +189,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   // next kernel in the stream relies on this one.  The CTAs of a cluster wait for one another at the end, so they run on with
   // every wait falling through instead.  Where this return stands changes the code of the softmax loop.  Above, behind a
   // griddep_wait of its own, calls of one or two key tiles per item are up to 3 % slower (64 x 16 heads x 100 x 64: 31.7 -> 32.8 us); here,
-  // long calls with turns are (8 heads x 32768 x 128, causal: 2346 -> 2414 us).
-  if (!kCluster && MODE != 1 && cta_skip != 0) {
+  // pairs with separate rings are no faster (8 heads x 32768 x 128, causal: 1846 and 1850 us).
+  if (!kCluster && MODE != 5 && cta_skip != 0) {
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem_base, C::kTmemCols);
     return;
@@ -217,6 +239,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   auto q_buf = [&](int ti) { return split ? (ti & 1) : 0; };
   auto q_use = [&](int ti) { return split ? (ti >> 1) : ti; };      // how often the buffer has been used before item ti
 
+  if (warp < 4) {
+  if constexpr (kMoveRegs) setmaxnreg_dec<C::kRegsAux>();
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer of K_j, V_j
     // With separate rings a K tile is free as soon as its scores are complete, a V tile only when the probabilities of its
@@ -326,7 +350,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     constexpr uint32_t idesc_s = idesc_bf16_f32(128, 128, 0, 0);   // both operands K-major
     const SmemDesc dscQ0 = make_smem_desc(smem_u32(sQ), 16, 1024);
     const SmemDesc dscK0 = make_smem_desc(smem_u32(sKV), 16, 1024);
-    int g = 0, ti = 0, cnt[2] = {0, 0};
+    int g = 0, ti = 0, cnt[2] = {0, 0}, last = -1;
     for (int lin = sched.next(); lin >= 0; lin = sched.next(), ++ti) {
       const Item it = decode(lin);
       const int T = it.n_kt;
@@ -342,8 +366,12 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           if (split ? ((j & 1) != t) : !active(it, t, j)) continue;
           // S_t may be overwritten once its previous contents are dead: copied to registers by the softmax (P~ has its
           // own columns), or, when P~ lives in the same columns, consumed by the previous P~V product.
-          if (cnt[t] > 0) {
-            if (C::kSepP) mbar_wait(&bar_s_free[t], (cnt[t] - 1) & 1, ab, kFwdWaitSFree);
+          // With one score tile for both warpgroups those are the scores issued last, whoever's they are.
+          if (M::kSharedS) {
+            if (last >= 0) mbar_wait(&bar_s_free[last], (cnt[last] - 1) & 1, ab, kFwdWaitSFree);
+            last = t;
+          } else if (cnt[t] > 0) {
+            if (M::kSepP) mbar_wait(&bar_s_free[t], (cnt[t] - 1) & 1, ab, kFwdWaitSFree);
             else          mbar_wait(&bar_pv_done[t], (cnt[t] - 1) & 1, ab, kFwdWaitSFree);
           }
           tc_fence_after();
@@ -352,7 +380,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 #pragma unroll
             for (int k = 0; k < D / 16; ++k) {
               const uint32_t off = (k / 4) * C::kSlabBytes + (k % 4) * 32;
-              umma_ss(tmem_base + C::kColS + 128 * t, dscQ.at(off), dscK.at(off), idesc_s, k > 0);
+              umma_ss(tmem_base + C::kColS + M::kSStride * t, dscQ.at(off), dscK.at(off), idesc_s, k > 0);
             }
             umma_commit(&bar_s_full[t]);
           }
@@ -387,7 +415,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           if (first && ti > 0) mbar_wait(&bar_o_free[t], (ti - 1) & 1, ab, kFwdWaitOFree);   // previous epilogue has read O_t
           mbar_wait(&bar_p_ready[t], cnt[t] & 1, ab, kFwdWaitP);
           tc_fence_after();
-          const uint32_t tP = tmem_base + (C::kSepP ? C::kColP + 64 * t : C::kColS + 128 * t);
+          const uint32_t tP = tmem_base + M::kColP + M::kPStride * t;
           const uint32_t acc = first ? 0u : 1u;
           if (elect_one_sync()) {
 #pragma unroll
@@ -404,15 +432,17 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       }
     }
     drain_mmas_if_aborted(&bar_drain[1], ab);
+  }
   } else {
+    if constexpr (kMoveRegs) setmaxnreg_inc<C::kRegsSoftmax>();
     // ---------------------------------------------------------------- softmax: warpgroup t <-> query tile t, thread <-> row
     const int t = (warp - 4) >> 2;
     const int row = 32 * (warp & 3) + lane;
     const uint32_t lane_addr = static_cast<uint32_t>(32 * (warp & 3)) << 16;
-    const uint32_t tS = tmem_base + C::kColS + 128 * t + lane_addr;
+    const uint32_t tS = tmem_base + C::kColS + M::kSStride * t + lane_addr;
     const uint32_t tO = tmem_base + C::kColO + D * t + lane_addr;
-    const uint32_t tP = tmem_base + (C::kSepP ? C::kColP + 64 * t : C::kColS + 128 * t) + lane_addr;
-    int ti = 0, cnt = 0, turn = 0;
+    const uint32_t tP = tmem_base + M::kColP + M::kPStride * t + lane_addr;
+    int ti = 0, cnt = 0;
     for (int lin = sched.next(); lin >= 0; lin = sched.next(), ++ti) {
       const int qb = q_buf(ti);
       mbar_wait(&bar_q_full[qb], q_use(ti) & 1, ab, kFwdWaitQ);   // the item's Q has landed, and with it its description
@@ -440,24 +470,14 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 #ifdef GPROJ_TRACE
       const unsigned long long ev_n0 = global_ns(); const long long ev_c0 = clock64();
 #endif
-      // Both tiles of the pair exist: the warpgroups alternate in the exponential phase, step by step, tile 0 first.
-      const bool take_turns = TURNS && it.nq == 2;
       const int cnt_item0 = cnt;
       for (int j = split ? 2 * crank + t : 0; j < T; j += split ? 2 * ncta : 1) {
         const bool first = split ? (j < 2 * crank + 2) : (j == 0);     // this warpgroup's first key tile of the item
-        if (!split && j > jl) {
-          // no work in this step (causal: the first tile of the pair ends one key tile earlier): pass the turn on
-          if (take_turns) {
-            if (t == 1 || turn > 0) mbar_wait(&bar_turn[t], (t == 1 ? turn : turn - 1) & 1, ab, kFwdWaitTurn);
-            mbar_arrive(&bar_turn[1 - t]);
-            ++turn;
-          }
-          continue;
-        }
+        if (!split && j > jl) continue;               // causal: the first tile of the pair ends one key tile earlier
         mbar_wait(&bar_s_full[t], cnt & 1, ab, kFwdWaitS);
         tc_fence_after();
         if (kCluster && !live) {
-          if (C::kSepP) mbar_arrive(&bar_s_free[t]);
+          if (M::kSepP) mbar_arrive(&bar_s_free[t]);
           if (!first) mbar_wait(&bar_pv_done[t], (cnt - 1) & 1, ab, kFwdWaitPV);
           mbar_arrive(&bar_p_ready[t]);
           ++cnt;
@@ -467,7 +487,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 #pragma unroll
         for (int c = 0; c < 4; ++c) tmem_ld32(tS + 32 * c, xr[c]);
         tmem_wait_ld();
-        if (C::kSepP) { tc_fence_before(); mbar_arrive(&bar_s_free[t]); }   // the next S_t may be issued while this one is in the ALUs
+        if (M::kSepP) { tc_fence_before(); mbar_arrive(&bar_s_free[t]); }   // the next S_t may be issued while this one is in the ALUs
         // Keys beyond the causal diagonal, and the zero-filled columns past the last key of a ragged tile, get -inf.
         if (j >= jm) {
           const int lim = rk - j * C::kBlockN;
@@ -505,13 +525,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         const float m_scaled = __fmul_rn(m_new, scale_log2);
         // P~ of the previous key tile must have been consumed (and O_t updated) before either is touched
         if (!first) { mbar_wait(&bar_pv_done[t], (cnt - 1) & 1, ab, kFwdWaitPV); tc_fence_after(); }
-        // The exponential phase is the only heavy user of the special-function unit (16 results per clock per SM, the
-        // forward's scarcest pipe).  With TURNS the two warpgroups alternate in it, so that one's exponentials run against
-        // the other's loads, maxima and barrier work instead of both phases colliding and then both leaving the unit idle
-        // (measured: +9 % at d = 128, -4 % at d = 64, so the host enables it for d = 128 with paired tiles only).
-        if (take_turns) { if (t == 1 || turn > 0) mbar_wait(&bar_turn[t], (t == 1 ? turn : turn - 1) & 1, ab, kFwdWaitTurn); }
         const float rs = softmax_exp_store<FMA_SOFTMAX>(xr, tP, m_new, scale_log2, m_scaled);
-        if (take_turns) { mbar_arrive(&bar_turn[1 - t]); ++turn; }
         l_run = l_run * corr + rs;
         if (!first && __any_sync(0xffffffffu, m_new != m_run)) {
 #pragma unroll

@@ -129,16 +129,18 @@ int device_state(DeviceState **out) {
       ok &= allow_smem(attn_fwd_kernel<64, false, true, 0>, FwdCfg<64>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<64, false, true, 2>, FwdCfg<64>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, true, false, 0>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
-      ok &= allow_smem(attn_fwd_kernel<128, true, false, 1>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, true, false, 2>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, true, true, 0>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, true, true, 2>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, false, false, 0>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
-      ok &= allow_smem(attn_fwd_kernel<128, false, false, 1>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, false, false, 2>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, false, true, 0>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, false, true, 2>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, true, false, 4>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
+      ok &= allow_smem(attn_fwd_kernel<128, true, true, 5>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
+      ok &= allow_smem(attn_fwd_kernel<128, true, false, 5>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
+      ok &= allow_smem(attn_fwd_kernel<128, false, true, 5>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
+      ok &= allow_smem(attn_fwd_kernel<128, false, false, 5>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, true, true, 4>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, false, false, 4>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, false, true, 4>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
@@ -434,7 +436,8 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
     tl_launch_count = 1;
     return GPROJ_OK;
   }
-  bool sep_rings = d == 128 && tiles_per_item == 1 && total_items <= st->sm_count;
+  // One item per CTA: the longest tile counts.
+  bool sep_rings = d == 128 && tiles_per_item == 1 && total_items <= st->sm_count && (seqs ? longest_keys(*seqs) : Nk) > 2 * 128;
   if (seqs && total_items > st->sm_count && total_items <= 16LL * st->sm_count) {
     const std::vector<int> key_tiles = tile_steps(*seqs, false, 128, 1);
     fwd_order.solo = solo_ctas(key_tiles, BH, st->sm_count, 2.1);
@@ -457,13 +460,13 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
   do { if (causal) GPROJ_LAUNCH_FWD(DD, true, FF, MM); else GPROJ_LAUNCH_FWD(DD, false, FF, MM); } while (0)
 #define GPROJ_LAUNCH_FWD_F(DD, MM)                                                                                  \
   do { if (fma) GPROJ_LAUNCH_FWD_C(DD, true, MM); else GPROJ_LAUNCH_FWD_C(DD, false, MM); } while (0)
-  // Single tiles: the two softmax warpgroups split the key range of the tile.  Pairs: one tile each, and at d = 128
-  // they alternate in the exponential phase (measured to pay there only) unless there is one tile to a head, and no pair.
-  const bool split = (tiles_per_item == 1), turns = (d == 128) && !split && !fma && n_qt > 1;
+  // Single tiles: the two softmax warpgroups split the key range of the tile.  Pairs: one tile each; at d = 128 with both
+  // warpgroups' scores in one place unless there is one tile to a head, and no pair.
+  const bool split = (tiles_per_item == 1);
   if (d == 64) { if (split) GPROJ_LAUNCH_FWD_F(64, 2); else GPROJ_LAUNCH_FWD_F(64, 0); }
   else if (split && sep_rings) GPROJ_LAUNCH_FWD_F(128, 4);
   else if (split) GPROJ_LAUNCH_FWD_F(128, 2);
-  else if (turns) GPROJ_LAUNCH_FWD_C(128, false, 1);
+  else if (n_qt > 1) GPROJ_LAUNCH_FWD_F(128, 5);
   else GPROJ_LAUNCH_FWD_F(128, 0);
 #undef GPROJ_LAUNCH_FWD_F
 #undef GPROJ_LAUNCH_FWD_C

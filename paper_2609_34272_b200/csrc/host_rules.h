@@ -26,10 +26,11 @@ inline long long fwd_key_tiles(int lq, int lk, bool causal) {
 }
 
 // Forward at d = 128 with the key range of a tile split between the warpgroups: separate rings for K and V (see attn_fwd.cuh)?
-// From three key tiles per item on (key_tiles, tiles: of one head, or of the items of one CTA), and always with one item per CTA.
+// From three key tiles per item on (key_tiles, tiles: of one head, or of the items of one CTA; with one item per CTA: of the longest item).
 // Measured, one ring -> two, 16 query / 4 KV heads, 40000 rows in sequences of one length, causal: 512 rows (2.5 key tiles per item)
-// 228 -> 239 us, 640 (3.0) 256 -> 256, 1024 (4.5) 332 -> 312; not causal: 256 (2) 177 -> 190, 384 (3) 240 -> 234; 16 heads x 500 (64
-// items): 11.0 -> 10.4.
+// 228 -> 239 us, 640 (3.0) 256 -> 256, 1024 (4.5) 332 -> 312; not causal: 256 (2) 177 -> 190, 384 (3) 240 -> 234.  With the scores of both
+// warpgroups in one place as well (FwdTmem): 64 heads x 384, causal (2.0) 12.3 -> 13.3, x 500 (2.5) 16.0 -> 15.6, not causal: 256 (2) 8.5
+// -> 8.6, 384 (3) 17.5 -> 15.2; one item per CTA, causal: 16 x 500 (4) 10.6 -> 9.3, 16 x 300 (3) 8.7 -> 8.2, 16 x 200 (2) 7.0 -> 7.2.
 inline bool fwd_separate_rings(long long key_tiles, long long tiles) { return key_tiles >= 3 * tiles; }
 
 // dQ side at d = 128: are the tiles so short that the compute warpgroups should prepare the row constants (SHORT in attn_bwd.cuh)?

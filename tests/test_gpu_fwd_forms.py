@@ -1,0 +1,52 @@
+"""Forward kernels without clusters, at the edges of their dispatch rules and of their tiles (through the C ABI, against the oracle).
+
+Tolerances as in test_gpu_clusters.py: BF16 operands and results leave up to 0.26 % relative L2 against FP64, one BF16 step of the
+largest value is 0.4 % of it; a wrong tile, part or rescale moves a result by several per cent.
+"""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2609_34272_b200 as g
+
+pytestmark = pytest.mark.gpu
+
+
+def tobits(t):
+    return t.contiguous().view(torch.int16).numpy().view(np.uint16)
+
+
+# Pairs of query tiles need 222 pairs; an odd tile at the end, one or two rows in the last tile, ends of key tiles.  Single
+# tiles: one item per CTA with two and with three key tiles, then more items than CTAs on both sides of three key tiles per item.
+SHAPES = [  # B, H, Hkv, Nq, Nk, causal
+    (1, 112, 112, 257, 257, True), (1, 112, 56, 258, 385, True), (2, 75, 25, 300, 130, True), (1, 222, 222, 256, 1, False), (1, 112, 112, 384, 640, False),
+    (1, 60, 60, 513, 513, True), (1, 223, 223, 129, 128, True), (3, 100, 100, 128, 200, True), (2, 150, 75, 77, 77, True),
+    (1, 3, 3, 256, 256, True), (1, 3, 3, 257, 257, True), (1, 16, 4, 300, 300, True), (1, 60, 60, 384, 384, True), (1, 40, 40, 640, 640, True), (1, 2, 2, 1, 385, False),
+    (1, 5, 5, 200, 64, True), (1, 3, 1, 130, 1030, True),
+]
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("fma", [0, 1])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_forward_forms(shape, d, fma):
+    B, H, Hkv, Nq, Nk, causal = shape
+    gen = torch.Generator().manual_seed(Nq * 7 + Nk + d)
+    Q = torch.randn(B, H, Nq, d, generator=gen).to(torch.bfloat16)
+    K = torch.randn(B, Hkv, Nk, d, generator=gen) + 0.5
+    K[:, :, Nk // 2:] *= 3.0                      # the running maximum moves on the way
+    K = K.to(torch.bfloat16)
+    V = torch.randn(B, Hkv, Nk, d, generator=gen).to(torch.bfloat16)
+    ex = oracle.attn_rect_f64(tobits(Q), tobits(K), tobits(V), tobits(torch.zeros_like(Q)), d ** -0.5, causal)
+    q, k, v = Q.cuda(), K.cuda(), V.cuda()
+    O, LSE = torch.full_like(q, float("nan")), torch.full(q.shape[:3], float("nan"), device="cuda")
+    g.gproj_attn_fwd_rect(q, k, v, d ** -0.5, causal, O=O, LSE=LSE, fwd_flags=fma * g.FWD_FLAG_FMA_SOFTMAX)
+    rc, detail = g.gproj_last_device_status()
+    assert rc == 0, hex(detail)
+    O, LSE = O.float().cpu().numpy().astype(np.float64), LSE.cpu().numpy().astype(np.float64)
+    empty = np.isinf(ex["LSE"])
+    assert np.array_equal(np.isposinf(LSE), empty) and np.all(O[empty] == 0.0) and np.all(np.isfinite(O))
+    assert np.all(np.abs(LSE[~empty] - ex["LSE"][~empty]) <= 1e-4 + 1e-5 * np.abs(ex["LSE"][~empty]))
+    assert oracle.rel_l2_percent(O, ex["O"]) <= 0.3
+    assert np.abs(O - ex["O"]).max() <= 0.01 * np.abs(ex["O"]).max()
