@@ -14,6 +14,7 @@
 #include "attn_bwd.cuh"
 #include "attn_bwd_w128.cuh"
 #include "attn_fwd.cuh"
+#include "attn_fwd_w64.cuh"
 #include "key_smoothing.cuh"
 #include "attn_fp32.cuh"
 #include "host_rules.h"
@@ -120,14 +121,8 @@ int device_state(DeviceState **out) {
       if (cudaGetSymbolAddress(reinterpret_cast<void **>(&st.status_ptr), g_device_status) != cudaSuccess)
         return GPROJ_ERR_CUDA;
       bool ok = true;
-      ok &= allow_smem(attn_fwd_kernel<64, true, false, 0>, FwdCfg<64>::kSmemBytes) == cudaSuccess;
-      ok &= allow_smem(attn_fwd_kernel<64, true, false, 2>, FwdCfg<64>::kSmemBytes) == cudaSuccess;
-      ok &= allow_smem(attn_fwd_kernel<64, true, true, 0>, FwdCfg<64>::kSmemBytes) == cudaSuccess;
-      ok &= allow_smem(attn_fwd_kernel<64, true, true, 2>, FwdCfg<64>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<64, false, false, 0>, FwdCfg<64>::kSmemBytes) == cudaSuccess;
-      ok &= allow_smem(attn_fwd_kernel<64, false, false, 2>, FwdCfg<64>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<64, false, true, 0>, FwdCfg<64>::kSmemBytes) == cudaSuccess;
-      ok &= allow_smem(attn_fwd_kernel<64, false, true, 2>, FwdCfg<64>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, true, false, 0>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, true, false, 2>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, true, true, 0>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
@@ -137,6 +132,10 @@ int device_state(DeviceState **out) {
       ok &= allow_smem(attn_fwd_kernel<128, false, true, 0>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, false, true, 2>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, true, false, 4>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
+      ok &= allow_smem(attn_fwd_w64_kernel<true, true>, FwdW64Cfg::kSmemBytes) == cudaSuccess;
+      ok &= allow_smem(attn_fwd_w64_kernel<true, false>, FwdW64Cfg::kSmemBytes) == cudaSuccess;
+      ok &= allow_smem(attn_fwd_w64_kernel<false, true>, FwdW64Cfg::kSmemBytes) == cudaSuccess;
+      ok &= allow_smem(attn_fwd_w64_kernel<false, false>, FwdW64Cfg::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, true, true, 5>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, true, false, 5>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, false, true, 5>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
@@ -339,45 +338,6 @@ int tile_group_of(bool packed, bool causal, int heads, int n_per_head, size_t st
   return best;
 }
 
-// Causal forward at d = 64: paired query tiles or single tiles with the key range split between the warpgroups?
-// Measured on B200 (in units of one key-tile step of a pair): a pair item costs its key tiles + 2.9 per item, a single
-// tile 0.855 x half its key tiles + 2.9 per item (the split steady state is faster, the per-item cost is paid twice as
-// often), and the kernel time is the longest CTA's sum under the static boustrophedon deal.  This replays the deal; the
-// constants reproduce the measured ratio of the two modes within 4 % for 8 to 128 heads and N from 1024 to 32768.
-bool fwd_prefers_single_tiles(int BH, int n_qt, int sms) {
-  const long long n_pairs = (n_qt + 1) / 2, items_p = BH * n_pairs, items_s = static_cast<long long>(BH) * n_qt;
-  if (items_s > (1 << 16)) return false;   // many items per SM: both deals balance, pairs have the lower per-item cost
-  static std::mutex memo_mutex;
-  static std::map<std::tuple<int, int, int>, bool> memo;
-  const auto key = std::make_tuple(BH, n_qt, sms);
-  {
-    std::lock_guard<std::mutex> lock(memo_mutex);
-    const auto hit = memo.find(key);
-    if (hit != memo.end()) return hit->second;
-  }
-  auto longest = [&](long long items, auto work_of) {
-    const int G = static_cast<int>(std::min<long long>(items, sms));
-    std::vector<double> load(static_cast<size_t>(G), 0.0);
-    for (long long lin = 0; lin < items; ++lin) {
-      const long long r = lin / G, pos = lin % G;
-      load[static_cast<size_t>((r & 1) ? G - 1 - pos : pos)] += work_of(lin);
-    }
-    return *std::max_element(load.begin(), load.end());
-  };
-  const double kItem = 2.9, kSplitStep = 0.855;
-  const double t_pairs = longest(items_p, [&](long long lin) {
-    const long long p = n_pairs - 1 - lin / BH;                       // longest pairs first, as the kernel orders them
-    return static_cast<double>(2 * p + std::min<long long>(2, n_qt - 2 * p)) + kItem;
-  });
-  const double t_single = longest(items_s, [&](long long lin) {
-    const long long t = n_qt - 1 - lin / BH;
-    return kSplitStep * 0.5 * static_cast<double>(t + 1) + kItem;
-  });
-  std::lock_guard<std::mutex> lock(memo_mutex);
-  if (memo.size() < 4096) memo[key] = t_single < t_pairs;
-  return t_single < t_pairs;
-}
-
 // Dense call: plan == nullptr, one sequence [0, N) per head.  Packed call: B = 1, N = total tokens, plan = device tile
 // list (query order) with n_plan_tiles entries, longest_keys = most keys of one sequence.
 int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE, int B, int H, int Hkv, int N, int Nk, int d,
@@ -411,16 +371,15 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
       !make_map(&mO, O, BH, N, d, 128))
     return GPROJ_ERR_CUDA;
   const float scale_log2 = static_cast<float>(static_cast<double>(softmax_scale) * 1.4426950408889634);
-  // One work item = a pair of query tiles of one head (two softmax warpgroups ping-pong on the tensor core); when
-  // that leaves too few items to balance the SMs, items are single tiles.
+  // One work item = a pair of query tiles of one head (two softmax warpgroups ping-pong on the tensor core), or a single tile: where
+  // pairs leave too few items to balance the SMs, and at d = 64 wherever the kernel of attn_fwd_w64.cuh is not slower.
   const int n_qt = plan ? n_plan_tiles : (N + 127) / 128;
   int tiles_per_item = (!plan && static_cast<long long>(BH) * ((n_qt + 1) / 2) * 2 >= 3LL * st->sm_count) ? 2 : 1;
-  if (fold > 0) tiles_per_item = 1;
-  if (tiles_per_item == 2 && d == 64 && causal && N == Nk && fwd_prefers_single_tiles(BH, n_qt, st->sm_count)) tiles_per_item = 1;
+  if (fold > 0 || (d == 64 && (causal || !fwd_prefers_pairs(BH, n_qt, (Nk + 127) / 128, st->sm_count)))) tiles_per_item = 1;
   const int total_items = BH * ((n_qt + tiles_per_item - 1) / tiles_per_item);
   if (total_items <= 0) return GPROJ_OK;   // nothing but empty sequences
   ItemOrder fwd_order = item_order(BH, total_items / BH, tile_group_of(plan != nullptr, causal != 0, BH, total_items / BH, 2 * static_cast<size_t>(BHkv) * Nk * d * 2, st->sm_count,
-                                                            tiles_per_item == 2 ? 1.45 : 6.8));
+                                                            tiles_per_item == 2 ? 1.45 : d == 64 ? 1.8 : 6.8));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   tl_form[GPROJ_FORM_FWD_HEADS] = Hkv == H ? Hq / Hkv : 1;
   const int (&fit)[4] = st->fwd_clusters[d == 128];
@@ -460,10 +419,18 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
   do { if (causal) GPROJ_LAUNCH_FWD(DD, true, FF, MM); else GPROJ_LAUNCH_FWD(DD, false, FF, MM); } while (0)
 #define GPROJ_LAUNCH_FWD_F(DD, MM)                                                                                  \
   do { if (fma) GPROJ_LAUNCH_FWD_C(DD, true, MM); else GPROJ_LAUNCH_FWD_C(DD, false, MM); } while (0)
-  // Single tiles: the two softmax warpgroups split the key range of the tile.  Pairs: one tile each; at d = 128 with both
+  // Single tiles: the softmax warpgroups split the key range of the tile (three of them at d = 64).  Pairs: one tile each; at d = 128 with both
   // warpgroups' scores in one place unless there is one tile to a head, and no pair.
   const bool split = (tiles_per_item == 1);
-  if (d == 64) { if (split) GPROJ_LAUNCH_FWD_F(64, 2); else GPROJ_LAUNCH_FWD_F(64, 0); }
+  if (d == 64 && split) {
+    CUtensorMap mK64, mV64;
+    if (!make_map(&mK64, K, BHkv, Nk, d, 64) || !make_map(&mV64, V, BHkv, Nk, d, 64)) return GPROJ_ERR_CUDA;
+    auto kernel = causal ? (fma ? attn_fwd_w64_kernel<true, true> : attn_fwd_w64_kernel<true, false>)
+                         : (fma ? attn_fwd_w64_kernel<false, true> : attn_fwd_w64_kernel<false, false>);
+    launch_after(kernel, grid, 1, FwdW64Cfg::kThreads, FwdW64Cfg::kSmemBytes, s, early, mQ, mK64, mV64, mO, static_cast<__nv_bfloat16 *>(O), plan, LSE, N, Nk,
+                 H, G, total_items, fwd_order, scale_log2, softmax_scale, st->status_ptr);
+  }
+  else if (d == 64) { if (fma) GPROJ_LAUNCH_FWD(64, false, true, 0); else GPROJ_LAUNCH_FWD(64, false, false, 0); }
   else if (split && sep_rings) GPROJ_LAUNCH_FWD_F(128, 4);
   else if (split) GPROJ_LAUNCH_FWD_F(128, 2);
   else if (n_qt > 1) GPROJ_LAUNCH_FWD_F(128, 5);

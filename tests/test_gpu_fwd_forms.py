@@ -50,3 +50,28 @@ def test_forward_forms(shape, d, fma):
     assert np.all(np.abs(LSE[~empty] - ex["LSE"][~empty]) <= 1e-4 + 1e-5 * np.abs(ex["LSE"][~empty]))
     assert oracle.rel_l2_percent(O, ex["O"]) <= 0.3
     assert np.abs(O - ex["O"]).max() <= 0.01 * np.abs(ex["O"]).max()
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("lens", [[1 + (7 * i) % 64 for i in range(300)], [64] * 40 + [65, 129, 1, 0, 193, 400, 63] * 12], ids=["one_step", "mixed"])
+def test_packed_forward_of_many_short_sequences(lens, d):
+    """Items of one, two and three 64-key steps behind one another on every CTA."""
+    H = 8
+    cu = np.concatenate([[0], np.cumsum(lens)])
+    T = int(cu[-1])
+    gen = torch.Generator().manual_seed(T + d)
+    Q, K, V = (torch.randn(H, T, d, generator=gen).to(torch.bfloat16) for _ in range(3))
+    plan = g.VarlenPlan([int(c) for c in cu], causal=True)
+    O, LSE = g.gproj_attn_fwd_varlen(Q.cuda(), K.cuda(), V.cuda(), plan, d ** -0.5)
+    rc, detail = g.gproj_last_device_status()
+    assert rc == 0, hex(detail)
+    O, LSE = O.double().cpu(), LSE.double().cpu()
+    for a, b in zip(cu[:-1], cu[1:]):
+        if a == b:
+            continue
+        s = (Q[:, a:b].double() @ K[:, a:b].double().transpose(1, 2)) * d ** -0.5
+        s = s.masked_fill(torch.ones(b - a, b - a, dtype=torch.bool).triu(1), -float("inf"))
+        ex = torch.softmax(s, -1) @ V[:, a:b].double()
+        assert float((O[:, a:b] - ex).norm() / ex.norm()) <= 3e-3
+        assert float((O[:, a:b] - ex).abs().max()) <= 0.01 * float(ex.abs().max())
+        assert float((LSE[:, a:b] - torch.logsumexp(s, -1)).abs().max()) <= 2e-4
