@@ -5,12 +5,15 @@ memory and the stream.  There is no CPU fallback: if the library is missing or t
 device is not sm_100a the calls raise.
 """
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 
 import torch
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libgproj_attn.so")
+CALLS_PATH = os.path.join(_PKG, "_torch_calls.so")
 
 GPROJ_OK = 0
 FLAG_NO_Q_CORRECTION = 1
@@ -33,6 +36,7 @@ EXPORTS = ("gproj_attn_fwd", "gproj_attn_bwd_workspace_bytes", "gproj_attn_bwd",
            "gproj_status_string", "gproj_last_launch_count", "gproj_last_form")
 
 _lib = None
+_calls = None       # the dense calls as one native step (csrc/torch_calls.cpp), once the library is loaded
 
 
 class GprojError(RuntimeError):
@@ -112,7 +116,27 @@ def load():
         lib.gproj_last_form.restype = i
         lib.gproj_last_form.argtypes = [i]
         _lib = lib
+        _bind_native_calls(lib)
     return _lib
+
+
+def _bind_native_calls(lib):
+    """Hand the library's entry points to the native call layer, if that was built; without it the calls below go through ctypes."""
+    global _calls
+    if not os.path.exists(CALLS_PATH):
+        return
+    loader = importlib.machinery.ExtensionFileLoader("_torch_calls", CALLS_PATH)
+    calls = importlib.util.module_from_spec(importlib.util.spec_from_file_location("_torch_calls", CALLS_PATH, loader=loader))
+    loader.exec_module(calls)
+    calls.bind(*(ctypes.cast(getattr(lib, n), ctypes.c_void_p).value for n in ("gproj_attn_fwd_rect", "gproj_attn_bwd_rect", "gproj_attn_bwd_workspace_bytes")))
+    _calls = calls
+
+
+def _native(name, result):
+    """What a native call returned: its output tensors, or None where it left the call to the checks below."""
+    if type(result) is int:
+        raise GprojError(result, name)
+    return result
 
 
 def status_string(status: int) -> str:
@@ -208,6 +232,10 @@ def gproj_attn_bwd_workspace_bytes(B, H, N, d) -> int:
 def gproj_attn_fwd(Q, K, V, softmax_scale, causal, O=None, LSE=None, fwd_flags=0):
     """O, LSE = attention forward.  Q: CUDA bfloat16 [B, H, N, d]; K, V: [B, Hkv, N, d] with H a multiple of Hkv
     (Hkv < H = grouped-query attention)."""
+    if O is None and LSE is None and _calls is not None:
+        out = _native("gproj_attn_fwd", _calls.fwd(Q, K, V, softmax_scale, causal, fwd_flags, True))
+        if out is not None:
+            return out
     _check_bf16("Q", Q)
     shape = Q.shape
     B, H, N, d = shape
@@ -230,6 +258,10 @@ def gproj_attn_fwd(Q, K, V, softmax_scale, causal, O=None, LSE=None, fwd_flags=0
 def gproj_attn_bwd(Q, K, V, O, LSE, dO, softmax_scale, causal, flags=0, workspace=None, dQ=None, dK=None, dV=None):
     """dQ, dK, dV = attention backward with the GProj correction (flags: FLAG_NO_*_CORRECTION).
     K, V (and dK, dV) may have fewer heads than Q (grouped-query attention)."""
+    if workspace is None and dQ is None and dK is None and dV is None and _calls is not None:
+        out = _native("gproj_attn_bwd", _calls.bwd(Q, K, V, O, LSE, dO, softmax_scale, causal, flags, True))
+        if out is not None:
+            return out
     _check_bf16("Q", Q)
     shape = Q.shape
     B, H, N, d = shape
@@ -262,6 +294,10 @@ def _rect_shapes(Q, K, V):
 def gproj_attn_fwd_rect(Q, K, V, softmax_scale, causal, O=None, LSE=None, fwd_flags=0):
     """Forward with Nq queries and Nk keys: Q [B, H, Nq, d]; K, V [B, Hkv, Nk, d].  Causal: query i sees the keys
     j <= i + (Nk - Nq); a query that sees none gets O = 0 and LSE = +inf."""
+    if O is None and LSE is None and _calls is not None:
+        out = _native("gproj_attn_fwd_rect", _calls.fwd(Q, K, V, softmax_scale, causal, fwd_flags, False))
+        if out is not None:
+            return out
     B, H, Hkv, Nq, Nk, d = _rect_shapes(Q, K, V)
     O = torch.empty_like(Q) if O is None else O
     LSE = _lse_out(LSE, Q, (B, H, Nq))
@@ -276,6 +312,10 @@ def gproj_attn_fwd_rect(Q, K, V, softmax_scale, causal, O=None, LSE=None, fwd_fl
 
 def gproj_attn_bwd_rect(Q, K, V, O, LSE, dO, softmax_scale, causal, flags=0, workspace=None, dQ=None, dK=None, dV=None):
     """Backward of gproj_attn_fwd_rect (same shapes; dK, dV like K).  Workspace: gproj_attn_bwd_workspace_bytes(B, H, Nq, d)."""
+    if workspace is None and dQ is None and dK is None and dV is None and _calls is not None:
+        out = _native("gproj_attn_bwd_rect", _calls.bwd(Q, K, V, O, LSE, dO, softmax_scale, causal, flags, False))
+        if out is not None:
+            return out
     B, H, Hkv, Nq, Nk, d = _rect_shapes(Q, K, V)
     for name, t in (("O", O), ("dO", dO)):
         _check_bf16(name, t, Q.shape)

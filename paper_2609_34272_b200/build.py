@@ -1,4 +1,4 @@
-"""Compile the CUDA library in-tree for sm_100a with nvcc (works without a GPU)."""
+"""Compile the CUDA library (nvcc, sm_100a) and the native call layer (g++, against torch) in-tree; works without a GPU."""
 import os
 import subprocess
 import sys
@@ -7,6 +7,8 @@ PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libgproj_attn.so")
+CALLS = os.path.join(PKG, "_torch_calls.so")
+CALLS_SOURCE = os.path.join(CSRC, "torch_calls.cpp")
 SOURCES = [os.path.join(CSRC, "gproj_attn.cu")]
 HEADERS = [os.path.join(CSRC, f) for f in ("host_rules.h", "tile_schedule.h", "wait_budget.h", "sm100_primitives.cuh", "attn_fwd.cuh", "attn_fwd_w64.cuh", "attn_bwd.cuh", "attn_bwd_w128.cuh", "key_smoothing.cuh", "attn_fp32.cuh")] + \
           [os.path.join(ROOT, "include", "gproj_attn.h")]
@@ -21,15 +23,34 @@ def nvcc_command(verbose: bool = False):
     return cmd
 
 
-def build(force: bool = False, verbose: bool = False) -> str:
-    deps = SOURCES + HEADERS
-    if not force and os.path.exists(LIB) and all(os.path.getmtime(LIB) >= os.path.getmtime(p) for p in deps):
-        return LIB
-    res = subprocess.run(nvcc_command(verbose), capture_output=True, text=True)
+def calls_command():
+    import sysconfig
+
+    import torch
+    from torch.utils.cpp_extension import CUDA_HOME, include_paths, library_paths
+
+    includes = include_paths() + [sysconfig.get_paths()["include"], os.path.join(CUDA_HOME or "/usr/local/cuda", "include")]
+    return ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"] + \
+        [f"-I{p}" for p in includes] + ["-o", CALLS, CALLS_SOURCE] + [f"-L{p}" for p in library_paths()] + ["-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+
+
+def _up_to_date(target, deps):
+    return os.path.exists(target) and all(os.path.getmtime(target) >= os.path.getmtime(p) for p in deps)
+
+
+def _run(cmd, verbose=False):
+    res = subprocess.run(cmd, capture_output=True, text=True)
     if verbose:
         sys.stderr.write(res.stderr)
     if res.returncode != 0:
-        raise RuntimeError("nvcc failed:\n" + res.stdout + res.stderr)
+        raise RuntimeError(f"{cmd[0]} failed:\n" + res.stdout + res.stderr)
+
+
+def build(force: bool = False, verbose: bool = False) -> str:
+    if force or not _up_to_date(LIB, SOURCES + HEADERS):
+        _run(nvcc_command(verbose), verbose)
+    if force or not _up_to_date(CALLS, [CALLS_SOURCE]):
+        _run(calls_command())
     return LIB
 
 
