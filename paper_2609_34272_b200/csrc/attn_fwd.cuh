@@ -158,7 +158,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   constexpr bool split = (MODE >= 2 && MODE <= 4);              // one query tile; warpgroup t takes the key tiles j = t (mod 2), merged at the end
   // Key tile j of the item belongs to CTA (j / 2) mod ncta of the cluster (ncta = 1 without a cluster), warpgroup j mod 2.
   const int ncta = kCluster ? cluster_size() : 1, crank = kCluster ? cluster_rank() : 0;
-  auto mine = [&](int j) { return !kCluster || ((j >> 1) % ncta) == crank; };
+  // The roles step through this CTA's key tiles alone.  (Walking over all of them with a division by ncta at each took an issuing
+  // warp longer than its products.)
+  const int j_first = 2 * crank;
+  auto j_next = [&](int j) { return kCluster && (j & 1) ? j + 2 * ncta - 1 : j + 1; };
   const int n_pairs = (n_qt + TPI - 1) / TPI;
   AbortState ab{status, &cta_abort};
   if (threadIdx.x == 0) {
@@ -262,7 +265,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         c.j = 0;
       };
       auto settle = [&](Cursor &c) {                         // on to the next key tile of this CTA's
-        while (c.more && !(c.j < c.it.n_kt && mine(c.j))) { if (c.j + 1 < c.it.n_kt) ++c.j; else next_item(c); }
+        while (c.more && c.j >= c.it.n_kt) next_item(c);
       };
       auto feed = [&](Cursor &c, uint64_t *full, uint64_t *empty, const CUtensorMap *map, uint8_t *ring) {
         const int st = c.g % S;
@@ -298,8 +301,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       for (int lin = sched.next(); lin >= 0; lin = sched.next()) {
         const Item it = decode(lin);
         const int bh = hix(lin), T = it.n_kt;
-        for (int j = 0; j < T; ++j) {
-          if (!mine(j)) continue;
+        for (int j = j_first; j < T; j = j_next(j)) {
           const int st = g % S;
           if (g >= S) mbar_wait(&bar_v_empty[st], ((g / S) - 1) & 1, ab, kFwdWaitKVEmpty);
           uint8_t *dK = sKV + st * 2 * C::kTileBytes, *dV = dK + C::kTileBytes;
@@ -356,8 +358,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       const int T = it.n_kt;
       const int qb = q_buf(ti);
       mbar_wait(&bar_q_full[qb], q_use(ti) & 1, ab, kFwdWaitQ);
-      for (int j = 0; j < T; ++j) {
-        if (!mine(j)) continue;
+      for (int j = j_first; j < T; j = j_next(j)) {
         const int st = g % S;
         mbar_wait(&bar_k_full[st], (g / S) & 1, ab, kFwdWaitK);
         const SmemDesc dscK = dscK0.advanced(st * 2 * C::kTileBytes);
@@ -403,8 +404,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     for (int lin = sched.next(); lin >= 0; lin = sched.next(), ++ti) {
       const Item it = decode(lin);
       const int T = it.n_kt;
-      for (int j = 0; j < T; ++j) {
-        if (!mine(j)) continue;
+      for (int j = j_first; j < T; j = j_next(j)) {
         const int st = g % S;
         mbar_wait(&bar_v_full[st], (g / S) & 1, ab, kFwdWaitV);
         const SmemDesc dscV = dscV0.advanced(st * 2 * C::kTileBytes);
