@@ -48,7 +48,7 @@ struct FwdCfg {
   static constexpr int kTmemCols = 512;
   static constexpr uint32_t kColS = 0, kColO = 256;    // O_t at 256 + D t; S_t and P~_t as in FwdTmem
   static constexpr int kThreads = 384;
-  // MODE 4 and 5 re-deal the 384 x 168 registers of the launch: with 168 the causal pairs spill 156 bytes (32 heads x 4096: 149 us, re-dealt
+  // MODE 4, 5 and 6 re-deal the 384 x 168 registers of the launch: with 168 the causal pairs spill 156 bytes (32 heads x 4096: 149 us, re-dealt
   // 138; 8 x 32768: 1960, 1845).  At d = 64 it does not pay (60.4 -> 62 us).
   static constexpr int kRegsSoftmax = 216, kRegsAux = 72;
   static_assert(2 * kRegsSoftmax + kRegsAux <= 3 * 168, "register shares");
@@ -58,18 +58,20 @@ struct FwdCfg {
 
 // TMEM columns of the scores and the probabilities.  At d = 64 there is room for S_0, S_1, P~_0 and P~_1.  At d = 128 there is
 // not.  With P~_t over S_t a warpgroup's key tile is a serial chain of scores (512 clk), softmax (2600) and P~_t V (512), since the
-// next scores have to wait for the last product: 3900 clk for two tiles in flight.  MODE 4 and 5 keep P~_0 and P~_1 apart and
+// next scores have to wait for the last product: 3900 clk for two tiles in flight.  MODE 4, 5 and 6 keep P~_0 and P~_1 apart and
 // one score tile that the warpgroups, half a tile apart, use in turn: it is free again as soon as one of them has copied its
 // scores to registers, and the other's are computed while that one is in its exponentials.  Bound then by the exponentials of
 // two warps per scheduler (2900 clk).  Measured (forward alone, calls back to back in a graph), P~ over S -> one score tile: pairs,
 // causal: 8 heads x 32768: 2260 -> 1845 us; 32 x 4096: 167 -> 138; 96 x 1000: 49.0 -> 42.0; 256 x 500: 50.9 -> 43.6; not causal: 32 x
 // 8192: 1050 -> 912; single tiles, causal: 8 x 4096: 42.6 -> 36; 8 x 2300: 25.3 -> 21.1; 24 packed documents, 16676 rows, 8 heads: 75.5
-// -> 68.6.  Where the second warpgroup would only wait for its first scores the old form is kept: tiles of one or two key tiles
-// (64 heads x 384, causal: 12.3 -> 13.3; 200 documents of 30 to 300 rows, 16 heads: 218 -> 227; 1000 heads x 64: 35.5 -> 37.8)
-// and clusters (8 x (16, 4 heads) x 16 queries behind 8192 keys: 38.5 -> 43).
+// -> 68.6; clusters and folded heads: 8 x (16, 4 heads) x 16 queries behind 8192 keys: 37.0 -> 29.9; 4 x 8 x 1 behind 16384: 58.1 ->
+// 45.4; 2 x 1000 behind 20000: 64.8 -> 42.7; 16 x (32, 8) x 1 behind 1000: 17.8 -> 13.6; 64 x (32, 8) x 64 behind 2048: 262 -> 204.
+// Where the second warpgroup would only wait for its first scores the old form is kept: tiles of one or two key tiles
+// (64 heads x 384, causal: 12.3 -> 13.3; 200 documents of 30 to 300 rows, 16 heads: 218 -> 227; 1000 heads x 64: 35.5 -> 37.8),
+// folded heads and clusters with fewer than four to a CTA (2 x (64, 8) x 100 behind 300: 9.4 -> 10.2).
 template <int D, int MODE>
 struct FwdTmem {
-  static constexpr bool kSepP = (D == 64) || MODE == 4 || MODE == 5;             // P~ in its own columns
+  static constexpr bool kSepP = (D == 64) || MODE == 4 || MODE == 5 || MODE == 6;   // P~ in its own columns
   static constexpr bool kSharedS = kSepP && D == 128;              // one score tile for both warpgroups
   static constexpr uint32_t kSStride = kSharedS ? 0 : 128;         // S_t at kSStride t
   static constexpr uint32_t kColP = !kSepP ? 0 : kSharedS ? 128 : 384, kPStride = kSepP ? 64 : 128;   // P~_t at kColP + kPStride t
@@ -112,7 +114,8 @@ __device__ __forceinline__ float softmax_exp_store(const uint32_t (&xr)[4][32], 
 
 // MODE: 0 = pairs of query tiles, 2 = single tiles with the key range split between the warpgroups, 3 = single tiles with the key
 // range split over the warpgroups of a cluster of CTAs (one tile per cluster; the parts of all CTAs are merged through
-// distributed shared memory), 4 = as 2, 5 = as 0, with separate rings for K and V and the scores of both warpgroups in one place (d = 128).
+// distributed shared memory), 4 = as 2, 5 = as 0, 6 = as 3, with separate rings for K and V and the scores of both warpgroups in one
+// place (d = 128).
 template <int D, bool CAUSAL, bool FMA_SOFTMAX, int MODE>
 __global__ void __launch_bounds__(384, 1)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
@@ -123,7 +126,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   // (grouped queries with few rows); row r then sees the keys of query r mod fold.
   using C = FwdCfg<D>;
   constexpr int S = C::kStages;
-  constexpr bool kCluster = (MODE == 3);
+  constexpr bool kCluster = (MODE == 3 || MODE == 6);
   // Separate K and V rings: with one ring the next K waits for the whole softmax and P~V of its stage, which is what a ring of
   // two stages (d = 128) is bound by while the warpgroups work on two key tiles.  Measured, one ring -> two: 8 heads x 4096 x 128, causal:
   // 49.1 -> 41.4 us; 12 packed pairs (4000 queries, 9000 keys, 12 heads): 62.2 -> 51.5.  With few key tiles to an item (fwd_separate_rings
@@ -131,7 +134,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   // thread that polls both rings cost more than they give (200 packed documents of 30 to 300 rows, 16 heads, d = 128: 230 -> 270 us;
   // 16 heads x 4096 x 64: 60.5 -> 62.5; clusters at d = 64: 33.0 -> 38).  With the scores in one place they pay at every length of
   // pairs: 32 heads x 4096, causal: 159 -> 141; 32 x 2048: 72.5 -> 66.0.
-  constexpr bool kSepRings = (MODE == 4 || MODE == 5);
+  constexpr bool kSepRings = (MODE == 4 || MODE == 5 || MODE == 6);
   using M = FwdTmem<D, MODE>;
   constexpr bool kMoveRegs = M::kSharedS;
   const int fold = kCluster ? fold_rows : 0;
@@ -155,7 +158,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 
   const int n_qt = (N + C::kBlockM - 1) / C::kBlockM;   // the last tile may be ragged: rows past N load as zero, stores clip
   const int TPI = tiles_per_item;                  // 2: a pair of query tiles per work item; 1: single tiles, key range split
-  constexpr bool split = (MODE >= 2 && MODE <= 4);              // one query tile; warpgroup t takes the key tiles j = t (mod 2), merged at the end
+  constexpr bool split = (MODE != 0 && MODE != 5);              // one query tile; warpgroup t takes the key tiles j = t (mod 2), merged at the end
   // Key tile j of the item belongs to CTA (j / 2) mod ncta of the cluster (ncta = 1 without a cluster), warpgroup j mod 2.
   const int ncta = kCluster ? cluster_size() : 1, crank = kCluster ? cluster_rank() : 0;
   // The roles step through this CTA's key tiles alone.  (Walking over all of them with a division by ncta at each took an issuing
@@ -262,7 +265,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         if (!c.more) return;
         c.it = decode(lin);
         c.kvh = kv_head_of(hix(lin), Hq, G);                 // grouped-query: the group's shared K / V head
-        c.j = 0;
+        c.j = j_first;
       };
       auto settle = [&](Cursor &c) {                         // on to the next key tile of this CTA's
         while (c.more && c.j >= c.it.n_kt) next_item(c);
@@ -274,7 +277,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         for (int s = 0; s < C::kSlabs; ++s)
           tma_load_3d(ring + st * 2 * C::kTileBytes + s * C::kSlabBytes, map, &full[st], s * 64, c.it.kseq0 + c.j * C::kBlockN, c.kvh);
         ++c.g;
-        ++c.j;
+        c.j = j_next(c.j);
         settle(c);
         return true;
       };

@@ -164,7 +164,9 @@ int device_state(DeviceState **out) {
       ok &= allow_smem(attn_fwd_kernel<64, true, false, 3>, FwdCfg<64>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<64, false, false, 3>, FwdCfg<64>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, true, false, 3>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
+      ok &= allow_smem(attn_fwd_kernel<128, true, false, 6>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, false, false, 3>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
+      ok &= allow_smem(attn_fwd_kernel<128, false, false, 6>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       if (!ok) { (void)cudaGetLastError(); return GPROJ_ERR_CUDA; }
       st.dq_clusters[0] = max_clusters(bwd_dq_kernel<64, true, 2, false>, 2, BwdCfg<64>::kDqThreads, BwdCfg<64>::kDqSmemBytes);
       st.dq_clusters[1] = max_clusters(bwd_dq_kernel<128, true, 2, false>, 2, BwdCfg<128>::kDqThreads, BwdCfg<128>::kDqSmemBytes);
@@ -172,7 +174,7 @@ int device_state(DeviceState **out) {
       st.dkv_clusters[1] = max_clusters(bwd_dkv_kernel<128, true, 2>, 2, BwdCfg<128>::kDkvThreads, BwdCfg<128>::kDkvSmemBytes);
       for (int lg = 1; lg < 4; ++lg) {
         st.fwd_clusters[0][lg] = max_clusters(attn_fwd_kernel<64, true, false, 3>, 1 << lg, FwdCfg<64>::kThreads, FwdCfg<64>::kSmemBytes);
-        st.fwd_clusters[1][lg] = max_clusters(attn_fwd_kernel<128, true, false, 3>, 1 << lg, FwdCfg<128>::kThreads, FwdCfg<128>::kSmemBytes);
+        st.fwd_clusters[1][lg] = max_clusters(attn_fwd_kernel<128, true, false, 6>, 1 << lg, FwdCfg<128>::kThreads, FwdCfg<128>::kSmemBytes);
       }
     }
     st.ready = true;
@@ -386,8 +388,10 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
   const int lg = (tiles_per_item == 1 && !fma && total_items <= fit[1]) ? fwd_cluster_log2(total_items, ((seqs ? longest_keys(*seqs) : Nk) + 127) / 128, fit) : 0;
   tl_form[GPROJ_FORM_FWD_CTAS] = 1 << lg;
   if (lg > 0 || fold > 0) {
+    const int key_tiles_per_cta = (((seqs ? longest_keys(*seqs) : Nk) + 127) / 128) >> lg;   // at d = 128: which form, see FwdTmem in attn_fwd.cuh
     auto kernel = d == 64 ? (causal ? attn_fwd_kernel<64, true, false, 3> : attn_fwd_kernel<64, false, false, 3>)
-                          : (causal ? attn_fwd_kernel<128, true, false, 3> : attn_fwd_kernel<128, false, false, 3>);
+              : key_tiles_per_cta < 4 ? (causal ? attn_fwd_kernel<128, true, false, 3> : attn_fwd_kernel<128, false, false, 3>)
+                                      : (causal ? attn_fwd_kernel<128, true, false, 6> : attn_fwd_kernel<128, false, false, 6>);
     launch_after(kernel, dim3(static_cast<unsigned>(total_items) << lg), 1 << lg, FwdCfg<64>::kThreads,
                  d == 64 ? FwdCfg<64>::kSmemBytes : FwdCfg<128>::kSmemBytes, s, true, mQ, mK, mV, mO, static_cast<__nv_bfloat16 *>(O), plan, LSE, N, Nk,
                  BH, H, G, fold, tiles_per_item, total_items, fwd_order, scale_log2, softmax_scale, st->status_ptr);
