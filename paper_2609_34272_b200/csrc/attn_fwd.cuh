@@ -143,7 +143,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   uint8_t *sQ = smem;                              // tile 0, then tile 1 (each later reused to stage O_t)
   uint8_t *sKV = sQ + 2 * C::kTileBytes;            // stage s: K tile, then V tile
 
-  __shared__ int s_item[4][2];
+  __shared__ int s_item[4][2];                     // rank and head of an item, from the Q loader to the softmax warps
   __shared__ uint64_t bar_q_full[2], bar_q_free[2], bar_k_full[S], bar_v_full[S], bar_k_empty[S], bar_v_empty[S];
   __shared__ uint64_t bar_s_full[2], bar_s_free[2], bar_p_ready[2], bar_pv_done[2], bar_o_free[2], bar_merge, bar_drain[2];
   __shared__ float s_m1[2][128], s_l1[2][128];   // split mode: running maximum and normaliser of the second warpgroup, by item parity (with a cluster: of both)
@@ -170,9 +170,11 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   if (threadIdx.x == 0) {
     cta_abort = kCluster ? cta_skip : 0;
     mbar_init(&bar_merge, 128);
+    // Whenever a warp reads a slot (after an abort it may be too early or too late), it finds an item of this launch.
+    for (auto &slot : s_item) slot[0] = slot[1] = 0;
     for (int b = 0; b < 2; ++b) {
       mbar_init(&bar_q_full[b], 1);
-      mbar_init(&bar_q_free[b], tiles_per_item);    // one arrival per query tile slot: its O store has left shared memory
+      mbar_init(&bar_q_free[b], 4 * tiles_per_item);    // one arrival per warp and query tile slot: its O store has left shared memory
     }
     for (int s = 0; s < S; ++s) { mbar_init(&bar_k_full[s], 1); mbar_init(&bar_v_full[s], 1); mbar_init(&bar_k_empty[s], 1); mbar_init(&bar_v_empty[s], 1); }
     for (int t = 0; t < 2; ++t) {
@@ -465,7 +467,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       if (!split && t >= it.nq) {
         // Odd number of query tiles: the last pair has no second tile.  This warpgroup is in step with the item (it has
         // waited for its Q above), so it may hand back the slot without any barrier running ahead of its waiters.
-        if (row == 0) mbar_arrive(&bar_q_free[0]);
+        if (lane == 0) mbar_arrive(&bar_q_free[0]);
         mbar_arrive(&bar_o_free[t]);
         continue;
       }
@@ -636,22 +638,23 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       if (split) mbar_arrive(&bar_o_free[1]);          // warpgroup 0 has read both accumulators
       const int qrow0 = it.seq0 + qt * C::kBlockM;      // first row of the tile inside the head
       if (qt * C::kBlockM + row < it.len) LSE[static_cast<size_t>(bh) * N + qrow0 + row] = (l_run > 0.f) ? fmaf(m_run, alpha, logf(l_run)) : INFINITY;
-      fence_proxy_async_smem();
-      named_bar_sync(1 + t, 128);
+      // Every warp writes its own 32 rows out: after an abort the warps of a warpgroup may be at different items, and a barrier among
+      // them, which has no limit, could wait for ever.
       const TileInfo tinfo{qrow0, it.seq0, it.seq0 + it.len, 0};
       if (tile_store_by_tma(tinfo, N)) {
-        if (row == 0) {
-          for (int sl = 0; sl < C::kSlabs; ++sl) tma_store_3d(&tmO, stage + sl * C::kSlabBytes, sl * 64, qrow0, bh);
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0 && qt * C::kBlockM + row < it.len) {
+          for (int sl = 0; sl < C::kSlabs; ++sl) tma_store_3d(&tmO, stage + sl * C::kSlabBytes + row * 128, sl * 64, qrow0 + row, bh);
           bulk_commit_group();
           bulk_wait_group_read0();
-          mbar_arrive(&bar_q_free[qb]);                // this tile's slot of the Q buffer may be reloaded
         }
       } else {
         // ragged last tile of a packed sequence that another sequence follows: rows past its end are not ours to write
         store_rows_clipped<D>(stage, C::kSlabBytes, Og + (static_cast<size_t>(bh) * N + qrow0) * D, row, it.len - qt * C::kBlockM);
-        named_bar_sync(1 + t, 128);
-        if (row == 0) mbar_arrive(&bar_q_free[qb]);
+        __syncwarp();
       }
+      if (lane == 0) mbar_arrive(&bar_q_free[qb]);     // this tile's slot of the Q buffer may be reloaded
 #ifdef GPROJ_TRACE
       if (row == 0) tile_event(20 + t, lin, T, ev_n0, ev_n0, ev_n2, global_ns(), ev_c0, clock64());
 #endif

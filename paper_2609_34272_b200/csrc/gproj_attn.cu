@@ -370,7 +370,7 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
   const int BHkv = B * Hkv;
   CUtensorMap mQ, mK, mV, mO;
   if (!make_map(&mQ, Q, BH, N, d, 128) || !make_map(&mK, K, BHkv, Nk, d, 128) || !make_map(&mV, V, BHkv, Nk, d, 128) ||
-      !make_map(&mO, O, BH, N, d, 128))
+      !make_map(&mO, O, BH, N, d, 32))
     return GPROJ_ERR_CUDA;
   const float scale_log2 = static_cast<float>(static_cast<double>(softmax_scale) * 1.4426950408889634);
   // One work item = a pair of query tiles of one head (two softmax warpgroups ping-pong on the tensor core), or a single tile: where

@@ -56,3 +56,17 @@ def test_a_cta_that_skips_its_work_still_waits_for_the_previous_kernel():
                 branch = body[skip.start():body.index("return;", skip.start())]
                 assert "griddep_wait();" in branch or "griddep_wait();" in body[:skip.start()], name
     assert found == 5
+
+
+def test_softmax_warps_that_disagree_about_an_item_neither_hang_nor_leave_the_tensors():
+    # the forward's Q loader leaves an item's rank and head in shared memory for the softmax warps.  After a wait has given up they
+    # may read a slot too early or too late, each warp something else: it has to be an item of the launch all the same, so the
+    # slots are written before the kernel's first barrier, and no barrier without a limit may depend on what the item is
+    for name in ("attn_fwd.cuh", "attn_fwd_w64.cuh"):
+        body = open(os.path.join(CSRC, name)).read().split("__global__")[1]
+        setup = body[:body.index("fence_mbar_init();")]
+        assert re.search(r"for \(auto &slot : s_item\) slot\[0\] = slot\[1\] = 0;", setup), name
+        role = body[body.index("setmaxnreg_inc"):]
+        barriers = re.findall(r"named_bar_sync\([^;]*;|__syncthreads\(\);", role)
+        # behind the item loop, and in the cluster form, whose single item every warp reaches the barrier of
+        assert barriers == (["named_bar_sync(3, 256);", "__syncthreads();", "__syncthreads();"] if name == "attn_fwd.cuh" else ["__syncthreads();"]), (name, barriers)
