@@ -1,0 +1,36 @@
+"""The native call layer is optional: what the binding and the build do where it is unusable (no GPU needed)."""
+import warnings
+
+import pytest
+
+import __graft_entry__ as entry
+from paper_2609_34272_b200 import binding
+
+
+@pytest.fixture
+def unloaded(monkeypatch):
+    """The binding as in a new process."""
+    entry.build()
+    monkeypatch.setattr(binding, "_lib", None)
+    monkeypatch.setattr(binding, "_calls", None)
+
+
+def test_a_file_that_does_not_load_leaves_the_calls_to_ctypes(unloaded, tmp_path, monkeypatch):
+    bad = tmp_path / "_torch_calls.so"
+    bad.write_bytes(b"not a shared object")
+    monkeypatch.setattr(binding, "CALLS_PATH", str(bad))
+    with pytest.warns(RuntimeWarning, match="ctypes"):
+        lib = binding.load()                       # the first call is as good as any later one ...
+    with warnings.catch_warnings():
+        warnings.simplefilter("error")
+        assert binding.load() is lib               # ... and says so once
+    assert binding._calls is None and lib.gproj_attn_bwd_workspace_bytes(1, 2, 256, 64) > 0
+
+
+def test_a_call_that_fails_half_way_through_loading_is_repeated(unloaded, monkeypatch):
+    def fail(lib):
+        raise MemoryError
+    monkeypatch.setattr(binding, "_bind_native_calls", fail)
+    for _ in range(2):
+        with pytest.raises(MemoryError):
+            binding.load()
