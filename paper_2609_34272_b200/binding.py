@@ -12,9 +12,11 @@ import warnings
 
 import torch
 
+from .build import calls_path
+
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libgproj_attn.so")
-CALLS_PATH = os.path.join(_PKG, "_torch_calls.so")
+CALLS_PATH = calls_path()
 
 GPROJ_OK = 0
 FLAG_NO_Q_CORRECTION = 1

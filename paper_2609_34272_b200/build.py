@@ -2,16 +2,23 @@
 import os
 import subprocess
 import sys
+import warnings
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libgproj_attn.so")
-CALLS = os.path.join(PKG, "_torch_calls.so")
 CALLS_SOURCE = os.path.join(CSRC, "torch_calls.cpp")
 SOURCES = [os.path.join(CSRC, "gproj_attn.cu")]
 HEADERS = [os.path.join(CSRC, f) for f in ("host_rules.h", "tile_schedule.h", "wait_budget.h", "sm100_primitives.cuh", "attn_fwd.cuh", "attn_fwd_w64.cuh", "attn_bwd.cuh", "attn_bwd_w128.cuh", "key_smoothing.cuh", "attn_fp32.cuh")] + \
           [os.path.join(ROOT, "include", "gproj_attn.h")]
+
+
+def calls_path() -> str:
+    """The native call layer of this Python and this torch: it is bound to the binary interfaces of both, so each pair has its own file."""
+    import torch
+
+    return os.path.join(PKG, f"_torch_calls.{sys.implementation.cache_tag}-torch{torch.__version__}.so")
 
 
 def nvcc_command(verbose: bool = False):
@@ -31,7 +38,7 @@ def calls_command():
 
     includes = include_paths() + [sysconfig.get_paths()["include"], os.path.join(CUDA_HOME or "/usr/local/cuda", "include")]
     return ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"] + \
-        [f"-I{p}" for p in includes] + ["-o", CALLS, CALLS_SOURCE] + [f"-L{p}" for p in library_paths()] + ["-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+        [f"-I{p}" for p in includes] + ["-o", calls_path(), CALLS_SOURCE] + [f"-L{p}" for p in library_paths()] + ["-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
 
 
 def _up_to_date(target, deps):
@@ -49,8 +56,13 @@ def _run(cmd, verbose=False):
 def build(force: bool = False, verbose: bool = False) -> str:
     if force or not _up_to_date(LIB, SOURCES + HEADERS):
         _run(nvcc_command(verbose), verbose)
-    if force or not _up_to_date(CALLS, [CALLS_SOURCE]):
-        _run(calls_command())
+    if force or not _up_to_date(calls_path(), [CALLS_SOURCE]):
+        try:                       # optional: without it the calls go through ctypes
+            _run(calls_command())
+        except (OSError, RuntimeError) as e:
+            if os.path.exists(calls_path()):
+                os.remove(calls_path())                     # out of date: it may call the library by another signature
+            warnings.warn(f"the native call layer was not built, so calls take more host time: {e}", RuntimeWarning, stacklevel=2)
     return LIB
 
 

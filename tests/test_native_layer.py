@@ -1,10 +1,12 @@
 """The native call layer is optional: what the binding and the build do where it is unusable (no GPU needed)."""
+import os
+import sys
 import warnings
 
 import pytest
 
 import __graft_entry__ as entry
-from paper_2609_34272_b200 import binding
+from paper_2609_34272_b200 import binding, build
 
 
 @pytest.fixture
@@ -34,3 +36,31 @@ def test_a_call_that_fails_half_way_through_loading_is_repeated(unloaded, monkey
     for _ in range(2):
         with pytest.raises(MemoryError):
             binding.load()
+
+
+def test_another_torch_or_python_gets_a_layer_of_its_own(monkeypatch):
+    entry.build()
+    made = []
+    monkeypatch.setattr(build, "_run", lambda cmd, verbose=False: made.append(cmd[0]))
+    build.build()
+    assert made == [] and build.calls_path() == binding.CALLS_PATH
+    for owner, name in ((sys.modules["torch"], "__version__"), (sys.implementation, "cache_tag")):
+        with monkeypatch.context() as m:
+            m.setattr(owner, name, "0.0")
+            assert build.calls_path() != binding.CALLS_PATH
+            build.build()
+            assert made == ["g++"]
+        made.clear()
+
+
+def test_a_host_compiler_that_fails_does_not_fail_the_build(monkeypatch, tmp_path):
+    entry.build()
+    stale = tmp_path / "_torch_calls.so"
+    monkeypatch.setattr(build, "calls_path", lambda: str(stale))
+    for command in (["false"], ["/nonexistent/g++"]):
+        stale.write_bytes(b"")
+        os.utime(stale, (0, 0))
+        monkeypatch.setattr(build, "calls_command", lambda: command)
+        with pytest.warns(RuntimeWarning, match="native call layer"):
+            assert build.build() == build.LIB
+        assert not stale.exists()                  # an old one might call the library by another signature
