@@ -10,8 +10,9 @@ CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libgproj_attn.so")
 CALLS_SOURCE = os.path.join(CSRC, "torch_calls.cpp")
 SOURCES = [os.path.join(CSRC, "gproj_attn.cu")]
+ABI_HEADER = os.path.join(ROOT, "include", "gproj_attn.h")
 HEADERS = [os.path.join(CSRC, f) for f in ("host_rules.h", "tile_schedule.h", "wait_budget.h", "sm100_primitives.cuh", "attn_fwd.cuh", "attn_fwd_w64.cuh", "attn_bwd.cuh", "attn_bwd_w128.cuh", "key_smoothing.cuh", "attn_fp32.cuh")] + \
-          [os.path.join(ROOT, "include", "gproj_attn.h")]
+          [ABI_HEADER]
 
 
 def calls_path() -> str:
@@ -36,7 +37,7 @@ def calls_command():
     import torch
     from torch.utils.cpp_extension import CUDA_HOME, include_paths, library_paths
 
-    includes = include_paths() + [sysconfig.get_paths()["include"], os.path.join(CUDA_HOME or "/usr/local/cuda", "include")]
+    includes = [os.path.dirname(ABI_HEADER)] + include_paths() + [sysconfig.get_paths()["include"], os.path.join(CUDA_HOME or "/usr/local/cuda", "include")]
     return ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"] + \
         [f"-I{p}" for p in includes] + ["-o", calls_path(), CALLS_SOURCE] + [f"-L{p}" for p in library_paths()] + ["-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
 
@@ -56,7 +57,7 @@ def _run(cmd, verbose=False):
 def build(force: bool = False, verbose: bool = False) -> str:
     if force or not _up_to_date(LIB, SOURCES + HEADERS):
         _run(nvcc_command(verbose), verbose)
-    if force or not _up_to_date(calls_path(), [CALLS_SOURCE]):
+    if force or not _up_to_date(calls_path(), [CALLS_SOURCE, ABI_HEADER]):
         try:                       # optional: without it the calls go through ctypes
             _run(calls_command())
         except (OSError, RuntimeError) as e:

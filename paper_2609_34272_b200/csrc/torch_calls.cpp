@@ -7,6 +7,8 @@
 // Python and ctypes and take 16.9 here (three launches, eleven tensor maps, six allocations), 20.3 with the GPU's share.
 #include <Python.h>
 
+#include "gproj_attn.h"
+
 #include <ATen/ATen.h>
 #include <ATen/PythonTorchFunctionTLS.h>
 #include <c10/core/impl/TorchDispatchModeTLS.h>
@@ -19,13 +21,10 @@
 
 namespace {
 
-using FwdFn = int (*)(const void *, const void *, const void *, void *, float *, int, int, int, int, int, int, float, int, unsigned, void *);
-using BwdFn = int (*)(const void *, const void *, const void *, const void *, const float *, const void *, void *, void *, void *, int, int, int, int, int, int,
-                      float, int, void *, size_t, unsigned, void *);
-using BytesFn = size_t (*)(int, int, int, int);
-FwdFn fwd_fn = nullptr;       // gproj_attn_fwd_rect
-BwdFn bwd_fn = nullptr;       // gproj_attn_bwd_rect
-BytesFn bytes_fn = nullptr;   // gproj_attn_bwd_workspace_bytes
+// In the library that binding.py loaded; its types are the header's, so a signature that changes there does not compile here.
+decltype(&gproj_attn_fwd_rect) fwd_fn = nullptr;
+decltype(&gproj_attn_bwd_rect) bwd_fn = nullptr;
+decltype(&gproj_attn_bwd_workspace_bytes) bytes_fn = nullptr;
 
 struct Unusual {};            // leave the call to binding.py
 
@@ -131,9 +130,9 @@ PyObject *bwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
 PyObject *bind(PyObject *, PyObject *args) {
   unsigned long long f, b, w;
   if (!PyArg_ParseTuple(args, "KKK", &f, &b, &w)) return nullptr;
-  fwd_fn = reinterpret_cast<FwdFn>(f);
-  bwd_fn = reinterpret_cast<BwdFn>(b);
-  bytes_fn = reinterpret_cast<BytesFn>(w);
+  fwd_fn = reinterpret_cast<decltype(fwd_fn)>(f);
+  bwd_fn = reinterpret_cast<decltype(bwd_fn)>(b);
+  bytes_fn = reinterpret_cast<decltype(bytes_fn)>(w);
   Py_RETURN_NONE;
 }
 

@@ -1,5 +1,6 @@
 """The native call layer is optional: what the binding and the build do where it is unusable (no GPU needed)."""
 import os
+import subprocess
 import sys
 import warnings
 
@@ -64,3 +65,20 @@ def test_a_host_compiler_that_fails_does_not_fail_the_build(monkeypatch, tmp_pat
         with pytest.warns(RuntimeWarning, match="native call layer"):
             assert build.build() == build.LIB
         assert not stale.exists()                  # an old one might call the library by another signature
+
+
+def test_the_layer_calls_by_the_headers_signatures(tmp_path, monkeypatch):
+    entry.build()
+    # a call that does not fit a changed signature no longer compiles ...
+    changed = tmp_path / "gproj_attn.h"
+    changed.write_text(open(build.ABI_HEADER).read().replace("int gproj_attn_bwd_rect(", "int gproj_attn_bwd_rect(long long added, ", 1))
+    command = [c for c in build.calls_command() if c != "-shared"]
+    out = command.index("-o")
+    done = subprocess.run([command[0], "-fsyntax-only", f"-I{tmp_path}"] + command[1:out] + [command[out + 2]], capture_output=True, text=True)
+    assert done.returncode != 0 and "bwd_fn" in done.stderr
+    # ... and a changed header makes the layer out of date
+    made = []
+    monkeypatch.setattr(build, "_run", lambda cmd, verbose=False: made.append(cmd[0]))
+    monkeypatch.setattr(build, "ABI_HEADER", str(changed))
+    build.build()
+    assert made == ["g++"]
