@@ -72,6 +72,12 @@ PyObject *tuple_of(std::initializer_list<at::Tensor> ts) {
   return out;
 }
 
+// Other Python threads may run while this lives; it ends by an exception as well.
+struct NoGil {
+  PyThreadState *state = PyEval_SaveThread();
+  ~NoGil() { PyEval_RestoreThread(state); }
+};
+
 template <typename Body>
 PyObject *guarded(Body body) {
   try {
@@ -94,10 +100,7 @@ PyObject *fwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
     at::Tensor O = at::empty_like(Q), LSE = at::empty({s.B, s.H, s.Nq}, Q.options().dtype(at::kFloat));
     void *out = O.mutable_data_ptr();
     float *lse = static_cast<float *>(LSE.mutable_data_ptr());
-    int rc;
-    Py_BEGIN_ALLOW_THREADS
-    rc = fwd_fn(q, k, v, out, lse, s.B, s.H, s.Hkv, s.Nq, s.Nk, s.d, o.scale, o.causal, o.flags, stream);
-    Py_END_ALLOW_THREADS
+    const int rc = [&] { const NoGil free; return fwd_fn(q, k, v, out, lse, s.B, s.H, s.Hkv, s.Nq, s.Nk, s.d, o.scale, o.causal, o.flags, stream); }();
     return rc == 0 ? tuple_of({O, LSE}) : PyLong_FromLong(rc);
   });
 }
@@ -118,10 +121,7 @@ PyObject *bwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
     at::Tensor ws = at::empty({static_cast<int64_t>(bytes)}, Q.options().dtype(at::kByte));
     at::Tensor dQ = at::empty_like(Q), dK = at::empty_like(K), dV = at::empty_like(V);
     void *pq = dQ.mutable_data_ptr(), *pk = dK.mutable_data_ptr(), *pv = dV.mutable_data_ptr(), *pw = ws.mutable_data_ptr();
-    int rc;
-    Py_BEGIN_ALLOW_THREADS
-    rc = bwd_fn(q, k, v, out, lse, u, pq, pk, pv, s.B, s.H, s.Hkv, s.Nq, s.Nk, s.d, o.scale, o.causal, pw, bytes, o.flags, stream);
-    Py_END_ALLOW_THREADS
+    const int rc = [&] { const NoGil free; return bwd_fn(q, k, v, out, lse, u, pq, pk, pv, s.B, s.H, s.Hkv, s.Nq, s.Nk, s.d, o.scale, o.causal, pw, bytes, o.flags, stream); }();
     return rc == 0 ? tuple_of({dQ, dK, dV}) : PyLong_FromLong(rc);
   });
 }

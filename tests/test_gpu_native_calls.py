@@ -1,4 +1,7 @@
 """The dense calls as one native step: same results and the same refusals as by way of ctypes."""
+import ctypes
+import subprocess
+
 import pytest
 import torch
 
@@ -57,6 +60,24 @@ def test_refusals_are_those_of_the_checks(x):
     with pytest.raises(g.GprojError):
         g.gproj_attn_bwd(Q, K, V, O, LSE, dO, 0.125, True, flags=1 << 10)
     assert all(torch.equal(a, b) for a, b in zip(g.gproj_attn_fwd(Q, K, V, torch.tensor(0.125), 1), (O, LSE)))     # numbers of other types
+
+
+def test_an_exception_out_of_the_library_leaves_the_call_to_the_checks(x, tmp_path):
+    source = tmp_path / "throws.cpp"
+    source.write_text('#include <new>\nextern "C" int f() { throw std::bad_alloc(); }\nextern "C" unsigned long bytes() { return 4096; }\n')
+    subprocess.run(["g++", "-shared", "-fPIC", "-o", str(tmp_path / "throws.so"), str(source)], check=True)
+    fake, lib = ctypes.CDLL(str(tmp_path / "throws.so")), binding.load()
+    address = lambda f: ctypes.cast(f, ctypes.c_void_p).value
+    Q, K, V, dO = x
+    O, LSE = g.gproj_attn_fwd(Q, K, V, 0.125, True)
+    expected = g.gproj_attn_bwd(Q, K, V, O, LSE, dO, 0.125, True)
+    try:
+        binding._calls.bind(address(fake.f), address(fake.f), address(fake.bytes))
+        assert binding._calls.fwd(Q, K, V, 0.125, True, 0, True) is None
+        assert all(torch.equal(a, b) for a, b in zip(g.gproj_attn_fwd(Q, K, V, 0.125, True), (O, LSE)))
+        assert all(torch.equal(a, b) for a, b in zip(g.gproj_attn_bwd(Q, K, V, O, LSE, dO, 0.125, True), expected))
+    finally:
+        binding._calls.bind(*(address(getattr(lib, n)) for n in ("gproj_attn_fwd_rect", "gproj_attn_bwd_rect", "gproj_attn_bwd_workspace_bytes")))
 
 
 def test_function_and_dispatch_modes_see_the_call(x):
