@@ -368,10 +368,6 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
   }
   const int BH = B * H;
   const int BHkv = B * Hkv;
-  CUtensorMap mQ, mK, mV, mO;
-  if (!make_map(&mQ, Q, BH, N, d, 128) || !make_map(&mK, K, BHkv, Nk, d, 128) || !make_map(&mV, V, BHkv, Nk, d, 128) ||
-      !make_map(&mO, O, BH, N, d, 32))
-    return GPROJ_ERR_CUDA;
   const float scale_log2 = static_cast<float>(static_cast<double>(softmax_scale) * 1.4426950408889634);
   // One work item = a pair of query tiles of one head (two softmax warpgroups ping-pong on the tensor core), or a single tile: where
   // pairs leave too few items to balance the SMs, and at d = 64 wherever the kernel of attn_fwd_w64.cuh is not slower.
@@ -387,6 +383,11 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
   const int (&fit)[4] = st->fwd_clusters[d == 128];
   const int lg = (tiles_per_item == 1 && !fma && total_items <= fit[1]) ? fwd_cluster_log2(total_items, ((seqs ? longest_keys(*seqs) : Nk) + 127) / 128, fit) : 0;
   tl_form[GPROJ_FORM_FWD_CTAS] = 1 << lg;
+  const bool three = d == 64 && tiles_per_item == 1 && lg == 0 && fold == 0;   // the kernel of attn_fwd_w64.cuh, whose steps have 64 keys
+  CUtensorMap mQ, mK, mV, mO;
+  if (!make_map(&mQ, Q, BH, N, d, 128) || !make_map(&mK, K, BHkv, Nk, d, three ? 64 : 128) || !make_map(&mV, V, BHkv, Nk, d, three ? 64 : 128) ||
+      !make_map(&mO, O, BH, N, d, 32))
+    return GPROJ_ERR_CUDA;
   if (lg > 0 || fold > 0) {
     const int key_tiles_per_cta = (((seqs ? longest_keys(*seqs) : Nk) + 127) / 128) >> lg;   // at d = 128: which form, see FwdTmem in attn_fwd.cuh
     auto kernel = d == 64 ? (causal ? attn_fwd_kernel<64, true, false, 3> : attn_fwd_kernel<64, false, false, 3>)
@@ -426,12 +427,10 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
   // Single tiles: the softmax warpgroups split the key range of the tile (three of them at d = 64).  Pairs: one tile each; at d = 128 with both
   // warpgroups' scores in one place unless there is one tile to a head, and no pair.
   const bool split = (tiles_per_item == 1);
-  if (d == 64 && split) {
-    CUtensorMap mK64, mV64;
-    if (!make_map(&mK64, K, BHkv, Nk, d, 64) || !make_map(&mV64, V, BHkv, Nk, d, 64)) return GPROJ_ERR_CUDA;
+  if (three) {
     auto kernel = causal ? (fma ? attn_fwd_w64_kernel<true, true> : attn_fwd_w64_kernel<true, false>)
                          : (fma ? attn_fwd_w64_kernel<false, true> : attn_fwd_w64_kernel<false, false>);
-    launch_after(kernel, grid, 1, FwdW64Cfg::kThreads, FwdW64Cfg::kSmemBytes, s, early, mQ, mK64, mV64, mO, static_cast<__nv_bfloat16 *>(O), plan, LSE, N, Nk,
+    launch_after(kernel, grid, 1, FwdW64Cfg::kThreads, FwdW64Cfg::kSmemBytes, s, early, mQ, mK, mV, mO, static_cast<__nv_bfloat16 *>(O), plan, LSE, N, Nk,
                  H, G, total_items, fwd_order, scale_log2, softmax_scale, st->status_ptr);
   }
   else if (d == 64) { if (fma) GPROJ_LAUNCH_FWD(64, false, true, 0); else GPROJ_LAUNCH_FWD(64, false, false, 0); }

@@ -82,3 +82,10 @@ def test_the_layer_calls_by_the_headers_signatures(tmp_path, monkeypatch):
     monkeypatch.setattr(build, "ABI_HEADER", str(changed))
     build.build()
     assert made == ["g++"]
+
+
+def test_the_forward_encodes_each_tensor_map_once():
+    # an encoded map is 0.15 us of host time; the smallest calls are bound by that
+    source = open(build.SOURCES[0]).read()
+    body = source[source.index("int launch_fwd(", source.index("int launch_fwd(") + 1):]
+    assert body[:body.index("\n}\n")].count("make_map(&") == 4
