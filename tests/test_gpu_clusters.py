@@ -23,8 +23,8 @@ def tobits(t):
 FWD = [  # B, H, Hkv, Nq, Nk, causal, CTAs per tile, query heads taken as one (at d = 64, at d = 128)
     (1, 2, 2, 128, 1921, True, 4, 1, 1), (1, 2, 2, 130, 2048, False, 4, 1, 1), (13, 3, 3, 1, 2047, True, 2, 1, 1), (1, 2, 2, 257, 4100, True, 8, 1, 1),
     (1, 1, 1, 64, 5000, False, 8, 1, 1), (1, 8, 2, 16, 4096, True, 8, 1, 1), (9, 6, 2, 127, 2500, True, 2, 1, 1), (1, 4, 1, 33, 300, True, 1, 1, 1),
-    (1, 4, 2, 100, 40, True, 1, 1, 1), (1, 6, 2, 200, 2100, False, 4, 3, 3), (1, 8, 1, 1, 1, True, 1, 8, 1), (3, 4, 1, 96, 2049, True, 4, 1, 1),
-    (40, 8, 2, 1, 300, True, 1, 4, 4), (50, 8, 2, 20, 130, True, 1, 4, 4), (70, 8, 1, 33, 300, True, 1, 8, 8), (3, 64, 8, 5, 2300, True, 4, 8, 8),
+    (1, 4, 2, 100, 40, True, 1, 1, 1), (1, 6, 2, 200, 2100, False, 4, 3, 3), (1, 8, 1, 1, 1, True, 1, 1, 1), (3, 4, 1, 96, 2049, True, 4, 1, 1),
+    (40, 8, 2, 1, 300, True, 1, 4, 4), (50, 8, 2, 20, 130, True, 1, 4, 4), (70, 8, 1, 33, 300, True, 1, 1, 8), (3, 64, 8, 5, 2300, True, 4, 8, 8),
     (20, 12, 3, 60, 2100, True, 1, 4, 4), (8, 16, 4, 16, 8192, True, 4, 4, 4), (60, 8, 1, 3, 2, True, 1, 8, 8),
 ]
 
