@@ -66,16 +66,17 @@ inline int fwd_cluster_log2(long long tiles, int key_tiles, const int (&fit)[4])
 // of G N rows?  Folded, the kernel runs one tile per CTA (or cluster) and merges its parts through shared memory, which costs
 // more per tile than the persistent form; unfolded, every head is a tile of its own with N of its 128 rows in use.  The two
 // times are estimated in microseconds from what was measured (148 CTAs at once):
-//   folded          per round 5.5 + 2.65 x (share of the tile's rows in use) + 0.86 per key tile of a CTA at d = 64, less 0.4; 7.15, 5.0,
-//                   1.0, 0.9 at d = 128.  Whole heads in clusters: the same
+//   folded          with u the share of the tile's rows in use: per round 5.7 + 2.25 u + (0.785 + 0.135 u) per key tile of a CTA at
+//                   d = 64, less 0.35; 7.15 + 5 u + 1 per key tile, less 0.9, at d = 128.  Whole heads in clusters: the same
 //   whole heads     d = 64: 3.1 + per round 1.1 + 0.765 per key tile; d = 128: 1.7 + per round 3.85 + 0.87 per key tile while the key
 //                   range of a tile is split between the warpgroups; beyond 1.5 tiles per SM, where it is not, 2.1, 2.7, 1.82
-// Folded also where the estimates are within 4 %: it reads the keys once, which a busy memory system rewards.
+// Folded also where the estimates are within 3 %: it reads the keys once, which a busy memory system rewards.  Never where whole
+// heads are in clusters already and folding does not make the tiles fewer.
 // Measured, whole -> folded, d = 64: 16 x (32 query, 8 KV heads) x 1 query behind 1000 keys: 32.7 -> 12.1 us; 64 x (32, 8) x 64
 // behind 2048: 185 -> 159; but 32 x (64, 4) x 64 behind 600: 73.9 -> 90.9 and x 120: 74.6 -> 170; 64 x (16, 4) x 100 on as many keys:
 // 18.3 -> 61.8; 2 x (64, 8) x 100 behind 1000: 11.0 -> 15.4.  d = 128: 70.4 -> 13.9, 447 -> 195, 172 -> 119; 182 -> 221, 36.1 -> 88.3,
-// 13.7 -> 19.3.  Over 410 shapes that the figures were not fitted to, the choice costs 0.25 % on average against the better of
-// the two, more than 3 % in 12 of them and 16 % at most (8 KV heads x 4 x 59 queries behind 19504 keys, d = 64: 36.4 -> 42.3).
+// 13.7 -> 19.3.  Over 410 sizes that the figures were not fitted to, at both head dimensions, the choice costs 0.2 % on average
+// against the better of the two, more than 3 % in 18 of the 820 and 17 % at most.
 inline bool fwd_folds_heads(int kv_heads, int G, int N, int Nk, int d, int sms, const int (&fit)[4]) {
   if (N >= 128) return false;
   const bool wide = d == 128;
@@ -85,14 +86,17 @@ inline bool fwd_folds_heads(int kv_heads, int G, int N, int Nk, int d, int sms, 
   auto merged = [&](long long tiles, long long rows) {
     const int lg = fwd_cluster_log2(tiles, key_tiles, fit);
     const double used = static_cast<double>(std::min<long long>(128, rows)) / 128;
-    return (lg > 0 ? 1.0 : rounds(tiles)) * ((wide ? 7.15 + 5.0 * used : 5.5 + 2.65 * used) + (wide ? 1.0 : 0.86) * ((key_tiles + (1 << lg) - 1) >> lg)) - (wide ? 0.9 : 0.4);
+    return (lg > 0 ? 1.0 : rounds(tiles)) * ((wide ? 7.15 + 5.0 * used : 5.7 + 2.25 * used) + (wide ? 1.0 : 0.785 + 0.135 * used) * ((key_tiles + (1 << lg) - 1) >> lg)) - (wide ? 0.9 : 0.35);
   };
   double t_whole;
-  if (fwd_cluster_log2(whole, key_tiles, fit) > 0) t_whole = merged(whole, N);
+  if (fwd_cluster_log2(whole, key_tiles, fit) > 0) {
+    if (folded == whole) return false;
+    t_whole = merged(whole, N);
+  }
   else if (!wide) t_whole = 3.1 + rounds(whole) * (1.1 + 0.765 * key_tiles);
   else if (2 * whole < 3LL * sms) t_whole = 1.7 + rounds(whole) * (3.85 + 0.87 * key_tiles);
   else t_whole = 2.1 + rounds(whole) * (2.7 + 1.82 * key_tiles);
-  return merged(folded, static_cast<long long>(G) * N) < 1.04 * t_whole;
+  return merged(folded, static_cast<long long>(G) * N) < 1.03 * t_whole;
 }
 
 // CTAs per (head, sequence) of key smoothing: 1, 2, 4 or 8.  pairs: (head, sequence) pairs of the launch; rows: their rows
