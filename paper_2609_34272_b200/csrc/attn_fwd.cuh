@@ -10,9 +10,9 @@
 //                 the other one (the tensor-core queue is only 1-2 instructions deep, hence two issuing warps: each
 //                 one's barrier polls overlap the other's MMAs).
 // Work items (template parameter MODE):
-//   pairs (0)     one item = two 128-row query tiles of one (batch, head), warpgroup t <-> tile t, every K / V tile
-//                 serves both.
-//   pairs (5)     the same with separate rings for K and V (d = 128).
+//   pairs (5)     one item = two 128-row query tiles of one (batch, head), warpgroup t <-> tile t, every K / V tile
+//                 serves both; separate rings for K and V.
+//   one tile (0)  the same with one ring, for heads of a single tile, of which there are many: the second warpgroup idles.
 //   split (2)     one item = one query tile; warpgroup t takes the key tiles j = t (mod 2) with its own running
 //                 maximum, normaliser and accumulator, and warpgroup 0 merges the two halves at the end.  Used when
 //                 pairs would leave SMs idle and for packed sequences.
@@ -20,6 +20,7 @@
 //   cluster (3)   one item = one query tile on a cluster of 2, 4 or 8 CTAs that share its key tiles in the same way and
 //                 merge 4, 8 or 16 parts through distributed shared memory.  Used when even single tiles leave SMs
 //                 idle: a block of new queries behind a key history, a short batch.
+//   cluster (6)   the same with separate rings for K and V (d = 128, four or more key tiles to a CTA).
 // Softmax arithmetic (FMA_SOFTMAX = false, the default): online softmax on the UNSCALED logits with the
 // subtract-before-scale rounding of
 // Eq. "gproj-forward": z = exp2(fl32[ fl32(x - x_max) * (alpha log2 e) ]); l accumulates the FP32 z, the value
@@ -112,10 +113,10 @@ __device__ __forceinline__ float softmax_exp_store(const uint32_t (&xr)[4][32], 
   return (r0 + r1) + (r2 + r3);
 }
 
-// MODE: 0 = pairs of query tiles, 2 = single tiles with the key range split between the warpgroups, 3 = single tiles with the key
+// MODE: 0 = pairs of query tiles (of heads with one tile), 2 = single tiles with the key range split between the warpgroups, 3 = single tiles with the key
 // range split over the warpgroups of a cluster of CTAs (one tile per cluster; the parts of all CTAs are merged through
 // distributed shared memory), 4 = as 2, 5 = as 0, 6 = as 3, with separate rings for K and V and the scores of both warpgroups in one
-// place (d = 128).
+// place.  All at d = 128; at d = 64 only 3, everything else is attn_fwd_w64.cuh's.
 template <int D, bool CAUSAL, bool FMA_SOFTMAX, int MODE>
 __global__ void __launch_bounds__(384, 1)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,

@@ -17,7 +17,7 @@
 // merge of an item runs in one warpgroup while the others are in the next, and short items cost a third of what they did.
 // Measured, forward alone, two warpgroups on 128 keys (pairs or split tiles) -> this: 16 heads x 4096, causal: 58.0 -> 51.5 us; 96 x
 // 1000: 35.5 -> 29.8; 32 x 8192: 422 -> 391; 24 packed documents, 16676 rows, 16 heads: 101.8 -> 78.1; 200 documents of 30 to 300
-// rows: 178.8 -> 113.8; 64 x 2000, not causal: 117.6 -> 95.6; 32 x 8192, not causal: 729 -> 738 (stays with pairs: fwd_prefers_pairs).
+// rows: 178.8 -> 113.8; 64 x 2000, not causal: 117.6 -> 92.9; 32 x 8192, not causal: 730 -> 677.
 // Tried: four warpgroups with P~_w over S_w (59 us on the first of these; each product P~V is then on its warpgroup's way), P~_w
 // apart from S_w (55; waits for P~V), a pool for the probabilities alone (57.5), P~V(n) and S(n + 5) from one thread (63).
 #pragma once

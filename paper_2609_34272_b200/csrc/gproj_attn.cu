@@ -121,8 +121,6 @@ int device_state(DeviceState **out) {
       if (cudaGetSymbolAddress(reinterpret_cast<void **>(&st.status_ptr), g_device_status) != cudaSuccess)
         return GPROJ_ERR_CUDA;
       bool ok = true;
-      ok &= allow_smem(attn_fwd_kernel<64, false, false, 0>, FwdCfg<64>::kSmemBytes) == cudaSuccess;
-      ok &= allow_smem(attn_fwd_kernel<64, false, true, 0>, FwdCfg<64>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, true, false, 0>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, true, false, 2>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
       ok &= allow_smem(attn_fwd_kernel<128, true, true, 0>, FwdCfg<128>::kSmemBytes) == cudaSuccess;
@@ -370,10 +368,11 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
   const int BHkv = B * Hkv;
   const float scale_log2 = static_cast<float>(static_cast<double>(softmax_scale) * 1.4426950408889634);
   // One work item = a pair of query tiles of one head (two softmax warpgroups ping-pong on the tensor core), or a single tile: where
-  // pairs leave too few items to balance the SMs, and at d = 64 wherever the kernel of attn_fwd_w64.cuh is not slower.
+  // pairs leave too few items to balance the SMs, and at d = 64 always.  (Pairs at d = 64 are slower than the kernel of attn_fwd_w64.cuh.
+  // Measured without a mask, pairs -> single tiles: 32 heads x 8192: 730 -> 676 us; 64 x 4096: 380 -> 348; 128 x 512: 21.1 -> 20.8; the one
+  // exception is two full rounds of pairs on two key tiles, 296 x 256: 14.7 -> 15.6.)
   const int n_qt = plan ? n_plan_tiles : (N + 127) / 128;
-  int tiles_per_item = (!plan && static_cast<long long>(BH) * ((n_qt + 1) / 2) * 2 >= 3LL * st->sm_count) ? 2 : 1;
-  if (fold > 0 || (d == 64 && (causal || !fwd_prefers_pairs(BH, n_qt, (Nk + 127) / 128, st->sm_count)))) tiles_per_item = 1;
+  const int tiles_per_item = (d == 128 && !plan && fold == 0 && static_cast<long long>(BH) * ((n_qt + 1) / 2) * 2 >= 3LL * st->sm_count) ? 2 : 1;
   const int total_items = BH * ((n_qt + tiles_per_item - 1) / tiles_per_item);
   if (total_items <= 0) return GPROJ_OK;   // nothing but empty sequences
   ItemOrder fwd_order = item_order(BH, total_items / BH, tile_group_of(plan != nullptr, causal != 0, BH, total_items / BH, 2 * static_cast<size_t>(BHkv) * Nk * d * 2, st->sm_count,
@@ -383,7 +382,7 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
   const int (&fit)[4] = st->fwd_clusters[d == 128];
   const int lg = (tiles_per_item == 1 && !fma && total_items <= fit[1]) ? fwd_cluster_log2(total_items, ((seqs ? longest_keys(*seqs) : Nk) + 127) / 128, fit) : 0;
   tl_form[GPROJ_FORM_FWD_CTAS] = 1 << lg;
-  const bool three = d == 64 && tiles_per_item == 1 && lg == 0 && fold == 0;   // the kernel of attn_fwd_w64.cuh, whose steps have 64 keys
+  const bool three = d == 64 && lg == 0 && fold == 0;   // the kernel of attn_fwd_w64.cuh, whose steps have 64 keys
   CUtensorMap mQ, mK, mV, mO;
   if (!make_map(&mQ, Q, BH, N, d, 128) || !make_map(&mK, K, BHkv, Nk, d, three ? 64 : 128) || !make_map(&mV, V, BHkv, Nk, d, three ? 64 : 128) ||
       !make_map(&mO, O, BH, N, d, 32))
@@ -433,7 +432,6 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
     launch_after(kernel, grid, 1, FwdW64Cfg::kThreads, FwdW64Cfg::kSmemBytes, s, early, mQ, mK, mV, mO, static_cast<__nv_bfloat16 *>(O), plan, LSE, N, Nk,
                  H, G, total_items, fwd_order, scale_log2, softmax_scale, st->status_ptr);
   }
-  else if (d == 64) { if (fma) GPROJ_LAUNCH_FWD(64, false, true, 0); else GPROJ_LAUNCH_FWD(64, false, false, 0); }
   else if (split && sep_rings) GPROJ_LAUNCH_FWD_F(128, 4);
   else if (split) GPROJ_LAUNCH_FWD_F(128, 2);
   else if (n_qt > 1) GPROJ_LAUNCH_FWD_F(128, 5);

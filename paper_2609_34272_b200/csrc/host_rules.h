@@ -38,17 +38,6 @@ inline bool fwd_separate_rings(long long key_tiles, long long tiles) { return ke
 // (3.5) 147 -> 133, 1000 (4.5) 83.3 -> 83.3, 2300 (9.5) 212 -> 219; not causal: 256 (2) 142 -> 125, 384 (3) 123 -> 125, 500 (4) 181 -> 192.
 inline bool dq_short_tiles(long long key_tiles, long long tiles, bool causal) { return 2 * key_tiles <= (causal ? 7 : 5) * tiles; }
 
-// Forward at d = 64, no mask, clusters apart: pairs of query tiles (attn_fwd.cuh) or single tiles on three warpgroups
-// (attn_fwd_w64.cuh)?  All items are alike, so the rounds over the SMs decide.  Measured, in microseconds: a pair takes 1.6 per
-// 128 keys and 2.5 besides, a single tile 0.401 per 64 keys and 1.47 besides, so the steady states are equal and single tiles lose
-// only where two of them need more than the rounds of one pair.  Pairs, single tiles: 128 heads x 512 (256 pairs, 512 tiles)
-// 20.6, 21.6 us; 32 x 8192: 729, 738; 64 x 2000 (4 rounds, 7) 117.6, 95.6.  With a causal mask single tiles are always ahead: 16 x
-// 4096: 58.0, 51.5; 32 x 8192: 422, 391; 8 x 32768: 1517, 1470; 96 x 1000: 35.5, 29.8; 300 x 200: 20.6, 17.0.
-inline bool fwd_prefers_pairs(long long heads, int n_qt, int key_tiles, int sms) {
-  auto rounds = [&](long long items) { return static_cast<double>((items + sms - 1) / sms); };
-  return rounds(heads * ((n_qt + 1) / 2)) * (1.6 * key_tiles + 2.5) < rounds(heads * n_qt) * (0.802 * key_tiles + 1.47);
-}
-
 // CTAs per query tile of the forward (its base-two logarithm): with few tiles and long key ranges a tile's key range is
 // split over a cluster of 2, 4 or 8 CTAs, as many as leave each of their two warpgroups at least two 128-key tiles and let
 // all clusters run at once (`fit`: how many clusters of 2^lg CTAs do).  Beyond one wave the split only adds its merge, and
