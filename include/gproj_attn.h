@@ -310,11 +310,20 @@ int gproj_last_launch_count(void);
  *   GPROJ_FORM_FWD_CTAS   CTAs that share a query tile of the forward (1, 2, 4 or 8)
  *   GPROJ_FORM_FWD_HEADS  query heads of a KV head taken as one head by the forward (1: none)
  *   GPROJ_FORM_DQ_CTAS    CTAs that share a query tile of the dQ side (0: not run, 1 or 2)
- *   GPROJ_FORM_DKV_CTAS   CTAs that share a key tile of the dK/dV side (0: not run, 1 or 2) */
+ *   GPROJ_FORM_DKV_CTAS   CTAs that share a key tile of the dK/dV side (0: not run, 1 or 2)
+ *   GPROJ_FORM_FWD_KERNEL kernel of the forward, one of GPROJ_FWD_KERNEL_* */
 #define GPROJ_FORM_FWD_CTAS 0
 #define GPROJ_FORM_FWD_HEADS 1
 #define GPROJ_FORM_DQ_CTAS 2
 #define GPROJ_FORM_DKV_CTAS 3
+#define GPROJ_FORM_FWD_KERNEL 4
+#define GPROJ_FWD_KERNEL_THREE 1         /* d = 64: single tiles, three softmax warpgroups on 64-key steps */
+#define GPROJ_FWD_KERNEL_PAIRS 2         /* d = 128 from here on: pairs of query tiles */
+#define GPROJ_FWD_KERNEL_ONE_TILE 3      /* heads of one query tile, many of them */
+#define GPROJ_FWD_KERNEL_SPLIT 4         /* single tiles, key range split between two warpgroups, one ring for K and V */
+#define GPROJ_FWD_KERNEL_SPLIT_RINGS 5   /* the same, a ring each */
+#define GPROJ_FWD_KERNEL_CLUSTER 6       /* single tiles, key range split over a cluster's warpgroups (both head dimensions) */
+#define GPROJ_FWD_KERNEL_CLUSTER_RINGS 7 /* the same, a ring each */
 int gproj_last_form(int what);
 
 #ifdef __cplusplus

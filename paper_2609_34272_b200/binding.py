@@ -24,7 +24,8 @@ FLAG_NO_K_CORRECTION = 2
 FLAG_ONLY_DQ_PASS = 4
 FLAG_ONLY_DKV_PASS = 8
 FWD_FLAG_FMA_SOFTMAX = 1
-FORM_FWD_CTAS, FORM_FWD_HEADS, FORM_DQ_CTAS, FORM_DKV_CTAS = range(4)
+FORM_FWD_CTAS, FORM_FWD_HEADS, FORM_DQ_CTAS, FORM_DKV_CTAS, FORM_FWD_KERNEL = range(5)
+FWD_KERNELS = (None, "three", "pairs", "one tile", "split", "split, rings", "cluster", "cluster, rings")     # by the value of FORM_FWD_KERNEL
 
 STATIC_SCRATCH_BYTES = 16 << 20
 

@@ -66,7 +66,7 @@ std::mutex g_pipe_mutex;   // serialises the host-buffer entry point's use of th
 DeviceState g_dev[kMaxDevices];
 EncodeTiledFn g_encode = nullptr;
 thread_local int tl_launch_count = 0;
-thread_local int tl_form[4] = {};   // gproj_last_form
+thread_local int tl_form[5] = {};   // gproj_last_form
 
 template <typename Kernel>
 cudaError_t allow_smem(Kernel kernel, int bytes) {
@@ -380,7 +380,8 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   tl_form[GPROJ_FORM_FWD_HEADS] = Hkv == H ? Hq / Hkv : 1;
   const int (&fit)[4] = st->fwd_clusters[d == 128];
-  const int lg = (tiles_per_item == 1 && !fma && total_items <= fit[1]) ? fwd_cluster_log2(total_items, ((seqs ? longest_keys(*seqs) : Nk) + 127) / 128, fit) : 0;
+  const int key_tiles = ((seqs ? longest_keys(*seqs) : Nk) + 127) / 128;      // of the longest sequence
+  const int lg = (tiles_per_item == 1 && !fma && total_items <= fit[1]) ? fwd_cluster_log2(total_items, key_tiles, fit) : 0;
   tl_form[GPROJ_FORM_FWD_CTAS] = 1 << lg;
   const bool three = d == 64 && lg == 0 && fold == 0;   // the kernel of attn_fwd_w64.cuh, whose steps have 64 keys
   CUtensorMap mQ, mK, mV, mO;
@@ -388,10 +389,11 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
       !make_map(&mO, O, BH, N, d, 32))
     return GPROJ_ERR_CUDA;
   if (lg > 0 || fold > 0) {
-    const int key_tiles_per_cta = (((seqs ? longest_keys(*seqs) : Nk) + 127) / 128) >> lg;   // at d = 128: which form, see FwdTmem in attn_fwd.cuh
+    const bool rings = d == 128 && fwd_cluster_separate_rings(key_tiles, lg);
+    tl_form[GPROJ_FORM_FWD_KERNEL] = rings ? GPROJ_FWD_KERNEL_CLUSTER_RINGS : GPROJ_FWD_KERNEL_CLUSTER;
     auto kernel = d == 64 ? (causal ? attn_fwd_kernel<64, true, false, 3> : attn_fwd_kernel<64, false, false, 3>)
-              : key_tiles_per_cta < 4 ? (causal ? attn_fwd_kernel<128, true, false, 3> : attn_fwd_kernel<128, false, false, 3>)
-                                      : (causal ? attn_fwd_kernel<128, true, false, 6> : attn_fwd_kernel<128, false, false, 6>);
+                : !rings  ? (causal ? attn_fwd_kernel<128, true, false, 3> : attn_fwd_kernel<128, false, false, 3>)
+                          : (causal ? attn_fwd_kernel<128, true, false, 6> : attn_fwd_kernel<128, false, false, 6>);
     launch_after(kernel, dim3(static_cast<unsigned>(total_items) << lg), 1 << lg, FwdCfg<64>::kThreads,
                  d == 64 ? FwdCfg<64>::kSmemBytes : FwdCfg<128>::kSmemBytes, s, true, mQ, mK, mV, mO, static_cast<__nv_bfloat16 *>(O), plan, LSE, N, Nk,
                  BH, H, G, fold, tiles_per_item, total_items, fwd_order, scale_log2, softmax_scale, st->status_ptr);
@@ -400,11 +402,11 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
     return GPROJ_OK;
   }
   // One item per CTA: the longest tile counts.
-  bool sep_rings = d == 128 && tiles_per_item == 1 && total_items <= st->sm_count && (seqs ? longest_keys(*seqs) : Nk) > 2 * 128;
+  bool sep_rings = d == 128 && tiles_per_item == 1 && total_items <= st->sm_count && key_tiles > 2;
   if (seqs && total_items > st->sm_count && total_items <= 16LL * st->sm_count) {
-    const std::vector<int> key_tiles = tile_steps(*seqs, false, 128, 1);
-    fwd_order.solo = solo_ctas(key_tiles, BH, st->sm_count, 2.1);
-    sep_rings = d == 128 && fwd_separate_rings(key_tiles, BH, st->sm_count, fwd_order.solo);
+    const std::vector<int> of_each = tile_steps(*seqs, false, 128, 1);
+    fwd_order.solo = solo_ctas(of_each, BH, st->sm_count, 2.1);
+    sep_rings = d == 128 && fwd_separate_rings(of_each, BH, st->sm_count, fwd_order.solo);
   } else if (d == 128 && !sep_rings && tiles_per_item == 1) {
     sep_rings = fwd_separate_rings(seqs ? walked_key_tiles(*seqs) : fwd_key_tiles(N, Nk, causal != 0), n_qt);
   }
@@ -426,6 +428,8 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
   // Single tiles: the softmax warpgroups split the key range of the tile (three of them at d = 64).  Pairs: one tile each; at d = 128 with both
   // warpgroups' scores in one place unless there is one tile to a head, and no pair.
   const bool split = (tiles_per_item == 1);
+  tl_form[GPROJ_FORM_FWD_KERNEL] = three ? GPROJ_FWD_KERNEL_THREE : split ? (sep_rings ? GPROJ_FWD_KERNEL_SPLIT_RINGS : GPROJ_FWD_KERNEL_SPLIT)
+                                 : n_qt > 1 ? GPROJ_FWD_KERNEL_PAIRS : GPROJ_FWD_KERNEL_ONE_TILE;
   if (three) {
     auto kernel = causal ? (fma ? attn_fwd_w64_kernel<true, true> : attn_fwd_w64_kernel<true, false>)
                          : (fma ? attn_fwd_w64_kernel<false, true> : attn_fwd_w64_kernel<false, false>);
@@ -986,7 +990,7 @@ const char *gproj_status_string(int status) {
 
 int gproj_last_launch_count(void) { return tl_launch_count; }
 
-int gproj_last_form(int what) { return what >= 0 && what < 4 ? tl_form[what] : -1; }
+int gproj_last_form(int what) { return what >= 0 && what < 5 ? tl_form[what] : -1; }
 
 // ---- fused FP32 attention (comparison arm; plain SIMT arithmetic) ------------------------------------------------------
 size_t gproj_fp32_attn_saved_bytes(int B, int H, int N, int d) {

@@ -33,6 +33,10 @@ inline long long fwd_key_tiles(int lq, int lk, bool causal) {
 // -> 8.6, 384 (3) 17.5 -> 15.2; one item per CTA, causal: 16 x 500 (4) 10.6 -> 9.3, 16 x 300 (3) 8.7 -> 8.2, 16 x 200 (2) 7.0 -> 7.2.
 inline bool fwd_separate_rings(long long key_tiles, long long tiles) { return key_tiles >= 3 * tiles; }
 
+// The same with a cluster of 2^lg CTAs (or query heads folded, lg = 0): from four key tiles to a CTA on, below that the second warpgroup
+// would only wait for its first scores (see FwdTmem in attn_fwd.cuh).
+inline bool fwd_cluster_separate_rings(int key_tiles, int lg) { return (key_tiles >> lg) >= 4; }
+
 // dQ side at d = 128: are the tiles so short that the compute warpgroups should prepare the row constants (SHORT in attn_bwd.cuh)?
 // key_tiles, tiles: of one head.  Measured, off -> on, causal, rows (key tiles per tile): 256 (1.5) 162 -> 124 us, 500 (2.5) 371 -> 293, 700
 // (3.5) 147 -> 133, 1000 (4.5) 83.3 -> 83.3, 2300 (9.5) 212 -> 219; not causal: 256 (2) 142 -> 125, 384 (3) 123 -> 125, 500 (4) 181 -> 192.

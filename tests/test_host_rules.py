@@ -19,6 +19,7 @@ int smooth(long long pairs, long long rows, int longest, int d) { return smooth_
 long long key_tiles(int lq, int lk, int causal) { return fwd_key_tiles(lq, lk, causal != 0); }
 int short_tiles(long long key_tiles, long long tiles, int causal) { return dq_short_tiles(key_tiles, tiles, causal != 0); }
 int packed_rings(const int *key_tiles, int n, int heads, int solo) { return fwd_separate_rings(std::vector<int>(key_tiles, key_tiles + n), heads, 148, solo); }
+int cluster_rings(int key_tiles, int lg) { return fwd_cluster_separate_rings(key_tiles, lg); }
 int rings(long long key_tiles, long long tiles) { return fwd_separate_rings(key_tiles, tiles); }
 double deal(const int *steps, int n, int heads, int ctas, int solo, double per_item) {
   return deal_tiles(std::vector<int>(steps, steps + n), heads, ctas, [&](int s) { return s + per_item; }, solo);
@@ -137,6 +138,11 @@ def test_tiles_are_not_listed_where_the_deal_does_not_matter(rules):
     short = [128 * i for i in range(101)]
     cu_q, cu_k = ((ctypes.c_int * 102)(0, *[first + x for x in short]) for first in (300, 9000))
     assert rules.form(cu_q, cu_k, 101, 0, 1, 0, 1, 12, 103) == 36                   # three long tiles of 12 heads, 1200 short ones
+
+
+def test_separate_rings_in_clusters_from_four_key_tiles_of_a_cta_on(rules):
+    assert [rules.cluster_rings(n, 0) for n in (1, 3, 4, 5)] == [0, 0, 1, 1]
+    assert [rules.cluster_rings(n, 2) for n in (15, 16)] == [0, 1] and rules.cluster_rings(16, 1) == 1
 
 
 def test_separate_rings_of_a_packed_call_follow_its_longest_cta(rules):
