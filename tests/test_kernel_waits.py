@@ -36,26 +36,30 @@ def test_every_wait_that_may_span_a_tile_has_the_tile_limit():
     # loaders of a stationary tile, epilogues, parts of another CTA (what waits for an epilogue waits for its last microseconds)
     bars = "res_free|acc_done|mass_ready|peer_mass|peer_ready|peer_full|peer_free|q_free"
     found = 0
-    for name in ("attn_fwd.cuh", "attn_bwd.cuh", "attn_bwd_w128.cuh"):
+    for name in ("attn_fwd.cuh", "attn_fwd_w64.cuh", "attn_bwd.cuh", "attn_bwd_w128.cuh"):
+        here = found
         for line in open(os.path.join(CSRC, name)):
             for call in re.findall(r"mbar_wait(?:_cluster)?\(&bar_(?:%s)\b[^;]*;" % bars, line):
                 found += 1
                 assert any(b in call for b in ("tile_budget()", "kTileBudget", "tile_wait_budget(")), (name, call)
-    assert found >= 16
+        assert found > here, name
+    assert found >= 17
 
 
 def test_a_cta_that_skips_its_work_still_waits_for_the_previous_kernel():
     # after a wait has given up, the CTAs of later launches return at once; one that was launched early (programmatic
     # dependent launch) must not let its grid end before the one in front of it, which may still be writing
     found = 0
-    for name, kernels in (("attn_fwd.cuh", 1), ("attn_bwd.cuh", 2), ("attn_bwd_w128.cuh", 1)):
-        for body in open(os.path.join(CSRC, name)).read().split("__global__")[1:]:
+    for name, kernels in (("attn_fwd.cuh", 1), ("attn_fwd_w64.cuh", 1), ("attn_bwd.cuh", 2), ("attn_bwd_w128.cuh", 1)):
+        bodies = open(os.path.join(CSRC, name)).read().split("__global__")[1:]
+        assert len(bodies) == kernels, name
+        for body in bodies:
             for skip in re.finditer(r"if \([^()]*cta_skip != 0\)", body):
                 found += 1
                 # the wait stands in the branch, in front of the return, or on everybody's way before the branch
                 branch = body[skip.start():body.index("return;", skip.start())]
                 assert "griddep_wait();" in branch or "griddep_wait();" in body[:skip.start()], name
-    assert found == 5
+    assert found == 6
 
 
 def test_softmax_warps_that_disagree_about_an_item_neither_hang_nor_leave_the_tensors():
