@@ -376,7 +376,7 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
   const int total_items = BH * ((n_qt + tiles_per_item - 1) / tiles_per_item);
   if (total_items <= 0) return GPROJ_OK;   // nothing but empty sequences
   ItemOrder fwd_order = item_order(BH, total_items / BH, tile_group_of(plan != nullptr, causal != 0, BH, total_items / BH, 2 * static_cast<size_t>(BHkv) * Nk * d * 2, st->sm_count,
-                                                            tiles_per_item == 2 ? 1.45 : d == 64 ? 1.8 : 6.8));
+                                                            fwd_item_cost(d, tiles_per_item == 2)));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   tl_form[GPROJ_FORM_FWD_HEADS] = Hkv == H ? Hq / Hkv : 1;
   const int (&fit)[4] = st->fwd_clusters[d == 128];
@@ -405,7 +405,7 @@ int launch_fwd(const void *Q, const void *K, const void *V, void *O, float *LSE,
   bool sep_rings = d == 128 && tiles_per_item == 1 && total_items <= st->sm_count && key_tiles > 2;
   if (seqs && total_items > st->sm_count && total_items <= 16LL * st->sm_count) {
     const std::vector<int> of_each = tile_steps(*seqs, false, 128, 1);
-    fwd_order.solo = solo_ctas(of_each, BH, st->sm_count, 2.1);
+    fwd_order.solo = solo_ctas(of_each, BH, st->sm_count, fwd_item_cost(d, false));
     sep_rings = d == 128 && fwd_separate_rings(of_each, BH, st->sm_count, fwd_order.solo);
   } else if (d == 128 && !sep_rings && tiles_per_item == 1) {
     sep_rings = fwd_separate_rings(seqs ? walked_key_tiles(*seqs) : fwd_key_tiles(N, Nk, causal != 0), n_qt);

@@ -25,6 +25,13 @@ inline long long fwd_key_tiles(int lq, int lk, bool causal) {
   return ones + n * (ones + 1 + e + tq + e) / 2 - (n > 0 ? std::max<long long>(0, tq + e - tk) : 0);
 }
 
+// What an item of the forward costs beside its key tiles, in key tiles; for a pair of query tiles in ranks, of two key tiles each.
+// Measured, in microseconds per item and per key tile: d = 64: 1.4 and 0.77; d = 128, single tiles: 3.1 and 1.45.  Pairs take 3 and 2.05,
+// which would be 0.7; the 1.45 of an older kernel stays.  It groups ranks (tile_group_of) in 30 of 557 sizes where 0.7 does not: 88 heads x
+// 3968 x 128, causal: 349 us (0.7: 352) in a short burst, 438 (391) under the power limit; 64 x 7424: 747 (790), 894 (874).  For the CTAs
+// with one item (solo_ctas) 1.2 to 2.4 are alike.
+inline double fwd_item_cost(int d, bool pairs) { return d == 64 ? 1.8 : pairs ? 1.45 : 2.1; }
+
 // Forward at d = 128 with the key range of a tile split between the warpgroups: separate rings for K and V (see attn_fwd.cuh)?
 // From three key tiles per item on (key_tiles, tiles: of one head, or of the items of one CTA; with one item per CTA: of the longest item).
 // Measured, one ring -> two, 16 query / 4 KV heads, 40000 rows in sequences of one length, causal: 512 rows (2.5 key tiles per item)
@@ -185,13 +192,14 @@ double deal_tiles(const std::vector<int> &steps, int heads, int ctas, CostOf cos
 }
 
 // fwd_separate_rings for a packed call of few items per CTA: what counts is the CTA that takes longest (its items' key tiles, and
-// 2.1 more for each), which has long tiles where the others have many short ones.  48 documents of 6288 rows together, 2 heads, causal: one
+// fwd_item_cost more for each), which has long tiles where the others have many short ones.  48 documents of 6288 rows together, 2 heads, causal: one
 // ring 23.5 us, two 19.8; 49 pairs of 3485 queries and 13379 keys, 4 heads: 26.9, 23.1.
 inline bool fwd_separate_rings(const std::vector<int> &key_tiles, int heads, int sms, int solo) {
-  const std::vector<double> load = deal_tile_loads(key_tiles, heads, sms, [](int n) { return n + 2.1; }, solo);
+  const double cost = fwd_item_cost(128, false);
+  const std::vector<double> load = deal_tile_loads(key_tiles, heads, sms, [&](int n) { return n + cost; }, solo);
   const std::vector<double> items = deal_tile_loads(key_tiles, heads, sms, [](int) { return 1.0; }, solo);
   const size_t c = static_cast<size_t>(std::max_element(load.begin(), load.end()) - load.begin());
-  return load[c] - 2.1 * items[c] >= 3.0 * items[c] - 1e-6;
+  return load[c] - cost * items[c] >= 3.0 * items[c] - 1e-6;
 }
 
 // TileSched's solo CTAs for `heads` copies of tiles with the given costs (decreasing): those whose first item is longer than

@@ -19,6 +19,7 @@ int smooth(long long pairs, long long rows, int longest, int d) { return smooth_
 long long key_tiles(int lq, int lk, int causal) { return fwd_key_tiles(lq, lk, causal != 0); }
 int short_tiles(long long key_tiles, long long tiles, int causal) { return dq_short_tiles(key_tiles, tiles, causal != 0); }
 int packed_rings(const int *key_tiles, int n, int heads, int solo) { return fwd_separate_rings(std::vector<int>(key_tiles, key_tiles + n), heads, 148, solo); }
+double item_cost(int d, int pairs) { return fwd_item_cost(d, pairs != 0); }
 int cluster_rings(int key_tiles, int lg) { return fwd_cluster_separate_rings(key_tiles, lg); }
 int rings(long long key_tiles, long long tiles) { return fwd_separate_rings(key_tiles, tiles); }
 double deal(const int *steps, int n, int heads, int ctas, int solo, double per_item) {
@@ -138,6 +139,14 @@ def test_tiles_are_not_listed_where_the_deal_does_not_matter(rules):
     short = [128 * i for i in range(101)]
     cu_q, cu_k = ((ctypes.c_int * 102)(0, *[first + x for x in short]) for first in (300, 9000))
     assert rules.form(cu_q, cu_k, 101, 0, 1, 0, 1, 12, 103) == 36                   # three long tiles of 12 heads, 1200 short ones
+
+
+def test_one_cost_of_an_item_in_every_weighing_of_the_forward(rules):
+    rules.item_cost.restype = ctypes.c_double
+    assert [rules.item_cost(64, 0), rules.item_cost(128, 0), rules.item_cost(128, 1)] == [1.8, 2.1, 1.45]
+    text = open(os.path.join(CSRC, "gproj_attn.cu")).read()
+    body = text[text.rindex("int launch_fwd("):text.index("gproj_attn_bwd_workspace_bytes(")]
+    assert re.findall(r"(?:solo_ctas|tile_group_of)\(.*?fwd_item_cost\(d, [^)]*\)", body, re.S).__len__() == 2
 
 
 def test_separate_rings_in_clusters_from_four_key_tiles_of_a_cta_on(rules):
