@@ -32,13 +32,12 @@ UNIT = "TFLOP/s"
 NCU_DRAM_BYTES_PER_LAUNCH = {
     ("bwd_dkv_w128_kernel", 2): (44.1e6 + 1.1e6, "profiles/bwd_fwd_kernels_cfg2_ncu.md"),
     ("bwd_dq_kernel", 2): (42.3e6 + 0.7e6, "profiles/bwd_fwd_kernels_cfg2_ncu.md"),
-    ("attn_fwd_kernel", 2): (25.2e6 + 0.0e6, "profiles/bwd_fwd_kernels_cfg2_ncu.md"),
+    ("attn_fwd_w64_kernel", 2): (25.2e6 + 0.0e6, "profiles/steps_4096_counters_ncu.md"),
+    ("attn_fwd_kernel", 3): (25.2e6 + 0.0e6, "profiles/steps_4096_counters_ncu.md"),
     ("bwd_dkv_kernel", 4): (1351.9e6 + 516.8e6, "profiles/bwd_fwd_kernels_cfg4_dram_ncu.md"),
     ("bwd_dq_kernel", 4): (1347.8e6 + 521.5e6, "profiles/bwd_fwd_kernels_cfg4_dram_ncu.md"),
-    ("attn_fwd_kernel", 4): (805.6e6 + 253.8e6, "profiles/bwd_fwd_kernels_cfg4_dram_ncu.md"),
     ("bwd_dkv_kernel", 5): (1552.6e6 + 110.8e6, "profiles/bwd_fwd_kernels_cfg4_dram_ncu.md"),
     ("bwd_dq_kernel", 5): (1057.8e6 + 114.4e6, "profiles/bwd_fwd_kernels_cfg4_dram_ncu.md"),
-    ("attn_fwd_kernel", 5): (557.8e6 + 61.1e6, "profiles/bwd_fwd_kernels_cfg4_dram_ncu.md"),
 }
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 
@@ -106,7 +105,7 @@ def flops(w):
 # Contractions per tile pair of each kernel: executed, and the share of the 7 the method itself needs (Algorithm 1: S, dP,
 # dV, tK, rK, t^T Q, r^T Z).  The dQ side computes S, dP, tK, rK (all four are the method's); the dK/dV side computes S^T,
 # dP^T again (recomputation of the two-kernel design) and dV, t^T Q, r^T Z (the method's).
-KERNEL_UNITS = {"bwd_dq_kernel": (4, 4), "bwd_dkv_w128_kernel": (5, 3), "bwd_dkv_kernel": (5, 3), "attn_fwd_kernel": (2, 2)}
+KERNEL_UNITS = {"bwd_dq_kernel": (4, 4), "bwd_dkv_w128_kernel": (5, 3), "bwd_dkv_kernel": (5, 3), "attn_fwd_w64_kernel": (2, 2), "attn_fwd_kernel": (2, 2)}
 
 
 def stats_ms(xs):
@@ -276,7 +275,7 @@ def main():
         return max_over_ranks(sum(e[0].elapsed_time(e[1]) for e in evk), world) / n_k
 
     kernels_ms = {"bwd_dq_kernel": alone(lambda: bwd(g.FLAG_ONLY_DQ_PASS)), dkv_name: alone(lambda: bwd(g.FLAG_ONLY_DKV_PASS)),
-                  "attn_fwd_kernel": alone(fwd)}
+                  "attn_fwd_w64_kernel" if w.d == 64 else "attn_fwd_kernel": alone(fwd)}
 
     # a second, long region: backward calls back to back (no L2 flush, no gaps) for a few seconds, with the SM clock
     # sampled throughout -- the rate the part sustains under its power limit, next to the burst number above
