@@ -12,7 +12,8 @@
 // What bounds it.  The exponentials of a key tile (128 x 128) keep the special-function unit busy for 1024 clk; with all that goes
 // with them (maximum, subtraction, scale, sum, packing, TMEM) two or more warps per scheduler sustain 1140.  Each warp also spends
 // 700 to 1000 clk per step on barriers, TMEM loads and the maximum, in which the others have the unit to themselves: with two
-// warps per scheduler it was busy 70 % of the time, and an item's epilogue idled it altogether.  Three warps per scheduler
+// warps per scheduler it idled a third of the time, and throughout an item's epilogue (its pipe over a launch of 16 heads x 4096, by ncu:
+// 59 % of the peak then, 65 % now).  Three warps per scheduler
 // hide that better (more than three do not fit: 64 columns of TMEM for each O_w and at least 64 for its scores), the
 // merge of an item runs in one warpgroup while the others are in the next, and short items cost a third of what they did.
 // Measured, forward alone, two warpgroups on 128 keys (pairs or split tiles) -> this: 16 heads x 4096, causal: 58.0 -> 51.5 us; 96 x

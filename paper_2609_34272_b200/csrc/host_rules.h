@@ -51,11 +51,11 @@ inline bool dq_short_tiles(long long key_tiles, long long tiles, bool causal) { 
 
 // CTAs per query tile of the forward (its base-two logarithm): with few tiles and long key ranges a tile's key range is
 // split over a cluster of 2, 4 or 8 CTAs, as many as leave each of their two warpgroups at least two 128-key tiles and let
-// all clusters run at once (`fit`: how many clusters of 2^lg CTAs do).  Beyond one wave the split only adds its merge, and
-// below 16 key tiles the launch and the merge of a cluster cost what they save.  Measured, one CTA per tile -> cluster: 8 x (16
-// query, 4 KV heads) x 16 queries behind 16384 keys, d = 64: 109.7 -> 45.7 us (with the query heads folded, see
-// fwd_folds_heads), behind 8192: 58.5 -> 27.2, behind 2048: 20.6 -> 13.6; 4 x 8 heads x 1 query behind 16384 keys, d = 128: 201 ->
-// 63 us; 4 heads x 1000 x 128 (8 key tiles, with a merge by scattered stores): 18.7 -> 20.7 us, hence the 16.
+// all clusters run at once (`fit`: how many clusters of 2^lg CTAs do).  Beyond one wave the split only adds its merge.  Measured, one
+// CTA per tile -> cluster, d = 64: 49 heads x 15 queries behind 17059 keys: 104 -> 59.3 us (two CTAs), 61 x 3 behind 6496: 42.6 ->
+// 27.1, 17 x 128 behind 8346: 53.1 -> 25.2 (four); d = 128: 56.6 -> 27.5, 13 x 128 behind 13398: 94.2 -> 26.8 (eight).  At 7 to 12 key
+// tiles it depends on the tiles: 64 x 128 behind 915: 10.6 -> 13.0, but 3 x 63 behind 1490: 13.0 -> 8.7 with eight CTAs and 16 x 1
+// behind 842: 9.1 -> 7.4 with four, which the limit of 16 key tiles, as an older merge needed it, leaves out.
 inline int fwd_cluster_log2(long long tiles, int key_tiles, const int (&fit)[4]) {
   int lg = 0;
   while (lg < 3 && key_tiles >= std::max(16, 4 << (lg + 1)) && tiles <= fit[lg + 1]) ++lg;
