@@ -147,3 +147,11 @@ def test_varlen_qk_plan_on_host(lib):
         assert wq == sorted(wq, reverse=True) and wk == sorted(wk, reverse=True)
     short = (ctypes.c_int * 2)(0, 0)
     assert lib.gproj_attn_varlen_qk_plan_bytes(aq, short, 1) == 0        # no keys at all
+
+
+def test_forms_are_numbered_as_the_header_says():
+    defines = dict(re.findall(r"#define GPROJ_(FORM_\w+|FWD_KERNEL_\w+) (\d+)", open(os.path.join(ROOT, "include", "gproj_attn.h")).read()))
+    forms = {k: int(v) for k, v in defines.items() if k.startswith("FORM_")}
+    assert forms and all(getattr(binding, k) == v for k, v in forms.items()) and sorted(forms.values()) == list(range(len(forms)))
+    kernels = {int(v): k[len("FWD_KERNEL_"):].lower().replace("_rings", ", rings").replace("_", " ") for k, v in defines.items() if k.startswith("FWD_KERNEL_")}
+    assert binding.FWD_KERNELS == (None, *(kernels[i] for i in sorted(kernels))) and sorted(kernels) == list(range(1, len(kernels) + 1))
