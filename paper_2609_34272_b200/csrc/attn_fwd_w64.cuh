@@ -323,8 +323,8 @@ attn_fwd_w64_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 
       __syncwarp();
       if (lane == 0) mbar_arrive(&bar_merge[par]);
       // The last tile's buffer is handed back only here: waiting for its store right away kept this item's merge waiting for this warp.
-      // Measured, with the stores by warps: 96 heads x 1000: 29.7 -> 29.1 us, 300 x 200: 17.4 -> 16.9, 64 x 2000, not causal: 95.5 -> 93.1, 24
-      // documents, 20585 rows, 16 / 4 heads: 125.8 -> 122.7; 16 x 4096 (four long items per CTA): 51.9 -> 52.2.
+      // Measured, a store of the whole tile waited for at once -> stores by warps, handed back here: 96 heads x 1000: 29.9 -> 28.8 us, 1000 x
+      // 64: 15.2 -> 14.3, 16 x 4096: 51.6 -> 51.1, 32 x 4096, not causal: 175.9 -> 172.6; 100 x 128 behind 1000 (one item per CTA): 11.1 -> 11.3.
       if (stored >= 0) {
         bulk_wait_group_read0();
         mbar_arrive(&bar_q_free[stored]);
@@ -377,9 +377,9 @@ attn_fwd_w64_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 
         const int qrow0 = it.seq0 + it.qt * C::kBlockM;
         if (qrow < it.len) LSE[static_cast<size_t>(bh) * N + qrow0 + row] = (L > 0.f) ? fmaf(M, alpha, logf(L)) : INFINITY;
         const TileInfo tinfo{qrow0, it.seq0, it.seq0 + it.len, 0, 0, 0};
+        fence_proxy_async_smem();
+        warp_bar_sync(warp);                                       // see there: more than __syncwarp
         if (tile_store_by_tma(tinfo, N)) {                         // by each warp for itself: see attn_fwd.cuh
-          fence_proxy_async_smem();
-          __syncwarp();
           if (lane == 0) {
             if (qrow < it.len) tma_store_3d(&tmO, stage + row * 128, 0, qrow0 + row, bh);
             bulk_commit_group();
@@ -388,7 +388,7 @@ attn_fwd_w64_kernel(const __grid_constant__ CUtensorMap tmQ,    // box 64 x 128 
         } else {
           // ragged last tile of a packed sequence that another sequence follows: rows past its end are not ours to write
           store_rows_clipped<C::D>(stage, C::kQBytes, Og + (static_cast<size_t>(bh) * N + qrow0) * C::D, row, it.len - it.qt * C::kBlockM);
-          __syncwarp();
+          warp_bar_sync(warp);
           if (lane == 0) mbar_arrive(&bar_q_free[qb]);
         }
       }

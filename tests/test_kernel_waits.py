@@ -72,5 +72,5 @@ def test_softmax_warps_that_disagree_about_an_item_neither_hang_nor_leave_the_te
         assert re.search(r"for \(auto &slot : s_item\) slot\[0\] = slot\[1\] = 0;", setup), name
         role = body[body.index("setmaxnreg_inc"):]
         barriers = re.findall(r"named_bar_sync\([^;]*;|__syncthreads\(\);", role)
-        # behind the item loop, and in the cluster form, whose single item every warp reaches the barrier of
+        # behind the item loop, and in the cluster form, whose single item every warp reaches the barrier of (warp_bar_sync is one warp's own)
         assert barriers == (["named_bar_sync(3, 256);", "__syncthreads();", "__syncthreads();"] if name == "attn_fwd.cuh" else ["__syncthreads();"]), (name, barriers)
